@@ -508,8 +508,8 @@ def _gmres(A, b, tol=1e-11, steps=300):
 def exact(case, seed):
     d = _inputs(case, seed)
     n, tau = d["n"], -1.0 if case["surface"] == "duct" else 1.0
-    if n > 160000:
-        return None
+    if n > 45000:
+        return None          # the dense rows take minutes
     t = lambda v, f=torch.complex128: torch.as_tensor(v, device=_DEV).to(f)  # noqa: E731
     one, zero = torch.ones(n, dtype=torch.complex128, device=_DEV), torch.zeros(n, dtype=torch.complex128, device=_DEV)
     if case["kind"] == "product":
