@@ -420,7 +420,7 @@ def residual_vs_fp64(W, p, args, nrows=48):
 #       python bench.py --steps 1 --warmup 3 --no-cpu-baseline --leaf-edge 0.0126
 # Valid only while the kernel's source and launch and the plan (near_nnz)
 # are the ones captured (the source hash below guards it).
-SPMV_TRAFFIC = {"source_sha256": "db2463538395424353b36850b2d41a4b78dc3f4392a9654b16dd22976cd5a783",
+SPMV_TRAFFIC = {"source_sha256": "072a1b81091cecf996027de780a3b1aa872908dd1618af338cd09a6791df839c",
                 "near_nnz": 35925668, "bytes": 291443712}
 
 

@@ -279,6 +279,8 @@ struct Lists {
     DevArr<int64_t> row_ptr;
     DevArr<int4> spmv_items;      // (leaf, first row, end row) work items of the product
     int n_spmv_items = 0;
+    DevArr<int4> fused_tasks;     // (leaf, first row, end row) of the recomputed product (internal rows)
+    int n_fused = 0, fused_s = 1; // ... and the parts of the columns
     int64_t nnz = 0;
     std::vector<std::unique_ptr<ListsLevelDev>> lev;
     // all levels together, for the one-launch far-field kernels
@@ -385,6 +387,7 @@ struct Frame {
     DevArr<float2> cp, cq, cp0, cq0, z, aq;    // column coefficients, known data (internal order)
     DevArr<int> err;                           // first element whose subdivision failed
     DevArr<float2> vtmp, vout;                 // scratch of the fused validation pass
+    DevArr<float2> fpart;                      // column parts of a recomputed product (stays with the stream)
     cudaStream_t s = nullptr;                  // stream of this frame's setup work
     bool known_nonzero = false;
 };
@@ -618,6 +621,17 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         }
         Ls->n_spmv_items = (int)items.size();
         Ls->spmv_items.upload(items, s);
+        std::vector<int4> ft;
+        for (int t = 0; t < nl; ++t) {
+            const int64_t a = leaf_start[t], cnt = Lf.count[t];
+            const int64_t nch = (cnt + kFusedRows - 1) / kFusedRows;
+            for (int64_t q = 0; q < nch; ++q)
+                ft.push_back(make_int4(t, (int)(a + cnt * q / nch), (int)(a + cnt * (q + 1) / nch), 0));
+        }
+        Ls->n_fused = (int)ft.size();
+        Ls->fused_s = fused_parts(Ls->n_fused, Ls->max_ncol);
+        Ls->fused_tasks.upload(ft, s);
+        ck(cudaStreamSynchronize(s), "sync");   // items and ft are uploaded before they go
     }
     std::vector<AggTask> all_tasks;
     std::vector<int2> all_reds, all_targets;
@@ -1157,6 +1171,48 @@ void store_near(bem_mesh_impl &M, Plan &P, const float2 *cp, const float2 *cq)
     check_err(M);
 }
 
+// Room for the column parts of a recomputed product with nr right-hand sides
+// (also before a graph capture, which may not allocate).
+void ensure_fused(bem_mesh_impl &M, int nr)
+{
+    const Lists &Ls = *fr(M).plan->lists;
+    if (Ls.fused_s > 1) fr(M).fpart.alloc((size_t)Ls.fused_s * std::min(nr, kMaxPlanes) * M.n);
+}
+
+// y = the recomputed near-field product of nr planes of x (transposed when
+// kt: one plane), on stream s of the calling thread's frame.
+void near_fused(bem_mesh_impl &M, const Plan &P, const NearArgs &a, const float2 *x, float2 *y, int nr, const int *skip,
+                cudaStream_t s, bool kt = false)
+{
+    const Lists &Ls = *P.lists;
+    if (Ls.n_fused == 0) return;
+    ensure_fused(M, nr);
+    int *err = fr(M).err.p;
+    const dim3 grid(Ls.n_fused, Ls.fused_s);
+    const char *name = kt ? "k_near_fused_t" : "k_near_fused";
+    for (int r = 0; r < nr;) {
+        const int g = nr - r >= 4 ? 4 : (nr - r >= 2 ? 2 : 1);
+        const float2 *xr = x + (int64_t)r * M.n;
+        float2 *yr = y + (int64_t)r * M.n, *o = Ls.fused_s > 1 ? fr(M).fpart.p : yr;
+        {
+            KTimer kt_(name, s);
+            if (kt) k_near_fused_t<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
+            else if (g == 4) k_near_fused_4<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
+            else if (g == 2) k_near_fused_2<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
+            else k_near_fused_1<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
+        }
+        ck_launch(name);
+        if (Ls.fused_s > 1) {
+            {
+                KTimer kt_("k_near_fused_sum", s);
+                k_near_fused_sum<<<nblocks((int64_t)g * M.n, 256), 256, 0, s>>>(o, Ls.fused_s, (int64_t)g * M.n, yr, skip);
+            }
+            ck_launch("k_near_fused_sum");
+        }
+        r += g;
+    }
+}
+
 // Make sure the stored near-field values match the current unknowns' coefficients.
 void ensure_near_values(bem_mesh_impl &M, const Coeffs &C)
 {
@@ -1176,11 +1232,7 @@ void ensure_near_values(bem_mesh_impl &M, const Coeffs &C)
             F.vout.alloc(M.n);
             ck(cudaMemsetAsync(F.vtmp.p, 0, M.n * sizeof(float2), F.s), "memset");
             NearArgs a = near_args(M, P, F.cp.p, F.cq.p);
-            {
-                KTimer kt_("k_near_fused", F.s);
-                k_near_fused<<<nblocks(M.n, 8), 256, 0, F.s>>>(a, F.vtmp.p, F.vout.p, F.err.p, nullptr);
-            }
-            ck_launch("k_near_fused");
+            near_fused(M, P, a, F.vtmp.p, F.vout.p, 1, nullptr, F.s);
             check_err(M);
             P.val_valid = true;
         }
@@ -1323,33 +1375,6 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
                 na, P.lists->spmv_items.p, P.val.p, M.xint.p, M.ynear.p, nr, n, cw, skip);
         }
         ck_launch("k_near_spmv");
-    } else if (nr > 1) {
-        // one right-hand side at a time (the values are streamed nr times)
-        for (int r = 0; r < nr; ++r) {
-            if (use_store && M.prm.near_store && !P.fp().direct &&
-                (size_t)P.lists->max_ncol * sizeof(float2) <= 160 * 1024) {
-                if (P.lists->n_spmv_items > 0) {
-                    KTimer kt_("k_near_spmv", s);
-                    k_near_spmv_items<<<P.lists->n_spmv_items, kSpmvThreads,
-                                        (size_t)P.lists->max_ncol * sizeof(float2), s>>>(
-                        na, P.lists->spmv_items.p, P.val.p, M.xint.p + r * n, M.ynear.p + r * n, skip);
-                }
-                ck_launch("k_near_spmv");
-            } else if (use_store && M.prm.near_store && !P.fp().direct) {
-                {
-                    KTimer kt_("k_near_spmv", s);
-                    k_near_spmv<<<nblocks(n, 8), 256, 0, s>>>(na, P.val.p, M.xint.p + r * n, M.ynear.p + r * n, skip);
-                }
-                ck_launch("k_near_spmv");
-            } else {
-                {
-                    KTimer kt_("k_near_fused", s);
-                    k_near_fused<<<nblocks(n, 8), 256, 0, s>>>(na, M.xint.p + r * n, M.ynear.p + r * n, fr(M).err.p,
-                                                                skip);
-                }
-                ck_launch("k_near_fused");
-            }
-        }
     } else if (use_store && M.prm.near_store && !P.fp().direct) {
         const size_t xs_bytes = (size_t)P.lists->max_ncol * sizeof(float2);
         if (xs_bytes <= 160 * 1024) {
@@ -1367,11 +1392,7 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
             ck_launch("k_near_spmv");
         }
     } else {
-        {
-            KTimer kt_("k_near_fused", s);
-            k_near_fused<<<nblocks(n, 8), 256, 0, s>>>(na, M.xint.p, M.ynear.p, fr(M).err.p, skip);
-        }
-        ck_launch("k_near_fused");
+        near_fused(M, P, na, M.xint.p, M.ynear.p, nr, skip, s);
     }
     DisaggArgs da;
     da.n = n;
@@ -1583,11 +1604,7 @@ void matvec_t_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, con
         ck_launch("k_near_spmv_t");
     } else {
         NearArgs na = near_args(M, P, cp, cq);
-        {
-            KTimer kt_("k_near_fused_t", s);
-            k_near_fused_t<<<nblocks(n, 8), 256, 0, s>>>(na, M.xint.p, M.ynear.p, nullptr, fr(M).err.p, skip);
-        }
-        ck_launch("k_near_fused_t");
+        near_fused(M, P, na, M.xint.p, M.ynear.p, 1, skip, s, true);
     }
     if (fork) {
         ck(cudaEventRecord(M.ev_join, sf), "record join");
@@ -2185,6 +2202,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     GmresResult R;
     if (transposed) M.rowf.alloc(n);   // before the Arnoldi steps are captured (no allocation in a capture)
     if (nr > 1) ensure_planes(M, nr);
+    ensure_fused(M, nr);
     // GMRES workspace, nr planes of each
     const int64_t vplane = (int64_t)(m + 1) * n, hplane = (int64_t)(m + 1) * m;
     M.V.alloc((size_t)nr * vplane);

@@ -77,6 +77,32 @@ __device__ __forceinline__ void sincos_turns(float t, float *s, float *c)
     __sincosf(r * 6.28318548f, s, c);
 }
 
+// sin and cos of 2 pi t to FP32 rounding, t in turns: the nearest quarter
+// turn removed exactly, then the Taylor series on [-pi/4, pi/4] (remainders
+// below 3e-8).  For the singular and near-singular entries, the largest of a
+// row: the SFU's cosine near phase 0 is off by about 2e-7 with one sign, which
+// showed as a bias of these entries.
+__device__ __forceinline__ void sincos_turns_nr(float t, float *s, float *c)
+{
+    const float m = __fadd_rn(4.0f * t, 12582912.f);        // 1.5 2^23 + quarters, |t| < 2^20
+    const int q = __float_as_int(m);                        // quarters in the low bits
+    const float x = 6.28318548f * fmaf(-0.25f, __fsub_rn(m, 12582912.f), t);
+    const float x2 = x * x;
+    const float sx = fmaf(x * x2, fmaf(x2, fmaf(x2, fmaf(x2, 2.75573192e-6f, -1.98412698e-4f), 8.33333333e-3f),
+                                       -1.66666667e-1f), x);
+    const float cx = fmaf(x2, fmaf(x2, fmaf(x2, fmaf(x2, 2.48015873e-5f, -1.38888889e-3f), 4.16666667e-2f), -0.5f), 1.0f);
+    const float a = (q & 1) ? cx : sx, b = (q & 1) ? sx : cx;
+    *s = __int_as_float(__float_as_int(a) ^ ((q & 2) << 30));
+    *c = __int_as_float(__float_as_int(b) ^ (((q + 1) & 2) << 30));
+}
+// 1 / sqrt(x) to FP32 rounding: one Newton step on the SFU's value (the
+// kernels near an element carry 1/r cubed).
+__device__ __forceinline__ float rsqrt_nr(float x)
+{
+    const float y = rsqrtf(x);
+    return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
+}
+
 // ------------------------------------------------------------------ kernels
 // Burton-Miller column kernels at one quadrature point (Eq. SystemI, tau = 1,
 // gamma = i/k), with d = y - x, weight w:
@@ -87,14 +113,16 @@ __device__ __forceinline__ void sincos_turns(float t, float *s, float *c)
 // With ir = 1/r, rx = d.nx/r, ry = d.ny/r, nn = nx.ny this is
 //   Kp = G [ ir (ry - 3 rx ry + nn) + i ( -k ry + (k - 3 ir^2/k) rx ry + (ir^2/k) nn ) ]
 //   Kq = G [ 1 - rx - i (ir/k) rx ].
+template <bool kNr = false>
 __device__ __forceinline__ void bm_point(float3 d, float3 nx, float3 ny, float k, float ik_inv, float w,
                                          float2 &Kp, float2 &Kq)
 {
     float r2 = dot3f(d, d);
-    float ir = rsqrtf(r2);
+    float ir = kNr ? rsqrt_nr(r2) : rsqrtf(r2);
     float r = r2 * ir;
     float s, c;
-    sincos_turns(k * r * 0.15915494309189535f, &s, &c);
+    if (kNr) sincos_turns_nr(k * r * 0.15915494309189535f, &s, &c);
+    else sincos_turns(k * r * 0.15915494309189535f, &s, &c);
     float g = w * ir * kInv4Pi;
     float2 G = make_float2(c * g, s * g);
     float rx = dot3f(d, nx) * ir, ry = dot3f(d, ny) * ir, nn = dot3f(nx, ny);
@@ -207,6 +235,37 @@ struct SubTri {
     int depth;
 };
 
+// Rule code of the part s of element j with centroid dc = y - x and area sa:
+// 0 = subdivide; FP64 (same formula, exact coordinates) near a threshold.
+__device__ __forceinline__ int sub_rule(const ElemDev &E, int64_t j, float3 dc, float sa, const SubTri &s,
+                                        const double *xd, const QuadTables &Q)
+{
+    const float rt = sqrtf(dot3f(dc, dc) / sa);
+    if (!rt_ambiguous(rt, Q)) return rule_from_rt(rt, Q);
+    double d[3];
+    const double cxd = ((double)s.x0 + (double)s.x1 + (double)s.x2) / 3.0;
+    const double cyd = ((double)s.y0 + (double)s.y1 + (double)s.y2) / 3.0;
+    for (int q = 0; q < 3; ++q)
+        d[q] = (xd[q] - E.cd[3 * j + q]) - (E.vad[3 * j + q] + cxd * E.e1d[3 * j + q] + cyd * E.e2d[3 * j + q]);
+    const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    return rule_from_rt_d(dist / sqrt(E.ad[j] * exp2(-2.0 * s.depth)), Q);
+}
+
+// Rule code of the whole element j seen from x (D0 = x_j - x): the same
+// decision as the first step of the subdivision (the unit triangle's centroid
+// is x_j).
+__device__ __forceinline__ int whole_rule(const ElemDev &E, int64_t j, float3 D0, float area, const double *xd,
+                                          const QuadTables &Q)
+{
+    const float rt = sqrtf(dot3f(D0, D0) / area);
+    if (!rt_ambiguous(rt, Q)) return rule_from_rt(rt, Q);
+    double d[3];
+    for (int q = 0; q < 3; ++q)
+        d[q] = (xd[q] - E.cd[3 * j + q]) -
+               (E.vad[3 * j + q] + (1.0 / 3.0) * E.e1d[3 * j + q] + (1.0 / 3.0) * E.e2d[3 * j + q]);
+    return rule_from_rt_d(sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) / sqrt(E.ad[j]), Q);
+}
+
 // Integrate kernels over element j from point x (high/low parts xhi, xlo;
 // FP64 copy xd), with the subdivision of Sec. 3.1.3 and the regular rule of
 // Sec. 3.1.4: acc.point(d, ny, w) adds the kernels at each quadrature point
@@ -233,20 +292,9 @@ __device__ bool integrate_regular_acc(const ElemDev &E, int64_t j, float3 xhi, f
         }
     }
     // Whole element under one regular rule (no subdivision): the common
-    // case, handled without the subdivision stack.  Same decision as the
-    // first step of the loop below (the unit triangle's centroid is x_j).
+    // case, handled without the subdivision stack.
     {
-        const float rt = sqrtf(dot3f(D0, D0) / area);
-        int code;
-        if (!rt_ambiguous(rt, Q)) {
-            code = rule_from_rt(rt, Q);
-        } else {
-            double d[3];
-            for (int q = 0; q < 3; ++q)
-                d[q] = (xd[q] - E.cd[3 * j + q]) -
-                       (E.vad[3 * j + q] + (1.0 / 3.0) * E.e1d[3 * j + q] + (1.0 / 3.0) * E.e2d[3 * j + q]);
-            code = rule_from_rt_d(sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) / sqrt(E.ad[j]), Q);
-        }
+        const int code = whole_rule(E, j, D0, area, xd, Q);
         if (code > 0) {
             const int nq = code * code;
             for (int q = 0; q < nq; ++q) {
@@ -266,21 +314,7 @@ __device__ bool integrate_regular_acc(const ElemDev &E, int64_t j, float3 xhi, f
         const float cx = (s.x0 + s.x1 + s.x2) * (1.0f / 3.0f), cy = (s.y0 + s.y1 + s.y2) * (1.0f / 3.0f);
         const float3 dc = mad3(cy, e2, mad3(cx, e1, base));              // centroid - x
         const float sa = area * exp2f(-2.0f * (float)s.depth);           // area / 4^depth
-        const float rt = sqrtf(dot3f(dc, dc) / sa);
-        int code;
-        if (!rt_ambiguous(rt, Q)) {
-            code = rule_from_rt(rt, Q);
-        } else {
-            // FP64 decision (same formula as in FP32, exact coordinates)
-            double d[3];
-            const double cxd = ((double)s.x0 + (double)s.x1 + (double)s.x2) / 3.0;
-            const double cyd = ((double)s.y0 + (double)s.y1 + (double)s.y2) / 3.0;
-            for (int q = 0; q < 3; ++q)
-                d[q] = (xd[q] - E.cd[3 * j + q]) - (E.vad[3 * j + q] + cxd * E.e1d[3 * j + q] + cyd * E.e2d[3 * j + q]);
-            const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-            const double rtd = dist / sqrt(E.ad[j] * exp2(-2.0 * s.depth));
-            code = rule_from_rt_d(rtd, Q);
-        }
+        const int code = sub_rule(E, j, dc, sa, s, xd, Q);
         if (code == 0) {
             if (s.depth >= Q.max_depth) { ok = false; break; }
             const float mx01 = 0.5f * (s.x0 + s.x1), my01 = 0.5f * (s.y0 + s.y1);
@@ -410,6 +444,80 @@ __device__ __forceinline__ void self_term(const ElemDev &E, int64_t j, float k, 
     }
     Gii = G;
     Eii = make_float2(Ee.x + k * k * G.x, Ee.y + k * k * G.y);
+}
+
+// The self term shared by the lanes of a warp: the points of self_term
+// numbered, Duffy points 0 .. 95 adding to G and edge points 0 .. 9
+// edge_parts - 1 to Ee, each to FP32 rounding (the recomputed product).
+constexpr int kDuffyPoints = 6 * 16;
+__device__ __forceinline__ void duffy_point(float3 va, float3 e1, float3 e2, float k, const QuadTables &Q, int q,
+                                            float2 &G)
+{
+    const int e = q >> 4, a = (q >> 2) & 3, b = q & 3;
+    // the ring a, m_ab, b, m_bc, c, m_ca as a - x + xi e1 + eta e2
+    auto ring = [&](int i) {
+        const float xi = i == 0 || i == 4 || i == 5 ? 0.f : (i == 2 ? 1.f : 0.5f);
+        const float et = i < 3 ? 0.f : (i == 4 ? 1.f : 0.5f);
+        return mad3(et, e2, mad3(xi, e1, va));
+    };
+    const float3 p1 = ring(e), dp = sub3f(ring(e == 5 ? 0 : e + 1), p1);
+    const float3 cr = make_float3(p1.y * dp.z - p1.z * dp.y, p1.z * dp.x - p1.x * dp.z, p1.x * dp.y - p1.y * dp.x);
+    const float twoA = sqrtf(dot3f(cr, cr));
+    const float u = Q.gl4_x[a], v = Q.gl4_x[b];
+    const float3 d = make_float3(u * (p1.x + v * dp.x), u * (p1.y + v * dp.y), u * (p1.z + v * dp.z));
+    const float r2 = dot3f(d, d);
+    const float ir = rsqrt_nr(r2);
+    float s, c;
+    sincosf(k * r2 * ir, &s, &c);
+    const float g = Q.gl4_w[a] * Q.gl4_w[b] * twoA * u * ir * kInv4Pi;
+    G.x = fmaf(c, g, G.x);
+    G.y = fmaf(s, g, G.y);
+}
+// hypersingular edge part: sum over edges (a->b, b->c, c->a) of
+// integral of dG/dr (d.m)/r ds, m = t x n the outward edge normal
+__device__ __forceinline__ void edge_point(float3 va, float3 e1, float3 e2, float3 n, float k, const QuadTables &Q,
+                                           int q, float2 &Ee)
+{
+    const int parts = Q.edge_parts, e = q / (3 * parts), sp = (q / 3) % parts, g3 = q % 3;
+    const float3 p = e == 0 ? va : (e == 1 ? add3(va, e1) : add3(va, e2));
+    const float3 p2 = e == 0 ? add3(va, e1) : (e == 1 ? add3(va, e2) : va);
+    const float3 pq = sub3f(p2, p);
+    const float len = sqrtf(dot3f(pq, pq));
+    const float3 t = make_float3(pq.x / len, pq.y / len, pq.z / len);
+    const float3 m = make_float3(t.y * n.z - t.z * n.y, t.z * n.x - t.x * n.z, t.x * n.y - t.y * n.x);
+    const float hm = dot3f(p, m);            // (y - x).m, constant on the edge
+    const float sg = ((float)sp + Q.gl3_x[g3]) / (float)parts;
+    const float wg = Q.gl3_w[g3] * len / (float)parts;
+    const float3 d = mad3(sg, pq, p);
+    const float r2 = dot3f(d, d);
+    const float ir = rsqrt_nr(r2);
+    float s, c;
+    sincosf(k * r2 * ir, &s, &c);
+    const float g = wg * ir * kInv4Pi * hm * ir;   // G (d.m)/r without the (ik - 1/r) factor
+    const float2 Gp = make_float2(c * g, s * g);
+    Ee = cfma(Gp, make_float2(-ir, k), Ee);
+}
+// Points lane, lane + 32, ... of the self term of element j (the caller adds
+// the lanes).
+__device__ __forceinline__ void self_points(const ElemDev &E, int64_t j, float k, const QuadTables &Q, int lane,
+                                            float2 &G, float2 &Ee)
+{
+    const float3 va = f3(E.va[j]), e1 = f3(E.e1[j]), e2 = f3(E.e2[j]), n = f3(E.nrm[j]);
+    G = Ee = make_float2(0.f, 0.f);
+    for (int q = lane; q < kDuffyPoints; q += 32) duffy_point(va, e1, e2, k, Q, q, G);
+    for (int q = lane; q < 9 * Q.edge_parts; q += 32) edge_point(va, e1, e2, n, k, Q, q, Ee);
+}
+// A_ii from the self term's sums: gamma E_ii cp + G_ii cq (Kp = gamma E, Kq =
+// G; H and H' vanish) and the identity half tau (cp - gamma cq) / 2 of the
+// coefficients without tau; E = Ee + k^2 G, gamma = i/k.
+__device__ __forceinline__ float2 self_entry(float2 Gii, float2 Ee, float k, float ik_inv, float tau, float2 cp,
+                                             float2 cq)
+{
+    const float2 Eii = make_float2(Ee.x + k * k * Gii.x, Ee.y + k * k * Gii.y);
+    const float2 gE = make_float2(-Eii.y * ik_inv, Eii.x * ik_inv);
+    const float2 v = cadd(cmul(cp, gE), cmul(cq, Gii));
+    const float2 gcq = make_float2(-cq.y * ik_inv, cq.x * ik_inv);
+    return cadd(v, cscale(csub(cp, gcq), 0.5f * tau));
 }
 
 // Entry A_ij of the Burton-Miller matrix for columns with coefficients

@@ -73,11 +73,11 @@ __global__ void k_near_classify(NearArgs a, int2 *__restrict__ heavy, unsigned l
 // with every value in registers.
 constexpr int kLightRows = 64;
 // the general rule out of line, so that the common path keeps few registers
-__device__ __noinline__ bool general_entry(const ElemDev &E, int64_t i, int64_t j, float3 xhi, float3 xlo,
-                                           const double *xd, float3 nx, float k, float ik_inv, float tau,
-                                           const QuadTables &Q, float2 cpj, float2 cqj, float2 *out)
+__device__ __noinline__ bool general_entry(const NearArgs &a, int64_t i, int64_t j, float2 *out)
 {
-    return bm_entry(E, i, j, xhi, xlo, xd, nx, k, ik_inv, tau, Q, cpj, cqj, *out);
+    const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
+    return bm_entry(a.E, i, j, f3(a.E.chi[i]), f3(a.E.clo[i]), xd, f3(a.E.nrm[i]), a.k, a.ik_inv, a.tau, *a.Q, a.cp[j],
+                    a.cq[j], *out);
 }
 // Entry A_ij of order 2 or 3 over the whole element j (no subdivision).
 __device__ __forceinline__ float2 order23_entry(const ElemDev &E, int j, float3 D0, float3 nx, float k, float ik_inv,
@@ -198,10 +198,8 @@ __global__ void __launch_bounds__(256, 4) k_near_store_light(NearArgs a, float2 
             } else if (code == 0) {
                 // subdivision or a high order (only when the heavy split is
                 // off, m_max <= 3): the general rule
-                const double xd[3] = {s_xd[q][0], s_xd[q][1], s_xd[q][2]};
                 float2 v;
-                if (!general_entry(a.E, i, j, f3(s_hi[q]), f3(s_lo[q]), xd, f3(s_n[q]), a.k, a.ik_inv, a.tau, Q, cpj,
-                                   cqj, &v)) {
+                if (!general_entry(a, i, j, &v)) {
                     atomicMin(err, j);
                     v = make_float2(0.f, 0.f);
                 }
@@ -609,36 +607,481 @@ __global__ void __launch_bounds__(kSpmvThreads) k_near_spmv_items_multi(NearArgs
     }
 }
 
-// Near-field product with the entries recomputed on the fly (no storage);
-// also the conventional dense BEM product when the near list is everything.
-__global__ void k_near_fused(NearArgs a, const float2 *__restrict__ x, float2 *__restrict__ y,
-                             int *__restrict__ err, const int *skip)
+// ------------------------------------------------------------------ recomputed near field
+// Kp and / or Kq of bm_point at one quadrature point (needp, needq uniform
+// over the warp: a sound-hard problem has no q-columns, the admittance
+// derivative's operator no p-columns).
+__device__ __forceinline__ void bm_point_sel(float3 d, float3 nx, float3 ny, float k, float ik_inv, float w, bool needp,
+                                             bool needq, float2 &Kp, float2 &Kq)
 {
-    if (skip_now(skip)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= a.E.n) return;
+    const float r2 = dot3f(d, d);
+    const float ir = rsqrtf(r2);
+    const float r = r2 * ir;
+    float s, c;
+    sincos_turns(k * r * 0.15915494309189535f, &s, &c);
+    const float g = w * ir * kInv4Pi;
+    const float2 G = make_float2(c * g, s * g);
+    const float rx = dot3f(d, nx) * ir;
+    if (needp) {
+        const float ry = dot3f(d, ny) * ir, nn = dot3f(nx, ny);
+        const float ir2k = ir * ir * ik_inv;
+        const float rxry = rx * ry;
+        const float2 P = make_float2(ir * (ry - 3.0f * rxry + nn), -k * ry + (k - 3.0f * ir2k) * rxry + ir2k * nn);
+        Kp = cfma(G, P, Kp);
+    }
+    if (needq) Kq = cfma(G, make_float2(1.0f - rx, -(ir * ik_inv) * rx), Kq);
+}
+
+// A part of a subdivided element, packed: the order in bits 24..26, the depth
+// in 20..23 and the children taken from the whole element down, two bits
+// each, in 0..19 (the first in bits 0, 1).
+constexpr int kPartDepth = 10;
+__device__ __forceinline__ SubTri part_triangle(unsigned code, int depth)
+{
+    SubTri s{0.f, 0.f, 1.f, 0.f, 0.f, 1.f, depth};
+    for (int d = 0; d < depth; ++d) {
+        const float mx01 = 0.5f * (s.x0 + s.x1), my01 = 0.5f * (s.y0 + s.y1);
+        const float mx12 = 0.5f * (s.x1 + s.x2), my12 = 0.5f * (s.y1 + s.y2);
+        const float mx20 = 0.5f * (s.x2 + s.x0), my20 = 0.5f * (s.y2 + s.y0);
+        switch ((code >> (2 * d)) & 3) {
+            case 0: s = SubTri{s.x0, s.y0, mx01, my01, mx20, my20, depth}; break;
+            case 1: s = SubTri{mx01, my01, s.x1, s.y1, mx12, my12, depth}; break;
+            case 2: s = SubTri{mx20, my20, mx12, my12, s.x2, s.y2, depth}; break;
+            default: s = SubTri{mx01, my01, mx12, my12, mx20, my20, depth}; break;
+        }
+    }
+    return s;
+}
+// The parts under one rule of element j seen from midpoint i (Sec. 3.1.3's
+// subdivision, the decisions of integrate_subdivided), without integrating:
+// their number, and their codes (with `row` set in the upper bits) when out
+// is given.  0 when the element is subdivided deeper than a code can say
+// (the caller then takes the general rule, which also reports the limit).
+__device__ __noinline__ int cut_pair(const NearArgs &a, int64_t i, int64_t j, unsigned *out, unsigned row)
+{
     const QuadTables &Q = *a.Q;
-    const float4 ch = a.E.chi[i], cl = a.E.clo[i];
-    const float3 xhi = f3(ch), xlo = f3(cl), nx = f3(a.E.nrm[i]);
+    const float4 ch = a.E.chi[j];
+    const float3 e1 = f3(a.E.e1[j]), e2 = f3(a.E.e2[j]);
+    const float3 D0 = add3(sub3f(f3(ch), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i])));
+    const float3 base = add3(D0, f3(a.E.va[j]));
     const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
-    const int t = a.N.leaf_of[i];
-    const int r_end = a.N.run_ptr[t + 1], nc = a.N.ncol[t];
-    int r = a.N.run_ptr[t];
-    float2 acc = make_float2(0.f, 0.f);
-    for (int p = lane; p < nc; p += 32) {
-        const int j = near_col(a.N, r_end, r, p);
-        const float2 cp = a.cp[j], cq = a.cq[j];
-        if (cp.x == 0.f && cp.y == 0.f && cq.x == 0.f && cq.y == 0.f) continue;
-        float2 v;
-        if (!bm_entry(a.E, i, j, xhi, xlo, xd, nx, a.k, a.ik_inv, a.tau, Q, cp, cq, v)) {
-            atomicMin(err, j);
+    int m = whole_rule(a.E, j, D0, ch.w, xd, Q);
+    if (m > 0) {
+        if (out) *out = row | (unsigned)m << 24;
+        return 1;
+    }
+    int n = 0, depth = 1;
+    unsigned path = 0;                     // the part at hand: child path[depth - 1] of its parent ...
+    if (Q.max_depth < 1) return 0;
+    for (;;) {
+        const SubTri s = part_triangle(path, depth);
+        const float cx = (s.x0 + s.x1 + s.x2) * (1.0f / 3.0f), cy = (s.y0 + s.y1 + s.y2) * (1.0f / 3.0f);
+        m = sub_rule(a.E, j, mad3(cy, e2, mad3(cx, e1, base)), ch.w * exp2f(-2.0f * (float)depth), s, xd, Q);
+        if (m == 0) {
+            if (depth >= kPartDepth || depth >= Q.max_depth) return 0;
+            ++depth;                       // down to its first child
             continue;
         }
-        acc = cfma(v, x[j], acc);
+        if (out) out[n] = row | (unsigned)m << 24 | (unsigned)depth << 20 | path;
+        ++n;
+        // the next sibling, or the next one of the nearest ancestor that has one
+        while (depth > 0 && ((path >> (2 * (depth - 1))) & 3u) == 3u) {
+            path &= ~(3u << (2 * (depth - 1)));
+            --depth;
+        }
+        if (depth == 0) return n;
+        path += 1u << (2 * (depth - 1));
     }
-    acc = warp_sum(acc);
-    if (lane == 0) y[i] = acc;
+}
+
+// Near-field product with the entries recomputed on the fly (no storage):
+// the conventional dense BEM product when the near list is everything, and
+// the known boundary data's product.  Bound by FP32 / SFU issue (one kernel
+// evaluation is about 55 instructions with three SFU operations), so the
+// layout keeps everything else out of the inner loop and the lanes together:
+//   - a lane holds one row (its midpoint and normal) in registers, the 32
+//     rows being neighbours in Morton order; the columns are staged in shared
+//     memory in tiles of kFusedTile and read as broadcasts, warp w taking
+//     columns [32 w, 32 w + 32) of a tile.  The rows of a warp see a column
+//     at nearly the same distance, so they mostly agree on its rule, and no
+//     sum crosses lanes until the end.  (Leaves of at most 16 rows put two
+//     or more columns side by side in a warp.)
+//   - orders 1 to 3 are evaluated in place; the expensive pairs (subdivided
+//     elements, orders 4 to 6, distances within rounding of a threshold) are
+//     queued per block and worked off after the tiles by all its threads:
+//     each pair is first cut into its parts under one rule (the subdivision
+//     without any integration), the parts are sorted by their order, and the
+//     lanes then take parts of one order, so that a warp's loops have one
+//     length.  (Pairs taken whole, one per thread, had lanes of a warp in
+//     different parts and orders: 7 times the instructions.)  The self terms
+//     take a warp each.  The sums of all these are FP64 additions in shared
+//     memory, so their order does not show.
+// A block takes the rows of one task and every gridDim.y-th part of the
+// tiles; with several parts, k_near_fused_sum adds them in order.  NR right-
+// hand sides share every entry.  One warp per row with lanes over the columns
+// (96 bytes of element data per pair through L1, all rules mixed in a warp)
+// took 721 us on 5120 elements; this takes 281 us (four blocks per SM; with
+// three 283, and 352 with half as many parts).
+// kT: the transposed product (the lists read backwards): a lane holds
+// column j, the rows i whose leaves are in the near list of j's own leaf are
+// staged, y_j = cp_j sum_i Kp_ij x_i + cq_j sum_i Kq_ij x_i.
+template <int NR, bool kT>
+__device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *__restrict__ tasks,
+                                                const float2 *__restrict__ x, float2 *__restrict__ out,
+                                                int *__restrict__ err)
+{
+    static_assert(!kT || NR == 1, "the transposed product has one right-hand side");
+    constexpr int kW = kFusedThreads / 32;
+    constexpr bool kFold = !kT && NR == 1;             // the column's x folded into its coefficients
+    static_assert(kFusedTile == kFusedThreads, "one staged element per thread");
+    // the staged tile (a transposed product stages rows: no vertices and
+    // coefficients), and afterwards the parts of the queued pairs
+    constexpr int kTileArrays = kT ? 3 : 7;
+    constexpr int kTileBytes = kTileArrays * kFusedTile * 16, kPartBytes = kFusedParts * 10;
+    __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
+    float4 *s_hi = reinterpret_cast<float4 *>(s_buf), *s_lo = s_hi + kFusedTile, *s_n = s_lo + kFusedTile;
+    float4 *s_va = kT ? s_hi : s_n + kFusedTile, *s_e1 = kT ? s_hi : s_va + kFusedTile;
+    float4 *s_e2 = kT ? s_hi : s_e1 + kFusedTile, *s_c = kT ? s_hi : s_e2 + kFusedTile;
+    int *s_pj = reinterpret_cast<int *>(s_buf);                        // part: staged element
+    unsigned *s_pc = reinterpret_cast<unsigned *>(s_pj + kFusedParts); // ... row, order, depth, path
+    unsigned short *s_po = reinterpret_cast<unsigned short *>(s_pc + kFusedParts);   // parts by order
+    __shared__ float2 s_x[NR][kFold ? 1 : kFusedTile];
+    __shared__ int s_j[kFusedTile];
+    __shared__ int s_qj[kFusedQueue];                  // expensive pairs: staged element and row
+    __shared__ unsigned char s_qr[kFusedQueue];
+    __shared__ int s_qn, s_pn[8];
+    __shared__ int s_self[kFusedRows];                 // the row's own element is in this block's part
+    __shared__ double2 s_h[NR][kFusedRows];
+    __shared__ float4 s_rule[91];                      // (xi, eta, 2 w) of orders 1 to 6, order m from rule_at(m)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const QuadTables &Q = *a.Q;
+    int t = 0;
+    int64_t e0, e1;
+    if (tasks) {
+        const int4 T = tasks[blockIdx.x];
+        t = T.x;
+        e0 = T.y;
+        e1 = T.z;
+    } else {                                           // one leaf holds every element
+        e0 = (int64_t)blockIdx.x * kFusedRows;
+        e1 = min(a.E.n, e0 + kFusedRows);
+    }
+    const int cnt = (int)(e1 - e0);
+    int w = 1;
+    while (w < cnt) w <<= 1;                           // cnt <= kFusedRows = 32
+    const int R = 32 / w, sub = lane / w, rr = lane % w;
+    const bool live = rr < cnt;
+    const int64_t e = e0 + (live ? rr : 0);
+    if (threadIdx.x == 0) s_qn = 0;
+    if (threadIdx.x < kFusedRows) s_self[threadIdx.x] = 0;
+    if (threadIdx.x < kFusedRows)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) s_h[r][threadIdx.x] = make_double2(0.0, 0.0);
+    // first point of order m: 0, 1, 5, 14, 30, 55
+    auto rule_at = [](int m) { return (m - 1) * m * (2 * m - 1) / 6; };
+    if (threadIdx.x < 91) {
+        int m = 1;
+        while (rule_at(m + 1) <= (int)threadIdx.x) ++m;
+        const int v = threadIdx.x - rule_at(m);
+        s_rule[threadIdx.x] = make_float4(Q.tri_xi[m][v], Q.tri_eta[m][v], 2.0f * Q.tri_w[m][v], 0.f);
+    }
+    // this lane's element
+    const float4 ehi = a.E.chi[e], elo = a.E.clo[e], en = a.E.nrm[e];
+    float3 eva = make_float3(0.f, 0.f, 0.f), ee1 = eva, ee2 = eva;
+    float2 ecp = make_float2(0.f, 0.f), ecq = ecp;
+    float einv = 0.f;
+    bool needp = true, needq = false;
+    if (kT) {
+        eva = f3(a.E.va[e]);
+        ee1 = f3(a.E.e1[e]);
+        ee2 = f3(a.E.e2[e]);
+        ecp = a.cp[e];
+        ecq = a.cq[e];
+        einv = __frcp_rn(ehi.w);
+        needp = __any_sync(0xffffffffu, ecp.x != 0.f || ecp.y != 0.f);
+        needq = __any_sync(0xffffffffu, ecq.x != 0.f || ecq.y != 0.f);
+    }
+    // thresholds on r~^2: order 1 clearly above R_1; orders 1 to 3 above
+    // heavy_rt2 and not within 2e-5 of R_1 or R_2 (m_max <= 3 has no such
+    // split: everything but order 1 goes to the general rule)
+    const bool split = Q.m_max > 3;
+    const float rt1 = Q.m_max > 1 ? Q.R2[1] * (1.0f + 2e-5f) : __int_as_float(0x7f800000);
+    const float rt1lo = Q.R2[1] * (1.0f - 2e-5f), rt2hi = Q.R2[2] * (1.0f + 2e-5f), rt2lo = Q.R2[2] * (1.0f - 2e-5f);
+    const float rth = Q.heavy_rt2;
+    const float k = a.k, ik_inv = a.ik_inv;
+    float2 acc[NR], accq = make_float2(0.f, 0.f);      // kT: acc[0] the p sum, accq the q sum
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r] = make_float2(0.f, 0.f);
+    // v times x of the pair (row, wj), added to the row's FP64 sums
+    auto add_pair = [&](int row, int wj, float2 v) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const float2 c = cmul(v, x[r * a.E.n + wj]);
+            atomicAdd(&s_h[r][row].x, (double)c.x);
+            atomicAdd(&s_h[r][row].y, (double)c.y);
+        }
+    };
+    // a pair or part that found no room in the queues: the general rule
+    auto general = [&](int row, int wj) {
+        const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
+        float2 v;
+        if (!general_entry(a, i, j, &v)) {
+            atomicMin(err, (int)j);
+            return;
+        }
+        add_pair(row, wj, v);
+    };
+    const int nc = a.N.ncol[t];
+    const int ntile = (nc + kFusedTile - 1) / kFusedTile;
+    const int run0 = a.N.run_ptr[t], run1 = a.N.run_ptr[t + 1];
+    // this block's part of the tiles: the parts that hold the rows' own
+    // columns, and with them the expensive pairs, are the first of the grid
+    // to start
+    int part = blockIdx.y;
+    if (gridDim.y > 1) {
+        int lo = run0, hi = run1 - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.N.runs[mid].x <= e0) lo = mid;
+            else hi = mid - 1;
+        }
+        const int64_t own = (a.N.runs[lo].y + (e0 - a.N.runs[lo].x)) / kFusedTile;
+        part = (int)((part + max((int64_t)0, min(own, (int64_t)ntile - 1)) * gridDim.y / ntile) % gridDim.y);
+    }
+    const int tb = (int)((int64_t)ntile * part / gridDim.y), te = (int)((int64_t)ntile * (part + 1) / gridDim.y);
+    for (int tile = tb; tile < te; ++tile) {
+        __syncthreads();
+        bool q_here = false;
+        {
+            const int p = tile * kFusedTile + threadIdx.x;
+            if (p < nc) {
+                int lo = run0, hi = run1 - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (a.N.runs[mid].y <= p) lo = mid;
+                    else hi = mid - 1;
+                }
+                const int2 rn = a.N.runs[lo];
+                const int j = rn.x + (p - rn.y);
+                const float4 h = a.E.chi[j];
+                float4 l = a.E.clo[j];
+                l.w = __frcp_rn(h.w);
+                s_hi[threadIdx.x] = h;
+                s_lo[threadIdx.x] = l;
+                s_n[threadIdx.x] = a.E.nrm[j];
+                s_j[threadIdx.x] = j;
+                if (!kT) {
+                    s_va[threadIdx.x] = a.E.va[j];
+                    s_e1[threadIdx.x] = a.E.e1[j];
+                    s_e2[threadIdx.x] = a.E.e2[j];
+                    float2 cp = a.cp[j], cq = a.cq[j];
+                    if (kFold) {
+                        const float2 xv = x[j];
+                        cp = cmul(cp, xv);
+                        cq = cmul(cq, xv);
+                    }
+                    s_c[threadIdx.x] = make_float4(cp.x, cp.y, cq.x, cq.y);
+                    q_here = cq.x != 0.f || cq.y != 0.f;
+                }
+                if (!kFold)
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) s_x[r][threadIdx.x] = x[r * a.E.n + j];
+            }
+        }
+        const bool q_tile = __syncthreads_or(q_here);
+        if (!kT) needq = q_tile;
+        const int c0 = warp * 32, c1 = min(c0 + 32, nc - tile * kFusedTile);
+        // the tile's own sum first: a long row's sum is then one of few terms
+        float2 ta[NR], tq = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) ta[r] = make_float2(0.f, 0.f);
+        for (int cb = c0; cb < c1; cb += R) {
+            const int c = cb + sub;
+            if (!live || c >= c1) continue;
+            const float4 whi = s_hi[c], wlo = s_lo[c];
+            float3 D0;                                  // x_j - x_i
+            const float rt2 = kT ? pair_rt2(f3(ehi), f3(elo), f3(whi), f3(wlo), einv, D0)
+                                 : pair_rt2(f3(whi), f3(wlo), f3(ehi), f3(elo), wlo.w, D0);
+            int code = 0;
+            if (rt2 > rt1) code = 1;
+            else if (split && rt2 > rth && rt2 < rt1lo && (rt2 > rt2hi || rt2 < rt2lo)) code = rt2 > rt2hi ? 2 : 3;
+            const float3 wn = f3(s_n[c]);
+            const float3 nx = kT ? wn : f3(en), ny = kT ? f3(en) : wn;
+            const float area = kT ? ehi.w : whi.w;
+            if (code == 0) {
+                if (s_j[c] == (int)e) {
+                    s_self[rr] = 1;
+                    continue;
+                }
+                const int slot = atomicAdd(&s_qn, 1);
+                if (slot < kFusedQueue) {
+                    s_qj[slot] = s_j[c];
+                    s_qr[slot] = (unsigned char)rr;
+                } else {
+                    general(rr, s_j[c]);
+                }
+                continue;
+            }
+            float2 Kp = make_float2(0.f, 0.f), Kq = Kp;
+            if (code == 1) {
+                // the 1 x 1 conical rule is the centroid rule
+                bm_point_sel(D0, nx, ny, k, ik_inv, area, needp, needq, Kp, Kq);
+            } else {
+                const float3 g1 = kT ? ee1 : f3(s_e1[c]), g2 = kT ? ee2 : f3(s_e2[c]);
+                const float3 base = add3(D0, kT ? eva : f3(s_va[c]));
+                const int u1 = code == 2 ? 5 : 14;
+                for (int u = code == 2 ? 1 : 5; u < u1; ++u) {
+                    const float4 rl = s_rule[u];
+                    bm_point_sel(mad3(rl.y, g2, mad3(rl.x, g1, base)), nx, ny, k, ik_inv, area * rl.z, needp, needq, Kp,
+                                 Kq);
+                }
+            }
+            if (kT) {
+                const float2 xv = s_x[0][c];
+                ta[0] = cfma(Kp, xv, ta[0]);
+                tq = cfma(Kq, xv, tq);
+            } else {
+                const float4 cc = s_c[c];
+                if (kFold) {
+                    ta[0] = cfma(Kp, make_float2(cc.x, cc.y), ta[0]);
+                    if (needq) ta[0] = cfma(Kq, make_float2(cc.z, cc.w), ta[0]);
+                } else {
+                    float2 v = cmul(make_float2(cc.x, cc.y), Kp);
+                    if (needq) v = cfma(make_float2(cc.z, cc.w), Kq, v);
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) ta[r] = cfma(v, s_x[r][c], ta[r]);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r] = cadd(acc[r], ta[r]);
+        accq = cadd(accq, tq);
+    }
+    if (kT) acc[0] = cadd(cmul(ecp, acc[0]), cmul(ecq, accq));
+    __syncthreads();
+    // the queued pairs, kFusedThreads at a time: cut into parts, the parts
+    // sorted by order, the parts integrated; then the self terms
+    {
+        const int nq = min(s_qn, kFusedQueue);
+        for (int q0 = 0; q0 < nq; q0 += kFusedThreads) {
+            __syncthreads();
+            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
+            __syncthreads();
+            if (q0 + (int)threadIdx.x < nq) {
+                const int row = s_qr[q0 + threadIdx.x], wj = s_qj[q0 + threadIdx.x];
+                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
+                // more parts than room for this pair: all of it by the general rule
+                const int np = cut_pair(a, i, j, nullptr, 0);
+                const int at = np > 0 ? atomicAdd(&s_pn[0], np) : 0;
+                if (np > 0 && at + np <= kFusedParts) {
+                    unsigned *pc = s_pc + at;
+                    cut_pair(a, i, j, pc, (unsigned)row << 27);
+                    for (int u = 0; u < np; ++u) {
+                        s_pj[at + u] = wj;
+                        atomicAdd(&s_pn[(pc[u] >> 24) & 7], 1);
+                    }
+                } else {
+                    if (np > 0)
+                        for (int u = at; u < min(at + np, kFusedParts); ++u) s_pc[u] = 0;   // order 0: no part
+                    general(row, wj);
+                }
+            }
+            __syncthreads();
+            const int n_all = min(s_pn[0], kFusedParts);
+            int start[8];                              // first slot of an order: the longest first
+            start[7] = 0;
+            start[6] = 0;
+#pragma unroll
+            for (int m = 5; m >= 1; --m) start[m] = start[m + 1] + s_pn[m + 1];
+            const int n_parts = start[1] + s_pn[1];
+            __syncthreads();
+            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
+            __syncthreads();
+            for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
+                const int m = (s_pc[u] >> 24) & 7;
+                if (m == 0) continue;
+                int at = start[1];
+#pragma unroll
+                for (int v = 2; v <= 6; ++v)
+                    if (m == v) at = start[v];
+                s_po[at + atomicAdd(&s_pn[m], 1)] = (unsigned short)u;
+            }
+            __syncthreads();
+            for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) {
+                const int pi = s_po[u], wj = s_pj[pi];
+                const unsigned pc = s_pc[pi];
+                const int row = pc >> 27, m = (pc >> 24) & 7, depth = (pc >> 20) & 15;
+                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
+                const SubTri T = part_triangle(pc, depth);
+                const float4 ch = a.E.chi[j];
+                const float3 g1 = f3(a.E.e1[j]), g2 = f3(a.E.e2[j]), ny = f3(a.E.nrm[j]), nx = f3(a.E.nrm[i]);
+                const float3 base = add3(add3(sub3f(f3(ch), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i]))),
+                                         f3(a.E.va[j]));
+                const float sa = ch.w * exp2f(-2.0f * (float)depth);
+                const float sx1 = T.x1 - T.x0, sy1 = T.y1 - T.y0, sx2 = T.x2 - T.x0, sy2 = T.y2 - T.y0;
+                float2 Kp = make_float2(0.f, 0.f), Kq = Kp;
+                const int r0 = rule_at(m), r1 = rule_at(m + 1);
+                for (int v = r0; v < r1; ++v) {
+                    const float4 rl = s_rule[v];
+                    const float px = T.x0 + rl.x * sx1 + rl.y * sx2, py = T.y0 + rl.x * sy1 + rl.y * sy2;
+                    bm_point<true>(mad3(py, g2, mad3(px, g1, base)), nx, ny, k, ik_inv, sa * rl.z, Kp, Kq);
+                }
+                add_pair(row, wj, cadd(cmul(a.cp[j], Kp), cmul(a.cq[j], Kq)));
+            }
+        }
+        for (int row = warp; row < cnt; row += kW) {
+            if (!s_self[row]) continue;
+            const int64_t j = e0 + row;
+            float2 G, Ee;
+            self_points(a.E, j, k, Q, lane, G, Ee);
+            G = warp_sum(G);
+            Ee = warp_sum(Ee);
+            if (lane == 0) add_pair(row, (int)j, self_entry(G, Ee, k, ik_inv, a.tau, a.cp[j], a.cq[j]));
+        }
+    }
+    // the lanes' sums of a row in (warp, side-by-side column) order
+    float2 *red = reinterpret_cast<float2 *>(s_buf);
+    float2 *dst = out + (int64_t)part * NR * a.E.n;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        __syncthreads();
+        red[threadIdx.x] = acc[r];
+        __syncthreads();
+        if (threadIdx.x < cnt) {
+            const double2 h = s_h[r][threadIdx.x];
+            float2 v = make_float2((float)h.x, (float)h.y);
+            for (int q = 0; q < kW; ++q)
+                for (int u = 0; u < R; ++u) v = cadd(v, red[q * 32 + u * w + threadIdx.x]);
+            dst[r * a.E.n + e0 + threadIdx.x] = v;
+        }
+    }
+}
+
+#define BEM_FUSED_KERNEL(NAME, NR, T)                                                                                \
+    __global__ void __launch_bounds__(kFusedThreads, 4)                                                             \
+        NAME(NearArgs a, const int4 *__restrict__ tasks, const float2 *__restrict__ x, float2 *__restrict__ out,    \
+             int *__restrict__ err, const int *skip)                                                                \
+    {                                                                                                                \
+        if (skip_now(skip)) return;                                                                                  \
+        near_fused_body<NR, T>(a, tasks, x, out, err);                                                               \
+    }
+BEM_FUSED_KERNEL(k_near_fused_1, 1, false)
+BEM_FUSED_KERNEL(k_near_fused_2, 2, false)
+BEM_FUSED_KERNEL(k_near_fused_4, 4, false)
+BEM_FUSED_KERNEL(k_near_fused_t, 1, true)
+#undef BEM_FUSED_KERNEL
+
+// y = the S column parts of a recomputed product (part[s][n] with n the rows
+// of every plane) in order.
+__global__ void k_near_fused_sum(const float2 *__restrict__ part, int S, int64_t n, float2 *__restrict__ y,
+                                 const int *skip)
+{
+    if (skip_now(skip)) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float2 v = part[i];
+    for (int s = 1; s < S; ++s) v = cadd(v, part[(int64_t)s * n + i]);
+    y[i] = v;
 }
 
 // Row scaling of Eq. SystemI (Sec. 3.2, the solver's row-scaling
@@ -818,48 +1261,6 @@ __global__ void __launch_bounds__(kBjMax) k_bj_apply(const int4 *__restrict__ bl
 }
 
 // ------------------------------------------------------------------ adjoint
-// Near part of the transposed product: y_j = sum_i A_ij x_i over the rows i
-// whose leaves are in the near list of j's own leaf (the lists read
-// backwards), with the entries recomputed by bm_entry (row i, column j; the
-// forward product's entries).  Where a pair's near/far verdict differs by
-// direction (the far test uses the source cluster's element areas), the
-// pair is taken here or in the far part, the other way than in A.  One warp
-// per column j, lanes over those rows.  zero (may be null): also cleared
-// at j.
-__global__ void k_near_fused_t(NearArgs a, const float2 *__restrict__ x, float2 *__restrict__ y,
-                               float2 *__restrict__ zero, int *__restrict__ err, const int *skip)
-{
-    if (skip_now(skip)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (j >= a.E.n) return;
-    const QuadTables &Q = *a.Q;
-    const float2 cp = a.cp[j], cq = a.cq[j];
-    float2 acc = make_float2(0.f, 0.f);
-    if (cp.x != 0.f || cp.y != 0.f || cq.x != 0.f || cq.y != 0.f) {
-        const int t = a.N.leaf_of[j];
-        const int r_end = a.N.run_ptr[t + 1], nc = a.N.ncol[t];
-        int r = a.N.run_ptr[t];
-        for (int p = lane; p < nc; p += 32) {
-            const int64_t i = near_col(a.N, r_end, r, p);
-            const float4 ch = a.E.chi[i], cl = a.E.clo[i];
-            const float3 xhi = f3(ch), xlo = f3(cl), nx = f3(a.E.nrm[i]);
-            const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
-            float2 v;
-            if (!bm_entry(a.E, i, j, xhi, xlo, xd, nx, a.k, a.ik_inv, a.tau, Q, cp, cq, v)) {
-                atomicMin(err, (int)j);
-                continue;
-            }
-            acc = cfma(v, x[i], acc);
-        }
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) {
-        y[j] = acc;
-        if (zero) zero[j] = make_float2(0.f, 0.f);
-    }
-}
-
 // Inputs of the transposed product's far field.  With the antipodal
 // symmetry of the sphere grid and D(-X, s) = D(X, -s) (Eq. FMMBase), the far
 // part of A^T x is the forward aggregation of the weights (alpha, c) =

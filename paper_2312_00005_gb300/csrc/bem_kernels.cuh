@@ -202,7 +202,32 @@ __global__ void k_near_transpose(const int64_t *leaf_start, const int *trow_ptr,
 constexpr int kSpmvMultiChunk = 512;
 __global__ void k_near_spmv_items_multi(NearArgs a, const int4 *items, const float2 *val, const float2 *x, float2 *y,
                                         int nr, int64_t plane, int cw, const int *skip);
-__global__ void k_near_fused(NearArgs a, const float2 *x, float2 *y, int *err, const int *skip);
+// Near-field product with recomputed entries for 1, 2 or 4 right-hand sides
+// (planes n apart in x and out) and its transpose: blocks of tasks (leaf,
+// first row, end row; at most kFusedRows rows; tasks null: one leaf holds
+// every element) times gridDim.y parts of the columns, each part into its own
+// [NR][n] plane of out; k_near_fused_sum adds the parts.
+constexpr int kFusedThreads = 256;
+constexpr int kFusedTile = 256;          // columns staged per pass
+constexpr int kFusedRows = 32;           // rows per block (the lanes of a warp)
+constexpr int kFusedQueue = 1024;        // expensive pairs queued per block
+constexpr int kFusedParts = 2560;        // ... and their parts under one rule, per kFusedThreads pairs
+__global__ void k_near_fused_1(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
+__global__ void k_near_fused_2(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
+__global__ void k_near_fused_4(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
+__global__ void k_near_fused_t(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
+__global__ void k_near_fused_sum(const float2 *part, int S, int64_t n, float2 *y, const int *skip);
+// Parts of the columns for ntasks row tasks of at most max_ncol columns:
+// blocks enough for several rounds of four per SM, and whole tiles in each part
+// (5120 elements: 20 parts of one tile 283 us, 10 of two 352 us).
+inline int fused_parts(int64_t ntasks, int64_t max_ncol)
+{
+    const int64_t ntile = (max_ncol + kFusedTile - 1) / kFusedTile;
+    const int64_t want = ntasks > 0 ? 3648 / ntasks : 1;
+    if (want <= 1 || ntile <= 1) return 1;
+    const int64_t per = (ntile + want - 1) / want;
+    return (int)((ntile + per - 1) / per);
+}
 __global__ void k_prep(PrepArgs a, const int *skip);
 // True when the product kernels of a finished GMRES cycle should skip.
 __device__ __forceinline__ bool skip_now(const int *skip) { return skip != nullptr && *(volatile const int *)skip != 0; }
@@ -348,7 +373,6 @@ __global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, 
 __global__ void k_field_eval_finish(const double *pts, int64_t M, float k, float tau, const SourceDev *src, int nsrc,
                                     const float2 *v, const int64_t *perm, float2 *out);
 
-__global__ void k_near_fused_t(NearArgs a, const float2 *x, float2 *y, float2 *zero, int *err, const int *skip);
 __global__ void k_prep_t(int64_t n, const float2 *x, float2 *xint, float4 *wts, float4 *rowf, const float4 *chi,
                          const float2 *cp, const float2 *cq, float k, const int *skip);
 __global__ void k_field_t(ElemDev E, const QuadTables *Qp, const double *pts, int64_t M, float k, const float2 *f,

@@ -60,7 +60,8 @@ size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // Scratch layout for n elements (each piece 256-byte aligned).
 struct Layout {
-    size_t chi, clo, nrm, va, e1, e2, cd, vad, e1d, e2d, ad, cp, cq, leaf_of, run_ptr, runs, ncol, Q, err, total;
+    size_t chi, clo, nrm, va, e1, e2, cd, vad, e1d, e2d, ad, cp, cq, leaf_of, run_ptr, runs, ncol, Q, err, part, total;
+    int parts;
     explicit Layout(int64_t n)
     {
         size_t o = 0;
@@ -71,6 +72,11 @@ struct Layout {
         cp = take(8 * n); cq = take(8 * n);
         leaf_of = take(4 * n); run_ptr = take(8); runs = take(8); ncol = take(4);
         Q = take(sizeof(QuadTables)); err = take(4);
+        // partial sums of the product's column parts, as many as the scratch
+        // array has room for (none: one part, written to y)
+        parts = fused_parts((n + kFusedRows - 1) / kFusedRows, n);
+        while (parts > 1 && o + align256(8 * (size_t)n * parts) > kScratchBytes) --parts;
+        part = parts > 1 ? take(8 * (size_t)n * parts) : o;
         total = o;
     }
 };
@@ -248,8 +254,12 @@ extern "C" int bem_matvec_direct_noalloc(const double *nodes_dev, int64_t n_node
     a.tau = 1.f;             // exterior problem
     a.cp = (const float2 *)(base + lay.cp);
     a.cq = (const float2 *)(base + lay.cq);
-    k_near_fused<<<(unsigned)((n_tris + 7) / 8), 256, 0, s>>>(a, (const float2 *)x_dev, (float2 *)y_dev,
-                                                               (int *)(base + lay.err), nullptr);
+    float2 *part = (float2 *)(base + lay.part);
+    k_near_fused_1<<<dim3((unsigned)((n_tris + kFusedRows - 1) / kFusedRows), (unsigned)lay.parts), kFusedThreads, 0, s>>>(
+        a, nullptr, (const float2 *)x_dev, lay.parts > 1 ? part : (float2 *)y_dev, (int *)(base + lay.err), nullptr);
+    if (lay.parts > 1)
+        k_near_fused_sum<<<(unsigned)((n_tris + 255) / 256), 256, 0, s>>>(part, lay.parts, n_tris, (float2 *)y_dev,
+                                                                          nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(BEM_E_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     int herr = INT_MAX;
