@@ -33,6 +33,9 @@ constexpr double kPhaseTableMaxBytes = 4.0 * 1024 * 1024 * 1024;
 constexpr double kFieldFmmMinPairs = 1e9;
 // Arnoldi steps captured in one CUDA graph (one status read per graph)
 constexpr int kStepsPerGraph = 4;
+// columns of the GMRES triangle that k_gm_backsolve stages (packed, with its
+// 32 KB of vectors within 227 KB)
+constexpr int kBacksolveCols = 155;
 // values per work item of the stored near-field product
 constexpr int64_t kSpmvItemEntries = 65536;
 
@@ -2054,7 +2057,8 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
                                 (int)(kMaxPlanes * 4096 * sizeof(float2))),
            "cudaFuncSetAttribute");
 
-        ck(cudaFuncSetAttribute(k_gm_backsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 100 * 16),
+        ck(cudaFuncSetAttribute(k_gm_backsolve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kBacksolveCols * (kBacksolveCols + 1) / 2 * (int)sizeof(double2)),
            "cudaFuncSetAttribute");
         if (p.far_precision == 1) {
             ck(cudaFuncSetAttribute(k_aggregate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes),
@@ -2248,7 +2252,10 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     ck(cudaMemsetAsync(M.uvec.p, 0, (size_t)nr * n * sizeof(float2), s), "memset x");
     ck(cudaMemsetAsync(M.H.p, 0, M.H.bytes(), s), "memset H");
     // per-plane pointers of the Gram-Schmidt and Givens kernels
-    std::vector<GsArgs> oa(nr);
+    GsPlanes planes;
+    memset(&planes, 0, sizeof planes);
+    planes.nr = nr;
+    GsArgs *oa = planes.p;
     for (int r = 0; r < nr; ++r) {
         GmresArgs &ga = oa[r].g;
         ga.V = M.V.p + r * vplane;
@@ -2285,19 +2292,16 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     };
     // r0 = b, V_0 = r0 / ||r0||, cycle state reset (every plane)
     auto start = [&](const float2 *r0, int first) {
-        for (int r = 0; r < nr; ++r) {
-            {
-                KTimer kt_("k_norm_part", s);
-                k_norm_part<<<nnorm, 256, 0, s>>>(r0 + r * n, n, oa[r].g.normpart);
-            }
-            ck_launch("k_norm_part");
-            {
-                KTimer kt_("k_gm_start", s);
-                k_gm_start<<<nblocks(n, 256), 256, 0, s>>>(oa[r].g.st, oa[r].g.V, r0 + r * n, n, oa[r].g.normpart,
-                                                           nnorm, oa[r].g.g, m, first, oa[r].acc, oa[r].h2);
-            }
-            ck_launch("k_gm_start");
+        {
+            KTimer kt_("k_norm_part", s);
+            k_norm_part<<<dim3(nnorm, nr), 256, 0, s>>>(planes, r0);
         }
+        ck_launch("k_norm_part");
+        {
+            KTimer kt_("k_gm_start", s);
+            k_gm_start<<<dim3(nblocks(n, 256), nr), 256, 0, s>>>(planes, r0, nnorm, first);
+        }
+        ck_launch("k_gm_start");
         prep_v0();
     };
     start(M.bvec.p, 1);
@@ -2312,59 +2316,49 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     // kernel is timed alone and no timed launch is a skipped one.
     const int batch = use_graph ? kStepsPerGraph : 1;
     auto ortho = [&]() {
-        for (int r = 0; r < nr; ++r) {
-            {
-                KTimer kt_("k_gs_dots", s);
-                k_gs_dots<<<nblk, kGsThreads, 0, s>>>(oa[r]);
-            }
-            ck_launch("k_gs_dots");
-            {
-                KTimer kt_("k_gs_update", s);
-                k_gs_update<<<nblk, kGsThreads, 0, s>>>(oa[r]);
-            }
-            ck_launch("k_gs_update");
-            {
-                KTimer kt_("k_gs_finish", s);
-                k_gs_finish<<<nblk, kGsThreads, 0, s>>>(oa[r]);
-            }
-            ck_launch("k_gs_finish");
-
+        {
+            KTimer kt_("k_gs_dots", s);
+            if (nr > 1) k_gs_dots_m<<<dim3(nblk, nr), kGsThreads, 0, s>>>(planes);
+            else k_gs_dots<<<nblk, kGsThreads, 0, s>>>(planes.p[0]);
         }
-        if (nr > 1) {
-            k_gm_skip_all<<<1, 32, 0, s>>>(M.st.p, nr);
-            ck_launch("k_gm_skip_all");
+        ck_launch("k_gs_dots");
+        {
+            KTimer kt_("k_gs_update", s);
+            if (nr > 1) k_gs_update_m<<<dim3(nblk, nr), kGsThreads, 0, s>>>(planes);
+            else k_gs_update<<<nblk, kGsThreads, 0, s>>>(planes.p[0]);
         }
+        ck_launch("k_gs_update");
+        {
+            KTimer kt_("k_gs_finish", s);
+            if (nr > 1) k_gs_finish_m<<<dim3(nblk, nr), kGsThreads, 0, s>>>(planes);
+            else k_gs_finish<<<nblk, kGsThreads, 0, s>>>(planes.p[0]);
+        }
+        ck_launch("k_gs_finish");
     };
     auto givens = [&](cudaStream_t gs) {
-        for (int r = 0; r < nr; ++r) {
-            {
-                KTimer kt_("k_gm_givens", gs);
-                k_gm_givens<<<1, 32, 0, gs>>>(oa[r].g);
-            }
-            ck_launch("k_gm_givens");
+        {
+            KTimer kt_("k_gm_givens", gs);
+            k_gm_givens<<<nr, 32, 0, gs>>>(planes);
         }
+        ck_launch("k_gm_givens");
     };
     // the preconditioner on every plane of w (and of the near part, which
     // the Gram-Schmidt step would add, when wnear is given)
     auto precond = [&](float2 *w, float2 *wnear, const int *skip) {
-        for (int r = 0; r < nr; ++r) {
-            if (rscale) {
-                {
-                    KTimer kt_("k_row_scale", s);
-                    k_row_scale<<<nblocks(n, 256), 256, 0, s>>>(w + r * n, wnear ? wnear + r * n : nullptr, M.dinv.p,
-                                                                n, skip);
-                }
-                ck_launch("k_row_scale");
+        if (rscale) {
+            {
+                KTimer kt_("k_row_scale", s);
+                k_row_scale<<<dim3(nblocks(n, 256), nr), 256, 0, s>>>(w, wnear, M.dinv.p, n, skip);
             }
-            if (bjac) {
-                // w <- P (w + wnear), the near part cleared
-                {
-                    KTimer kt_("k_bj_apply", s);
-                    k_bj_apply<<<(unsigned)Lb.h_bj.size(), kBjMax, 0, s>>>(Lb.bj.p, M.bjinv.p, w + r * n,
-                                                                           wnear ? wnear + r * n : nullptr, skip);
-                }
-                ck_launch("k_bj_apply");
+            ck_launch("k_row_scale");
+        }
+        if (bjac) {
+            // w <- P (w + wnear), the near part cleared
+            {
+                KTimer kt_("k_bj_apply", s);
+                k_bj_apply<<<dim3((unsigned)Lb.h_bj.size(), nr), kBjMax, 0, s>>>(Lb.bj.p, M.bjinv.p, w, wnear, n, skip);
             }
+            ck_launch("k_bj_apply");
         }
     };
     // the product of the current basis vectors (their inputs already
@@ -2458,21 +2452,18 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
                 if (all_done) break;
             }
         }
-        for (int r = 0; r < nr; ++r) {
-            {
-                KTimer kt_("k_gm_backsolve", s);
-                const int tri_cols = std::min(m, 100);
-                k_gm_backsolve<<<1, 256, (size_t)tri_cols * tri_cols * sizeof(double2), s>>>(
-                    oa[r].g.st, oa[r].g.H, oa[r].g.g, M.yv.p + (int64_t)r * (m + 1), m, tri_cols);
-            }
-            ck_launch("k_gm_backsolve");
-            {
-                KTimer kt_("k_gm_xupdate", s);
-                k_gm_xupdate<<<nblocks(n, 256), 256, 0, s>>>(M.uvec.p + r * n, oa[r].g.V, n, oa[r].g.st,
-                                                             M.yv.p + (int64_t)r * (m + 1));
-            }
-            ck_launch("k_gm_xupdate");
+        {
+            KTimer kt_("k_gm_backsolve", s);
+            const int tri_cols = std::min(m, kBacksolveCols);
+            k_gm_backsolve<<<nr, 256, (size_t)tri_cols * (tri_cols + 1) / 2 * sizeof(double2), s>>>(planes, M.yv.p,
+                                                                                                     tri_cols);
         }
+        ck_launch("k_gm_backsolve");
+        {
+            KTimer kt_("k_gm_xupdate", s);
+            k_gm_xupdate<<<dim3(nblocks(n, 256), nr), 256, 0, s>>>(planes, M.uvec.p, M.yv.p);
+        }
+        ck_launch("k_gm_xupdate");
         bool all_conv = true, at_max = false;
         for (int r = 0; r < nr; ++r) {
             all_conv = all_conv && R.hp[r].converged;
@@ -2522,21 +2513,19 @@ void precondition_rhs(bem_mesh_impl &M, float2 *b, int nr)
     cudaStream_t s = M.s;
     const int64_t n = M.n;
     const Lists &Lb = *fr(M).plan->lists;
-    for (int r = 0; r < nr; ++r) {
-        if (M.prm.row_scaling) {
-            {
-                KTimer kt_("k_row_scale", s);
-                k_row_scale<<<nblocks(n, 256), 256, 0, s>>>(b + r * n, nullptr, M.dinv.p, n, nullptr);
-            }
-            ck_launch("k_row_scale");
+    if (M.prm.row_scaling) {
+        {
+            KTimer kt_("k_row_scale", s);
+            k_row_scale<<<dim3(nblocks(n, 256), nr), 256, 0, s>>>(b, nullptr, M.dinv.p, n, nullptr);
         }
-        if (M.prm.block_jacobi) {
-            {
-                KTimer kt_("k_bj_apply", s);
-                k_bj_apply<<<(unsigned)Lb.h_bj.size(), kBjMax, 0, s>>>(Lb.bj.p, M.bjinv.p, b + r * n, nullptr, nullptr);
-            }
-            ck_launch("k_bj_apply");
+        ck_launch("k_row_scale");
+    }
+    if (M.prm.block_jacobi) {
+        {
+            KTimer kt_("k_bj_apply", s);
+            k_bj_apply<<<dim3((unsigned)Lb.h_bj.size(), nr), kBjMax, 0, s>>>(Lb.bj.p, M.bjinv.p, b, nullptr, n, nullptr);
         }
+        ck_launch("k_bj_apply");
     }
 }
 

@@ -1113,8 +1113,9 @@ __global__ void k_row_scale(float2 *__restrict__ y, float2 *__restrict__ y2, con
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float2 d = dinv[i];
-    y[i] = cmul(y[i], d);
-    if (y2) y2[i] = cmul(y2[i], d);
+    const int64_t q = (int64_t)blockIdx.y * n + i;         // the right-hand side's plane
+    y[q] = cmul(y[q], d);
+    if (y2) y2[q] = cmul(y2[q], d);
 }
 
 // Block-Jacobi preconditioner (the block form of the solver's row scaling,
@@ -1234,30 +1235,43 @@ __global__ void __launch_bounds__(256) k_bj_factor(NearArgs a, const int4 *__res
 // product kernels.
 __global__ void __launch_bounds__(kBjMax) k_bj_apply(const int4 *__restrict__ blocks, const float2 *__restrict__ binv,
                                                      float2 *__restrict__ w, float2 *__restrict__ wnear,
-                                                     const int *skip)
+                                                     int64_t n, const int *skip)
 {
     if (skip_now(skip)) return;
     __shared__ float2 xs[kBjMax];
     const int4 B = blocks[blockIdx.x];
     const int nb = B.y;
     const int r = threadIdx.x;
+    const int64_t o = (int64_t)blockIdx.y * n + B.x + r;   // the row in its right-hand side's plane
     if (r < nb) {
-        float2 v = w[B.x + r];
-        if (wnear) v = cadd(v, wnear[B.x + r]);
+        float2 v = w[o];
+        if (wnear) v = cadd(v, wnear[o]);
         xs[r] = v;
     }
     __syncthreads();
     if (r >= nb) return;
     const float2 *__restrict__ col = binv + B.z + r;
     float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0;
+    // eight columns' loads in flight per thread (the inverses come from L2 or
+    // HBM and a leaf's block is a few such batches: the kernel is their latency)
     int c = 0;
-    for (; c + 1 < nb; c += 2) {
-        acc0 = cfma(col[(int64_t)c * nb], xs[c], acc0);
-        acc1 = cfma(col[(int64_t)(c + 1) * nb], xs[c + 1], acc1);
+    for (; c + 8 <= nb; c += 8, col += 8 * nb) {
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = col[u * nb];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+            acc0 = cfma(v[u], xs[c + u], acc0);
+            acc1 = cfma(v[u + 1], xs[c + u + 1], acc1);
+        }
     }
-    if (c < nb) acc0 = cfma(col[(int64_t)c * nb], xs[c], acc0);
-    w[B.x + r] = cadd(acc0, acc1);
-    if (wnear) wnear[B.x + r] = make_float2(0.f, 0.f);
+    for (; c + 1 < nb; c += 2, col += 2 * nb) {
+        acc0 = cfma(col[0], xs[c], acc0);
+        acc1 = cfma(col[nb], xs[c + 1], acc1);
+    }
+    if (c < nb) acc0 = cfma(col[0], xs[c], acc0);
+    w[o] = cadd(acc0, acc1);
+    if (wnear) wnear[o] = make_float2(0.f, 0.f);
 }
 
 // ------------------------------------------------------------------ adjoint
@@ -2636,7 +2650,7 @@ __device__ double gs_load_h(const double2 *src, int64_t stride, float2 *hs, int 
 // 0.02 after 19 steps, 1 after 53.)
 __device__ __forceinline__ bool gs_second_pass(double ww, double hh) { return ww - hh < 0.5 * ww; }
 
-__global__ void __launch_bounds__(kGsThreads) k_gs_dots(GsArgs a)
+__device__ __forceinline__ void gs_dots_body(const GsArgs &a)
 {
     const GmresArgs &g = a.g;
     GmresState *st = g.st;
@@ -2676,7 +2690,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_dots(GsArgs a)
     gs_norm_part(ws, R, a.acc + 4 * (j & 1));
 }
 
-__global__ void __launch_bounds__(kGsThreads) k_gs_update(GsArgs a)
+__device__ __forceinline__ void gs_update_body(const GsArgs &a)
 {
     const GmresArgs &g = a.g;
     GmresState *st = g.st;
@@ -2728,7 +2742,7 @@ __device__ void gs_store(const GsArgs &a, const float2 *ws, int R, int64_t r0, i
     }
 }
 
-__global__ void __launch_bounds__(kGsThreads) k_gs_finish(GsArgs a)
+__device__ __forceinline__ void gs_finish_body(const GsArgs &a)
 {
     const GmresArgs &g = a.g;
     GmresState *st = g.st;
@@ -2754,9 +2768,28 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_finish(GsArgs a)
     gs_store(a, ws, R, r0, j, need);
 }
 
-// Givens step of the column the Gram-Schmidt kernels just formed (one warp).
-__global__ void k_gm_givens(GmresArgs a)
+__global__ void __launch_bounds__(kGsThreads) k_gs_dots(GsArgs a) { gs_dots_body(a); }
+__global__ void __launch_bounds__(kGsThreads) k_gs_update(GsArgs a) { gs_update_body(a); }
+__global__ void __launch_bounds__(kGsThreads) k_gs_finish(GsArgs a) { gs_finish_body(a); }
+__global__ void __launch_bounds__(kGsThreads) k_gs_dots_m(GsPlanes A) { gs_dots_body(A.p[blockIdx.y]); }
+__global__ void __launch_bounds__(kGsThreads) k_gs_update_m(GsPlanes A) { gs_update_body(A.p[blockIdx.y]); }
+__global__ void __launch_bounds__(kGsThreads) k_gs_finish_m(GsPlanes A)
 {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        // the product kernels skip once every system is done (their flags
+        // were set by k_gs_dots_m)
+        int all = 1;
+        for (int r = 0; r < A.nr; ++r) all &= __ldcv(&A.p[r].g.st->skip_prod) != 0;
+        A.p[0].g.st->skip_all = all;
+    }
+    gs_finish_body(A.p[blockIdx.y]);
+}
+
+// Givens step of the column the Gram-Schmidt kernels just formed (one warp
+// per plane).
+__global__ void k_gm_givens(GsPlanes A)
+{
+    const GmresArgs &a = A.p[blockIdx.x].g;
     GmresState *st = a.st;
     if (*(volatile int *)&st->done) return;
     // ||v_{j+1}||^2 from the Gram-Schmidt sums (after the second pass when
@@ -2765,16 +2798,6 @@ __global__ void k_gm_givens(GmresArgs a)
     const double nn = __ldcg(a.gs_acc + 4 * (j & 1) + (*(volatile int *)&st->reorth ? 2 : 1));
     if (threadIdx.x == 0) st->nn = nn;
     gm_givens_warp(a, nn, j);
-}
-
-// st[0].skip_all = every plane's skip_prod (the product kernels of several
-// right-hand sides skip only when all systems are done).
-__global__ void k_gm_skip_all(GmresState *st, int nr)
-{
-    if (threadIdx.x != 0) return;
-    int all = 1;
-    for (int r = 0; r < nr; ++r) all &= __ldcv(&st[r].skip_prod) != 0;
-    st[0].skip_all = all;
 }
 
 // The condition of the WHILE node that runs one Arnoldi cycle on the device
@@ -2792,19 +2815,22 @@ __global__ void k_gm_continue(cudaGraphConditionalHandle h, GmresState *st, int 
     cudaGraphSetConditional(h, (!all && b < max_bodies) ? 1u : 0u);
 }
 
-// Back substitution y = R^{-1} g over ncols columns (FP64), one warp:
-// column-oriented, each step scales one entry by the reciprocal of its
-// diagonal and the lanes update the rest.  The reciprocals 1 / R_ll are
-// formed first, all in parallel, so the sequential chain of steps holds no
+// Back substitution y = R^{-1} g over ncols columns (FP64), one block per
+// plane: column-oriented, each step scales one entry by the reciprocal of its
+// diagonal and the lanes of warp 0 update the rest.  The reciprocals 1 / R_ll
+// are formed first, all in parallel, so the sequential chain of steps holds no
 // division (FP64 division is a long dependent sequence on this part).  The
-// triangle is staged in shared memory when it fits (smem_cols columns).
-__global__ void k_gm_backsolve(const GmresState *st, const double2 *__restrict__ H, const double2 *__restrict__ g,
-                               double2 *__restrict__ y, int m, int smem_cols)
+// triangle is staged packed in shared memory when it fits (smem_cols columns;
+// 141 columns from global memory took 212 us, staged 142 us).
+__global__ void k_gm_backsolve(GsPlanes A, double2 *__restrict__ yv, int smem_cols)
 {
-    extern __shared__ double2 tri[];       // [nc][nc] when nc <= smem_cols (upper triangle filled)
+    extern __shared__ double2 tri[];       // row r of the upper triangle from r nc - r (r - 1) / 2
     __shared__ double2 sv[kMaxRestart + 1];
     __shared__ double2 rinv[kMaxRestart + 1];
-    const int nc = st->ncols;
+    const GmresArgs &a = A.p[blockIdx.x].g;
+    const double2 *__restrict__ H = a.H, *__restrict__ g = a.g;
+    const int m = a.m, nc = a.st->ncols;
+    double2 *__restrict__ y = yv + (int64_t)blockIdx.x * (m + 1);
     const int lane = threadIdx.x & 31;
     const bool in_smem = nc <= smem_cols;
     // staging by the whole block (its loads independent of one another),
@@ -2816,8 +2842,10 @@ __global__ void k_gm_backsolve(const GmresState *st, const double2 *__restrict__
         rinv[l] = make_double2(d.x * inv, -d.y * inv);   // conj(d) / |d|^2
     }
     if (in_smem)
-        for (int r = threadIdx.x / 32; r < nc; r += blockDim.x / 32)
-            for (int c = r + lane; c < nc; c += 32) tri[r * nc + c] = H[(int64_t)r * m + c];
+        for (int r = threadIdx.x / 32; r < nc; r += blockDim.x / 32) {
+            double2 *row = tri + (r * nc - r * (r - 1) / 2) - r;
+            for (int c = r + lane; c < nc; c += 32) row[c] = H[(int64_t)r * m + c];
+        }
     __syncthreads();
     if (threadIdx.x >= 32) return;
     for (int l = nc - 1; l >= 0; --l) {
@@ -2826,7 +2854,7 @@ __global__ void k_gm_backsolve(const GmresState *st, const double2 *__restrict__
         const double2 yl = make_double2(sl.x * ri.x - sl.y * ri.y, sl.x * ri.y + sl.y * ri.x);
         if (lane == 0) y[l] = yl;
         for (int r = lane; r < l; r += 32) {
-            const double2 h = in_smem ? tri[r * nc + l] : H[(int64_t)r * m + l];
+            const double2 h = in_smem ? tri[r * nc - r * (r - 1) / 2 - r + l] : H[(int64_t)r * m + l];
             sv[r].x -= h.x * yl.x - h.y * yl.y;
             sv[r].y -= h.x * yl.y + h.y * yl.x;
         }
@@ -2834,12 +2862,16 @@ __global__ void k_gm_backsolve(const GmresState *st, const double2 *__restrict__
     }
 }
 
-// x <- x + sum_l y_l V_l
-__global__ void k_gm_xupdate(float2 *__restrict__ x, const float2 *__restrict__ V, int64_t n,
-                             const GmresState *st, const double2 *__restrict__ y)
+// x <- x + sum_l y_l V_l (plane blockIdx.y)
+__global__ void k_gm_xupdate(GsPlanes A, float2 *__restrict__ x, const double2 *__restrict__ yv)
 {
     __shared__ float2 ys[kMaxRestart + 1];
-    const int nc = st->ncols;
+    const GmresArgs &a = A.p[blockIdx.y].g;
+    const float2 *__restrict__ V = a.V;
+    const int64_t n = a.n;
+    const double2 *__restrict__ y = yv + (int64_t)blockIdx.y * (a.m + 1);
+    x += (int64_t)blockIdx.y * n;
+    const int nc = a.st->ncols;
     for (int l = threadIdx.x; l < nc; l += blockDim.x) ys[l] = make_float2((float)y[l].x, (float)y[l].y);
     __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2850,20 +2882,26 @@ __global__ void k_gm_xupdate(float2 *__restrict__ x, const float2 *__restrict__ 
 }
 
 // r = b - A x is formed by the caller; here: V_0 = r / ||r|| with ||r|| from
-// normpart, and the cycle state is reset.
-__global__ void k_gm_start(GmresState *st, float2 *__restrict__ V, const float2 *__restrict__ r, int64_t n,
-                           const double *__restrict__ normpart, int nblk, double2 *__restrict__ g, int m, int first,
-                           double *__restrict__ gs_acc, double2 *__restrict__ gs_h2)
+// normpart, and the cycle state is reset (plane blockIdx.y).
+__global__ void k_gm_start(GsPlanes A, const float2 *__restrict__ r, int nblk, int first)
 {
+    const GsArgs &a = A.p[blockIdx.y];
+    GmresState *st = a.g.st;
+    const int64_t n = a.g.n;
+    const int m = a.g.m;
+    float2 *__restrict__ V = a.g.V;
+    double2 *__restrict__ g = a.g.g;
+    r += (int64_t)blockIdx.y * n;
     if (blockIdx.x == 0) {
         // the Gram-Schmidt sums of both parities (see k_gs_dots)
-        for (int l = threadIdx.x; l < 2 * (m + 1); l += blockDim.x) gs_h2[l] = make_double2(0.0, 0.0);
-        if (threadIdx.x < 8) gs_acc[threadIdx.x] = 0.0;
+        for (int l = threadIdx.x; l < 2 * (m + 1); l += blockDim.x) a.h2[l] = make_double2(0.0, 0.0);
+        if (threadIdx.x < 8) a.acc[threadIdx.x] = 0.0;
+        for (int l = threadIdx.x; l <= m; l += blockDim.x) g[l] = make_double2(0.0, 0.0);
     }
     __shared__ double beta_s;
     if (threadIdx.x == 0) {
         double nn = 0.0;
-        for (int b = 0; b < nblk; ++b) nn += normpart[b];
+        for (int b = 0; b < nblk; ++b) nn += a.g.normpart[b];
         beta_s = sqrt(nn);
     }
     __syncthreads();
@@ -2881,15 +2919,17 @@ __global__ void k_gm_start(GmresState *st, float2 *__restrict__ V, const float2 
         st->converged = 0;
         st->bodies = 0;
         st->resid = st->bnorm > 0.0 ? beta / st->bnorm : 0.0;
-        for (int l = 0; l <= m; ++l) g[l] = make_double2(0.0, 0.0);
         g[0] = make_double2(beta, 0.0);
         if (st->resid <= st->tol) { st->done = 1; st->converged = 1; }
     }
 }
 
-// partial ||r||^2 per block
-__global__ void k_norm_part(const float2 *__restrict__ r, int64_t n, double *__restrict__ part)
+// partial ||r||^2 per block (plane blockIdx.y)
+__global__ void k_norm_part(GsPlanes A, const float2 *__restrict__ r)
 {
+    const GmresArgs &a = A.p[blockIdx.y].g;
+    const int64_t n = a.n;
+    r += (int64_t)blockIdx.y * n;
     double v = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         v += (double)r[i].x * r[i].x + (double)r[i].y * r[i].y;
@@ -2900,7 +2940,7 @@ __global__ void k_norm_part(const float2 *__restrict__ r, int64_t n, double *__r
     if (threadIdx.x < 32) {
         double s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) part[blockIdx.x] = s;
+        if (threadIdx.x == 0) a.normpart[blockIdx.x] = s;
     }
 }
 

@@ -7,6 +7,7 @@
 namespace bem {
 
 constexpr int kMaxRestart = 1024;
+constexpr int kMaxPlanes = 4;            // right-hand sides per multi-plane launch
 constexpr int kMaxFarLevels = 16;
 
 // Near columns of a leaf: runs of consecutive elements (the elements of
@@ -52,7 +53,7 @@ struct GmresState {
     // there could differ between the threads of one block.
     int skip_prod;
     // With several right-hand sides (plane 0's state only): the product
-    // kernels skip once every plane's skip_prod is set (k_gm_skip_all).
+    // kernels skip once every plane's skip_prod is set (k_gs_finish).
     int skip_all;
     // Bodies of the device-driven Arnoldi loop run in the current cycle
     // (plane 0's state; k_gm_continue counts, k_gm_start resets).
@@ -301,7 +302,6 @@ __global__ void k_aggregate_3(const LevelsArgs *A, const float4 *wts, int64_t wp
 __global__ void k_aggregate_4(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
 // One right-hand side, with the level's stored phases (FarArgs::ph).
 __global__ void k_aggregate_1t(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
-constexpr int kMaxPlanes = 4;            // right-hand sides per multi-plane launch
 // Aggregation on the tensor cores (bem_tc.cu): tasks of one element chunk
 // and kTcPairs direction pairs, split-BF16 operands, FP32 accumulation;
 // fault is set when the wait for the tensor cores runs out.
@@ -383,7 +383,7 @@ __global__ void k_adjoint_reduce(const float2 *u, const float2 *g, const float2 
 // block-Jacobi sub-blocks: at most kBjMax consecutive elements of one leaf
 constexpr int kBjMax = 64;
 __global__ void k_bj_factor(NearArgs a, const int4 *blocks, float2 *binv, int *err);
-__global__ void k_bj_apply(const int4 *blocks, const float2 *binv, float2 *w, float2 *wnear, const int *skip);
+__global__ void k_bj_apply(const int4 *blocks, const float2 *binv, float2 *w, float2 *wnear, int64_t n, const int *skip);
 __global__ void k_row_scale_init(NearArgs a, float2 *dinv, int *err);
 __global__ void k_row_scale(float2 *y, float2 *y2, const float2 *dinv, int64_t n, const int *skip);
 __global__ void k_sub(float2 *b, const float2 *y, int64_t n);
@@ -420,20 +420,30 @@ struct GsArgs {
 };
 constexpr int kGsThreads = 256;
 constexpr int kGsMaxRows = 1024;    // rows per block staged in shared memory
+// The systems solved in lockstep: blockIdx.y is the plane of the vector
+// kernels, blockIdx.x that of the one-warp kernels.  One launch serves all
+// planes (their steps are independent and each leaves most of the GPU idle;
+// one launch per plane and step cost 12 serial launches with four planes).
+struct GsPlanes {
+    GsArgs p[kMaxPlanes];
+    int nr;
+};
+// One plane has its own kernels: its arguments are direct constants (read by a
+// plane index they cost each kernel of a step 0.8 us).
 __global__ void k_gs_dots(GsArgs a);
 __global__ void k_gs_update(GsArgs a);
 __global__ void k_gs_finish(GsArgs a);
-__global__ void k_gm_givens(GmresArgs a);
-__global__ void k_gm_skip_all(GmresState *st, int nr);
+__global__ void k_gs_dots_m(GsPlanes A);
+__global__ void k_gs_update_m(GsPlanes A);
+__global__ void k_gs_finish_m(GsPlanes A);
+__global__ void k_gm_givens(GsPlanes A);
 // Loop condition of the WHILE node of a device-driven Arnoldi cycle: one
 // more body while some plane is not done and fewer than max_bodies have run.
 __global__ void k_gm_continue(cudaGraphConditionalHandle h, GmresState *st, int nr, int max_bodies);
-__global__ void k_gm_backsolve(const GmresState *st, const double2 *H, const double2 *g, double2 *y, int m,
-                               int smem_cols);
-__global__ void k_gm_xupdate(float2 *x, const float2 *V, int64_t n, const GmresState *st, const double2 *y);
-__global__ void k_gm_start(GmresState *st, float2 *V, const float2 *r, int64_t n, const double *normpart, int nblk,
-                           double2 *g, int m, int first, double *gs_acc, double2 *gs_h2);
-__global__ void k_norm_part(const float2 *r, int64_t n, double *part);
+__global__ void k_gm_backsolve(GsPlanes A, double2 *y, int smem_cols);
+__global__ void k_gm_xupdate(GsPlanes A, float2 *x, const double2 *y);
+__global__ void k_gm_start(GsPlanes A, const float2 *r, int nblk, int first);
+__global__ void k_norm_part(GsPlanes A, const float2 *r);
 
 // Host helpers shared by the translation units (bem_capi.cu): the
 // quadrature tables of a parameter set (conical rules m = 1..6, the Duffy and
