@@ -33,6 +33,7 @@ constexpr double kPhaseTableMaxBytes = 4.0 * 1024 * 1024 * 1024;
 constexpr double kFieldFmmMinPairs = 1e9;
 // Arnoldi steps captured in one CUDA graph (one status read per graph)
 constexpr int kStepsPerGraph = 4;
+constexpr int kNoErr = 0x7f7f7f7f;       // an error flag that no element has lowered (set by bytes)
 // columns of the GMRES triangle that k_gm_backsolve stages (packed, with its
 // 32 KB of vectors within 227 KB)
 constexpr int kBacksolveCols = 155;
@@ -371,15 +372,10 @@ struct Plan {
     DevArr<float2> valT;          // A^T in A's layout (near_transpose), made from val
     bool valT_valid = false;
     bool has_phases = false;      // every level's stored phases built (far_table)
-    std::vector<float> val_key;   // host copy of the coefficients the stored values were made with
+    std::vector<double> val_key;  // what the stored values' column coefficients depend on (coeff_key)
     bool val_valid = false;
     int64_t nnz() const { return lists->nnz; }
     const FreqPlan &fp() const { return lists->fp; }
-};
-
-struct Coeffs {
-    std::vector<float2> cp, cq, cp0, cq0, z, aq;   // internal order
-    bool known_nonzero = false;
 };
 
 }  // namespace
@@ -393,6 +389,9 @@ struct Frame {
     DevArr<float2> fpart;                      // column parts of a recomputed product (stays with the stream)
     cudaStream_t s = nullptr;                  // stream of this frame's setup work
     bool known_nonzero = false;
+    std::vector<double> coef_key;              // what the coefficients above were made from
+    DevArr<double> adm;                        // region admittances
+    int *h_err = nullptr;                      // pinned copies of the error flags (stay with the stream)
 };
 
 // Device data of the FMM field evaluation at points (one call's plan).
@@ -442,6 +441,14 @@ struct bem_mesh_impl {
     DevArr<int64_t> perm;
     DevArr<QuadTables> Q;
     DevArr<int> type;
+    // boundary data (internal order) and what the host asks of it
+    DevArr<double2> bcv_d;
+    DevArr<int> region_d;
+    bool has_admi = false, bcv_nan = false;
+    int max_region = -1;         // of the ADMI elements
+    double vmax = 0.0, pmax = 0.0;             // largest |component| of the velocities and of the pressures given
+    int *h_err = nullptr;        // pinned: error flag per frame, tensor-core fault
+    cudaEvent_t ev_user = nullptr;             // joins with the caller's stream
     DevArr<float2> xint, ynear, tmp, tmp2, bvec, uvec;
     DevArr<float2> dinv;         // row scaling 1 / A_ii (internal order) when row_scaling is on
     DevArr<float2> bjinv;        // block-Jacobi inverses of the diagonal sub-blocks when block_jacobi is on
@@ -477,6 +484,7 @@ struct bem_mesh_impl {
     DevArr<float2> spare_val;
     std::vector<std::unique_ptr<DevArr<float2>>> spare_bufs;
     DevArr<SourceDev> srcbuf;
+    std::vector<SourceDev> src_key;   // the sources srcbuf holds
     DevArr<float2> fieldpart;     // per-point partial sums of the field (point-major)
     std::unique_ptr<EvalDev> eval;  // FMM field evaluation
     DevArr<double> ptsbuf;
@@ -494,7 +502,6 @@ struct bem_mesh_impl {
     // pinned host copies of every plane's state (room for two copies)
     GmresState *h_st = nullptr;
     int h_st_planes = 0;                       // planes h_st holds per copy (two copies)
-    std::vector<float> coef_key;
 
     ElemDev elem() const
     {
@@ -511,6 +518,8 @@ struct bem_mesh_impl {
             if (ev_giv[t]) cudaEventDestroy(ev_giv[t]);
         }
         if (h_st) cudaFreeHost(h_st);
+        if (h_err) cudaFreeHost(h_err);
+        if (ev_user) cudaEventDestroy(ev_user);
         if (s_giv) cudaStreamDestroy(s_giv);
         if (s_setup) cudaStreamDestroy(s_setup);
         if (ev_fork) cudaEventDestroy(ev_fork);
@@ -1020,70 +1029,52 @@ NearArgs near_args(const bem_mesh_impl &M, const Plan &P, const float2 *cp, cons
     return a;
 }
 
-// coefficient sets (Eq. SystemI with the boundary conditions folded in)
-void make_coeffs(bem_mesh_impl &M, double k, double omega, double c, double rho, const double *adm, int nreg, Coeffs &C)
+// What the unknowns' column coefficients (cp, cq) of a plan depend on besides
+// its wavenumber: the admittances and rho c when the mesh has ADMI elements.
+std::vector<double> coeff_key(const bem_mesh_impl &M, double c, double rho, const double *adm)
 {
-    const int64_t n = M.n;
-    C.cp.assign(n, make_float2(0.f, 0.f));
-    C.cq = C.cp0 = C.cq0 = C.z = C.aq = C.cp;
-    C.known_nonzero = false;
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t e = M.t.perm[i];
-        const int ty = M.bct[e];
-        const double vr = M.bcv[2 * e], vi = M.bcv[2 * e + 1];
-        if (ty == BEM_PRES) {
-            C.cq[i] = make_float2(1.f, 0.f);
-            C.cp0[i] = make_float2(1.f, 0.f);
-            C.z[i] = make_float2((float)vr, (float)vi);
-        } else {
-            C.cp[i] = make_float2(1.f, 0.f);
-            C.cq0[i] = make_float2(1.f, 0.f);
-            // g = i w rho v
-            C.z[i] = make_float2((float)(-omega * rho * vi), (float)(omega * rho * vr));
-            if (ty == BEM_ADMI) {
-                const int r = M.region[e];
-                const double yr = adm[2 * r], yi = adm[2 * r + 1];
-                // a = -tau i k beta, beta = rho c Y, Y = velocity into the
-                // wall / p (the wall lies along the normal for the interior
-                // problem, against it for the exterior problem)
-                const double t = M.prm.tau < 0 ? -1.0 : 1.0;
-                const double br = t * rho * c * yr, bi = t * rho * c * yi;
-                C.cq[i] = make_float2((float)(k * bi), (float)(-k * br));
-                C.aq[i] = C.cq[i];
-            }
-        }
-        if (C.z[i].x != 0.f || C.z[i].y != 0.f) C.known_nonzero = true;
+    std::vector<double> k;
+    if (M.has_admi) {
+        k = {c, rho};
+        k.insert(k.end(), adm, adm + 2 * ((size_t)M.max_region + 1));
     }
-    // tau (Eq. SystemI: +1 exterior, -1 interior) multiplies every integral
-    // operator: it is folded into the column coefficients of the unknowns
-    // and of the known data (the self entry takes it out of its identity
-    // half again); aq, the physical relation q = a p, keeps its sign
-    if (M.prm.tau < 0)
-        for (int64_t i = 0; i < n; ++i) {
-            C.cp[i] = make_float2(-C.cp[i].x, -C.cp[i].y);
-            C.cq[i] = make_float2(-C.cq[i].x, -C.cq[i].y);
-            C.cp0[i] = make_float2(-C.cp0[i].x, -C.cp0[i].y);
-            C.cq0[i] = make_float2(-C.cq0[i].x, -C.cq0[i].y);
-        }
+    return k;
 }
 
-void upload_coeffs(bem_mesh_impl &M, const Coeffs &C)
+// Coefficient sets of the current plan's frequency (Eq. SystemI with the
+// boundary conditions folded in), formed on the device from the boundary data
+// there when anything they depend on has changed.
+void ensure_coeffs(bem_mesh_impl &M, double omega, double c, double rho, const double *adm)
 {
-    fr(M).cp.upload(C.cp, fr(M).s);
-    fr(M).cq.upload(C.cq, fr(M).s);
-    fr(M).cp0.upload(C.cp0, fr(M).s);
-    fr(M).cq0.upload(C.cq0, fr(M).s);
-    fr(M).z.upload(C.z, fr(M).s);
-    fr(M).aq.upload(C.aq, fr(M).s);
-    fr(M).known_nonzero = C.known_nonzero;
+    Frame &F = fr(M);
+    const double k = F.plan->k;
+    std::vector<double> key = coeff_key(M, c, rho, adm);
+    key.insert(key.end(), {k, omega, rho});
+    if (F.cp.n == (size_t)M.n && key == F.coef_key) return;
+    F.coef_key.clear();
+    for (DevArr<float2> *a : {&F.cp, &F.cq, &F.cp0, &F.cq0, &F.z, &F.aq}) a->alloc(M.n);
+    if (M.has_admi) {
+        std::vector<double> h(adm, adm + 2 * ((size_t)M.max_region + 1));
+        F.adm.upload(h, F.s);
+    }
+    {
+        KTimer kt_("k_coeffs", F.s);
+        k_coeffs<<<nblocks(M.n, 256), 256, 0, F.s>>>(M.n, M.type.p, M.bcv_d.p, M.region_d.p, F.adm.p, k, omega, rho, c,
+                                                    M.prm.tau < 0 ? -1.0 : 1.0, F.cp.p, F.cq.p, F.cp0.p, F.cq0.p, F.z.p,
+                                                    F.aq.p);
+    }
+    ck_launch("k_coeffs");
+    // some known datum is nonzero (i w rho v, or a given pressure) in FP32
+    F.known_nonzero = M.bcv_nan || (float)(omega * rho * M.vmax) != 0.f || (float)M.pmax != 0.f;
+    F.coef_key.swap(key);
 }
 
 void check_err(bem_mesh_impl &M)
 {
-    int e = INT_MAX;
-    ck(cudaMemcpyAsync(&e, fr(M).err.p, sizeof(int), cudaMemcpyDeviceToHost, fr(M).s), "D2H err");
+    ck(cudaMemcpyAsync(fr(M).h_err, fr(M).err.p, sizeof(int), cudaMemcpyDeviceToHost, fr(M).s), "D2H err");
     ck(cudaStreamSynchronize(fr(M).s), "sync");
-    if (e != INT_MAX) {
+    const int e = *fr(M).h_err;
+    if (e != kNoErr) {
         char buf[160];
         snprintf(buf, sizeof buf,
                  "number of subelements which are subdivided in a loop exceeds %d at element %lld",
@@ -1098,10 +1089,9 @@ void check_err(bem_mesh_impl &M)
 void check_tc_fault(bem_mesh_impl &M)
 {
     if (M.prm.far_precision != 1) return;
-    int f = 0;
-    ck(cudaMemcpyAsync(&f, M.tc_fault.p, sizeof(int), cudaMemcpyDeviceToHost, M.s), "D2H fault");
+    ck(cudaMemcpyAsync(M.h_err + 2, M.tc_fault.p, sizeof(int), cudaMemcpyDeviceToHost, M.s), "D2H fault");
     ck(cudaStreamSynchronize(M.s), "sync");
-    if (f) {
+    if (M.h_err[2]) {
         ck(cudaMemsetAsync(M.tc_fault.p, 0, sizeof(int), M.s), "memset");
         g_err = "tensor-core aggregation: the wait for the tensor cores gave up";
         throw Fail{BEM_E_TIMEOUT};
@@ -1110,8 +1100,7 @@ void check_tc_fault(bem_mesh_impl &M)
 
 void reset_err(bem_mesh_impl &M)
 {
-    const int v = INT_MAX;
-    ck(cudaMemcpyAsync(fr(M).err.p, &v, sizeof(int), cudaMemcpyHostToDevice, fr(M).s), "H2D err");
+    ck(cudaMemsetAsync(fr(M).err.p, 0x7f, sizeof(int), fr(M).s), "memset err");
 }
 
 // Stored near-field entries of plan P for the column coefficients (cp, cq):
@@ -1217,15 +1206,9 @@ void near_fused(bem_mesh_impl &M, const Plan &P, const NearArgs &a, const float2
 }
 
 // Make sure the stored near-field values match the current unknowns' coefficients.
-void ensure_near_values(bem_mesh_impl &M, const Coeffs &C)
+void ensure_near_values(bem_mesh_impl &M, double c, double rho, const double *adm)
 {
     Plan &P = *fr(M).plan;
-    std::vector<float> key;
-    key.reserve(4 * M.n);
-    for (int64_t i = 0; i < M.n; ++i) {
-        key.push_back(C.cp[i].x); key.push_back(C.cp[i].y);
-        key.push_back(C.cq[i].x); key.push_back(C.cq[i].y);
-    }
     if (!M.prm.near_store || P.fp().direct) {
         if (!P.val_valid) {
             // one fused pass validates the subdivision limit for this plan
@@ -1241,6 +1224,7 @@ void ensure_near_values(bem_mesh_impl &M, const Coeffs &C)
         }
         return;
     }
+    std::vector<double> key = coeff_key(M, c, rho, adm);
     if (P.val_valid && key == P.val_key) return;
     P.valT_valid = false;
     store_near(M, P, fr(M).cp.p, fr(M).cq.p);
@@ -1745,24 +1729,20 @@ void ensure_work(bem_mesh_impl &M)
     M.tmp2.alloc(M.n);
 }
 
-void prepare(bem_mesh_impl &M, double freq, const bem_medium *med, const double *adm, int nreg, Coeffs &C)
+void prepare(bem_mesh_impl &M, double freq, const bem_medium *med, const double *adm, int nreg)
 {
     double c, rho;
     medium_of(med, c, rho);
     if (!(freq > 0) || !std::isfinite(freq)) { g_err = "frequency must be positive"; throw Fail{BEM_E_ARG}; }
-    for (int64_t e = 0; e < M.n; ++e)
-        if (M.bct[e] == BEM_ADMI) {
-            if (!adm || M.region[e] >= nreg) {
-                g_err = "admittance missing for an ADMI element's region";
-                throw Fail{BEM_E_ARG};
-            }
-        }
+    if (M.has_admi && (!adm || M.max_region >= nreg)) {
+        g_err = "admittance missing for an ADMI element's region";
+        throw Fail{BEM_E_ARG};
+    }
     ck(cudaSetDevice(M.device), "cudaSetDevice");
     ensure_work(M);
     build_plan_dev(M, freq, c);
-    make_coeffs(M, fr(M).plan->k, 2.0 * M_PI * freq, c, rho, adm, nreg, C);
-    upload_coeffs(M, C);
-    ensure_near_values(M, C);
+    ensure_coeffs(M, 2.0 * M_PI * freq, c, rho, adm);
+    ensure_near_values(M, c, rho, adm);
 }
 
 int resolution_warning(const bem_mesh_impl &M, double freq, const bem_medium *med)
@@ -1796,13 +1776,36 @@ std::vector<SourceDev> sources_of(const bem_source *srcs, int n)
     return v;
 }
 
-void join_streams(cudaStream_t from, cudaStream_t to)
+// The device copy of the sources, uploaded when they differ from the last
+// ones (on the mesh's stream, which alone reads them).
+SourceDev *upload_sources(bem_mesh_impl &M, const bem_source *srcs, int n)
 {
-    cudaEvent_t ev;
-    ck(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
-    ck(cudaEventRecord(ev, from), "record");
-    ck(cudaStreamWaitEvent(to, ev, 0), "wait");
-    cudaEventDestroy(ev);
+    std::vector<SourceDev> v = sources_of(srcs, n);
+    auto same = [](const SourceDev &a, const SourceDev &b) {
+        return a.kind == b.kind && !memcmp(a.v, b.v, sizeof a.v) && !memcmp(a.amp, b.amp, sizeof a.amp);
+    };
+    if (v.empty() || v.size() != M.src_key.size() || !std::equal(v.begin(), v.end(), M.src_key.begin(), same)) {
+        M.src_key.clear();
+        M.srcbuf.upload(v, M.s);
+        M.src_key.swap(v);
+    }
+    return M.srcbuf.p;
+}
+
+// The points on the device (from the caller's array: the copy is staged, or
+// awaited with the call's own work, before the call returns).
+const double *upload_points(bem_mesh_impl &M, const double *pts, int64_t n)
+{
+    M.ptsbuf.alloc(3 * (size_t)n);
+    ck(cudaMemcpyAsync(M.ptsbuf.p, pts, 3 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, M.s), "H2D points");
+    return M.ptsbuf.p;
+}
+
+// to waits for what from holds (the mesh's event is recorded anew each time)
+void join_streams(bem_mesh_impl &M, cudaStream_t from, cudaStream_t to)
+{
+    ck(cudaEventRecord(M.ev_user, from), "record");
+    ck(cudaStreamWaitEvent(to, M.ev_user, 0), "wait");
 }
 
 
@@ -2019,6 +2022,10 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
             }
             ck(cudaMallocHost(&M->h_st, 2 * sizeof(GmresState)), "cudaMallocHost");
             M->h_st_planes = 1;
+            ck(cudaMallocHost(&M->h_err, 3 * sizeof(int)), "cudaMallocHost");
+            M->cur.h_err = M->h_err;
+            M->next.h_err = M->h_err + 1;
+            ck(cudaEventCreateWithFlags(&M->ev_user, cudaEventDisableTiming), "event");
         }
         const int64_t n = n_tris;
         std::vector<float4> chi(n), clo(n), nr(n), va(n), e1(n), e2(n);
@@ -2070,11 +2077,28 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
         std::vector<QuadTables> qt(1, make_tables(p));
         M->Q.upload(qt, s);
         {
-            const int none = INT_MAX;
             for (Frame *F : {&M->cur, &M->next}) {
                 F->err.alloc(1);
-                ck(cudaMemcpyAsync(F->err.p, &none, sizeof none, cudaMemcpyHostToDevice, s), "H2D err");
+                ck(cudaMemsetAsync(F->err.p, 0x7f, sizeof(int), s), "memset err");
             }
+            // boundary data in the internal order, for the coefficient kernel
+            std::vector<double2> bv(n);
+            std::vector<int> rg(n);
+            for (int64_t i = 0; i < n; ++i) {
+                const int64_t j = M->t.perm[i];
+                bv[i] = make_double2(M->bcv[2 * j], M->bcv[2 * j + 1]);
+                rg[i] = M->region[j];
+                double &top = M->bct[j] == BEM_PRES ? M->pmax : M->vmax;
+                top = std::max({top, std::fabs(bv[i].x), std::fabs(bv[i].y)});
+                if (!(bv[i].x == bv[i].x) || !(bv[i].y == bv[i].y)) M->bcv_nan = true;
+                if (M->bct[j] == BEM_ADMI) {
+                    M->has_admi = true;
+                    M->max_region = std::max(M->max_region, rg[i]);
+                }
+            }
+            M->bcv_d.upload(bv, s);
+            M->region_d.upload(rg, s);
+            ck(cudaStreamSynchronize(s), "sync");
         }
         ck(cudaStreamSynchronize(s), "sync");
         *out = M.release();
@@ -2104,9 +2128,8 @@ int bem_matvec(void *mesh, double freq_hz, const bem_medium *medium, const doubl
     auto &M = *(bem_mesh_impl *)mesh;
     try {
         cudaStream_t us = (cudaStream_t)stream;
-        Coeffs C;
-        join_streams(us, M.s);
-        prepare(M, freq_hz, medium, admittance, n_regions, C);
+        join_streams(M, us, M.s);
+        prepare(M, freq_hz, medium, admittance, n_regions);
         // up to kMaxPlanes right-hand sides per pass: one stream of the stored
         // near field and one phase per element and direction for all of them
         for (int r = 0; r < n_rhs; r += kMaxPlanes) {
@@ -2117,7 +2140,7 @@ int bem_matvec(void *mesh, double freq_hz, const bem_medium *medium, const doubl
                             nr);
         }
         check_tc_fault(M);
-        join_streams(M.s, us);
+        join_streams(M, M.s, us);
         return resolution_warning(M, freq_hz, medium);
     } catch (Fail &f) {
         return f.code;
@@ -2132,9 +2155,8 @@ int bem_matvec_transpose(void *mesh, double freq_hz, const bem_medium *medium, c
     auto &M = *(bem_mesh_impl *)mesh;
     try {
         cudaStream_t us = (cudaStream_t)stream;
-        Coeffs C;
-        join_streams(us, M.s);
-        prepare(M, freq_hz, medium, admittance, n_regions, C);
+        join_streams(M, us, M.s);
+        prepare(M, freq_hz, medium, admittance, n_regions);
         reset_err(M);
         M.tmp.alloc(M.n);
         {
@@ -2145,7 +2167,7 @@ int bem_matvec_transpose(void *mesh, double freq_hz, const bem_medium *medium, c
         ensure_transposed_values(M);
         matvec_t_internal(M, fr(M).cp.p, fr(M).cq.p, M.tmp.p, (float2 *)y_dev, true, false, nullptr, M.s);
         check_err(M);
-        join_streams(M.s, us);
+        join_streams(M, M.s, us);
         return resolution_warning(M, freq_hz, medium);
     } catch (Fail &f) {
         return f.code;
@@ -2642,9 +2664,7 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
         cudaStream_t s = M.s;
         const int64_t n = M.n;
         // right-hand side: incident field minus the known boundary data
-        std::vector<SourceDev> sv = sources_of(srcs, n_src);
-        DevArr<SourceDev> &sdev = M.srcbuf;
-        sdev.upload(sv, s);
+        SourceDev *sdev = upload_sources(M, srcs, n_src);
         M.bvec.alloc((size_t)nr * n);
         M.uvec.alloc((size_t)nr * n);
         if (nr > 1) {
@@ -2652,14 +2672,14 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
             for (int r = 0; r < nr; ++r) {
                 {
                     KTimer kt_("k_rhs", s);
-                    k_rhs<<<nblocks(n, 256), 256, 0, s>>>(M.cd.p, M.nrm.p, n, P.k, sdev.p + r, 1, M.bvec.p + r * n);
+                    k_rhs<<<nblocks(n, 256), 256, 0, s>>>(M.cd.p, M.nrm.p, n, P.k, sdev + r, 1, M.bvec.p + r * n);
                 }
                 ck_launch("k_rhs");
             }
         } else if (n_src > 0) {
             {
                 KTimer kt_("k_rhs", s);
-                k_rhs<<<nblocks(n, 256), 256, 0, s>>>(M.cd.p, M.nrm.p, n, P.k, sdev.p, n_src, M.bvec.p);
+                k_rhs<<<nblocks(n, 256), 256, 0, s>>>(M.cd.p, M.nrm.p, n, P.k, sdev, n_src, M.bvec.p);
             }
             ck_launch("k_rhs");
         } else {
@@ -2724,7 +2744,7 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
             ck_launch("k_pq");
         }
         check_err(M);
-        join_streams(s, us);
+        join_streams(M, s, us);
         ck(cudaStreamSynchronize(us), "sync");
         resolve_timing();
         bool all_conv = true;
@@ -2786,6 +2806,7 @@ void swap_frames(Frame &a, Frame &b)
     a.vtmp.swap(b.vtmp);
     a.vout.swap(b.vout);
     std::swap(a.known_nonzero, b.known_nonzero);
+    a.coef_key.swap(b.coef_key);
 }
 
 }  // namespace
@@ -2801,9 +2822,8 @@ int bem_solve(void *mesh, double freq_hz, const bem_medium *medium, const double
     auto &M = *(bem_mesh_impl *)mesh;
     try {
         cudaStream_t us = (cudaStream_t)stream;
-        Coeffs C;
-        join_streams(us, M.s);
-        prepare(M, freq_hz, medium, admittance, n_regions, C);
+        join_streams(M, us, M.s);
+        prepare(M, freq_hz, medium, admittance, n_regions);
         ck(cudaStreamSynchronize(M.s), "sync");
         return solve_frame(M, freq_hz, medium, srcs, n_src, tol, max_iter, p_dev, q_dev, info, us, t0,
                            std::chrono::steady_clock::now());
@@ -2824,9 +2844,8 @@ int bem_solve_multi(void *mesh, double freq_hz, const bem_medium *medium, const 
     auto &M = *(bem_mesh_impl *)mesh;
     try {
         cudaStream_t us = (cudaStream_t)stream;
-        Coeffs C;
-        join_streams(us, M.s);
-        prepare(M, freq_hz, medium, admittance, n_regions, C);
+        join_streams(M, us, M.s);
+        prepare(M, freq_hz, medium, admittance, n_regions);
         ck(cudaStreamSynchronize(M.s), "sync");
         return solve_frame(M, freq_hz, medium, srcs, n_rhs, tol, max_iter, p_dev, q_dev, infos, us, t0,
                            std::chrono::steady_clock::now(), n_rhs);
@@ -2853,11 +2872,10 @@ int bem_solve_sweep(void *mesh, const double *freqs_hz, int32_t n_freq, const be
     std::string worst_msg;
     try {
         cudaStream_t us = (cudaStream_t)stream;
-        join_streams(us, M.s);
+        join_streams(M, us, M.s);
         auto t0 = std::chrono::steady_clock::now();
         {
-            Coeffs C;
-            prepare(M, freqs_hz[0], medium, admittance, n_regions, C);
+            prepare(M, freqs_hz[0], medium, admittance, n_regions);
             ck(cudaStreamSynchronize(M.s), "sync");
         }
         for (int32_t i = 0; i < n_freq; ++i) {
@@ -2873,8 +2891,7 @@ int bem_solve_sweep(void *mesh, const double *freqs_hz, int32_t n_freq, const be
                     t_frame = &M.next;
                     try {
                         ck(cudaSetDevice(M.device), "cudaSetDevice");
-                        Coeffs Cn;
-                        prepare(M, fn, medium, admittance, n_regions, Cn);
+                        prepare(M, fn, medium, admittance, n_regions);
                         ck(cudaStreamSynchronize(M.s_setup), "sync");
                     } catch (Fail &f) {
                         next_code = f.code;
@@ -2941,7 +2958,7 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
     if (!M.eval) M.eval = std::make_unique<EvalDev>();
     EvalDev &V = *M.eval;
     if (V.valid && V.np == np && V.key_k == k && V.key_depth == M.leaf_depth && V.key_trunc == M.prm.trunc_factor &&
-        std::equal(pts, pts + 3 * np, V.key_pts.begin()))
+        !memcmp(pts, V.key_pts.data(), 3 * (size_t)np * sizeof(double)))
         return;
     V.valid = false;
     EvalPlan ep;
@@ -3219,35 +3236,27 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
         ck(cudaSetDevice(M.device), "cudaSetDevice");
         ensure_work(M);
         cudaStream_t us = (cudaStream_t)stream;
-        join_streams(us, M.s);
+        join_streams(M, us, M.s);
         cudaStream_t s = M.s;
         const int64_t n = M.n;
         {
             KTimer kt_("k_gather", s);
-            k_gather<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)p_dev, M.perm.p, n, M.tmp.p);
+            k_gather2<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)p_dev, (const float2 *)q_dev, M.perm.p, n, M.tmp.p,
+                                                      M.tmp2.p);
         }
         ck_launch("k_gather");
-        {
-            KTimer kt_("k_gather", s);
-            k_gather<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)q_dev, M.perm.p, n, M.tmp2.p);
-        }
-        ck_launch("k_gather");
-        std::vector<double> hp(pts, pts + 3 * M_pts);
-        DevArr<double> &dp = M.ptsbuf;
-        dp.upload(hp, s);
-        std::vector<SourceDev> sv = sources_of(srcs, n_src);
-        DevArr<SourceDev> &sdev = M.srcbuf;
-        sdev.upload(sv, s);
+        SourceDev *sdev = upload_sources(M, srcs, n_src);
         reset_err(M);
         const double k = wavenumber(freq_hz, c);
         if (M.prm.mode == BEM_MODE_FMM &&
             (M.prm.field_mode == 2 || (M.prm.field_mode == 0 && (double)M_pts * (double)n >= kFieldFmmMinPairs))) {
-            field_fmm(M, k, pts, M_pts, M.tmp.p, M.tmp2.p, sdev.p, n_src, (float2 *)out_dev, s);
+            field_fmm(M, k, pts, M_pts, M.tmp.p, M.tmp2.p, sdev, n_src, (float2 *)out_dev, s);
             check_err(M);
-            join_streams(s, us);
+            join_streams(M, s, us);
             resolve_timing();
             return BEM_OK;
         }
+        const double *dp = upload_points(M, pts, M_pts);
         // each point's element sum split over S blocks when the points alone
         // would leave SMs idle (partials added in slice order)
         int nsm = 0;
@@ -3258,9 +3267,9 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
         if (S > 1) M.fieldpart.alloc((size_t)M_pts * S);
         {
             KTimer kt_("k_field", s);
-            k_field<<<dim3((unsigned)M_pts, (unsigned)S), 256, 0, s>>>(M.elem(), M.Q.p, dp.p, M_pts, (float)k,
+            k_field<<<dim3((unsigned)M_pts, (unsigned)S), 256, 0, s>>>(M.elem(), M.Q.p, dp, M_pts, (float)k,
                                                                       (float)M.prm.tau, M.tmp.p, M.tmp2.p,
-                                                                      sdev.p, n_src,
+                                                                      sdev, n_src,
                                                                       M.fieldpart.p, (float2 *)out_dev,
                                                                       fr(M).err.p);
         }
@@ -3268,13 +3277,13 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
         if (S > 1) {
             {
                 KTimer kt_("k_field", s);
-                k_field_finish<<<nblocks(M_pts, 128), 128, 0, s>>>(dp.p, M_pts, S, (float)k, sdev.p, n_src,
+                k_field_finish<<<nblocks(M_pts, 128), 128, 0, s>>>(dp, M_pts, S, (float)k, sdev, n_src,
                                                                   M.fieldpart.p, (float2 *)out_dev);
             }
             ck_launch("k_field_finish");
         }
         check_err(M);
-        join_streams(s, us);
+        join_streams(M, s, us);
         resolve_timing();
         return BEM_OK;
     } catch (Fail &f) {
@@ -3299,28 +3308,20 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         ck(cudaSetDevice(M.device), "cudaSetDevice");
         ensure_work(M);
         cudaStream_t us = (cudaStream_t)stream;
-        join_streams(us, M.s);
+        join_streams(M, us, M.s);
         cudaStream_t s = M.s;
         const int64_t n = M.n;
         {
             KTimer kt_("k_gather", s);
-            k_gather<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)p_dev, M.perm.p, n, M.tmp.p);
+            k_gather2<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)p_dev, (const float2 *)q_dev, M.perm.p, n, M.tmp.p,
+                                                      M.tmp2.p);
         }
         ck_launch("k_gather");
-        {
-            KTimer kt_("k_gather", s);
-            k_gather<<<nblocks(n, 256), 256, 0, s>>>((const float2 *)q_dev, M.perm.p, n, M.tmp2.p);
-        }
-        ck_launch("k_gather");
-        std::vector<double> hp(pts, pts + 3 * M_pts);
-        DevArr<double> &dp = M.ptsbuf;
-        dp.upload(hp, s);
-        std::vector<SourceDev> sv = sources_of(srcs, n_src);
-        DevArr<SourceDev> &sdev = M.srcbuf;
-        sdev.upload(sv, s);
+        SourceDev *sdev = upload_sources(M, srcs, n_src);
         reset_err(M);
         const double k = wavenumber(freq_hz, c);
         const float inv_omega_rho = (float)(1.0 / (2.0 * 3.14159265358979323846 * freq_hz * rho));
+        const double *dp = upload_points(M, pts, M_pts);
         // blocks per point as for the field (partials added in slice order)
         int nsm = 0;
         ck(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, M.device), "attribute");
@@ -3331,8 +3332,8 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         {
             KTimer kt_("k_field_velocity", s);
             k_field_velocity<<<dim3((unsigned)M_pts, (unsigned)S), 256, 0, s>>>(
-                M.elem(), M.Q.p, dp.p, M_pts, (float)k, (float)M.prm.tau, inv_omega_rho, M.tmp.p, M.tmp2.p,
-                sdev.p, n_src,
+                M.elem(), M.Q.p, dp, M_pts, (float)k, (float)M.prm.tau, inv_omega_rho, M.tmp.p, M.tmp2.p,
+                sdev, n_src,
                 M.fieldpart.p, (float2 *)v_out_dev, fr(M).err.p);
         }
         ck_launch("k_field_velocity");
@@ -3340,12 +3341,12 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
             {
                 KTimer kt_("k_field_velocity", s);
                 k_field_velocity_finish<<<nblocks(M_pts, 128), 128, 0, s>>>(
-                    dp.p, M_pts, S, (float)k, inv_omega_rho, sdev.p, n_src, M.fieldpart.p, (float2 *)v_out_dev);
+                    dp, M_pts, S, (float)k, inv_omega_rho, sdev, n_src, M.fieldpart.p, (float2 *)v_out_dev);
             }
             ck_launch("k_field_velocity_finish");
         }
         check_err(M);
-        join_streams(s, us);
+        join_streams(M, s, us);
         resolve_timing();
         return BEM_OK;
     } catch (Fail &f) {
@@ -3379,16 +3380,15 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         M.uadj.alloc(n);
         M.fadj.alloc(n_pts);
         M.gadj.alloc(n);
-        join_streams(us, s);
+        join_streams(M, us, s);
         ck(cudaMemcpyAsync(M.uadj.p, M.uvec.p, n * sizeof(float2), cudaMemcpyDeviceToDevice, s), "D2D u");
-        join_streams(s, us);
+        join_streams(M, s, us);
         const int ev = bem_evaluate(mesh, freq_hz, medium, srcs, n_src, p_dev, q_dev, pts, n_pts, M.fadj.p, stream);
         if (ev < 0) return ev;
-        join_streams(us, s);
+        join_streams(M, us, s);
         reset_err(M);
         // adjoint right-hand side F^T conj(f) into b, and G_f^T conj(f)
-        std::vector<double> hp(pts, pts + 3 * n_pts);
-        M.ptsbuf.upload(hp, s);
+        upload_points(M, pts, n_pts);
         M.bvec.alloc(n);
         {
             KTimer kt_("k_field_t", s);
@@ -3401,17 +3401,20 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         GmresResult R = run_gmres(M, tol, max_iter, true);
         // aq = A_q^T lambda: the transposed product with c^p = 0 and c^q = 1
         // (tau folded in as for the unknowns' coefficients)
-        std::vector<float2> h0((size_t)n, make_float2(0.f, 0.f)), hq((size_t)n, make_float2(tau, 0.f));
-        M.adj_cp.upload(h0, s);
-        M.adj_cq.upload(hq, s);
+        if (M.adjreg.n != (size_t)n) {
+            // the same for every gradient of the mesh
+            std::vector<float2> h0((size_t)n, make_float2(0.f, 0.f)), hq((size_t)n, make_float2(tau, 0.f));
+            M.adj_cp.upload(h0, s);
+            M.adj_cq.upload(hq, s);
+            std::vector<int> reg((size_t)n);
+            for (int64_t i = 0; i < n; ++i) {
+                const int64_t e = M.t.perm[i];
+                reg[i] = M.bct[e] == BEM_ADMI ? M.region[e] : -1;
+            }
+            M.adjreg.upload(reg, s);
+        }
         matvec_t_internal(M, M.adj_cp.p, M.adj_cq.p, M.uvec.p, M.w.p, false, false, nullptr, s);
         // per-region sums and the loss
-        std::vector<int> reg((size_t)n);
-        for (int64_t i = 0; i < n; ++i) {
-            const int64_t e = M.t.perm[i];
-            reg[i] = M.bct[e] == BEM_ADMI ? M.region[e] : -1;
-        }
-        M.adjreg.upload(reg, s);
         const int nacc = 2 * n_regions + 1;
         M.adjacc.alloc(nacc);
         ck(cudaMemsetAsync(M.adjacc.p, 0, nacc * sizeof(double), s), "memset acc");
@@ -3425,7 +3428,7 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         std::vector<double> hacc(nacc);
         ck(cudaMemcpyAsync(hacc.data(), M.adjacc.p, nacc * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H acc");
         check_err(M);
-        join_streams(s, us);
+        join_streams(M, s, us);
         ck(cudaStreamSynchronize(s), "sync");
         resolve_timing();
         *loss = hacc[2 * n_regions];

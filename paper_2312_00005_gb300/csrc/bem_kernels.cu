@@ -2267,6 +2267,62 @@ __global__ void k_gather(const float2 *__restrict__ x, const int64_t *__restrict
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) y[i] = x[perm[i]];
 }
+__global__ void k_gather2(const float2 *__restrict__ x0, const float2 *__restrict__ x1,
+                          const int64_t *__restrict__ perm, int64_t n, float2 *__restrict__ y0, float2 *__restrict__ y1)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int64_t j = perm[i];
+    y0[i] = x0[j];
+    y1[i] = x1[j];
+}
+// The boundary conditions folded into column coefficients (Eq. SystemI):
+// column j enters as p_j = cp u_j, q_j = cq u_j, with (1, 0) for VELO, (1, a)
+// for ADMI, a = -tau i k rho c Y (Y = velocity into the wall / p; the wall lies
+// along the normal for the interior problem, against it for the exterior
+// one), and (0, 1) for PRES; (cp0, cq0) and z the same for the known data
+// g = i w rho v and p.  tau multiplies every integral operator, so all but
+// aq and z carry it.  Formed here from the boundary data on the device: on
+// the host, the six vectors, their uploads and a comparison with the last
+// call's took 0.17 ms of every product on 20,480 elements and 2.9 ms on
+// 158,420; this takes one launch when something changed.
+__global__ void k_coeffs(int64_t n, const int *__restrict__ type, const double2 *__restrict__ bcv,
+                         const int *__restrict__ region, const double *__restrict__ adm, double k, double omega,
+                         double rho, double c, double tau, float2 *__restrict__ cp, float2 *__restrict__ cq,
+                         float2 *__restrict__ cp0, float2 *__restrict__ cq0, float2 *__restrict__ z,
+                         float2 *__restrict__ aq)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int ty = type[i];
+    const double2 v = bcv[i];
+    const float2 one = make_float2(1.f, 0.f), zero = make_float2(0.f, 0.f);
+    float2 p = zero, q = zero, p0 = zero, q0 = zero, zz, a = zero;
+    if (ty == BEM_PRES) {
+        q = p0 = one;
+        zz = make_float2((float)v.x, (float)v.y);
+    } else {
+        p = q0 = one;
+        zz = make_float2((float)(-omega * rho * v.y), (float)(omega * rho * v.x));
+        if (ty == BEM_ADMI) {
+            const int r = region[i];
+            const double br = tau * rho * c * adm[2 * r], bi = tau * rho * c * adm[2 * r + 1];
+            q = a = make_float2((float)(k * bi), (float)(-k * br));
+        }
+    }
+    z[i] = zz;
+    aq[i] = a;
+    if (tau < 0) {
+        p = make_float2(-p.x, -p.y);
+        q = make_float2(-q.x, -q.y);
+        p0 = make_float2(-p0.x, -p0.y);
+        q0 = make_float2(-q0.x, -q0.y);
+    }
+    cp[i] = p;
+    cq[i] = q;
+    cp0[i] = p0;
+    cq0[i] = q0;
+}
 // Iterative refinement of a mixed-precision solve: r = b - y in FP64 from the
 // FP32 right-hand side and product (y = A x with the FP32 products), stored
 // as FP32 in r; part[blockIdx.x] = the block's ||r||^2 in FP64.

@@ -365,6 +365,12 @@ __global__ void k_field_velocity(ElemDev E, const QuadTables *Q, const double *p
 __global__ void k_field_velocity_finish(const double *pts, int64_t M, int S, float k, float inv_omega_rho,
                                         const SourceDev *src, int nsrc, const float2 *part, float2 *out);
 __global__ void k_gather(const float2 *x, const int64_t *perm, int64_t n, float2 *y);
+__global__ void k_gather2(const float2 *x0, const float2 *x1, const int64_t *perm, int64_t n, float2 *y0, float2 *y1);
+// Column coefficients of the unknowns (cp, cq) and of the known data (cp0,
+// cq0), the known data z and the relation q = aq p, from the boundary data.
+__global__ void k_coeffs(int64_t n, const int *type, const double2 *bcv, const int *region, const double *adm, double k,
+                         double omega, double rho, double c, double tau, float2 *cp, float2 *cq, float2 *cp0, float2 *cq0,
+                         float2 *z, float2 *aq);
 // FMM evaluation of the field at points (see the definitions)
 __global__ void k_field_weights(int64_t n, const float2 *p, const float2 *q, const float4 *chi, float k, float4 *wts);
 __global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, const float2 *p,
