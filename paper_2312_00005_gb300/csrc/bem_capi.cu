@@ -1358,7 +1358,7 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
         const int cw = std::max(2, std::min(ncp, M.prm.near_chunk > 0 ? M.prm.near_chunk : kSpmvMultiChunk));
         if (P.lists->n_spmv_items > 0) {
             KTimer kt_("k_near_spmv", s);
-            k_near_spmv_items_multi<<<P.lists->n_spmv_items, kSpmvThreads, (size_t)nr * cw * sizeof(float2), s>>>(
+            k_near_spmv_items_multi<<<P.lists->n_spmv_items, kSpmvMultiThreads, (size_t)nr * cw * sizeof(float2), s>>>(
                 na, P.lists->spmv_items.p, P.val.p, M.xint.p, M.ynear.p, nr, n, cw, skip);
         }
         ck_launch("k_near_spmv");

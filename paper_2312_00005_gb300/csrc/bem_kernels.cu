@@ -546,7 +546,7 @@ __device__ __forceinline__ void spmv_segment_multi(const float2 *__restrict__ v,
     for (int r = 0; r < kMaxPlanes; ++r) out[r] = warp_sum(cadd(acc0[r], acc1[r]));
 }
 
-__global__ void __launch_bounds__(kSpmvThreads) k_near_spmv_items_multi(NearArgs a, const int4 *__restrict__ items,
+__global__ void __launch_bounds__(kSpmvMultiThreads) k_near_spmv_items_multi(NearArgs a, const int4 *__restrict__ items,
                                                                         const float2 *__restrict__ val,
                                                                         const float2 *__restrict__ x,
                                                                         float2 *__restrict__ y, int nr, int64_t plane,
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_near_spmv_items_multi(NearArgs
 {
     if (skip_now(skip)) return;
     extern __shared__ float2 xs[];            // [nr][cw]: one chunk of the leaf's columns
-    constexpr int kW = kSpmvThreads / 32;
+    constexpr int kW = kSpmvMultiThreads / 32;
     __shared__ float2 part[kMaxPlanes][kSpmvMaxItemRows][kW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 W = items[blockIdx.x];
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_near_spmv_items_multi(NearArgs
     const int nc = a.N.ncol[t];
     const int ncp = (nc + 1) & ~1;
     const int run0 = a.N.run_ptr[t], run1 = a.N.run_ptr[t + 1];
-    for (int q = threadIdx.x; q < kMaxPlanes * kSpmvMaxItemRows * kW; q += kSpmvThreads)
+    for (int q = threadIdx.x; q < kMaxPlanes * kSpmvMaxItemRows * kW; q += kSpmvMultiThreads)
         (&part[0][0][0])[q] = make_float2(0.f, 0.f);
     const int64_t i0 = a.N.leaf_start[t] + W.y;
     const int nrow = min(W.z - W.y, kSpmvMaxItemRows);
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(kSpmvThreads) k_near_spmv_items_multi(NearArgs
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < nrow * nr; q += kSpmvThreads) {
+    for (int q = threadIdx.x; q < nrow * nr; q += kSpmvMultiThreads) {
         const int row = q % nrow, pl = q / nrow;
         float2 sum = part[pl][row][0];
 #pragma unroll

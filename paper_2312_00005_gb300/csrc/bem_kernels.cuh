@@ -200,7 +200,12 @@ __global__ void k_near_transpose(const int64_t *leaf_start, const int *trow_ptr,
 // apart in x and y): the stored values are streamed once for all of them.
 // The leaf's columns are staged in chunks of cw (even) columns: dynamic
 // shared memory nr * cw * 8 bytes, small enough for several blocks per SM.
-constexpr int kSpmvMultiChunk = 512;
+// Eight warps share a chunk of 1024 (four planes: 71 us on 10,580 elements,
+// 594 on 158,420); with four warps and 512 the block waits more often for its
+// columns (102 and 602 us), larger chunks leave too few blocks on an SM beside
+// the far-field kernels (alone 64 us, but 10 % slower GMRES steps).
+constexpr int kSpmvMultiChunk = 1024;
+constexpr int kSpmvMultiThreads = 256;
 __global__ void k_near_spmv_items_multi(NearArgs a, const int4 *items, const float2 *val, const float2 *x, float2 *y,
                                         int nr, int64_t plane, int cw, const int *skip);
 // Near-field product with recomputed entries for 1, 2 or 4 right-hand sides
