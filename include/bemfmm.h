@@ -138,7 +138,8 @@ typedef struct bem_params {
                                of the row sums.  Other values: BEM_E_ARG.                     */
     int32_t gs_rows;        /* GMRES Gram-Schmidt step: rows of the basis per block (its sums
                                are FP64 atomic additions of the blocks' partials, one per
-                               basis column and block).  0 (default): 128, or more to keep the
+                               basis column and block).  0 (default): 128 (64 up to
+                               4096 elements), or more to keep the
                                blocks at most 1024; 64..1024 otherwise.  Results agree to the
                                summation order.  Other values: BEM_E_ARG.                     */
     int32_t field_mode;     /* bem_evaluate: 1 the direct sum over every element with the rules

@@ -39,6 +39,7 @@ constexpr int kNoErr = 0x7f7f7f7f;       // an error flag that no element has lo
 constexpr int kBacksolveCols = 155;
 // values per work item of the stored near-field product
 constexpr int64_t kSpmvItemEntries = 65536;
+constexpr int64_t kSpmvMinEntries = 4096;   // smaller items: mostly staging of x
 
 // ------------------------------------------------------------------ errors
 static thread_local std::string g_err;
@@ -283,6 +284,8 @@ struct Lists {
     DevArr<int64_t> row_ptr;
     DevArr<int4> spmv_items;      // (leaf, first row, end row) work items of the product
     int n_spmv_items = 0;
+    DevArr<int4> multi_items;     // the same for several right-hand sides
+    int n_multi_items = 0;
     DevArr<int4> fused_tasks;     // (leaf, first row, end row) of the recomputed product (internal rows)
     int n_fused = 0, fused_s = 1; // ... and the parts of the columns
     int64_t nnz = 0;
@@ -619,20 +622,37 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
     Ls->runs.upload(runs, s);
     Ls->row_ptr.upload(row_ptr, s);
     {
-        // about kSpmvItemEntries values per item (at most kSpmvMaxItemRows
-        // rows), a leaf's rows split evenly
-        std::vector<int4> items;
-        for (int t = 0; t < nl; ++t) {
-            const int rows = (int)Lf.count[t];
-            if (rows == 0) continue;
-            const int rpi = (int)std::max<int64_t>(1, std::min<int64_t>(kSpmvMaxItemRows,
-                                                                        kSpmvItemEntries / std::max(1, ncol[t])));
-            const int nit = (rows + rpi - 1) / rpi;
-            for (int q = 0; q < nit; ++q)
-                items.push_back(make_int4(t, (int)((int64_t)rows * q / nit), (int)((int64_t)rows * (q + 1) / nit), 0));
-        }
+        // at most `entries` values per item (and kSpmvMaxItemRows rows), a
+        // leaf's rows split evenly
+        auto cut = [&](int64_t entries) {
+            std::vector<int4> items;
+            for (int t = 0; t < nl; ++t) {
+                const int rows = (int)Lf.count[t];
+                if (rows == 0) continue;
+                const int rpi =
+                    (int)std::max<int64_t>(1, std::min<int64_t>(kSpmvMaxItemRows, entries / std::max(1, ncol[t])));
+                const int nit = (rows + rpi - 1) / rpi;
+                for (int q = 0; q < nit; ++q)
+                    items.push_back(make_int4(t, (int)((int64_t)rows * q / nit), (int)((int64_t)rows * (q + 1) / nit), 0));
+            }
+            return items;
+        };
+        // One right-hand side: kSpmvItemEntries, and less where that leaves an
+        // SM under 4 items (2240 elements: product 18 -> 10 us alone, solve 8.2
+        // -> 7.7 ms; 2880: steps 76 -> 66 us) or, where the near field is most
+        // of the product (over 2500 columns a row; 3200 on 9680 elements: 75 ->
+        // 65 us, gradient 14.6 -> 13.6 ms), under 8.  With 1700 columns a row
+        // the far-field kernels set the step's time, and 8 items an SM beside
+        // them cost 4 % (13,520 and 20,480 elements).
+        int nsm = 0;
+        ck(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, M.device), "attribute");
+        const int64_t per_sm = row_ptr[M.n] > 2500 * M.n ? 8 : 4;
+        const int64_t fine = std::max(kSpmvMinEntries, row_ptr[M.n] / (per_sm * nsm));
+        const std::vector<int4> items = cut(std::min(kSpmvItemEntries, fine)), multi = cut(kSpmvItemEntries);
         Ls->n_spmv_items = (int)items.size();
         Ls->spmv_items.upload(items, s);
+        Ls->n_multi_items = (int)multi.size();
+        Ls->multi_items.upload(multi, s);
         std::vector<int4> ft;
         for (int t = 0; t < nl; ++t) {
             const int64_t a = leaf_start[t], cnt = Lf.count[t];
@@ -1356,10 +1376,10 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
         // columns staged in chunks
         const int ncp = (P.lists->max_ncol + 1) & ~1;
         const int cw = std::max(2, std::min(ncp, M.prm.near_chunk > 0 ? M.prm.near_chunk : kSpmvMultiChunk));
-        if (P.lists->n_spmv_items > 0) {
+        if (P.lists->n_multi_items > 0) {
             KTimer kt_("k_near_spmv", s);
-            k_near_spmv_items_multi<<<P.lists->n_spmv_items, kSpmvMultiThreads, (size_t)nr * cw * sizeof(float2), s>>>(
-                na, P.lists->spmv_items.p, P.val.p, M.xint.p, M.ynear.p, nr, n, cw, skip);
+            k_near_spmv_items_multi<<<P.lists->n_multi_items, kSpmvMultiThreads, (size_t)nr * cw * sizeof(float2), s>>>(
+                na, P.lists->multi_items.p, P.val.p, M.xint.p, M.ynear.p, nr, n, cw, skip);
         }
         ck_launch("k_near_spmv");
     } else if (use_store && M.prm.near_store && !P.fp().direct) {
@@ -2241,11 +2261,12 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     // the Gram-Schmidt step: block b owns rows [b R, b R + R), R <= kGsMaxRows
     // (staged in shared memory); 128 rows per block (measured against 64,
     // 256 and 512: 64 made twice the atomic additions, the larger ones kept
-    // fewer loads of the basis in flight), and more when that would exceed
-    // about 1024 blocks
+    // fewer loads of the basis in flight), 64 up to 4096 rows, where 128 keep
+    // only a fifth of the SMs busy (2240: steps 53 -> 50 us; 5120: equal), and
+    // more when that would exceed about 1024 blocks
     int nblk = 0;
     {
-        const int64_t rows = M.prm.gs_rows > 0 ? (int64_t)M.prm.gs_rows : std::max<int64_t>(128, (n + 1023) / 1024);
+        const int64_t rows = M.prm.gs_rows > 0 ? (int64_t)M.prm.gs_rows : std::max<int64_t>(n <= 4096 ? 64 : 128, (n + 1023) / 1024);
         nblk = (int)std::max<int64_t>(1, (n + rows - 1) / rows);
     }
     const int orows = (int)((n + nblk - 1) / nblk);
