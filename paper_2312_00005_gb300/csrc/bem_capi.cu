@@ -424,7 +424,7 @@ struct EvalDev {
     DevArr<unsigned int> red_cnt;
     DevArr<int4> tgroups;
     DevArr<LevelsArgs> largs;
-    DevArr<int> pleaf, nptr;
+    DevArr<int> pleaf, nptr, ntot;
     DevArr<double> pts;
     DevArr<int64_t> perm;
     DevArr<float4> wts, zeros;
@@ -1821,6 +1821,10 @@ const double *upload_points(bem_mesh_impl &M, const double *pts, int64_t n)
     return M.ptsbuf.p;
 }
 
+// Parts of the elements of a direct field sum: blocks enough for several
+// rounds on every SM (at most 64 parts, which one thread per point adds).
+int field_parts(int64_t M_pts, int64_t n) { return std::min(64, fused_parts((M_pts + 31) / 32, n)); }
+
 // to waits for what from holds (the mesh's event is recorded anew each time)
 void join_streams(bem_mesh_impl &M, cudaStream_t from, cudaStream_t to)
 {
@@ -2999,19 +3003,21 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         for (int64_t i = ep.leaf_start[c]; i < ep.leaf_start[c + 1]; ++i) pleaf[i] = c;
     V.pleaf.upload(pleaf, s);
     const Level &EL = M.t.lv[ep.leaf_depth];
-    std::vector<int> nptr(npl + 1, 0);
-    std::vector<int2> nruns;
+    std::vector<int> nptr(npl + 1, 0), ntot(npl, 0);
+    std::vector<int2> nruns;                   // (first element, first position in the leaf's list)
     for (int c = 0; c < npl; ++c) {
-        int prev = -2;
+        int prev = -2, pos = 0;
         for (int q2 = ep.near_ptr[c]; q2 < ep.near_ptr[c + 1]; ++q2) {
             const int sl = ep.near_src[q2];
             if (EL.count[sl] == 0) continue;
-            if (sl == prev + 1) nruns.back().y += (int)EL.count[sl];   // consecutive leaves: one run
-            else nruns.push_back(make_int2((int)EL.start[sl], (int)EL.count[sl]));
+            if (sl != prev + 1) nruns.push_back(make_int2((int)EL.start[sl], pos));   // consecutive leaves: one run
+            pos += (int)EL.count[sl];
             prev = sl;
         }
         nptr[c + 1] = (int)nruns.size();
+        ntot[c] = pos;
     }
+    V.ntot.upload(ntot, s);
     V.nptr.upload(nptr, s);
     V.nruns.upload(nruns, s);
     V.vnear.alloc(np);
@@ -3198,7 +3204,7 @@ void field_fmm(bem_mesh_impl &M, double k, const double *pts, int64_t np, const 
     {
         KTimer kt_("k_field_near", s);
         k_field_near<<<nblocks(np, 8), 256, 0, s>>>(M.elem(), M.Q.p, V.pts.p, np, (float)k, p, q, V.pleaf.p,
-                                                   V.nptr.p, V.nruns.p, V.vnear.p, fr(M).err.p);
+                                                   V.nptr.p, V.ntot.p, V.nruns.p, V.vnear.p, fr(M).err.p);
     }
     ck_launch("k_field_near");
     const float2 *vres = V.vnear.p;
@@ -3278,17 +3284,11 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
             return BEM_OK;
         }
         const double *dp = upload_points(M, pts, M_pts);
-        // each point's element sum split over S blocks when the points alone
-        // would leave SMs idle (partials added in slice order)
-        int nsm = 0;
-        ck(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, M.device), "attribute");
-        const int64_t want = 8 * (int64_t)nsm;
-        const int S = (int)std::max<int64_t>(1, std::min<int64_t>({16, (want + M_pts - 1) / M_pts,
-                                                                   (n + 255) / 256}));
+        const int S = field_parts(M_pts, n);
         if (S > 1) M.fieldpart.alloc((size_t)M_pts * S);
         {
             KTimer kt_("k_field", s);
-            k_field<<<dim3((unsigned)M_pts, (unsigned)S), 256, 0, s>>>(M.elem(), M.Q.p, dp, M_pts, (float)k,
+            k_field<<<dim3(nblocks(M_pts, 32), (unsigned)S), kFusedThreads, 0, s>>>(M.elem(), M.Q.p, dp, M_pts, (float)k,
                                                                       (float)M.prm.tau, M.tmp.p, M.tmp2.p,
                                                                       sdev, n_src,
                                                                       M.fieldpart.p, (float2 *)out_dev,
@@ -3343,16 +3343,11 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         const double k = wavenumber(freq_hz, c);
         const float inv_omega_rho = (float)(1.0 / (2.0 * 3.14159265358979323846 * freq_hz * rho));
         const double *dp = upload_points(M, pts, M_pts);
-        // blocks per point as for the field (partials added in slice order)
-        int nsm = 0;
-        ck(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, M.device), "attribute");
-        const int64_t want = 8 * (int64_t)nsm;
-        const int S = (int)std::max<int64_t>(1, std::min<int64_t>({16, (want + M_pts - 1) / M_pts,
-                                                                   (n + 255) / 256}));
+        const int S = field_parts(M_pts, n);
         if (S > 1) M.fieldpart.alloc((size_t)M_pts * S * 3);
         {
             KTimer kt_("k_field_velocity", s);
-            k_field_velocity<<<dim3((unsigned)M_pts, (unsigned)S), 256, 0, s>>>(
+            k_field_velocity<<<dim3(nblocks(M_pts, 32), (unsigned)S), kFusedThreads, 0, s>>>(
                 M.elem(), M.Q.p, dp, M_pts, (float)k, (float)M.prm.tau, inv_omega_rho, M.tmp.p, M.tmp2.p,
                 sdev, n_src,
                 M.fieldpart.p, (float2 *)v_out_dev, fr(M).err.p);

@@ -2026,11 +2026,8 @@ __global__ void k_rhs(const double *__restrict__ cd, const float4 *__restrict__ 
 
 // ------------------------------------------------------------------ field evaluation
 // p(x) = p_inc(x) + tau sum_j [H(x)_j p_j - G(x)_j q_j] (Eq. BIE_I, lambda =
-// 1; tau = +1 at exterior points, -1 at interior points).  Block (m, s)
-// takes field point m and every S-th slice of blockDim elements from slice
-// s, threads over elements.  With S = 1 the block adds
-// the incident field and writes p(x_m); otherwise it leaves its partial sum
-// in part[m S + s] and k_field_finish adds the S partials in slice order.
+// 1; tau = +1 at exterior points, -1 at interior points): the incident field
+// of the sources at x, added to (br, bi).
 __device__ void field_incident(const double *xd, float k, const SourceDev *__restrict__ src, int nsrc, double &br,
                                double &bi)
 {
@@ -2050,128 +2047,6 @@ __device__ void field_incident(const double *xd, float k, const SourceDev *__res
         br += S.amp[0] * gr - S.amp[1] * gi;
         bi += S.amp[0] * gi + S.amp[1] * gr;
     }
-}
-
-__global__ void k_field(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, int64_t M,
-                        float k, float tau, const float2 *__restrict__ p, const float2 *__restrict__ q,
-                        const SourceDev *__restrict__ src, int nsrc, float2 *__restrict__ part,
-                        float2 *__restrict__ out, int *err)
-{
-    const int64_t m = blockIdx.x;
-    const int S = gridDim.y, sl = blockIdx.y;
-    if (m >= M) return;
-    const QuadTables &Q = *Qp;
-    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
-    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
-    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
-                                   (float)(xd[2] - (double)xhi.z));
-    float2 acc = make_float2(0.f, 0.f);
-    for (int64_t j = (int64_t)sl * blockDim.x + threadIdx.x; j < E.n; j += (int64_t)S * blockDim.x) {
-        float2 G = make_float2(0.f, 0.f), H = make_float2(0.f, 0.f);
-        if (!integrate_regular<true>(E, j, xhi, xlo, xd, make_float3(0.f, 0.f, 1.f), k, 1.0f / k, Q, G, H)) {
-            atomicMin(err, (int)j);
-            continue;
-        }
-        acc = cadd(acc, csub(cmul(H, p[j]), cmul(G, q[j])));
-    }
-    __shared__ float2 red[32];
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float2 v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : make_float2(0.f, 0.f);
-        v = warp_sum(v);
-        v = cscale(v, tau);      // tau on the integral part (Eq. BIE_I)
-        if (threadIdx.x == 0) {
-            if (S > 1) {
-                part[m * S + sl] = v;
-            } else {
-                double br = v.x, bi = v.y;
-                field_incident(xd, k, src, nsrc, br, bi);
-                out[m] = make_float2((float)br, (float)bi);
-            }
-        }
-    }
-}
-
-// The S partial sums of each field point in slice order, plus the incident
-// field; one thread per point.
-__global__ void k_field_finish(const double *__restrict__ pts, int64_t M, int S, float k,
-                               const SourceDev *__restrict__ src, int nsrc, const float2 *__restrict__ part,
-                               float2 *__restrict__ out)
-{
-    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    float2 v = part[m * S];
-    for (int s = 1; s < S; ++s) v = cadd(v, part[m * S + s]);
-    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
-    double br = v.x, bi = v.y;
-    field_incident(xd, k, src, nsrc, br, bi);
-    out[m] = make_float2((float)br, (float)bi);
-}
-
-// Far-field weights of the representation formula (Eq. BIE with lambda = 1)
-// for the aggregation T(l) (Sec. 3.3.3): with the one-point element rule,
-//   H_j p_j - G_j q_j ~ A_j (-q_j - ik (n_j.s) p_j) e^{ik (z_s - y_j).s} (...),
-// i.e. (alpha, c) = (-A q, -ik A p) in the form sum_j E_pj (alpha_j + t_pj c_j)
-// of the aggregation (internal element order).
-__global__ void k_field_weights(int64_t n, const float2 *__restrict__ p, const float2 *__restrict__ q,
-                                const float4 *__restrict__ chi, float k, float4 *__restrict__ wts)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float A = chi[i].w;
-    const float2 pv = p[i], qv = q[i];
-    wts[i] = make_float4(-A * qv.x, -A * qv.y, k * A * pv.y, -k * A * pv.x);
-}
-
-// Near part of the field at points (internal point order): the element
-// rules of k_field over the element runs (first element, count) of the
-// point's leaf near list, one warp per point; v_m = sum_j H_j p_j - G_j q_j.
-__global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, int64_t M,
-                             float k, const float2 *__restrict__ p, const float2 *__restrict__ q,
-                             const int *__restrict__ pleaf, const int *__restrict__ nptr,
-                             const int2 *__restrict__ nruns, float2 *__restrict__ v, int *err)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t m = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (m >= M) return;
-    const QuadTables &Q = *Qp;
-    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
-    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
-    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
-                                   (float)(xd[2] - (double)xhi.z));
-    const int pl = pleaf[m];
-    float2 acc = make_float2(0.f, 0.f);
-    for (int r = nptr[pl]; r < nptr[pl + 1]; ++r) {
-        const int2 run = nruns[r];
-        for (int u = lane; u < run.y; u += 32) {
-            const int64_t j = run.x + u;
-            float2 G = make_float2(0.f, 0.f), H = make_float2(0.f, 0.f);
-            if (!integrate_regular<true>(E, j, xhi, xlo, xd, make_float3(0.f, 0.f, 1.f), k, 1.0f / k, Q, G, H)) {
-                atomicMin(err, (int)j);
-                continue;
-            }
-            acc = cadd(acc, csub(cmul(H, p[j]), cmul(G, q[j])));
-        }
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) v[m] = acc;
-}
-
-// The field at the points: tau (near + far) plus the incident field (FP64),
-// written in caller order.
-__global__ void k_field_eval_finish(const double *__restrict__ pts, int64_t M, float k, float tau,
-                                    const SourceDev *__restrict__ src, int nsrc, const float2 *__restrict__ v,
-                                    const int64_t *__restrict__ perm, float2 *__restrict__ out)
-{
-    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
-    const float2 w = cscale(v[m], tau);
-    double br = w.x, bi = w.y;
-    field_incident(xd, k, src, nsrc, br, bi);
-    out[perm[m]] = make_float2((float)br, (float)bi);
 }
 
 // Gradient of the incident fields at x (FP64): plane wave grad p = ik d p,
@@ -2206,67 +2081,310 @@ __device__ void incident_grad(const double *xd, float k, const SourceDev *__rest
     }
 }
 
+// The quantity and its pair sums: the field (G and H, one complex sum) or its
+// gradient (grad G and grad H, three).
+template <bool kGrad> struct FieldPair;
+template <> struct FieldPair<false> {
+    static constexpr int kN = 1;
+    GhAcc acc;
+    __device__ __forceinline__ explicit FieldPair(float k) { acc = GhAcc{k, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+    // A1 = H, A0 = G
+    __device__ __forceinline__ void add(float2 *v, float2 p, float2 q) const
+    {
+        v[0] = cadd(v[0], csub(cmul(acc.A1, p), cmul(acc.A0, q)));
+    }
+};
+template <> struct FieldPair<true> {
+    static constexpr int kN = 3;
+    GradAcc acc;
+    __device__ __forceinline__ explicit FieldPair(float k)
+    {
+        acc.k = k;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) acc.gG[a] = acc.gH[a] = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ void add(float2 *v, float2 p, float2 q) const
+    {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a] = cadd(v[a], csub(cmul(acc.gH[a], p), cmul(acc.gG[a], q)));
+    }
+};
+// The contribution of element j at x by the general element rules.
+template <bool kGrad>
+__device__ __noinline__ bool field_entry(const ElemDev &E, const QuadTables &Q, int64_t j, const double *xd, float k,
+                                         float2 p, float2 q, float2 *v)
+{
+    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
+    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
+                                   (float)(xd[2] - (double)xhi.z));
+    FieldPair<kGrad> f(k);
+    const bool ok = integrate_regular_acc(E, j, xhi, xlo, xd, Q, f.acc);
+    for (int a = 0; a < FieldPair<kGrad>::kN; ++a) v[a] = make_float2(0.f, 0.f);
+    f.add(v, p, q);
+    return ok;
+}
+
+// Direct sum over every element at M points: p (k_field) or v (k_field_
+// velocity).  Bound by FP32 / SFU issue.  As in the recomputed product, a lane
+// holds a point, the elements are staged in shared memory and read as
+// broadcasts, and the far pairs (one quadrature point, nearly all) are
+// evaluated in place; the others are queued per block and worked off by all
+// its threads when the queue has filled and at the end, their sums FP64
+// additions.  Block (x, y) takes 32 points and every gridDim.y-th part of the
+// elements; with several parts they go to part[(m S + s) N + a] and the finish
+// kernels add them in order.  Lanes over the elements, one point per block
+// (112 bytes of element data through L1 per pair): 1000 points and 5120
+// elements 64 + 72 us (field + velocity); this 40 + 60; 8000 points and 8000
+// elements 640 -> 280 us.
+template <bool kGrad>
+__device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q, const double *__restrict__ pts,
+                                           int64_t M, float k, float tau, float inv_omega_rho,
+                                           const float2 *__restrict__ p, const float2 *__restrict__ q,
+                                           const SourceDev *__restrict__ src, int nsrc, float2 *__restrict__ part,
+                                           float2 *__restrict__ out, int *err)
+{
+    constexpr int kW = kFusedThreads / 32, kN = FieldPair<kGrad>::kN;
+    __shared__ float4 s_hi[kFusedTile], s_lo[kFusedTile], s_n[kFusedTile], s_pq[kFusedTile];
+    __shared__ int s_qj[kFieldQueue];
+    __shared__ unsigned char s_qr[kFieldQueue];
+    __shared__ int s_qn;
+    __shared__ double2 s_h[kN][32];
+    __shared__ double s_x[32][3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t m0 = (int64_t)blockIdx.x * 32;
+    const int cnt = (int)min((int64_t)32, M - m0);
+    int w = 1;
+    while (w < cnt) w <<= 1;
+    const int R = 32 / w, sub = lane / w, rr = lane % w;   // R elements side by side for fewer than 32 points
+    const bool live = rr < cnt;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int a = 0; a < kN; ++a) s_h[a][threadIdx.x] = make_double2(0.0, 0.0);
+        for (int a = 0; a < 3; ++a) s_x[threadIdx.x][a] = (int)threadIdx.x < cnt ? pts[3 * (m0 + threadIdx.x) + a] : 0.0;
+    }
+    if (threadIdx.x == 0) s_qn = 0;
+    __syncthreads();
+    const double *xd = s_x[live ? rr : 0];
+    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
+    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
+                                   (float)(xd[2] - (double)xhi.z));
+    const float rt1 = Q.m_max > 1 ? Q.R2[1] * (1.0f + 2e-5f) : __int_as_float(0x7f800000);
+    auto general = [&](int row, int j) {
+        float2 v[kN];
+        if (!field_entry<kGrad>(E, Q, j, s_x[row], k, p[j], q[j], v)) {
+            atomicMin(err, j);
+            return;
+        }
+#pragma unroll
+        for (int a = 0; a < kN; ++a) {
+            atomicAdd(&s_h[a][row].x, (double)v[a].x);
+            atomicAdd(&s_h[a][row].y, (double)v[a].y);
+        }
+    };
+    // (called by the whole block after a barrier)
+    auto drain = [&]() {
+        const int n = min(s_qn, kFieldQueue);
+        for (int u = threadIdx.x; u < n; u += kFusedThreads) general(s_qr[u], s_qj[u]);
+        __syncthreads();
+        if (threadIdx.x == 0) s_qn = 0;
+    };
+    float2 acc[kN];
+#pragma unroll
+    for (int a = 0; a < kN; ++a) acc[a] = make_float2(0.f, 0.f);
+    const int S = gridDim.y, sl = blockIdx.y;
+    const int64_t ntile = (E.n + kFusedTile - 1) / kFusedTile;
+    const int64_t tb = ntile * sl / S, te = ntile * (sl + 1) / S;
+    for (int64_t tile = tb; tile < te; ++tile) {
+        __syncthreads();
+        if (s_qn > kFieldQueue / 2) drain();               // the same in every thread: no pushes since the barrier
+        const int64_t j = tile * kFusedTile + threadIdx.x;
+        if (j < E.n) {
+            const float4 h = E.chi[j];
+            float4 l = E.clo[j];
+            l.w = __frcp_rn(h.w);
+            const float2 pj = p[j], qj = q[j];
+            s_hi[threadIdx.x] = h;
+            s_lo[threadIdx.x] = l;
+            s_n[threadIdx.x] = E.nrm[j];
+            s_pq[threadIdx.x] = make_float4(pj.x, pj.y, qj.x, qj.y);
+        }
+        __syncthreads();
+        const int c0 = warp * 32, c1 = (int)min((int64_t)c0 + 32, E.n - tile * kFusedTile);
+        float2 ta[kN];                                      // the tile's own sum first
+#pragma unroll
+        for (int a = 0; a < kN; ++a) ta[a] = make_float2(0.f, 0.f);
+        for (int cb = c0; cb < c1; cb += R) {
+            const int c = cb + sub;
+            if (!live || c >= c1) continue;
+            const float4 eh = s_hi[c], el = s_lo[c];
+            float3 D0;
+            const float rt2 = pair_rt2(f3(eh), f3(el), xhi, xlo, el.w, D0);
+            if (rt2 > rt1) {
+                const float4 pq = s_pq[c];
+                FieldPair<kGrad> f(k);
+                f.acc.point(D0, f3(s_n[c]), eh.w);
+                f.add(ta, make_float2(pq.x, pq.y), make_float2(pq.z, pq.w));
+            } else {
+                const int je = (int)(tile * kFusedTile) + c;
+                const int slot = atomicAdd(&s_qn, 1);
+                if (slot < kFieldQueue) {
+                    s_qj[slot] = je;
+                    s_qr[slot] = (unsigned char)rr;
+                } else {
+                    general(rr, je);
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < kN; ++a) acc[a] = cadd(acc[a], ta[a]);
+    }
+    __syncthreads();
+    drain();
+    // the lanes' sums of a point in (warp, side-by-side element) order
+    float2 *red = reinterpret_cast<float2 *>(s_hi);
+    float2 tot[kN];
+#pragma unroll
+    for (int a = 0; a < kN; ++a) {
+        __syncthreads();
+        red[threadIdx.x] = acc[a];
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) {
+            const double2 h = s_h[a][threadIdx.x];
+            float2 v = make_float2((float)h.x, (float)h.y);
+            for (int u = 0; u < kW; ++u)
+                for (int t = 0; t < R; ++t) v = cadd(v, red[u * 32 + t * w + threadIdx.x]);
+            tot[a] = cscale(v, tau);                        // tau on the integral part (Eq. BIE_I)
+        }
+    }
+    if ((int)threadIdx.x >= cnt) return;
+    const int64_t m = m0 + threadIdx.x;
+    if (S > 1) {
+#pragma unroll
+        for (int a = 0; a < kN; ++a) part[(m * S + sl) * kN + a] = tot[a];
+    } else if (!kGrad) {
+        double br = tot[0].x, bi = tot[0].y;
+        field_incident(s_x[threadIdx.x], k, src, nsrc, br, bi);
+        out[m] = make_float2((float)br, (float)bi);
+    } else {
+        double gr[3], gi[3];
+#pragma unroll
+        for (int a = 0; a < kN; ++a) {
+            gr[a] = tot[a].x;
+            gi[a] = tot[a].y;
+        }
+        incident_grad(s_x[threadIdx.x], k, src, nsrc, gr, gi);
+        // v = grad p / (i w rho) = -i grad p / (w rho)
+        for (int a = 0; a < kN; ++a)
+            out[3 * m + a] = make_float2((float)(gi[a] * inv_omega_rho), (float)(-gr[a] * inv_omega_rho));
+    }
+}
+
+__global__ void __launch_bounds__(kFusedThreads, 3) k_field(ElemDev E, const QuadTables *__restrict__ Q,
+                                                         const double *__restrict__ pts, int64_t M, float k, float tau,
+                                                         const float2 *__restrict__ p, const float2 *__restrict__ q,
+                                                         const SourceDev *__restrict__ src, int nsrc,
+                                                         float2 *__restrict__ part, float2 *__restrict__ out, int *err)
+{
+    field_body<false>(E, *Q, pts, M, k, tau, 0.f, p, q, src, nsrc, part, out, err);
+}
+
 // Particle velocity at field points, v = grad p / (i w rho) (Eq. utopandv),
 // with grad p = grad p_inc + tau sum_j [grad H(x)_j p_j - grad G(x)_j q_j]
 // (Eq. BIE_I, lambda = 1, differentiated under the integral; the element
-// rules of the field).  Blocks as in k_field: block (m, s) takes field point
-// m and every S-th slice of blockDim elements from slice s; with S = 1 it
-// writes v(x_m), otherwise its partial gradient part[(m S + s) 3 + a] for
-// k_field_velocity_finish.  out: [M][3] (x, y, z components).
-__global__ void k_field_velocity(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts,
-                                 int64_t M, float k, float tau, float inv_omega_rho, const float2 *__restrict__ p,
-                                 const float2 *__restrict__ q, const SourceDev *__restrict__ src, int nsrc,
-                                 float2 *__restrict__ part, float2 *__restrict__ out, int *err)
+// rules of the field).  out: [M][3] (x, y, z components).
+__global__ void __launch_bounds__(kFusedThreads, 3) k_field_velocity(ElemDev E, const QuadTables *__restrict__ Q,
+                                                                  const double *__restrict__ pts, int64_t M, float k,
+                                                                  float tau, float inv_omega_rho,
+                                                                  const float2 *__restrict__ p,
+                                                                  const float2 *__restrict__ q,
+                                                                  const SourceDev *__restrict__ src, int nsrc,
+                                                                  float2 *__restrict__ part, float2 *__restrict__ out,
+                                                                  int *err)
 {
-    const int64_t m = blockIdx.x;
-    const int S = gridDim.y, sl = blockIdx.y;
+    field_body<true>(E, *Q, pts, M, k, tau, inv_omega_rho, p, q, src, nsrc, part, out, err);
+}
+
+// The S partial sums of each field point in slice order, plus the incident
+// field; one thread per point.
+__global__ void k_field_finish(const double *__restrict__ pts, int64_t M, int S, float k,
+                               const SourceDev *__restrict__ src, int nsrc, const float2 *__restrict__ part,
+                               float2 *__restrict__ out)
+{
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= M) return;
+    float2 v = part[m * S];
+    for (int s = 1; s < S; ++s) v = cadd(v, part[m * S + s]);
+    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
+    double br = v.x, bi = v.y;
+    field_incident(xd, k, src, nsrc, br, bi);
+    out[m] = make_float2((float)br, (float)bi);
+}
+
+// Far-field weights of the representation formula (Eq. BIE with lambda = 1)
+// for the aggregation T(l) (Sec. 3.3.3): with the one-point element rule,
+//   H_j p_j - G_j q_j ~ A_j (-q_j - ik (n_j.s) p_j) e^{ik (z_s - y_j).s} (...),
+// i.e. (alpha, c) = (-A q, -ik A p) in the form sum_j E_pj (alpha_j + t_pj c_j)
+// of the aggregation (internal element order).
+__global__ void k_field_weights(int64_t n, const float2 *__restrict__ p, const float2 *__restrict__ q,
+                                const float4 *__restrict__ chi, float k, float4 *__restrict__ wts)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float A = chi[i].w;
+    const float2 pv = p[i], qv = q[i];
+    wts[i] = make_float4(-A * qv.x, -A * qv.y, k * A * pv.y, -k * A * pv.x);
+}
+
+// Near part of the field at points (internal point order): the element rules
+// of the direct sum over the point's leaf near list, one warp per point; v_m =
+// sum_j H_j p_j - G_j q_j.  The list's runs (first element, first position)
+// are walked by position, so that all lanes have an element whatever the
+// runs' lengths (a run is often a leaf of a dozen elements; run by run,
+// 24,874 points took 75 us, this 72).
+__global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, int64_t M,
+                             float k, const float2 *__restrict__ p, const float2 *__restrict__ q,
+                             const int *__restrict__ pleaf, const int *__restrict__ nptr, const int *__restrict__ ntot,
+                             const int2 *__restrict__ nruns, float2 *__restrict__ v, int *err)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t m = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (m >= M) return;
     const QuadTables &Q = *Qp;
     const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
     const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
     const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
                                    (float)(xd[2] - (double)xhi.z));
-    float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    for (int64_t j = (int64_t)sl * blockDim.x + threadIdx.x; j < E.n; j += (int64_t)S * blockDim.x) {
-        GradAcc g;
-        g.k = k;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) g.gG[a] = g.gH[a] = make_float2(0.f, 0.f);
-        if (!integrate_regular_acc(E, j, xhi, xlo, xd, Q, g)) {
+    const int pl = pleaf[m], tot = ntot[pl], r1 = nptr[pl + 1];
+    int r = nptr[pl];
+    float2 acc = make_float2(0.f, 0.f);
+    for (int c = lane; c < tot; c += 32) {
+        while (r + 1 < r1 && nruns[r + 1].y <= c) ++r;
+        const int2 run = nruns[r];
+        const int64_t j = run.x + (c - run.y);
+        float2 G = make_float2(0.f, 0.f), H = make_float2(0.f, 0.f);
+        if (!integrate_regular<true>(E, j, xhi, xlo, xd, make_float3(0.f, 0.f, 1.f), k, 1.0f / k, Q, G, H)) {
             atomicMin(err, (int)j);
             continue;
         }
-        const float2 pj = p[j], qj = q[j];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) acc[a] = cadd(acc[a], csub(cmul(g.gH[a], pj), cmul(g.gG[a], qj)));
+        acc = cadd(acc, csub(cmul(H, p[j]), cmul(G, q[j])));
     }
-    __shared__ float2 red[3][32];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float2 v = warp_sum(acc[a]);
-        if ((threadIdx.x & 31) == 0) red[a][threadIdx.x >> 5] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double gr[3], gi[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float2 v = threadIdx.x < (blockDim.x >> 5) ? red[a][threadIdx.x] : make_float2(0.f, 0.f);
-            v = warp_sum(v);
-            gr[a] = tau * v.x;   // tau on the integral part (Eq. BIE_I)
-            gi[a] = tau * v.y;
-        }
-        if (threadIdx.x == 0) {
-            if (S > 1) {
-                for (int a = 0; a < 3; ++a) part[(m * S + sl) * 3 + a] = make_float2((float)gr[a], (float)gi[a]);
-            } else {
-                incident_grad(xd, k, src, nsrc, gr, gi);
-                // v = grad p / (i w rho) = -i grad p / (w rho)
-                for (int a = 0; a < 3; ++a)
-                    out[3 * m + a] = make_float2((float)(gi[a] * inv_omega_rho), (float)(-gr[a] * inv_omega_rho));
-            }
-        }
-    }
+    acc = warp_sum(acc);
+    if (lane == 0) v[m] = acc;
+}
+
+// The field at the points: tau (near + far) plus the incident field (FP64),
+// written in caller order.
+__global__ void k_field_eval_finish(const double *__restrict__ pts, int64_t M, float k, float tau,
+                                    const SourceDev *__restrict__ src, int nsrc, const float2 *__restrict__ v,
+                                    const int64_t *__restrict__ perm, float2 *__restrict__ out)
+{
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= M) return;
+    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
+    const float2 w = cscale(v[m], tau);
+    double br = w.x, bi = w.y;
+    field_incident(xd, k, src, nsrc, br, bi);
+    out[perm[m]] = make_float2((float)br, (float)bi);
 }
 
 // The S partial gradients of each field point in slice order, the incident

@@ -217,6 +217,7 @@ constexpr int kFusedThreads = 256;
 constexpr int kFusedTile = 256;          // columns staged per pass
 constexpr int kFusedRows = 32;           // rows per block (the lanes of a warp)
 constexpr int kFusedQueue = 1024;        // expensive pairs queued per block
+constexpr int kFieldQueue = 2048;        // near pairs of field points queued per block
 constexpr int kFusedParts = 2560;        // ... and their parts under one rule, per kFusedThreads pairs
 __global__ void k_near_fused_1(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
 __global__ void k_near_fused_2(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
@@ -379,8 +380,8 @@ __global__ void k_coeffs(int64_t n, const int *type, const double2 *bcv, const i
 // FMM evaluation of the field at points (see the definitions)
 __global__ void k_field_weights(int64_t n, const float2 *p, const float2 *q, const float4 *chi, float k, float4 *wts);
 __global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, const float2 *p,
-                             const float2 *q, const int *pleaf, const int *nptr, const int2 *nruns, float2 *v,
-                             int *err);
+                             const float2 *q, const int *pleaf, const int *nptr, const int *ntot, const int2 *nruns,
+                             float2 *v, int *err);
 __global__ void k_field_eval_finish(const double *pts, int64_t M, float k, float tau, const SourceDev *src, int nsrc,
                                     const float2 *v, const int64_t *perm, float2 *out);
 
