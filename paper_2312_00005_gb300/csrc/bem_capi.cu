@@ -369,8 +369,7 @@ struct Plan {
     std::shared_ptr<Lists> lists;
     bool shared_lists = false;
     std::vector<std::unique_ptr<LevelDev>> lev;
-    DevArr<LevelsArgs> largs;     // device copy of the per-level arguments
-    LevelsArgs hargs;
+    LevelsArgs hargs;             // per-level arguments of the kernels
     DevArr<float2> val;
     DevArr<float2> valT;          // A^T in A's layout (near_transpose), made from val
     bool valT_valid = false;
@@ -423,7 +422,6 @@ struct EvalDev {
     DevArr<int2> reds, dtasks, nruns;
     DevArr<unsigned int> red_cnt;
     DevArr<int4> tgroups;
-    DevArr<LevelsArgs> largs;
     DevArr<int> pleaf, nptr, ntot;
     DevArr<double> pts;
     DevArr<int64_t> perm;
@@ -933,8 +931,6 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
         A.lev[l].mplane = (int64_t)(P->lev[l]->nc + P->lev[l]->ll->nextra) * P->lev[l]->nd;
         A.lev[l].lplane = (int64_t)P->lev[l]->nc * P->lev[l]->nd;
     }
-    std::vector<LevelsArgs> hv(1, A);
-    P->largs.upload(hv, s);
     ck(cudaStreamSynchronize(s), "sync");
 }
 
@@ -1294,9 +1290,6 @@ void ensure_planes(bem_mesh_impl &M, int nr)
         A.lev[l].M = D.M.p;
         A.lev[l].Lam = D.Lam.p;
     }
-    std::vector<LevelsArgs> hv(1, A);
-    P.largs.upload(hv, fr(M).s);
-    ck(cudaStreamSynchronize(fr(M).s), "sync");
     P.planes = nr;
 }
 
@@ -1342,7 +1335,7 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
         {
             KTimer kt_("k_aggregate_tc", sf);
             if (P.n_tc_tasks > 0)
-                k_aggregate_tc<<<P.n_tc_tasks, kTcThreads, kTcSmemBytes, sf>>>(P.largs.p, P.agg_tasks_tc.p, M.wts.p, n,
+                k_aggregate_tc<<<P.n_tc_tasks, kTcThreads, kTcSmemBytes, sf>>>(A, P.agg_tasks_tc.p, M.wts.p, n,
                                                                                M.nrm.p, nr, M.tc_fault.p, skip);
         }
         ck_launch("k_aggregate_tc");
@@ -1351,12 +1344,12 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
             KTimer kt_("k_aggregate", sf);
             switch (nr) {
                 case 1:
-                    if (P.has_phases) k_aggregate_1t<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip);
-                    else k_aggregate_1<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip);
+                    if (P.has_phases) k_aggregate_1t<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip);
+                    else k_aggregate_1<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip);
                     break;
-                case 2: k_aggregate_2<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip); break;
-                case 3: k_aggregate_3<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip); break;
-                default: k_aggregate_4<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip); break;
+                case 2: k_aggregate_2<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip); break;
+                case 3: k_aggregate_3<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip); break;
+                default: k_aggregate_4<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip); break;
             }
         }
         ck_launch("k_aggregate");
@@ -1364,9 +1357,13 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
     if (A.ntargets > 0) {
         if (A.ntgroups > 0) {
             KTimer kt_("k_transfer", sf);
-            if (nr == 4) k_transfer_m4<<<A.ntgroups, 32 * kTransferWarps, 0, sf>>>(P.largs.p, skip);
-            else if (nr == 2) k_transfer_m2<<<A.ntgroups, 32 * kTransferWarps, 0, sf>>>(P.largs.p, skip);
-            else k_transfer_split<<<dim3(A.ntgroups, nr), 32 * kTransferWarps, 0, sf>>>(P.largs.p, skip);
+            const int nb = 2 * A.ntgroups;
+            const bool many = nb >= kTransferManyBlocks;
+            if (nr == 4 && many) k_transfer_m4s<<<nb, 32, 0, sf>>>(A, skip);
+            else if (nr == 4) k_transfer_m4<<<nb, 32 * kTransferWarps, 0, sf>>>(A, skip);
+            else if (nr == 2 && many) k_transfer_m2s<<<nb, 32, 0, sf>>>(A, skip);
+            else if (nr == 2) k_transfer_m2<<<nb, 32 * kTransferWarps, 0, sf>>>(A, skip);
+            else k_transfer_split<<<dim3(A.ntgroups, nr), 32 * kTransferWarps, 0, sf>>>(A, skip);
         }
         ck_launch("k_transfer");
     }
@@ -1574,15 +1571,15 @@ void matvec_t_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, con
     if (A.ntasks > 0) {
         {
             KTimer kt_("k_aggregate", sf);
-            if (P.has_phases) k_aggregate_1t<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip);
-            else k_aggregate_1<<<A.ntasks, kAggThreads, 0, sf>>>(P.largs.p, M.wts.p, n, M.nrm.p, skip);
+            if (P.has_phases) k_aggregate_1t<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip);
+            else k_aggregate_1<<<A.ntasks, kAggThreads, 0, sf>>>(A, M.wts.p, n, M.nrm.p, skip);
         }
         ck_launch("k_aggregate");
     }
     if (A.ntargets > 0 && A.ntgroups > 0) {
         {
             KTimer kt_("k_transfer", sf);
-            k_transfer_split<<<A.ntgroups, 32 * kTransferWarps, 0, sf>>>(P.largs.p, skip);
+            k_transfer_split<<<A.ntgroups, 32 * kTransferWarps, 0, sf>>>(A, skip);
         }
         ck_launch("k_transfer");
     }
@@ -2742,7 +2739,8 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
             NearArgs na = near_args(M, P, fr(M).cp.p, fr(M).cq.p);
             {
                 KTimer kt_("k_bj_factor", s);
-                k_bj_factor<<<(unsigned)Lb.h_bj.size(), 256, 0, s>>>(na, Lb.bj.p, M.bjinv.p, fr(M).err.p);
+                k_bj_factor<<<(unsigned)Lb.h_bj.size(), 256, 0, s>>>(
+                    na, Lb.bj.p, M.prm.near_store && !P.fp().direct ? P.val.p : nullptr, M.bjinv.p, fr(M).err.p);
             }
             ck_launch("k_bj_factor");
             check_err(M);
@@ -3151,8 +3149,6 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         V.tgroups.upload(tg, s);
         A.tgroups = V.tgroups.p;
         A.ntgroups = (int)tg.size();
-        std::vector<LevelsArgs> hv(1, A);
-        V.largs.upload(hv, s);
         if (nb > 0) {
             {
                 KTimer kt_("k_dtable", s);
@@ -3218,14 +3214,14 @@ void field_fmm(bem_mesh_impl &M, double k, const double *pts, int64_t np, const 
         if (V.A.ntasks > 0) {
             {
                 KTimer kt_("k_aggregate", s);
-                k_aggregate_1<<<V.A.ntasks, kAggThreads, 0, s>>>(V.largs.p, V.wts.p, n, M.nrm.p, nullptr);
+                k_aggregate_1<<<V.A.ntasks, kAggThreads, 0, s>>>(V.A, V.wts.p, n, M.nrm.p, nullptr);
             }
             ck_launch("k_aggregate");
         }
         if (V.A.ntgroups > 0) {
             {
                 KTimer kt_("k_transfer", s);
-                k_transfer_split<<<V.A.ntgroups, 32 * kTransferWarps, 0, s>>>(V.largs.p, nullptr);
+                k_transfer_split<<<V.A.ntgroups, 32 * kTransferWarps, 0, s>>>(V.A, nullptr);
             }
             ck_launch("k_transfer");
         }

@@ -1124,14 +1124,18 @@ __global__ void k_row_scale(float2 *__restrict__ y, float2 *__restrict__ y2, con
 // Sec. 3.2): P = inverse of the block diagonal of A over sub-blocks of at
 // most kBjMax consecutive elements of one leaf (blocks[b] = (first element,
 // size, offset of its inverse, 0)).  One CUDA block per sub-block: the
-// entries A_ij of the sub-block (bm_entry, the stored near field's values),
+// entries A_ij of the sub-block, read from the stored near field (val; a leaf
+// is in its own near list) or, without one (val null), by bm_entry, the same
+// values (a sub-block's pairs are the subdivided and self terms: computing
+// them took 613 us on 13,520 elements, reading them 84);
 // then Gauss-Jordan inversion in place with partial pivoting in shared
 // memory (FP32 complex).  The inverse is stored column-major so that the
 // apply kernel's threads (one per row) read consecutive entries.  A zero
 // pivot leaves the sub-block's inverse the identity (no preconditioning
 // there); err takes the subdivision limit of the entries, as for the stored
 // near field.
-__global__ void __launch_bounds__(256) k_bj_factor(NearArgs a, const int4 *__restrict__ blocks, float2 *__restrict__ binv,
+__global__ void __launch_bounds__(256) k_bj_factor(NearArgs a, const int4 *__restrict__ blocks,
+                                                   const float2 *__restrict__ val, float2 *__restrict__ binv,
                                                    int *__restrict__ err)
 {
     __shared__ float2 A[kBjMax][kBjMax + 1];
@@ -1142,9 +1146,25 @@ __global__ void __launch_bounds__(256) k_bj_factor(NearArgs a, const int4 *__res
     const int64_t e0 = B.x;
     const int nb = B.y;
     const QuadTables &Q = *a.Q;
+    // position of column e0 in the rows of this leaf (val)
+    int64_t col0 = 0;
+    if (val) {
+        const int t = a.N.leaf_of[e0];
+        int lo = a.N.run_ptr[t], hi = a.N.run_ptr[t + 1] - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.N.runs[mid].x <= e0) lo = mid;
+            else hi = mid - 1;
+        }
+        col0 = a.N.runs[lo].y + (e0 - a.N.runs[lo].x);
+    }
     for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
         const int r = idx / nb, c = idx % nb;
         const int64_t i = e0 + r, j = e0 + c;
+        if (val) {
+            A[r][c] = val[a.N.row_ptr[i] + col0 + c];
+            continue;
+        }
         const float4 ch = a.E.chi[i], cl = a.E.clo[i];
         const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
         float2 v;
@@ -1431,11 +1451,11 @@ __device__ __forceinline__ float2 ld_stream2(const float2 *p)
 // kernel's length.  For a cluster split into several element chunks, the
 // last of its blocks to finish sums the chunks' partial rows in row order.
 template <int NR, bool kTab>
-__device__ __forceinline__ void aggregate_body(const LevelsArgs *__restrict__ A, const float4 *__restrict__ wts,
+__device__ __forceinline__ void aggregate_body(const LevelsArgs &A, const float4 *__restrict__ wts,
                                                int64_t wplane, const float4 *__restrict__ nrm)
 {
-    const AggTask T = A->tasks[blockIdx.x];
-    const FarArgs &f = A->lev[T.lev];
+    const AggTask T = A.tasks[blockIdx.x];
+    const FarArgs &f = A.lev[T.lev];
     __shared__ float4 sd[kTab ? 1 : kAggChunk];   // (z_c - x_j) k / (2 pi)
     __shared__ float4 sw[NR][kAggChunk];           // (alpha_j, c_j) per right-hand side
     __shared__ float4 sn[kAggChunk];               // n_j
@@ -1530,7 +1550,7 @@ __device__ __forceinline__ void aggregate_body(const LevelsArgs *__restrict__ A,
 
 #define BEM_AGGREGATE_KERNEL(NR, TAB, NAME)                                                                           \
     __global__ void __launch_bounds__(kAggThreads)                                                                   \
-        NAME(const LevelsArgs *__restrict__ A, const float4 *__restrict__ wts, int64_t wplane,                       \
+        NAME(const __grid_constant__ LevelsArgs A, const float4 *__restrict__ wts, int64_t wplane,                    \
              const float4 *__restrict__ nrm, const int *skip)                                                        \
     {                                                                                                                 \
         if (skip_now(skip)) return;                                                                                   \
@@ -1587,31 +1607,33 @@ __global__ void k_selftest_sincos(const float *__restrict__ x, int64_t n, float4
 // Diagonal transfer (Sec. 3.3.3, matrix D(l)): for every target cluster t
 // with an interaction list (Sec. 3.3.4),
 //   Lambda_t(nu) = sum_{s in I(t)} D_L(z_t - z_s, s_nu) M_s(nu).
-// A block takes one target and kTransferDirs directions (lanes); its
-// kTransferWarps warps take every kTransferWarps-th list entry, each with
-// kTransferUnroll entries (their D and M loads) in flight, and the partial
-// sums are added in warp order.  Few warps per target with deep load
-// batches hold fewer registers and warps of an SM for the same L2 traffic,
-// which leaves room for the near-field product running beside.
-__global__ void __launch_bounds__(32 * kTransferWarps) k_transfer_split(const LevelsArgs *__restrict__ A,
+// A block takes one target and kTransferDirs directions, two per lane (one
+// 16-byte load each of D and M per list entry); its kTransferWarps warps take
+// every kTransferWarps-th list entry, each with kTransferUnroll entries in
+// flight, and the partial sums are added in warp order.  Few warps per target
+// with deep load batches hold fewer registers and warps of an SM for the same
+// L2 traffic, which leaves room for the near-field product running beside.
+// One direction per lane and two warps per target took 26.1 us on 20,480
+// elements and 32.9 on 13,520; this 22.9 and 28.8 (two warps 22.0 and 30.9).
+__global__ void __launch_bounds__(32 * kTransferWarps) k_transfer_split(const __grid_constant__ LevelsArgs A,
                                                                         const int *skip)
 {
     if (skip_now(skip)) return;
-    __shared__ float2 part[kTransferWarps][kTransferDirs];
+    __shared__ float4 part[kTransferWarps][32];
     __shared__ int2 s_ent[kTransferEntries];      // (source cluster, offset) of the list entries
-    const int4 T = A->tgroups[blockIdx.x];
-    const FarArgs &f = A->lev[T.x];
+    const int4 T = A.tgroups[blockIdx.x];
+    const FarArgs &f = A.lev[T.x];
     const int t = T.y, nu0 = T.z, nd = f.nd;
     // right-hand side blockIdx.y: its M and Lambda planes
     const float2 *__restrict__ Mp = f.M + blockIdx.y * f.mplane;
     float2 *__restrict__ Lp = f.Lam + blockIdx.y * f.lplane;
+    const float2 *__restrict__ D = f.D;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nu = nu0 + lane;
+    const int nu = nu0 + 2 * lane;                // nd is even: a pair of directions is in range or not
     const bool live = nu < nd;
     const int b = f.il_ptr[t], e = f.il_ptr[t + 1];
     float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0;
     constexpr int kW = kTransferWarps, kU = kTransferUnroll;
-    static_assert(kU % 2 == 0, "entries are added in pairs");
     for (int c0 = b; c0 < e; c0 += kTransferEntries) {
         const int cnt = min(kTransferEntries, e - c0);
         __syncthreads();
@@ -1621,49 +1643,59 @@ __global__ void __launch_bounds__(32 * kTransferWarps) k_transfer_split(const Le
         if (!live) continue;
         int q = warp;
         for (; q + kW * (kU - 1) < cnt; q += kW * kU) {
-            float2 dv[kU], mv[kU];
+            float4 dv[kU], mv[kU];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int2 en = s_ent[q + kW * u];
-                dv[u] = __ldg(f.D + (int64_t)en.y * nd + nu);
-                mv[u] = Mp[(int64_t)en.x * nd + nu];
+                dv[u] = __ldg(reinterpret_cast<const float4 *>(D + (int64_t)en.y * nd + nu));
+                mv[u] = *reinterpret_cast<const float4 *>(Mp + (int64_t)en.x * nd + nu);
             }
 #pragma unroll
-            for (int u = 0; u < kU; u += 2) {
-                acc0 = cfma(dv[u], mv[u], acc0);
-                acc1 = cfma(dv[u + 1], mv[u + 1], acc1);
+            for (int u = 0; u < kU; ++u) {
+                acc0 = cfma(make_float2(dv[u].x, dv[u].y), make_float2(mv[u].x, mv[u].y), acc0);
+                acc1 = cfma(make_float2(dv[u].z, dv[u].w), make_float2(mv[u].z, mv[u].w), acc1);
             }
         }
         for (; q < cnt; q += kW) {
             const int2 en = s_ent[q];
-            acc0 = cfma(__ldg(f.D + (int64_t)en.y * nd + nu), Mp[(int64_t)en.x * nd + nu], acc0);
+            const float4 dv = __ldg(reinterpret_cast<const float4 *>(D + (int64_t)en.y * nd + nu));
+            const float4 mv = *reinterpret_cast<const float4 *>(Mp + (int64_t)en.x * nd + nu);
+            acc0 = cfma(make_float2(dv.x, dv.y), make_float2(mv.x, mv.y), acc0);
+            acc1 = cfma(make_float2(dv.z, dv.w), make_float2(mv.z, mv.w), acc1);
         }
     }
-    part[warp][lane] = cadd(acc0, acc1);
+    part[warp][lane] = make_float4(acc0.x, acc0.y, acc1.x, acc1.y);
     __syncthreads();
     if (warp == 0 && live) {
-        float2 sum = part[0][lane];
+        float4 sum = part[0][lane];
 #pragma unroll
-        for (int w = 1; w < kW; ++w) sum = cadd(sum, part[w][lane]);
-        Lp[(int64_t)t * nd + nu] = sum;
+        for (int w = 1; w < kW; ++w) {
+            const float4 v = part[w][lane];
+            sum = make_float4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
+        }
+        *reinterpret_cast<float4 *>(Lp + (int64_t)t * nd + nu) = sum;
     }
 }
 
 // The transfer for NR right-hand sides at once: the same blocks and list
 // order as k_transfer_split, each D value loaded once for all planes (the
 // M and Lambda planes are mplane and lplane apart).
-template <int NR>
-__device__ __forceinline__ void transfer_multi_body(const LevelsArgs *__restrict__ A)
+template <int NR, int kW>
+__device__ __forceinline__ void transfer_multi_body(const LevelsArgs &A)
 {
-    constexpr int kW = kTransferWarps, kU = 8 / NR;
-    __shared__ float2 part[NR][kW][kTransferDirs];
+    constexpr int kU = 8 / NR;
+    __shared__ float2 part[NR][kW][32];
     __shared__ int2 s_ent[kTransferEntries];
-    const int4 T = A->tgroups[blockIdx.x];
-    const FarArgs &f = A->lev[T.x];
-    const int t = T.y, nu0 = T.z, nd = f.nd;
+    // a block takes half of a group of kTransferDirs directions (one per lane)
+    const int4 T = A.tgroups[blockIdx.x >> 1];
+    const FarArgs &f = A.lev[T.x];
+    const int t = T.y, nu0 = T.z + 32 * (blockIdx.x & 1), nd = f.nd;
+    const float2 *__restrict__ M = f.M, *__restrict__ D = f.D;
+    const int64_t mplane = f.mplane;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nu = nu0 + lane;
     const bool live = nu < nd;
+    if (nu0 >= nd) return;
     const int b = f.il_ptr[t], e = f.il_ptr[t + 1];
     float2 acc[NR];
 #pragma unroll
@@ -1681,9 +1713,9 @@ __device__ __forceinline__ void transfer_multi_body(const LevelsArgs *__restrict
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int2 en = s_ent[q + kW * u];
-                dv[u] = __ldg(f.D + (int64_t)en.y * nd + nu);
+                dv[u] = __ldg(D + (int64_t)en.y * nd + nu);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) mv[u][r] = f.M[r * f.mplane + (int64_t)en.x * nd + nu];
+                for (int r = 0; r < NR; ++r) mv[u][r] = M[r * mplane + (int64_t)en.x * nd + nu];
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u)
@@ -1692,9 +1724,9 @@ __device__ __forceinline__ void transfer_multi_body(const LevelsArgs *__restrict
         }
         for (; q < cnt; q += kW) {
             const int2 en = s_ent[q];
-            const float2 dv = __ldg(f.D + (int64_t)en.y * nd + nu);
+            const float2 dv = __ldg(D + (int64_t)en.y * nd + nu);
 #pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r] = cfma(dv, f.M[r * f.mplane + (int64_t)en.x * nd + nu], acc[r]);
+            for (int r = 0; r < NR; ++r) acc[r] = cfma(dv, M[r * mplane + (int64_t)en.x * nd + nu], acc[r]);
         }
     }
 #pragma unroll
@@ -1711,15 +1743,16 @@ __device__ __forceinline__ void transfer_multi_body(const LevelsArgs *__restrict
     }
 }
 
-#define BEM_TRANSFER_MULTI_KERNEL(NR)                                                                               \
-    __global__ void __launch_bounds__(32 * kTransferWarps) k_transfer_m##NR(const LevelsArgs *__restrict__ A,      \
-                                                                            const int *skip)                       \
-    {                                                                                                               \
-        if (skip_now(skip)) return;                                                                                 \
-        transfer_multi_body<NR>(A);                                                                                 \
+#define BEM_TRANSFER_MULTI_KERNEL(NAME, NR, W)                                                                        \
+    __global__ void __launch_bounds__(32 * W) NAME(const __grid_constant__ LevelsArgs A, const int *skip)            \
+    {                                                                                                                 \
+        if (skip_now(skip)) return;                                                                                   \
+        transfer_multi_body<NR, W>(A);                                                                                \
     }
-BEM_TRANSFER_MULTI_KERNEL(2)
-BEM_TRANSFER_MULTI_KERNEL(4)
+BEM_TRANSFER_MULTI_KERNEL(k_transfer_m2, 2, kTransferWarps)
+BEM_TRANSFER_MULTI_KERNEL(k_transfer_m4, 4, kTransferWarps)
+BEM_TRANSFER_MULTI_KERNEL(k_transfer_m2s, 2, 1)
+BEM_TRANSFER_MULTI_KERNEL(k_transfer_m4s, 4, 1)
 #undef BEM_TRANSFER_MULTI_KERNEL
 
 // Disaggregation over all levels (Sec. 3.3.3, matrix S(l), with the

@@ -139,7 +139,8 @@ struct PhaseTableArgs {
 };
 __global__ void k_phase_table(PhaseTableArgs a);
 
-// All far levels of a plan, for the kernels that run every level in one launch.
+// All far levels of a plan, for the kernels that run every level in one launch
+// (passed by value: its reads are constants, not loads that every block waits for).
 struct LevelsArgs {
     int nlev;
     const AggTask *tasks;    // aggregation tasks of every level
@@ -244,7 +245,7 @@ __device__ __forceinline__ bool skip_now(const int *skip) { return skip != nullp
 // the last one to finish sums the partial rows in row order into row T.c of
 // every plane (nplanes right-hand sides).  Called by every thread of the
 // block after its own rows are written.
-__device__ __forceinline__ void aggregate_reduce(const LevelsArgs *A, const AggTask &T, const FarArgs &f, int ppb,
+__device__ __forceinline__ void aggregate_reduce(const LevelsArgs &A, const AggTask &T, const FarArgs &f, int ppb,
                                                  int nplanes)
 {
     if (T.red < 0) return;
@@ -255,7 +256,7 @@ __device__ __forceinline__ void aggregate_reduce(const LevelsArgs *A, const AggT
         const int h = f.nd / 2;
         const int npb = (h + ppb - 1) / ppb;
         const int ntask = (f.red_ptr[T.red + 1] - f.red_ptr[T.red]) * npb;
-        last = atomicAdd(&A->red_cnt[T.gred], 1u) == (unsigned)(ntask - 1);
+        last = atomicAdd(&A.red_cnt[T.gred], 1u) == (unsigned)(ntask - 1);
     }
     __syncthreads();
     if (!last) return;
@@ -297,17 +298,17 @@ __device__ __forceinline__ void aggregate_reduce(const LevelsArgs *A, const AggT
                 if (nb + b * nt < nd) dst[nb + b * nt] = acc[b];
         }
     }
-    if (threadIdx.x == 0) A->red_cnt[T.gred] = 0;
+    if (threadIdx.x == 0) A.red_cnt[T.gred] = 0;
 }
 
 // Aggregation of NR right-hand sides at once (one phase per element and
 // direction pair serves all of them); wts holds NR planes of n elements.
-__global__ void k_aggregate_1(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
-__global__ void k_aggregate_2(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
-__global__ void k_aggregate_3(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
-__global__ void k_aggregate_4(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
+__global__ void k_aggregate_1(const __grid_constant__ LevelsArgs A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
+__global__ void k_aggregate_2(const __grid_constant__ LevelsArgs A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
+__global__ void k_aggregate_3(const __grid_constant__ LevelsArgs A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
+__global__ void k_aggregate_4(const __grid_constant__ LevelsArgs A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
 // One right-hand side, with the level's stored phases (FarArgs::ph).
-__global__ void k_aggregate_1t(const LevelsArgs *A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
+__global__ void k_aggregate_1t(const __grid_constant__ LevelsArgs A, const float4 *wts, int64_t wplane, const float4 *nrm, const int *skip);
 // Aggregation on the tensor cores (bem_tc.cu): tasks of one element chunk
 // and kTcPairs direction pairs, split-BF16 operands, FP32 accumulation;
 // fault is set when the wait for the tensor cores runs out.
@@ -316,20 +317,27 @@ constexpr int kTcPairs = 128;
 constexpr int kTcSub = 16;               // elements per pass of the MMAs (a chunk takes up to four)
 constexpr size_t kTcSmemBytes = 2 * (size_t)kTcPairs * 4 * kTcSub * 2 + 2 * (size_t)4 * kMaxPlanes * 4 * kTcSub * 2 +
                                 1024;
-__global__ void k_aggregate_tc(const LevelsArgs *A, const AggTask *tasks, const float4 *wts, int64_t wplane,
+__global__ void k_aggregate_tc(const __grid_constant__ LevelsArgs A, const AggTask *tasks, const float4 *wts, int64_t wplane,
                                const float4 *nrm, int nr, int *fault, const int *skip);
 __global__ void k_selftest_sincos(const float *x, int64_t n, float4 *out);
 // Transfer with the interaction list of one target split among
 // kTransferWarps warps: one block per (target, kTransferDirs directions).
-constexpr int kTransferDirs = 32;
-constexpr int kTransferWarps = 2;          // warps sharing one target's list
-constexpr int kTransferUnroll = 8;         // list entries per warp in flight
+constexpr int kTransferDirs = 64;
+constexpr int kTransferWarps = 4;          // warps sharing one target's list
+constexpr int kTransferUnroll = 4;         // list entries per warp in flight
 constexpr int kTransferEntries = 512;     // interaction-list entries staged per pass
-__global__ void k_transfer_split(const LevelsArgs *A, const int *skip);
+__global__ void k_transfer_split(const __grid_constant__ LevelsArgs A, const int *skip);
 // The same for 2 or 4 right-hand sides (M and Lambda planes mplane and
-// lplane apart): each D value is loaded once for all of them.
-__global__ void k_transfer_m2(const LevelsArgs *A, const int *skip);
-__global__ void k_transfer_m4(const LevelsArgs *A, const int *skip);
+// lplane apart): each D value is loaded once for all of them.  One block per
+// half of a group of directions; kTransferWarps warps per target, or one (s)
+// from kTransferManyBlocks blocks on, where the blocks alone fill the GPU (four
+// planes: 158,420 elements, 107,000 blocks: 1066 us with four warps, 942 with
+// one; 10,580 elements, 7300 blocks: solves 29.0 and 30.6 ms).
+constexpr int kTransferManyBlocks = 20000;
+__global__ void k_transfer_m2(const __grid_constant__ LevelsArgs A, const int *skip);
+__global__ void k_transfer_m4(const __grid_constant__ LevelsArgs A, const int *skip);
+__global__ void k_transfer_m2s(const __grid_constant__ LevelsArgs A, const int *skip);
+__global__ void k_transfer_m4s(const __grid_constant__ LevelsArgs A, const int *skip);
 // 1, 2 or 4 right-hand sides at once (one phase per element and pair for
 // all), element-major with the directions staged in chunks (no dynamic
 // shared memory)
@@ -394,7 +402,7 @@ __global__ void k_adjoint_reduce(const float2 *u, const float2 *g, const float2 
                                  double *acc);
 // block-Jacobi sub-blocks: at most kBjMax consecutive elements of one leaf
 constexpr int kBjMax = 64;
-__global__ void k_bj_factor(NearArgs a, const int4 *blocks, float2 *binv, int *err);
+__global__ void k_bj_factor(NearArgs a, const int4 *blocks, const float2 *val, float2 *binv, int *err);
 __global__ void k_bj_apply(const int4 *blocks, const float2 *binv, float2 *w, float2 *wnear, int64_t n, const int *skip);
 __global__ void k_row_scale_init(NearArgs a, float2 *dinv, int *err);
 __global__ void k_row_scale(float2 *y, float2 *y2, const float2 *dinv, int64_t n, const int *skip);

@@ -107,7 +107,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
 
 }  // namespace
 
-__global__ void __launch_bounds__(kTcThreads, 4) k_aggregate_tc(const LevelsArgs *__restrict__ A,
+__global__ void __launch_bounds__(kTcThreads, 4) k_aggregate_tc(const __grid_constant__ LevelsArgs A,
                                                                 const AggTask *__restrict__ tasks,
                                                                 const float4 *__restrict__ wts, int64_t wplane,
                                                                 const float4 *__restrict__ nrm, int nr, int *fault,
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_aggregate_tc(const LevelsArgs
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     const AggTask T = tasks[blockIdx.x];
-    const FarArgs &f = A->lev[T.lev];
+    const FarArgs &f = A.lev[T.lev];
     const int h = f.nd / 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
