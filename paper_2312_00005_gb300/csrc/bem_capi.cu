@@ -3199,7 +3199,7 @@ void field_fmm(bem_mesh_impl &M, double k, const double *pts, int64_t np, const 
     const int64_t n = M.n;
     {
         KTimer kt_("k_field_near", s);
-        k_field_near<<<nblocks(np, 8), 256, 0, s>>>(M.elem(), M.Q.p, V.pts.p, np, (float)k, p, q, V.pleaf.p,
+        k_field_near<<<(unsigned)np, 32 * kFieldNearWarps, 0, s>>>(M.elem(), M.Q.p, V.pts.p, np, (float)k, p, q, V.pleaf.p,
                                                    V.nptr.p, V.ntot.p, V.nruns.p, V.vnear.p, fr(M).err.p);
     }
     ck_launch("k_field_near");

@@ -72,7 +72,9 @@ __global__ void k_near_classify(NearArgs a, int2 *__restrict__ heavy, unsigned l
 // a warp then write 32 consecutive values of one row.  r~ is compared in
 // squared form (FP64 when within 2e-5 of a threshold).  Four blocks per SM
 // (64 registers, a few spilled) keep more warps issuing than two blocks
-// with every value in registers.
+// with every value in registers.  (Orders 2 and 3 in place instead of queued, as
+// in the recomputed product: 633 us against 502 on 20,480 elements, since only
+// two thirds of a warp's lanes agree on the order.)
 constexpr int kLightRows = 64;
 // the general rule out of line, so that the common path keeps few registers
 __device__ __noinline__ bool general_entry(const NearArgs &a, int64_t i, int64_t j, float2 *out)
@@ -2372,16 +2374,17 @@ __global__ void k_field_weights(int64_t n, const float2 *__restrict__ p, const f
 // of the direct sum over the point's leaf near list, one warp per point; v_m =
 // sum_j H_j p_j - G_j q_j.  The list's runs (first element, first position)
 // are walked by position, so that all lanes have an element whatever the
-// runs' lengths (a run is often a leaf of a dozen elements; run by run,
-// 24,874 points took 75 us, this 72).
+// runs' lengths (a run is often a leaf of a dozen elements).  kFieldNearWarps
+// warps share a point: the points nearest to the surface have lists many times
+// the mean, and set the kernel's length (24,874 points, one warp each 74 us,
+// four 46).
 __global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, int64_t M,
                              float k, const float2 *__restrict__ p, const float2 *__restrict__ q,
                              const int *__restrict__ pleaf, const int *__restrict__ nptr, const int *__restrict__ ntot,
                              const int2 *__restrict__ nruns, float2 *__restrict__ v, int *err)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t m = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (m >= M) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t m = blockIdx.x;
     const QuadTables &Q = *Qp;
     const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
     const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
@@ -2390,7 +2393,7 @@ __global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const
     const int pl = pleaf[m], tot = ntot[pl], r1 = nptr[pl + 1];
     int r = nptr[pl];
     float2 acc = make_float2(0.f, 0.f);
-    for (int c = lane; c < tot; c += 32) {
+    for (int c = threadIdx.x; c < tot; c += 32 * kFieldNearWarps) {
         while (r + 1 < r1 && nruns[r + 1].y <= c) ++r;
         const int2 run = nruns[r];
         const int64_t j = run.x + (c - run.y);
@@ -2401,8 +2404,15 @@ __global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const
         }
         acc = cadd(acc, csub(cmul(H, p[j]), cmul(G, q[j])));
     }
+    __shared__ float2 red[kFieldNearWarps];
     acc = warp_sum(acc);
-    if (lane == 0) v[m] = acc;
+    if (lane == 0) red[warp] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < kFieldNearWarps; ++w) acc = cadd(acc, red[w]);
+        v[m] = acc;
+    }
 }
 
 // The field at the points: tau (near + far) plus the incident field (FP64),
@@ -2906,10 +2916,10 @@ __device__ __forceinline__ void gs_dots_body(const GsArgs &a)
     const int j = jd.x, done = jd.y;
     if (blockIdx.x == 0 && threadIdx.x == 0) st->skip_prod = done;
     if (done) return;
-    // v_j was stored unnormalised (||v_j||^2 = st->nn, set by k_gm_givens of
+    // v_j was stored unnormalised (1 / ||v_j|| = st->rnorm, set by k_gm_givens of
     // step j - 1, or 1 by k_gm_start): scale the block's rows of v_j and of
     // the product
-    const float sc = (float)(1.0 / sqrt(__ldcv(&st->nn)));
+    const float sc = __ldcv(&st->rnorm);
     float2 *vj = g.V + (int64_t)j * g.n + r0;
     __shared__ float2 ws[kGsMaxRows];
 #pragma unroll
@@ -3033,7 +3043,7 @@ __global__ void k_gm_givens(GsPlanes A)
     // there was one); k_gs_dots of step j + 1 scales v_{j+1} by it
     const int j = st->j;
     const double nn = __ldcg(a.gs_acc + 4 * (j & 1) + (*(volatile int *)&st->reorth ? 2 : 1));
-    if (threadIdx.x == 0) st->nn = nn;
+    if (threadIdx.x == 0) st->rnorm = (float)(1.0 / sqrt(nn));
     gm_givens_warp(a, nn, j);
 }
 
@@ -3149,7 +3159,7 @@ __global__ void k_gm_start(GsPlanes A, const float2 *__restrict__ r, int nblk, i
         if (first) st->bnorm = beta;
         st->beta = beta;
         st->j = 0;
-        st->nn = 1.0;      // v_0 is stored normalised
+        st->rnorm = 1.f;   // v_0 is stored normalised
         st->ncols = 0;
         st->done = 0;
         st->skip_prod = 0;

@@ -46,7 +46,7 @@ struct GmresState {
     int reorth;              // second Gram-Schmidt pass needed for the current column
     int n_reorth;            // columns that needed it
     int fault;               // unused (kept zero)
-    double nn;               // ||w||^2 after orthogonalisation (k_gs_finish -> k_gm_givens)
+    float rnorm;             // 1 / ||v_{j+1}||, for k_gs_dots (its FP64 root and division off every block's path)
     // Skip flag of the product kernels: a copy of done taken by k_gs_dots
     // (in stream order before the next product).  done itself is set by
     // k_gm_givens on a side stream while that product runs, so reading it
@@ -386,6 +386,7 @@ __global__ void k_coeffs(int64_t n, const int *type, const double2 *bcv, const i
                          double omega, double rho, double c, double tau, float2 *cp, float2 *cq, float2 *cp0, float2 *cq0,
                          float2 *z, float2 *aq);
 // FMM evaluation of the field at points (see the definitions)
+constexpr int kFieldNearWarps = 4;     // warps per point
 __global__ void k_field_weights(int64_t n, const float2 *p, const float2 *q, const float4 *chi, float k, float4 *wts);
 __global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, const float2 *p,
                              const float2 *q, const int *pleaf, const int *nptr, const int *ntot, const int2 *nruns,
