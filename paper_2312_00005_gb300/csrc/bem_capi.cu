@@ -271,6 +271,8 @@ struct ListsLevelDev {
     DevArr<AggTask> tasks;        // aggregation work items (element chunks)
     DevArr<int> red_ptr, red_c;   // split clusters: partial rows to sum
     int ntasks = 0, nred = 0, nextra = 0;
+    DevArr<int4> pair, pair_ent;  // pairs of targets and their merged lists (ensure_pairs)
+    int npairs = -1;              // -1: not built yet
 };
 
 struct Lists {
@@ -362,6 +364,7 @@ struct LevelDev {
 struct Plan {
     int planes = 1;               // right-hand sides the M and Lambda buffers hold
     DevArr<int4> tgroups;         // transfer blocks (level, target, first direction)
+    DevArr<int4> tpairs;          // the same of four right-hand sides (level, pair of targets, first direction)
     DevArr<AggTask> agg_tasks;    // aggregation blocks (element chunk, first direction pair)
     DevArr<AggTask> agg_tasks_tc; // the same with kTcPairs pairs per block (tensor-core aggregation)
     int n_tc_tasks = 0;
@@ -369,7 +372,7 @@ struct Plan {
     std::shared_ptr<Lists> lists;
     bool shared_lists = false;
     std::vector<std::unique_ptr<LevelDev>> lev;
-    LevelsArgs hargs;             // per-level arguments of the kernels
+    LevelsArgs hargs{};           // per-level arguments of the kernels
     DevArr<float2> val;
     DevArr<float2> valT;          // A^T in A's layout (near_transpose), made from val
     bool valT_valid = false;
@@ -1271,6 +1274,50 @@ PrepArgs prep_args(bem_mesh_impl &M, const float2 *cp, const float2 *cq, const f
     return pa;
 }
 
+// Pairs of targets of the current plan (the transfer of four right-hand
+// sides): consecutive targets of a level, with merged lists in the place of
+// the two.  The lists are built once, by the first plan on them that needs
+// pairs.
+void ensure_pairs(bem_mesh_impl &M)
+{
+    Plan &P = *fr(M).plan;
+    Lists &Ls = *P.lists;
+    cudaStream_t s = fr(M).s;
+    std::vector<std::vector<int4>> pt(P.lev.size());
+    bool build = false;
+    for (size_t l = 0; l < P.lev.size(); ++l) build = build || Ls.lev[l]->npairs < 0;
+    if (build) {
+        for (const int2 &lt : Ls.h_targets) {
+            auto &q = pt[lt.x];
+            if (q.empty() || q.back().y >= 0) q.push_back(make_int4(lt.y, -1, 0, 0));
+            else q.back().y = lt.y;
+        }
+        for (size_t l = 0; l < P.lev.size(); ++l) {
+            ListsLevelDev &L = *Ls.lev[l];
+            L.pair.upload(pt[l], s);
+            L.pair_ent.alloc(L.il_src.n);
+            if (!pt[l].empty())
+                k_pair_lists<<<(unsigned)pt[l].size(), 128, 0, s>>>(L.il_ptr.p, L.il_src.p, L.il_off.p, L.pair.p,
+                                                                    L.pair_ent.p);
+        }
+        ck_launch("k_pair_lists");
+        ck(cudaStreamSynchronize(s), "sync");
+        for (size_t l = 0; l < P.lev.size(); ++l) Ls.lev[l]->npairs = (int)pt[l].size();
+    }
+    std::vector<int4> tp;
+    for (size_t l = 0; l < P.lev.size(); ++l) {
+        const ListsLevelDev &L = *Ls.lev[l];
+        P.hargs.lev[l].pair = L.pair.p;
+        P.hargs.lev[l].pair_ent = L.pair_ent.p;
+        for (int g = 0; g < L.npairs; ++g)
+            for (int nu0 = 0; nu0 < P.lev[l]->nd; nu0 += 32) tp.push_back(make_int4((int)l, g, nu0, 0));
+    }
+    P.tpairs.upload(tp, s);
+    ck(cudaStreamSynchronize(s), "sync");
+    P.hargs.tpairs = P.tpairs.p;
+    P.hargs.ntpairs = (int)tp.size();
+}
+
 // Room for nr right-hand sides in the current plan's M and Lambda buffers
 // and in the product's work vectors (xint, ynear, wts: nr planes of n).
 void ensure_planes(bem_mesh_impl &M, int nr)
@@ -1281,6 +1328,7 @@ void ensure_planes(bem_mesh_impl &M, int nr)
         M.ynear.alloc((size_t)M.n * nr);
         M.wts.alloc((size_t)M.n * nr);
     }
+    if (nr == 4 && !P.hargs.tpairs && P.hargs.ntgroups > 0) ensure_pairs(M);
     if (P.planes >= nr) return;
     LevelsArgs &A = P.hargs;
     for (size_t l = 0; l < P.lev.size(); ++l) {
@@ -1357,11 +1405,10 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
     if (A.ntargets > 0) {
         if (A.ntgroups > 0) {
             KTimer kt_("k_transfer", sf);
-            const int nb = 2 * A.ntgroups;
-            const bool many = nb >= kTransferManyBlocks;
-            if (nr == 4 && many) k_transfer_m4s<<<nb, 32, 0, sf>>>(A, skip);
-            else if (nr == 4) k_transfer_m4<<<nb, 32 * kTransferWarps, 0, sf>>>(A, skip);
-            else if (nr == 2 && many) k_transfer_m2s<<<nb, 32, 0, sf>>>(A, skip);
+            const int nb = 2 * A.ntgroups, np = A.ntpairs;
+            if (nr == 4 && np >= kPairManyBlocks) k_transfer_p4s<<<np, 32 * kPairManyWarps, 0, sf>>>(A, skip);
+            else if (nr == 4) k_transfer_p4<<<np, 32 * kTransferWarps, 0, sf>>>(A, skip);
+            else if (nr == 2 && nb >= kTransferManyBlocks) k_transfer_m2s<<<nb, 32, 0, sf>>>(A, skip);
             else if (nr == 2) k_transfer_m2<<<nb, 32 * kTransferWarps, 0, sf>>>(A, skip);
             else k_transfer_split<<<dim3(A.ntgroups, nr), 32 * kTransferWarps, 0, sf>>>(A, skip);
         }

@@ -1679,8 +1679,8 @@ __global__ void __launch_bounds__(32 * kTransferWarps) k_transfer_split(const __
     }
 }
 
-// The transfer for NR right-hand sides at once: the same blocks and list
-// order as k_transfer_split, each D value loaded once for all planes (the
+// The transfer for NR = 2 right-hand sides at once: the same blocks and list
+// order as k_transfer_split, each D value loaded once for both planes (the
 // M and Lambda planes are mplane and lplane apart).
 template <int NR, int kW>
 __device__ __forceinline__ void transfer_multi_body(const LevelsArgs &A)
@@ -1752,10 +1752,142 @@ __device__ __forceinline__ void transfer_multi_body(const LevelsArgs &A)
         transfer_multi_body<NR, W>(A);                                                                                \
     }
 BEM_TRANSFER_MULTI_KERNEL(k_transfer_m2, 2, kTransferWarps)
-BEM_TRANSFER_MULTI_KERNEL(k_transfer_m4, 4, kTransferWarps)
 BEM_TRANSFER_MULTI_KERNEL(k_transfer_m2s, 2, 1)
-BEM_TRANSFER_MULTI_KERNEL(k_transfer_m4s, 4, 1)
 #undef BEM_TRANSFER_MULTI_KERNEL
+
+// The merged lists of pairs of targets (FarArgs::pair), one block per pair: the
+// first target's sources in their order, then those that only the second
+// lists.  Runs once per set of lists, 10^6 entries in tens of microseconds;
+// built on the host, 158,420 elements took 9 ms.
+__global__ void __launch_bounds__(128) k_pair_lists(const int *__restrict__ il_ptr, const int *__restrict__ il_src,
+                                                    const int *__restrict__ il_off, int4 *__restrict__ pair,
+                                                    int4 *__restrict__ ent)
+{
+    __shared__ int s_n[4];
+    const int4 T = pair[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int a0 = il_ptr[T.x], a1 = il_ptr[T.x + 1];
+    const int b0 = T.y >= 0 ? il_ptr[T.y] : 0, b1 = T.y >= 0 ? il_ptr[T.y + 1] : 0;
+    for (int q = a0 + threadIdx.x; q < a1; q += 128) {
+        const int src = il_src[q];
+        int off = -1;
+        for (int r = b0; r < b1; ++r)
+            if (il_src[r] == src) off = il_off[r];
+        ent[q] = make_int4(src, il_off[q], off, 0);
+    }
+    int end = a1;
+    for (int c = b0; c < b1; c += 128) {
+        const int r = c + threadIdx.x, src = r < b1 ? il_src[r] : -1;
+        bool only = r < b1;
+        for (int q = a0; q < a1; ++q) only = only && il_src[q] != src;
+        const unsigned m = __ballot_sync(0xffffffffu, only);
+        if (lane == 0) s_n[warp] = __popc(m);
+        __syncthreads();
+        int pos = end + __popc(m & ((1u << lane) - 1u));
+        for (int w = 0; w < 4; ++w) {
+            if (w < warp) pos += s_n[w];
+            end += s_n[w];
+        }
+        if (only) ent[pos] = make_int4(src, -1, il_off[r], 0);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) pair[blockIdx.x] = make_int4(T.x, T.y, a0, end - a0);
+}
+
+// The transfer for four right-hand sides at once.  Each D value serves all of
+// them (the M and Lambda planes are mplane and lplane apart), so the bytes are
+// mostly M's, 32 per list entry and direction, and they leave L2 near the rate
+// that the SMs take.  A block therefore takes two targets, neighbours in
+// Morton order that share most of their sources, and 32 directions (lanes): a
+// source's M is read once for both.  kU sources in flight per warp.  One target
+// per block took 49.4 us on 10,580 elements and 942 on 158,420; this 43.2 and
+// 827.  (Groups of four targets need registers that cost more warps than the
+// bytes they save; for two right-hand sides M weighs less, and pairs took 638 us
+// against 575.)
+template <int NR, int kW, int kU>
+__device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
+{
+    __shared__ float2 part[kW][2][NR][32];
+    __shared__ int4 s_ent[kTransferEntries];
+    const int4 T = A.tpairs[blockIdx.x];
+    const FarArgs &f = A.lev[T.x];
+    const int nd = f.nd, nu = T.z + (threadIdx.x & 31);
+    const float2 *__restrict__ M = f.M + nu, *__restrict__ D = f.D + nu;
+    const int64_t mplane = f.mplane;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool live = nu < nd;
+    const int b = f.pair[T.y].z, e = b + f.pair[T.y].w;
+    float2 acc[2][NR];
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[g][r] = make_float2(0.f, 0.f);
+    for (int c0 = b; c0 < e; c0 += kTransferEntries) {
+        const int cnt = min(kTransferEntries, e - c0);
+        __syncthreads();
+        for (int q = threadIdx.x; q < cnt; q += 32 * kW) s_ent[q] = f.pair_ent[c0 + q];
+        __syncthreads();
+        if (!live) continue;
+        for (int q = warp; q < cnt; q += kW * kU) {
+            float2 mv[kU][NR], dv[kU][2];
+            int off[kU][2];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                off[u][0] = off[u][1] = -1;
+                if (q + kW * u < cnt) {
+                    const int4 en = s_ent[q + kW * u];
+                    off[u][0] = en.y;
+                    off[u][1] = en.z;
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) mv[u][r] = M[r * mplane + (int64_t)en.x * nd];
+#pragma unroll
+                    for (int g = 0; g < 2; ++g)
+                        if (off[u][g] >= 0) dv[u][g] = __ldg(D + (int64_t)off[u][g] * nd);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+#pragma unroll
+                for (int g = 0; g < 2; ++g)
+                    if (off[u][g] >= 0)
+#pragma unroll
+                        for (int r = 0; r < NR; ++r) acc[g][r] = cfma(dv[u][g], mv[u][r], acc[g][r]);
+        }
+    }
+    const int4 tg = f.pair[T.y];                   // the second target may be absent (-1)
+    {
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) part[warp][g][r][lane] = acc[g][r];
+        __syncthreads();
+        if (warp > 0) return;
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+#pragma unroll
+                for (int w = 1; w < kW; ++w) acc[g][r] = cadd(acc[g][r], part[w][g][r][lane]);
+    }
+    if (!live) return;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const int t = g ? tg.y : tg.x;
+        if (t < 0) continue;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) f.Lam[r * f.lplane + (int64_t)t * nd + nu] = acc[g][r];
+    }
+}
+
+#define BEM_TRANSFER_PAIRS_KERNEL(NAME, W)                                                                            \
+    __global__ void __launch_bounds__(32 * W) NAME(const __grid_constant__ LevelsArgs A, const int *skip)            \
+    {                                                                                                                 \
+        if (skip_now(skip)) return;                                                                                   \
+        transfer_pairs_body<4, W, 3>(A);                                                                              \
+    }
+BEM_TRANSFER_PAIRS_KERNEL(k_transfer_p4, kTransferWarps)
+BEM_TRANSFER_PAIRS_KERNEL(k_transfer_p4s, kPairManyWarps)
+#undef BEM_TRANSFER_PAIRS_KERNEL
 
 // Disaggregation over all levels (Sec. 3.3.3, matrix S(l), with the
 // Burton-Miller row operator 1 + s.n_i) and the sum with the near field

@@ -106,6 +106,10 @@ struct FarArgs {
     int nred;
     const float4 *dirs;      // (s, w)
     const int *il_ptr, *il_src, *il_off;
+    // pairs of targets for the transfer of four right-hand sides: (target, target
+    // or -1, first entry, entries), and their merged lists: (source, translation
+    // row for each target or -1, 0)
+    const int4 *pair, *pair_ent;
     const float2 *D;         // [noff][nd]
     float2 *M, *Lam;         // [nc][nd]
     const int64_t *cstart;   // [nc + 1] element ranges
@@ -151,6 +155,8 @@ struct LevelsArgs {
     int ntargets;
     const int4 *tgroups;     // transfer blocks: (level, target cluster, first direction, 0)
     int ntgroups;
+    const int4 *tpairs;      // its blocks: (level, pair, first direction, 0); null until needed
+    int ntpairs;
     unsigned int *red_cnt;   // arrival counters of the split clusters (zero between uses)
     FarArgs lev[kMaxFarLevels];
 };
@@ -327,17 +333,23 @@ constexpr int kTransferWarps = 4;          // warps sharing one target's list
 constexpr int kTransferUnroll = 4;         // list entries per warp in flight
 constexpr int kTransferEntries = 512;     // interaction-list entries staged per pass
 __global__ void k_transfer_split(const __grid_constant__ LevelsArgs A, const int *skip);
-// The same for 2 or 4 right-hand sides (M and Lambda planes mplane and
-// lplane apart): each D value is loaded once for all of them.  One block per
-// half of a group of directions; kTransferWarps warps per target, or one (s)
-// from kTransferManyBlocks blocks on, where the blocks alone fill the GPU (four
-// planes: 158,420 elements, 107,000 blocks: 1066 us with four warps, 942 with
-// one; 10,580 elements, 7300 blocks: solves 29.0 and 30.6 ms).
+// The same for 2 right-hand sides (M and Lambda planes mplane and lplane
+// apart): each D value is loaded once for both.  One block per half of a group
+// of directions; kTransferWarps warps per target, or one (s) from
+// kTransferManyBlocks blocks on, where the blocks alone fill the GPU.
 constexpr int kTransferManyBlocks = 20000;
 __global__ void k_transfer_m2(const __grid_constant__ LevelsArgs A, const int *skip);
-__global__ void k_transfer_m4(const __grid_constant__ LevelsArgs A, const int *skip);
 __global__ void k_transfer_m2s(const __grid_constant__ LevelsArgs A, const int *skip);
-__global__ void k_transfer_m4s(const __grid_constant__ LevelsArgs A, const int *skip);
+// For 4 right-hand sides: one block per pair of targets and 32 directions;
+// kTransferWarps warps, or kPairManyWarps (s) from kPairManyBlocks blocks on,
+// where the blocks alone fill the GPU (10,580 elements, 4,800 blocks: 43.2 us
+// with four warps, 49.5 with two; 40,500, 17,400 blocks: 182 and 178; 158,420,
+// 70,000 blocks: 855 and 827).
+constexpr int kPairManyBlocks = 12000;
+constexpr int kPairManyWarps = 2;
+__global__ void k_pair_lists(const int *il_ptr, const int *il_src, const int *il_off, int4 *pair, int4 *ent);
+__global__ void k_transfer_p4(const __grid_constant__ LevelsArgs A, const int *skip);
+__global__ void k_transfer_p4s(const __grid_constant__ LevelsArgs A, const int *skip);
 // 1, 2 or 4 right-hand sides at once (one phase per element and pair for
 // all), element-major with the directions staged in chunks (no dynamic
 // shared memory)
