@@ -17,15 +17,6 @@ __device__ __forceinline__ float2 warp_sum(float2 v)
     }
     return v;
 }
-__device__ __forceinline__ double2 warp_sum_d(double2 v)
-{
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    return v;
-}
-
 
 // ------------------------------------------------------------------ near field
 // Expensive pairs (heavy_rt2) of the stored near field, listed by kind so
@@ -2793,64 +2784,6 @@ __device__ void gm_givens_warp(const GmresArgs &a, double nn, int j)
     }
     __syncwarp();
     for (int l = lane; l <= j + 1; l += 32) a.H[(int64_t)l * m + j] = shr[l];
-}
-
-// Compensated FP32 ("float-float") sums: s + e holds the running sum to
-// about 2^-44 relative.  The reductions below are issued by every block in
-// a fixed order, so all blocks derive identical values without FP64, whose
-// issue rate and latency on this part would dominate the step.
-struct FF {
-    float2 hi, lo;
-};
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ void ff_add1(float &hi, float &lo, float xh, float xl)
-{
-    float s, e;
-    two_sum(hi, xh, s, e);
-    e = __fadd_rn(e, __fadd_rn(lo, xl));
-    hi = __fadd_rn(s, e);
-    lo = __fsub_rn(e, __fsub_rn(hi, s));
-}
-__device__ __forceinline__ void ff_add(FF &a, const FF &b)
-{
-    ff_add1(a.hi.x, a.lo.x, b.hi.x, b.lo.x);
-    ff_add1(a.hi.y, a.lo.y, b.hi.y, b.lo.y);
-}
-// sum of p[0..n), n <= 32 kFFLoads (float2, written by other blocks before
-// the reduction: read through L2) by one warp: lane order, then a fixed
-// xor tree.  All loads are issued before the first add.
-constexpr int kFFLoads = 16;
-__device__ __forceinline__ FF warp_sum_ff(const float2 *p, int n)
-{
-    FF v = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    const int lane = threadIdx.x & 31;
-    float2 x[kFFLoads];
-#pragma unroll
-    for (int u = 0; u < kFFLoads; ++u) {
-        const int q = lane + 32 * u;
-        x[u] = q < n ? __ldcg(p + q) : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < kFFLoads; ++u) {
-        const FF t = {x[u], make_float2(0.f, 0.f)};
-        ff_add(v, t);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        FF x;
-        x.hi.x = __shfl_xor_sync(0xffffffffu, v.hi.x, o);
-        x.hi.y = __shfl_xor_sync(0xffffffffu, v.hi.y, o);
-        x.lo.x = __shfl_xor_sync(0xffffffffu, v.lo.x, o);
-        x.lo.y = __shfl_xor_sync(0xffffffffu, v.lo.y, o);
-        // both partners add in the same operand order: identical results
-        if ((threadIdx.x & o) == 0) ff_add(v, x);
-        else { ff_add(x, v); v = x; }
-    }
-    return v;
 }
 
 // ------------------------------------------------------------------ Gram-Schmidt
