@@ -2501,8 +2501,8 @@ __global__ void k_field_weights(int64_t n, const float2 *__restrict__ p, const f
 // warps share a point: the points nearest to the surface have lists many times
 // the mean, and set the kernel's length (24,874 points, one warp each 74 us,
 // four 46).
-__global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, int64_t M,
-                             float k, const float2 *__restrict__ p, const float2 *__restrict__ q,
+__global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, float k,
+                             const float2 *__restrict__ p, const float2 *__restrict__ q,
                              const int *__restrict__ pleaf, const int *__restrict__ nptr, const int *__restrict__ ntot,
                              const int2 *__restrict__ nruns, float2 *__restrict__ v, int *err)
 {

@@ -400,7 +400,7 @@ __global__ void k_coeffs(int64_t n, const int *type, const double2 *bcv, const i
 // FMM evaluation of the field at points (see the definitions)
 constexpr int kFieldNearWarps = 4;     // warps per point
 __global__ void k_field_weights(int64_t n, const float2 *p, const float2 *q, const float4 *chi, float k, float4 *wts);
-__global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, const float2 *p,
+__global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, float k, const float2 *p,
                              const float2 *q, const int *pleaf, const int *nptr, const int *ntot, const int2 *nruns,
                              float2 *v, int *err);
 __global__ void k_field_eval_finish(const double *pts, int64_t M, float k, float tau, const SourceDev *src, int nsrc,
