@@ -1289,20 +1289,24 @@ void ensure_pairs(bem_mesh_impl &M)
     if (build) {
         for (const int2 &lt : Ls.h_targets) {
             auto &q = pt[lt.x];
-            if (q.empty() || q.back().y >= 0) q.push_back(make_int4(lt.y, -1, 0, 0));
-            else q.back().y = lt.y;
+            if (q.empty() || q[q.size() - 2].y >= 0) {
+                q.push_back(make_int4(lt.y, -1, 0, 0));
+                q.push_back(make_int4(0, 0, 0, 0));
+            } else {
+                q[q.size() - 2].y = lt.y;
+            }
         }
         for (size_t l = 0; l < P.lev.size(); ++l) {
             ListsLevelDev &L = *Ls.lev[l];
             L.pair.upload(pt[l], s);
             L.pair_ent.alloc(L.il_src.n);
             if (!pt[l].empty())
-                k_pair_lists<<<(unsigned)pt[l].size(), 128, 0, s>>>(L.il_ptr.p, L.il_src.p, L.il_off.p, L.pair.p,
+                k_pair_lists<<<(unsigned)(pt[l].size() / 2), 128, 0, s>>>(L.il_ptr.p, L.il_src.p, L.il_off.p, L.pair.p,
                                                                     L.pair_ent.p);
         }
         ck_launch("k_pair_lists");
         ck(cudaStreamSynchronize(s), "sync");
-        for (size_t l = 0; l < P.lev.size(); ++l) Ls.lev[l]->npairs = (int)pt[l].size();
+        for (size_t l = 0; l < P.lev.size(); ++l) Ls.lev[l]->npairs = (int)(pt[l].size() / 2);
     }
     std::vector<int4> tp;
     for (size_t l = 0; l < P.lev.size(); ++l) {

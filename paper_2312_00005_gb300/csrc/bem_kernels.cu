@@ -1747,54 +1747,62 @@ BEM_TRANSFER_MULTI_KERNEL(k_transfer_m2s, 2, 1)
 #undef BEM_TRANSFER_MULTI_KERNEL
 
 // The merged lists of pairs of targets (FarArgs::pair), one block per pair: the
-// first target's sources in their order, then those that only the second
-// lists.  Runs once per set of lists, 10^6 entries in tens of microseconds;
+// sources that both list, then the first target's others, then the second's,
+// each in list order.  Runs once per set of lists, 10^6 entries in tens of microseconds;
 // built on the host, 158,420 elements took 9 ms.
 __global__ void __launch_bounds__(128) k_pair_lists(const int *__restrict__ il_ptr, const int *__restrict__ il_src,
                                                     const int *__restrict__ il_off, int4 *__restrict__ pair,
                                                     int4 *__restrict__ ent)
 {
     __shared__ int s_n[4];
-    const int4 T = pair[blockIdx.x];
+    const int4 T = pair[2 * blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int a0 = il_ptr[T.x], a1 = il_ptr[T.x + 1];
     const int b0 = T.y >= 0 ? il_ptr[T.y] : 0, b1 = T.y >= 0 ? il_ptr[T.y + 1] : 0;
-    for (int q = a0 + threadIdx.x; q < a1; q += 128) {
-        const int src = il_src[q];
-        int off = -1;
-        for (int r = b0; r < b1; ++r)
-            if (il_src[r] == src) off = il_off[r];
-        ent[q] = make_int4(src, il_off[q], off, 0);
-    }
-    int end = a1;
-    for (int c = b0; c < b1; c += 128) {
-        const int r = c + threadIdx.x, src = r < b1 ? il_src[r] : -1;
-        bool only = r < b1;
-        for (int q = a0; q < a1; ++q) only = only && il_src[q] != src;
-        const unsigned m = __ballot_sync(0xffffffffu, only);
-        if (lane == 0) s_n[warp] = __popc(m);
-        __syncthreads();
-        int pos = end + __popc(m & ((1u << lane) - 1u));
-        for (int w = 0; w < 4; ++w) {
-            if (w < warp) pos += s_n[w];
-            end += s_n[w];
+    // entries [c0, c1) of one list whose source is (both) or is not in [o0, o1)
+    // of the other, appended at end
+    int end = a0;
+    auto append = [&](int c0, int c1, int o0, int o1, bool both, bool second) {
+        for (int c = c0; c < c1; c += 128) {
+            const int r = c + threadIdx.x, src = r < c1 ? il_src[r] : -1;
+            int off = -1;
+            for (int q = o0; q < o1; ++q)
+                if (il_src[q] == src) off = il_off[q];
+            const bool take = r < c1 && (off >= 0) == both;
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            if (lane == 0) s_n[warp] = __popc(m);
+            __syncthreads();
+            int pos = end + __popc(m & ((1u << lane) - 1u));
+            for (int w = 0; w < 4; ++w) {
+                if (w < warp) pos += s_n[w];
+                end += s_n[w];
+            }
+            if (take) ent[pos] = second ? make_int4(src, -1, il_off[r], 0) : make_int4(src, il_off[r], off, 0);
+            __syncthreads();
         }
-        if (only) ent[pos] = make_int4(src, -1, il_off[r], 0);
-        __syncthreads();
+    };
+    append(a0, a1, b0, b1, true, false);
+    const int both = end - a0;
+    append(a0, a1, b0, b1, false, false);
+    append(b0, b1, a0, a1, false, true);
+    if (threadIdx.x == 0) {
+        pair[2 * blockIdx.x] = make_int4(T.x, T.y, a0, both);
+        pair[2 * blockIdx.x + 1] = make_int4(end - a0, 0, 0, 0);
     }
-    if (threadIdx.x == 0) pair[blockIdx.x] = make_int4(T.x, T.y, a0, end - a0);
 }
 
 // The transfer for four right-hand sides at once.  Each D value serves all of
 // them (the M and Lambda planes are mplane and lplane apart), so the bytes are
-// mostly M's, 32 per list entry and direction, and they leave L2 near the rate
-// that the SMs take.  A block therefore takes two targets, neighbours in
-// Morton order that share most of their sources, and 32 directions (lanes): a
-// source's M is read once for both.  kU sources in flight per warp.  One target
-// per block took 49.4 us on 10,580 elements and 942 on 158,420; this 43.2 and
-// 827.  (Groups of four targets need registers that cost more warps than the
-// bytes they save; for two right-hand sides M weighs less, and pairs took 638 us
-// against 575.)
+// mostly M's, 32 per list entry and direction.  A block therefore takes two
+// targets, neighbours in Morton order that share most of their sources, and 32
+// directions (lanes): a source's M is read once for both.  The sources of both
+// come first, in a loop without tests, since issue (67% of the slots) is what
+// bounds the kernel then.  kU sources in flight per warp at 72 registers, 28 warps
+// per SM (three in flight spill, and take 1065 us at 80 registers or 841 at 96).  One target per block
+// took 49.4 us on 10,580 elements and 942 on 158,420; pairs with every source
+// tested 43.3 and 827; this 42.5 and 796.  (Groups of four targets need
+// registers that cost more warps than the bytes they save; for two right-hand
+// sides M weighs less, and pairs took 638 us against 575.)
 template <int NR, int kW, int kU>
 __device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
 {
@@ -1807,7 +1815,7 @@ __device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
     const int64_t mplane = f.mplane;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool live = nu < nd;
-    const int b = f.pair[T.y].z, e = b + f.pair[T.y].w;
+    const int b = f.pair[2 * T.y].z, eb = b + f.pair[2 * T.y].w, e = b + f.pair[2 * T.y + 1].x;
     float2 acc[2][NR];
 #pragma unroll
     for (int g = 0; g < 2; ++g)
@@ -1819,7 +1827,28 @@ __device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
         for (int q = threadIdx.x; q < cnt; q += 32 * kW) s_ent[q] = f.pair_ent[c0 + q];
         __syncthreads();
         if (!live) continue;
-        for (int q = warp; q < cnt; q += kW * kU) {
+        int q = warp;
+        const int nboth = min(cnt, eb - c0) - kW * (kU - 1);
+#pragma unroll 1
+        for (; q < nboth; q += kW * kU) {                // sources of both
+            float2 mv[kU][NR], dv[kU][2];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int4 en = s_ent[q + kW * u];
+#pragma unroll
+                for (int r = 0; r < NR; ++r) mv[u][r] = M[r * mplane + (int64_t)en.x * nd];
+                dv[u][0] = __ldg(D + (int64_t)en.y * nd);
+                dv[u][1] = __ldg(D + (int64_t)en.z * nd);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+#pragma unroll
+                for (int g = 0; g < 2; ++g)
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) acc[g][r] = cfma(dv[u][g], mv[u][r], acc[g][r]);
+        }
+#pragma unroll 1
+        for (; q < cnt; q += kW * kU) {
             float2 mv[kU][NR], dv[kU][2];
             int off[kU][2];
 #pragma unroll
@@ -1845,7 +1874,7 @@ __device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
                         for (int r = 0; r < NR; ++r) acc[g][r] = cfma(dv[u][g], mv[u][r], acc[g][r]);
         }
     }
-    const int4 tg = f.pair[T.y];                   // the second target may be absent (-1)
+    const int4 tg = f.pair[2 * T.y];                   // the second target may be absent (-1)
     {
 #pragma unroll
         for (int g = 0; g < 2; ++g)
@@ -1871,10 +1900,10 @@ __device__ __forceinline__ void transfer_pairs_body(const LevelsArgs &A)
 }
 
 #define BEM_TRANSFER_PAIRS_KERNEL(NAME, W)                                                                            \
-    __global__ void __launch_bounds__(32 * W) NAME(const __grid_constant__ LevelsArgs A, const int *skip)            \
+    __global__ void __launch_bounds__(32 * W, 28 / W) NAME(const __grid_constant__ LevelsArgs A, const int *skip)            \
     {                                                                                                                 \
         if (skip_now(skip)) return;                                                                                   \
-        transfer_pairs_body<4, W, 3>(A);                                                                              \
+        transfer_pairs_body<4, W, 2>(A);                                                                              \
     }
 BEM_TRANSFER_PAIRS_KERNEL(k_transfer_p4, kTransferWarps)
 BEM_TRANSFER_PAIRS_KERNEL(k_transfer_p4s, kPairManyWarps)

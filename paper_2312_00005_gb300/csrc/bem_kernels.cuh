@@ -106,9 +106,10 @@ struct FarArgs {
     int nred;
     const float4 *dirs;      // (s, w)
     const int *il_ptr, *il_src, *il_off;
-    // pairs of targets for the transfer of four right-hand sides: (target, target
-    // or -1, first entry, entries), and their merged lists: (source, translation
-    // row for each target or -1, 0)
+    // pairs of targets for the transfer of four right-hand sides, two rows each:
+    // (target, target or -1, first entry, entries that both list) and (entries, 0,
+    // 0, 0), and their merged lists: (source, translation row for each target or
+    // -1, 0)
     const int4 *pair, *pair_ent;
     const float2 *D;         // [noff][nd]
     float2 *M, *Lam;         // [nc][nd]
@@ -342,9 +343,9 @@ __global__ void k_transfer_m2(const __grid_constant__ LevelsArgs A, const int *s
 __global__ void k_transfer_m2s(const __grid_constant__ LevelsArgs A, const int *skip);
 // For 4 right-hand sides: one block per pair of targets and 32 directions;
 // kTransferWarps warps, or kPairManyWarps (s) from kPairManyBlocks blocks on,
-// where the blocks alone fill the GPU (10,580 elements, 4,800 blocks: 43.2 us
-// with four warps, 49.5 with two; 40,500, 17,400 blocks: 182 and 178; 158,420,
-// 70,000 blocks: 855 and 827).
+// where the blocks alone fill the GPU (pairs with every source tested: 10,580
+// elements, 4,800 blocks: 43.2 us with four warps, 49.5 with two; 40,500, 17,400
+// blocks: 182 and 178; 158,420, 70,000 blocks: 855 and 827).
 constexpr int kPairManyBlocks = 12000;
 constexpr int kPairManyWarps = 2;
 __global__ void k_pair_lists(const int *il_ptr, const int *il_src, const int *il_off, int4 *pair, int4 *ent);
