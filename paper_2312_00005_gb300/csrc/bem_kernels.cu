@@ -3257,6 +3257,9 @@ __global__ void k_gm_start(GsPlanes A, const float2 *__restrict__ r, int nblk, i
         st->ncols = 0;
         st->done = 0;
         st->skip_prod = 0;
+        // the last cycle may have ended inside a graph body, whose further
+        // steps set it: the product of the new v_0 must not skip
+        st->skip_all = 0;
         st->converged = 0;
         st->bodies = 0;
         st->resid = st->bnorm > 0.0 ? beta / st->bnorm : 0.0;
