@@ -689,6 +689,41 @@ __device__ __noinline__ int cut_pair(const NearArgs &a, int64_t i, int64_t j, un
     }
 }
 
+// first point of order m in a table of orders 1 to 6: 0, 1, 5, 14, 30, 55
+__device__ __forceinline__ int rule_at(int m) { return (m - 1) * m * (2 * m - 1) / 6; }
+// The part's share of A_ij, to FP32 rounding; rule: (xi, eta, 2 w) of the
+// points of orders 1 to 6.
+__device__ __forceinline__ float2 part_entry(const NearArgs &a, int64_t i, int64_t j, unsigned code, const float4 *rule)
+{
+    const int m = (code >> 24) & 7, depth = (code >> 20) & 15;
+    const SubTri T = part_triangle(code, depth);
+    const float4 ch = a.E.chi[j];
+    const float3 g1 = f3(a.E.e1[j]), g2 = f3(a.E.e2[j]), ny = f3(a.E.nrm[j]), nx = f3(a.E.nrm[i]);
+    const float3 base = add3(add3(sub3f(f3(ch), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i]))), f3(a.E.va[j]));
+    const float sa = ch.w * exp2f(-2.0f * (float)depth);
+    const float sx1 = T.x1 - T.x0, sy1 = T.y1 - T.y0, sx2 = T.x2 - T.x0, sy2 = T.y2 - T.y0;
+    float2 Kp = make_float2(0.f, 0.f), Kq = Kp;
+    const int r1 = rule_at(m + 1);
+    for (int v = rule_at(m); v < r1; ++v) {
+        const float4 rl = rule[v];
+        const float px = T.x0 + rl.x * sx1 + rl.y * sx2, py = T.y0 + rl.x * sy1 + rl.y * sy2;
+        bm_point<true>(mad3(py, g2, mad3(px, g1, base)), nx, ny, a.k, a.ik_inv, sa * rl.z, Kp, Kq);
+    }
+    return cadd(cmul(a.cp[j], Kp), cmul(a.cq[j], Kq));
+}
+// v times x_w for every right-hand side, added to a row's FP64 sums (h[r][row]
+// in shared memory, h at the row).
+template <int NR>
+__device__ __forceinline__ void add_entry(double2 *h, const float2 *__restrict__ x, int64_t n, int64_t w, float2 v)
+{
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const float2 c = cmul(v, x[r * n + w]);
+        atomicAdd(&h[r * kFusedRows].x, (double)c.x);
+        atomicAdd(&h[r * kFusedRows].y, (double)c.y);
+    }
+}
+
 // Near-field product with the entries recomputed on the fly (no storage):
 // the conventional dense BEM product when the near list is everything, and
 // the known boundary data's product.  Bound by FP32 / SFU issue (one kernel
@@ -703,14 +738,17 @@ __device__ __noinline__ int cut_pair(const NearArgs &a, int64_t i, int64_t j, un
 //     or more columns side by side in a warp.)
 //   - orders 1 to 3 are evaluated in place; the expensive pairs (subdivided
 //     elements, orders 4 to 6, distances within rounding of a threshold) are
-//     queued per block and worked off after the tiles by all its threads:
+//     queued per block and worked off after the tiles (and between two when
+//     the queue is half full) by all its threads:
 //     each pair is first cut into its parts under one rule (the subdivision
 //     without any integration), the parts are sorted by their order, and the
 //     lanes then take parts of one order, so that a warp's loops have one
 //     length.  (Pairs taken whole, one per thread, had lanes of a warp in
 //     different parts and orders: 7 times the instructions.)  The self terms
-//     take a warp each.  The sums of all these are FP64 additions in shared
-//     memory, so their order does not show.
+//     take a warp each.  The sums of all these are FP64 additions of FP32
+//     terms in shared memory, exact while a row's terms lie within a factor of
+//     2^20, so their order does not show; a pair that finds the queue full
+//     waits for its next filling, so that every pair is taken the same way.
 // A block takes the rows of one task and every gridDim.y-th part of the
 // tiles; with several parts, k_near_fused_sum adds them in order.  NR right-
 // hand sides share every entry.  One warp per row with lanes over the columns
@@ -772,8 +810,6 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     if (threadIdx.x < kFusedRows)
 #pragma unroll
         for (int r = 0; r < NR; ++r) s_h[r][threadIdx.x] = make_double2(0.0, 0.0);
-    // first point of order m: 0, 1, 5, 14, 30, 55
-    auto rule_at = [](int m) { return (m - 1) * m * (2 * m - 1) / 6; };
     if (threadIdx.x < 91) {
         int m = 1;
         while (rule_at(m + 1) <= (int)threadIdx.x) ++m;
@@ -807,24 +843,72 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     float2 acc[NR], accq = make_float2(0.f, 0.f);      // kT: acc[0] the p sum, accq the q sum
 #pragma unroll
     for (int r = 0; r < NR; ++r) acc[r] = make_float2(0.f, 0.f);
-    // v times x of the pair (row, wj), added to the row's FP64 sums
-    auto add_pair = [&](int row, int wj, float2 v) {
+    // the queued pairs, kFusedThreads at a time: cut into parts, the parts
+    // sorted by order, the parts integrated; pairs whose parts found no room go
+    // into another round (called by the whole block after a barrier; takes the
+    // staged tile's place)
+    auto drain = [&]() {
+        const int nq = min(s_qn, kFusedQueue);
+        int q = threadIdx.x;                           // this thread's next pair
+        while (__syncthreads_or(q < nq)) {
+            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
+            __syncthreads();
+            if (q < nq) {
+                const int row = s_qr[q], wj = s_qj[q];
+                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
+                const int np = cut_pair(a, i, j, nullptr, 0);
+                if (np > 0 && np <= kFusedParts) {
+                    const int at = atomicAdd(&s_pn[0], np);
+                    if (at + np <= kFusedParts) {
+                        unsigned *pc = s_pc + at;
+                        cut_pair(a, i, j, pc, (unsigned)row << 27);
+                        for (int u = 0; u < np; ++u) {
+                            s_pj[at + u] = wj;
+                            atomicAdd(&s_pn[(pc[u] >> 24) & 7], 1);
+                        }
+                        q += kFusedThreads;
+                    } else {
+                        for (int u = at; u < min(at + np, kFusedParts); ++u) s_pc[u] = 0;   // order 0: no part
+                    }
+                } else {
+                    // cut deeper than a code can say
+                    float2 v;
+                    if (general_entry(a, i, j, &v)) add_entry<NR>(&s_h[0][row], x, a.E.n, wj, v);
+                    else atomicMin(err, (int)j);
+                    q += kFusedThreads;
+                }
+            }
+            __syncthreads();
+            const int n_all = min(s_pn[0], kFusedParts);
+            int start[8];                              // first slot of an order: the longest first
+            start[7] = 0;
+            start[6] = 0;
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const float2 c = cmul(v, x[r * a.E.n + wj]);
-            atomicAdd(&s_h[r][row].x, (double)c.x);
-            atomicAdd(&s_h[r][row].y, (double)c.y);
+            for (int m = 5; m >= 1; --m) start[m] = start[m + 1] + s_pn[m + 1];
+            const int n_parts = start[1] + s_pn[1];
+            __syncthreads();
+            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
+            __syncthreads();
+            for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
+                const int m = (s_pc[u] >> 24) & 7;
+                if (m == 0) continue;
+                int at = start[1];
+#pragma unroll
+                for (int v = 2; v <= 6; ++v)
+                    if (m == v) at = start[v];
+                s_po[at + atomicAdd(&s_pn[m], 1)] = (unsigned short)u;
+            }
+            __syncthreads();
+            for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) {
+                const int pi = s_po[u], wj = s_pj[pi];
+                const unsigned pc = s_pc[pi];
+                const int row = pc >> 27;
+                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
+                add_entry<NR>(&s_h[0][row], x, a.E.n, wj, part_entry(a, i, j, pc, s_rule));
+            }
         }
-    };
-    // a pair or part that found no room in the queues: the general rule
-    auto general = [&](int row, int wj) {
-        const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
-        float2 v;
-        if (!general_entry(a, i, j, &v)) {
-            atomicMin(err, (int)j);
-            return;
-        }
-        add_pair(row, wj, v);
+        __syncthreads();
+        if (threadIdx.x == 0) s_qn = 0;
     };
     const int nc = a.N.ncol[t];
     const int ntile = (nc + kFusedTile - 1) / kFusedTile;
@@ -844,8 +928,26 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         part = (int)((part + max((int64_t)0, min(own, (int64_t)ntile - 1)) * gridDim.y / ntile) % gridDim.y);
     }
     const int tb = (int)((int64_t)ntile * part / gridDim.y), te = (int)((int64_t)ntile * (part + 1) / gridDim.y);
-    for (int tile = tb; tile < te; ++tile) {
-        __syncthreads();
+    unsigned pend = 0;                                 // columns of this lane that found the queue full
+    for (int tile = tb;; ++tile) {
+        // the queue is worked off after the last tile, before one that may fill
+        // it, and where it was too short for the last one (s_qn is the same in
+        // every thread: no pushes since the barrier)
+        for (;;) {
+            const bool full = __syncthreads_or(pend != 0);
+            if (!full && tile < te && s_qn <= kFusedQueue / 2) break;
+            drain();
+            __syncthreads();
+            if (!full) break;
+            for (unsigned left = pend; left; left &= left - 1) {
+                const int b = __ffs((int)left) - 1, slot = atomicAdd(&s_qn, 1);
+                if (slot >= kFusedQueue) break;
+                s_qj[slot] = s_j[warp * 32 + b];
+                s_qr[slot] = (unsigned char)rr;
+                pend &= ~(1u << b);
+            }
+        }
+        if (tile >= te) break;
         bool q_here = false;
         {
             const int p = tile * kFusedTile + threadIdx.x;
@@ -913,7 +1015,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
                     s_qj[slot] = s_j[c];
                     s_qr[slot] = (unsigned char)rr;
                 } else {
-                    general(rr, s_j[c]);
+                    pend |= 1u << (c - c0);
                 }
                 continue;
             }
@@ -953,86 +1055,14 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         accq = cadd(accq, tq);
     }
     if (kT) acc[0] = cadd(cmul(ecp, acc[0]), cmul(ecq, accq));
-    __syncthreads();
-    // the queued pairs, kFusedThreads at a time: cut into parts, the parts
-    // sorted by order, the parts integrated; then the self terms
-    {
-        const int nq = min(s_qn, kFusedQueue);
-        for (int q0 = 0; q0 < nq; q0 += kFusedThreads) {
-            __syncthreads();
-            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
-            __syncthreads();
-            if (q0 + (int)threadIdx.x < nq) {
-                const int row = s_qr[q0 + threadIdx.x], wj = s_qj[q0 + threadIdx.x];
-                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
-                // more parts than room for this pair: all of it by the general rule
-                const int np = cut_pair(a, i, j, nullptr, 0);
-                const int at = np > 0 ? atomicAdd(&s_pn[0], np) : 0;
-                if (np > 0 && at + np <= kFusedParts) {
-                    unsigned *pc = s_pc + at;
-                    cut_pair(a, i, j, pc, (unsigned)row << 27);
-                    for (int u = 0; u < np; ++u) {
-                        s_pj[at + u] = wj;
-                        atomicAdd(&s_pn[(pc[u] >> 24) & 7], 1);
-                    }
-                } else {
-                    if (np > 0)
-                        for (int u = at; u < min(at + np, kFusedParts); ++u) s_pc[u] = 0;   // order 0: no part
-                    general(row, wj);
-                }
-            }
-            __syncthreads();
-            const int n_all = min(s_pn[0], kFusedParts);
-            int start[8];                              // first slot of an order: the longest first
-            start[7] = 0;
-            start[6] = 0;
-#pragma unroll
-            for (int m = 5; m >= 1; --m) start[m] = start[m + 1] + s_pn[m + 1];
-            const int n_parts = start[1] + s_pn[1];
-            __syncthreads();
-            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
-            __syncthreads();
-            for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
-                const int m = (s_pc[u] >> 24) & 7;
-                if (m == 0) continue;
-                int at = start[1];
-#pragma unroll
-                for (int v = 2; v <= 6; ++v)
-                    if (m == v) at = start[v];
-                s_po[at + atomicAdd(&s_pn[m], 1)] = (unsigned short)u;
-            }
-            __syncthreads();
-            for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) {
-                const int pi = s_po[u], wj = s_pj[pi];
-                const unsigned pc = s_pc[pi];
-                const int row = pc >> 27, m = (pc >> 24) & 7, depth = (pc >> 20) & 15;
-                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
-                const SubTri T = part_triangle(pc, depth);
-                const float4 ch = a.E.chi[j];
-                const float3 g1 = f3(a.E.e1[j]), g2 = f3(a.E.e2[j]), ny = f3(a.E.nrm[j]), nx = f3(a.E.nrm[i]);
-                const float3 base = add3(add3(sub3f(f3(ch), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i]))),
-                                         f3(a.E.va[j]));
-                const float sa = ch.w * exp2f(-2.0f * (float)depth);
-                const float sx1 = T.x1 - T.x0, sy1 = T.y1 - T.y0, sx2 = T.x2 - T.x0, sy2 = T.y2 - T.y0;
-                float2 Kp = make_float2(0.f, 0.f), Kq = Kp;
-                const int r0 = rule_at(m), r1 = rule_at(m + 1);
-                for (int v = r0; v < r1; ++v) {
-                    const float4 rl = s_rule[v];
-                    const float px = T.x0 + rl.x * sx1 + rl.y * sx2, py = T.y0 + rl.x * sy1 + rl.y * sy2;
-                    bm_point<true>(mad3(py, g2, mad3(px, g1, base)), nx, ny, k, ik_inv, sa * rl.z, Kp, Kq);
-                }
-                add_pair(row, wj, cadd(cmul(a.cp[j], Kp), cmul(a.cq[j], Kq)));
-            }
-        }
-        for (int row = warp; row < cnt; row += kW) {
-            if (!s_self[row]) continue;
-            const int64_t j = e0 + row;
-            float2 G, Ee;
-            self_points(a.E, j, k, Q, lane, G, Ee);
-            G = warp_sum(G);
-            Ee = warp_sum(Ee);
-            if (lane == 0) add_pair(row, (int)j, self_entry(G, Ee, k, ik_inv, a.tau, a.cp[j], a.cq[j]));
-        }
+    for (int row = warp; row < cnt; row += kW) {       // the self terms
+        if (!s_self[row]) continue;
+        const int64_t j = e0 + row;
+        float2 G, Ee;
+        self_points(a.E, j, k, Q, lane, G, Ee);
+        G = warp_sum(G);
+        Ee = warp_sum(Ee);
+        if (lane == 0) add_entry<NR>(&s_h[0][row], x, a.E.n, j, self_entry(G, Ee, k, ik_inv, a.tau, a.cp[j], a.cq[j]));
     }
     // the lanes' sums of a row in (warp, side-by-side column) order
     float2 *red = reinterpret_cast<float2 *>(s_buf);
