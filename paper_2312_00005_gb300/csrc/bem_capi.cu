@@ -88,7 +88,8 @@ QuadTables make_tables(const bem_params &p)
         Q.Rd[m] = R[m];
         Q.R2[m] = (float)(R[m] * R[m]);
     }
-    Q.heavy_rt2 = p.m_max > 3 ? (float)((R[3] * (1.0 + 1e-5)) * (R[3] * (1.0 + 1e-5))) : 0.f;
+    Q.heavy_rt2 = p.m_max > 3 ? (float)heavy_threshold(p.rt_subdiv, R) : 0.f;
+    Q.whole_rt2 = (float)((p.rt_subdiv * (1.0 + 1e-5)) * (p.rt_subdiv * (1.0 + 1e-5)));
     Q.rt_sub = (float)p.rt_subdiv;
     Q.rt_sub_d = p.rt_subdiv;
     Q.m_max = p.m_max;

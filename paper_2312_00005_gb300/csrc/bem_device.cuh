@@ -19,9 +19,10 @@ struct QuadTables {
     float rt_sub;
     double rt_sub_d;
     // squared thresholds of the light / heavy split: a pair is light when
-    // r~^2 > heavy_rt2 = (R_3 (1 + 1e-5))^2; R2[m] = R_m^2
+    // r~^2 > heavy_rt2 = (max(R_3, rt_sub) (1 + 1e-5))^2; R2[m] = R_m^2; no
+    // element is subdivided above whole_rt2 = (rt_sub (1 + 1e-5))^2
     float R2[kRules];
-    float heavy_rt2;
+    float heavy_rt2, whole_rt2;
     int m_max;
     int max_depth;
     int edge_parts;
@@ -220,8 +221,8 @@ __device__ __forceinline__ float pair_rt2(float3 xj_hi, float3 xj_lo, float3 xi_
     return __fmul_rn(__fmaf_rn(D0.x, D0.x, __fmaf_rn(D0.y, D0.y, __fmul_rn(D0.z, D0.z))), inv_area);
 }
 // Expensive pair: the self term, or an element whose r~ (whole element) is
-// not clearly above R_3, i.e. that may need subdivision or a rule of order
-// >= 4.  The cheap pairs take 1 to 9 quadrature points.
+// not clearly above R_3 and rt_sub, i.e. that may need subdivision or a rule of
+// order >= 4.  The cheap pairs take 1 to 9 quadrature points.
 __device__ __forceinline__ bool heavy_rt2(int64_t i, int64_t j, float rt2, const QuadTables &Q)
 {
     if (i == j) return true;
@@ -281,12 +282,12 @@ __device__ bool integrate_regular_acc(const ElemDev &E, int64_t j, float3 xhi, f
     const float3 va = f3(E.va[j]), e1 = f3(E.e1[j]), e2 = f3(E.e2[j]), ny = f3(E.nrm[j]);
     const float3 base = add3(D0, va);                                   // a - x
     const float area = ch.w;
-    // Fast path: r~ of the whole element clearly above R_1 (order m = 1, no
-    // subdivision).  The 1 x 1 conical rule is the centroid rule (node
+    // Fast path: r~ of the whole element clearly above R_1 and rt_sub (order m =
+    // 1, no subdivision).  The 1 x 1 conical rule is the centroid rule (node
     // (1/3, 1/3), weight 1/2), so the integral is A_j K(x, x_j).
     if (Q.m_max > 1) {
         const float rt0 = sqrtf(dot3f(D0, D0) / area);
-        if (rt0 > Q.R[1] * (1.0f + 1e-5f)) {
+        if (rt0 > fmaxf(Q.R[1], Q.rt_sub) * (1.0f + 1e-5f)) {
             acc.point(D0, ny, area);
             return true;
         }

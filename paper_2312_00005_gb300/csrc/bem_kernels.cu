@@ -832,11 +832,11 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         needp = __any_sync(0xffffffffu, ecp.x != 0.f || ecp.y != 0.f);
         needq = __any_sync(0xffffffffu, ecq.x != 0.f || ecq.y != 0.f);
     }
-    // thresholds on r~^2: order 1 clearly above R_1; orders 1 to 3 above
+    // thresholds on r~^2: order 1 clearly above R_1 and rt_sub; orders 1 to 3 above
     // heavy_rt2 and not within 2e-5 of R_1 or R_2 (m_max <= 3 has no such
     // split: everything but order 1 goes to the general rule)
     const bool split = Q.m_max > 3;
-    const float rt1 = Q.m_max > 1 ? Q.R2[1] * (1.0f + 2e-5f) : __int_as_float(0x7f800000);
+    const float rt1 = Q.m_max > 1 ? fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2) : __int_as_float(0x7f800000);
     const float rt1lo = Q.R2[1] * (1.0f - 2e-5f), rt2hi = Q.R2[2] * (1.0f + 2e-5f), rt2lo = Q.R2[2] * (1.0f - 2e-5f);
     const float rth = Q.heavy_rt2;
     const float k = a.k, ik_inv = a.ik_inv;
@@ -2385,7 +2385,7 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
     const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
     const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
                                    (float)(xd[2] - (double)xhi.z));
-    const float rt1 = Q.m_max > 1 ? Q.R2[1] * (1.0f + 2e-5f) : __int_as_float(0x7f800000);
+    const float rt1 = Q.m_max > 1 ? fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2) : __int_as_float(0x7f800000);
     auto general = [&](int row, int j) {
         float2 v[kN];
         if (!field_entry<kGrad>(E, Q, j, s_x[row], k, p[j], q[j], v)) {

@@ -237,6 +237,12 @@ void order_thresholds(double tol, int m_max, double *R)
     }
 }
 
+double heavy_threshold(double rt_subdiv, const double *R)
+{
+    const double r = std::max(R[3], rt_subdiv) * (1.0 + 1e-5);
+    return r * r;
+}
+
 void sphere_grid(int L, std::vector<double> &s, std::vector<double> &w)
 {
     std::vector<double> t, wt;
@@ -979,9 +985,7 @@ NearCount count_near_points(const Geometry &g, const Tree &t, const FreqPlan &fp
     NearCount c;
     double R[kMaxRule + 1] = {0};
     order_thresholds(p.quad_tol, std::max(2, p.m_max), R);
-    // the light / heavy split of the entry kernels: light when r~ is above
-    // R_3 (1 + 1e-5), so that one rule of order 1..3 covers the element
-    const double heavy_rt2 = p.m_max > 3 ? (R[3] * (1.0 + 1e-5)) * (R[3] * (1.0 + 1e-5)) : 0.0;
+    const double heavy_rt2 = p.m_max > 3 ? heavy_threshold(p.rt_subdiv, R) : 0.0;
     const Level &Lf = t.lv[fp.leaf_depth];
     const int nl = (int)Lf.start.size();
     for (int a = 0; a < nl; ++a) {

@@ -61,6 +61,9 @@ void conical_rule(int m, std::vector<double> &xi, std::vector<double> &eta, std:
 // R[m] for m = 1..m_max-1: the regular order is the smallest m with r~ > R[m]
 // (all three a-priori estimates of Sec. 3.1.4 below tol), else m_max.
 void order_thresholds(double tol, int m_max, double *R);
+// The light / heavy split of the entry kernels (m_max > 3): light when r~^2
+// exceeds this, so that one rule of order 1..3 covers the whole element.
+double heavy_threshold(double rt_subdiv, const double *R);
 // unit-sphere grid: L Gauss-Legendre nodes in cos(theta) x 2L azimuths
 // phi = pi b / L; weights w_GL * pi / L (sum 4 pi).  s: 3 * 2L^2, ordered in
 // antipodal halves: for q < L^2, s_{q + L^2} = -s_q exactly (same weight),
