@@ -832,13 +832,13 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         needp = __any_sync(0xffffffffu, ecp.x != 0.f || ecp.y != 0.f);
         needq = __any_sync(0xffffffffu, ecq.x != 0.f || ecq.y != 0.f);
     }
-    // thresholds on r~^2: order 1 clearly above R_1 and rt_sub; orders 1 to 3 above
-    // heavy_rt2 and not within 2e-5 of R_1 or R_2 (m_max <= 3 has no such
-    // split: everything but order 1 goes to the general rule)
-    const bool split = Q.m_max > 3;
-    const float rt1 = Q.m_max > 1 ? fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2) : __int_as_float(0x7f800000);
+    // thresholds on r~^2: order 1 clearly above R_1 and rt_sub; orders 2 and 3
+    // above heavy_rt2 (m_max <= 3: rt_sub, all regular orders being among them)
+    // and not within 2e-5 of R_1 or R_2 (R2[m] = 0 from m_max on: m_max = 2 has
+    // no order 3 and m_max = 1 no order 2 here)
+    const float rt1 = fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2);
     const float rt1lo = Q.R2[1] * (1.0f - 2e-5f), rt2hi = Q.R2[2] * (1.0f + 2e-5f), rt2lo = Q.R2[2] * (1.0f - 2e-5f);
-    const float rth = Q.heavy_rt2;
+    const float rth = Q.m_max > 3 ? Q.heavy_rt2 : Q.whole_rt2;
     const float k = a.k, ik_inv = a.ik_inv;
     float2 acc[NR], accq = make_float2(0.f, 0.f);      // kT: acc[0] the p sum, accq the q sum
 #pragma unroll
@@ -1001,7 +1001,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
                                  : pair_rt2(f3(whi), f3(wlo), f3(ehi), f3(elo), wlo.w, D0);
             int code = 0;
             if (rt2 > rt1) code = 1;
-            else if (split && rt2 > rth && rt2 < rt1lo && (rt2 > rt2hi || rt2 < rt2lo)) code = rt2 > rt2hi ? 2 : 3;
+            else if (rt2 > rth && rt2 < rt1lo && (rt2 > rt2hi || rt2 < rt2lo)) code = rt2 > rt2hi ? 2 : 3;
             const float3 wn = f3(s_n[c]);
             const float3 nx = kT ? wn : f3(en), ny = kT ? f3(en) : wn;
             const float area = kT ? ehi.w : whi.w;
@@ -2385,7 +2385,7 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
     const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
     const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
                                    (float)(xd[2] - (double)xhi.z));
-    const float rt1 = Q.m_max > 1 ? fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2) : __int_as_float(0x7f800000);
+    const float rt1 = fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2);   // R2[1] = 0 with m_max = 1
     auto general = [&](int row, int j) {
         float2 v[kN];
         if (!field_entry<kGrad>(E, Q, j, s_x[row], k, p[j], q[j], v)) {
