@@ -290,7 +290,8 @@ struct Lists {
     DevArr<int4> multi_items;     // the same for several right-hand sides
     int n_multi_items = 0;
     DevArr<int4> fused_tasks;     // (leaf, first row, end row) of the recomputed product (internal rows)
-    int n_fused = 0, fused_s = 1; // ... and the parts of the columns
+    int n_fused = 0;              // ... their number
+    FusedSplit fused;             // ... rows per task, columns per tile and parts of the columns
     int64_t nnz = 0;
     std::vector<std::unique_ptr<ListsLevelDev>> lev;
     // all levels together, for the one-launch far-field kernels
@@ -655,15 +656,15 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         Ls->spmv_items.upload(items, s);
         Ls->n_multi_items = (int)multi.size();
         Ls->multi_items.upload(multi, s);
+        Ls->fused = fused_split(Lf.count, Ls->max_ncol);
         std::vector<int4> ft;
         for (int t = 0; t < nl; ++t) {
             const int64_t a = leaf_start[t], cnt = Lf.count[t];
-            const int64_t nch = (cnt + kFusedRows - 1) / kFusedRows;
+            const int64_t nch = (cnt + Ls->fused.rows - 1) / Ls->fused.rows;
             for (int64_t q = 0; q < nch; ++q)
                 ft.push_back(make_int4(t, (int)(a + cnt * q / nch), (int)(a + cnt * (q + 1) / nch), 0));
         }
         Ls->n_fused = (int)ft.size();
-        Ls->fused_s = fused_parts(Ls->n_fused, Ls->max_ncol);
         Ls->fused_tasks.upload(ft, s);
         ck(cudaStreamSynchronize(s), "sync");   // items and ft are uploaded before they go
     }
@@ -1188,7 +1189,7 @@ void store_near(bem_mesh_impl &M, Plan &P, const float2 *cp, const float2 *cq)
 void ensure_fused(bem_mesh_impl &M, int nr)
 {
     const Lists &Ls = *fr(M).plan->lists;
-    if (Ls.fused_s > 1) fr(M).fpart.alloc((size_t)Ls.fused_s * std::min(nr, kMaxPlanes) * M.n);
+    if (Ls.fused.parts > 1) fr(M).fpart.alloc((size_t)Ls.fused.parts * std::min(nr, kMaxPlanes) * M.n);
 }
 
 // y = the recomputed near-field product of nr planes of x (transposed when
@@ -1200,24 +1201,25 @@ void near_fused(bem_mesh_impl &M, const Plan &P, const NearArgs &a, const float2
     if (Ls.n_fused == 0) return;
     ensure_fused(M, nr);
     int *err = fr(M).err.p;
-    const dim3 grid(Ls.n_fused, Ls.fused_s);
+    const dim3 grid(Ls.n_fused, Ls.fused.parts);
+    const int rows = Ls.fused.rows, cols = Ls.fused.cols;
     const char *name = kt ? "k_near_fused_t" : "k_near_fused";
     for (int r = 0; r < nr;) {
         const int g = nr - r >= 4 ? 4 : (nr - r >= 2 ? 2 : 1);
         const float2 *xr = x + (int64_t)r * M.n;
-        float2 *yr = y + (int64_t)r * M.n, *o = Ls.fused_s > 1 ? fr(M).fpart.p : yr;
+        float2 *yr = y + (int64_t)r * M.n, *o = Ls.fused.parts > 1 ? fr(M).fpart.p : yr;
         {
             KTimer kt_(name, s);
-            if (kt) k_near_fused_t<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
-            else if (g == 4) k_near_fused_4<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
-            else if (g == 2) k_near_fused_2<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
-            else k_near_fused_1<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, xr, o, err, skip);
+            if (kt) k_near_fused_t<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, rows, cols, xr, o, err, skip);
+            else if (g == 4) k_near_fused_4<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, rows, cols, xr, o, err, skip);
+            else if (g == 2) k_near_fused_2<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, rows, cols, xr, o, err, skip);
+            else k_near_fused_1<<<grid, kFusedThreads, 0, s>>>(a, Ls.fused_tasks.p, rows, cols, xr, o, err, skip);
         }
         ck_launch(name);
-        if (Ls.fused_s > 1) {
+        if (Ls.fused.parts > 1) {
             {
                 KTimer kt_("k_near_fused_sum", s);
-                k_near_fused_sum<<<nblocks((int64_t)g * M.n, 256), 256, 0, s>>>(o, Ls.fused_s, (int64_t)g * M.n, yr, skip);
+                k_near_fused_sum<<<nblocks((int64_t)g * M.n, 256), 256, 0, s>>>(o, Ls.fused.parts, (int64_t)g * M.n, yr, skip);
             }
             ck_launch("k_near_fused_sum");
         }

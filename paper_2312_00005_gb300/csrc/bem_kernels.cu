@@ -731,8 +731,8 @@ __device__ __forceinline__ void add_entry(double2 *h, const float2 *__restrict__
 // layout keeps everything else out of the inner loop and the lanes together:
 //   - a lane holds one row (its midpoint and normal) in registers, the 32
 //     rows being neighbours in Morton order; the columns are staged in shared
-//     memory in tiles of kFusedTile and read as broadcasts, warp w taking
-//     columns [32 w, 32 w + 32) of a tile.  The rows of a warp see a column
+//     memory in tiles of `cols` and read as broadcasts, each warp taking an
+//     eighth of a tile.  The rows of a warp see a column
 //     at nearly the same distance, so they mostly agree on its rule, and no
 //     sum crosses lanes until the end.  (Leaves of at most 16 rows put two
 //     or more columns side by side in a warp.)
@@ -759,7 +759,7 @@ __device__ __forceinline__ void add_entry(double2 *h, const float2 *__restrict__
 // column j, the rows i whose leaves are in the near list of j's own leaf are
 // staged, y_j = cp_j sum_i Kp_ij x_i + cq_j sum_i Kq_ij x_i.
 template <int NR, bool kT>
-__device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *__restrict__ tasks,
+__device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *__restrict__ tasks, int rows, int cols,
                                                 const float2 *__restrict__ x, float2 *__restrict__ out,
                                                 int *__restrict__ err)
 {
@@ -796,8 +796,8 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         e0 = T.y;
         e1 = T.z;
     } else {                                           // one leaf holds every element
-        e0 = (int64_t)blockIdx.x * kFusedRows;
-        e1 = min(a.E.n, e0 + kFusedRows);
+        e0 = (int64_t)blockIdx.x * rows;
+        e1 = min(a.E.n, e0 + rows);
     }
     const int cnt = (int)(e1 - e0);
     int w = 1;
@@ -911,7 +911,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         if (threadIdx.x == 0) s_qn = 0;
     };
     const int nc = a.N.ncol[t];
-    const int ntile = (nc + kFusedTile - 1) / kFusedTile;
+    const int ntile = (nc + cols - 1) / cols, chunk = cols / kW;
     const int run0 = a.N.run_ptr[t], run1 = a.N.run_ptr[t + 1];
     // this block's part of the tiles: the parts that hold the rows' own
     // columns, and with them the expensive pairs, are the first of the grid
@@ -924,7 +924,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
             if (a.N.runs[mid].x <= e0) lo = mid;
             else hi = mid - 1;
         }
-        const int64_t own = (a.N.runs[lo].y + (e0 - a.N.runs[lo].x)) / kFusedTile;
+        const int64_t own = (a.N.runs[lo].y + (e0 - a.N.runs[lo].x)) / cols;
         part = (int)((part + max((int64_t)0, min(own, (int64_t)ntile - 1)) * gridDim.y / ntile) % gridDim.y);
     }
     const int tb = (int)((int64_t)ntile * part / gridDim.y), te = (int)((int64_t)ntile * (part + 1) / gridDim.y);
@@ -942,7 +942,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
             for (unsigned left = pend; left; left &= left - 1) {
                 const int b = __ffs((int)left) - 1, slot = atomicAdd(&s_qn, 1);
                 if (slot >= kFusedQueue) break;
-                s_qj[slot] = s_j[warp * 32 + b];
+                s_qj[slot] = s_j[warp * chunk + b];
                 s_qr[slot] = (unsigned char)rr;
                 pend &= ~(1u << b);
             }
@@ -950,8 +950,8 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         if (tile >= te) break;
         bool q_here = false;
         {
-            const int p = tile * kFusedTile + threadIdx.x;
-            if (p < nc) {
+            const int p = tile * cols + threadIdx.x;
+            if ((int)threadIdx.x < cols && p < nc) {
                 int lo = run0, hi = run1 - 1;
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
@@ -987,7 +987,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         }
         const bool q_tile = __syncthreads_or(q_here);
         if (!kT) needq = q_tile;
-        const int c0 = warp * 32, c1 = min(c0 + 32, nc - tile * kFusedTile);
+        const int c0 = warp * chunk, c1 = min(c0 + chunk, nc - tile * cols);
         // the tile's own sum first: a long row's sum is then one of few terms
         float2 ta[NR], tq = make_float2(0.f, 0.f);
 #pragma unroll
@@ -1084,11 +1084,11 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
 
 #define BEM_FUSED_KERNEL(NAME, NR, T)                                                                                \
     __global__ void __launch_bounds__(kFusedThreads, 4)                                                             \
-        NAME(NearArgs a, const int4 *__restrict__ tasks, const float2 *__restrict__ x, float2 *__restrict__ out,    \
-             int *__restrict__ err, const int *skip)                                                                \
+        NAME(NearArgs a, const int4 *__restrict__ tasks, int rows, int cols, const float2 *__restrict__ x,          \
+             float2 *__restrict__ out, int *__restrict__ err, const int *skip)                                      \
     {                                                                                                                \
         if (skip_now(skip)) return;                                                                                  \
-        near_fused_body<NR, T>(a, tasks, x, out, err);                                                               \
+        near_fused_body<NR, T>(a, tasks, rows, cols, x, out, err);                                                               \
     }
 BEM_FUSED_KERNEL(k_near_fused_1, 1, false)
 BEM_FUSED_KERNEL(k_near_fused_2, 2, false)

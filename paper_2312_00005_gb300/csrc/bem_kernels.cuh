@@ -3,6 +3,7 @@
 
 #include "../../include/bemfmm.h"
 #include "bem_device.cuh"
+#include "bem_plan.hpp"
 
 namespace bem {
 
@@ -219,30 +220,23 @@ __global__ void k_near_spmv_items_multi(NearArgs a, const int4 *items, const flo
 // Near-field product with recomputed entries for 1, 2 or 4 right-hand sides
 // (planes n apart in x and out) and its transpose: blocks of tasks (leaf,
 // first row, end row; at most kFusedRows rows; tasks null: one leaf holds
-// every element) times gridDim.y parts of the columns, each part into its own
-// [NR][n] plane of out; k_near_fused_sum adds the parts.
+// every element, `rows` rows a block) times gridDim.y parts of the columns, in
+// tiles of `cols` (32 to kFusedTile), each part into its own [NR][n] plane of
+// out; k_near_fused_sum adds the parts.  fused_split (bem_plan.hpp) gives rows,
+// cols and parts.
 constexpr int kFusedThreads = 256;
-constexpr int kFusedTile = 256;          // columns staged per pass
-constexpr int kFusedRows = 32;           // rows per block (the lanes of a warp)
 constexpr int kFusedQueue = 1024;        // expensive pairs queued per block
 constexpr int kFieldQueue = 2048;        // near pairs of field points queued per block
 constexpr int kFusedParts = 2560;        // ... and their parts under one rule, per kFusedThreads pairs
-__global__ void k_near_fused_1(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
-__global__ void k_near_fused_2(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
-__global__ void k_near_fused_4(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
-__global__ void k_near_fused_t(NearArgs a, const int4 *tasks, const float2 *x, float2 *out, int *err, const int *skip);
+__global__ void k_near_fused_1(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
+                               int *err, const int *skip);
+__global__ void k_near_fused_2(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
+                               int *err, const int *skip);
+__global__ void k_near_fused_4(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
+                               int *err, const int *skip);
+__global__ void k_near_fused_t(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
+                               int *err, const int *skip);
 __global__ void k_near_fused_sum(const float2 *part, int S, int64_t n, float2 *y, const int *skip);
-// Parts of the columns for ntasks row tasks of at most max_ncol columns:
-// blocks enough for several rounds of four per SM, and whole tiles in each part
-// (5120 elements: 20 parts of one tile 283 us, 10 of two 352 us).
-inline int fused_parts(int64_t ntasks, int64_t max_ncol)
-{
-    const int64_t ntile = (max_ncol + kFusedTile - 1) / kFusedTile;
-    const int64_t want = ntasks > 0 ? 3648 / ntasks : 1;
-    if (want <= 1 || ntile <= 1) return 1;
-    const int64_t per = (ntile + want - 1) / want;
-    return (int)((ntile + per - 1) / per);
-}
 __global__ void k_prep(PrepArgs a, const int *skip);
 // True when the product kernels of a finished GMRES cycle should skip.
 __device__ __forceinline__ bool skip_now(const int *skip) { return skip != nullptr && *(volatile const int *)skip != 0; }

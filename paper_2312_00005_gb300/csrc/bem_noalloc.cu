@@ -61,7 +61,7 @@ size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 // Scratch layout for n elements (each piece 256-byte aligned).
 struct Layout {
     size_t chi, clo, nrm, va, e1, e2, cd, vad, e1d, e2d, ad, cp, cq, leaf_of, run_ptr, runs, ncol, Q, err, part, total;
-    int parts;
+    FusedSplit split;
     explicit Layout(int64_t n)
     {
         size_t o = 0;
@@ -74,9 +74,9 @@ struct Layout {
         Q = take(sizeof(QuadTables)); err = take(4);
         // partial sums of the product's column parts, as many as the scratch
         // array has room for (none: one part, written to y)
-        parts = fused_parts((n + kFusedRows - 1) / kFusedRows, n);
-        while (parts > 1 && o + align256(8 * (size_t)n * parts) > kScratchBytes) --parts;
-        part = parts > 1 ? take(8 * (size_t)n * parts) : o;
+        split = fused_split({n}, n);
+        while (split.parts > 1 && o + align256(8 * (size_t)n * split.parts) > kScratchBytes) --split.parts;
+        part = split.parts > 1 ? take(8 * (size_t)n * split.parts) : o;
         total = o;
     }
 };
@@ -255,11 +255,12 @@ extern "C" int bem_matvec_direct_noalloc(const double *nodes_dev, int64_t n_node
     a.cp = (const float2 *)(base + lay.cp);
     a.cq = (const float2 *)(base + lay.cq);
     float2 *part = (float2 *)(base + lay.part);
-    k_near_fused_1<<<dim3((unsigned)((n_tris + kFusedRows - 1) / kFusedRows), (unsigned)lay.parts), kFusedThreads, 0, s>>>(
-        a, nullptr, (const float2 *)x_dev, lay.parts > 1 ? part : (float2 *)y_dev, (int *)(base + lay.err), nullptr);
-    if (lay.parts > 1)
-        k_near_fused_sum<<<(unsigned)((n_tris + 255) / 256), 256, 0, s>>>(part, lay.parts, n_tris, (float2 *)y_dev,
-                                                                          nullptr);
+    const FusedSplit f = lay.split;
+    k_near_fused_1<<<dim3((unsigned)((n_tris + f.rows - 1) / f.rows), (unsigned)f.parts), kFusedThreads, 0, s>>>(
+        a, nullptr, f.rows, f.cols, (const float2 *)x_dev, f.parts > 1 ? part : (float2 *)y_dev, (int *)(base + lay.err),
+        nullptr);
+    if (f.parts > 1)
+        k_near_fused_sum<<<(unsigned)((n_tris + 255) / 256), 256, 0, s>>>(part, f.parts, n_tris, (float2 *)y_dev, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(BEM_E_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     int herr = INT_MAX;

@@ -323,6 +323,40 @@ double auto_leaf_edge(const Geometry &g, const bem_params &p)
     return std::max(r1 / 5.0, 2.0 * g.mean_edge);
 }
 
+// Blocks enough for several rounds of four per SM, and whole tiles in each part
+// (5120 elements: 20 parts of one tile 283 us, 10 of two 352 us).
+int fused_parts(int64_t ntasks, int64_t max_ncol)
+{
+    const int64_t ntile = (max_ncol + kFusedTile - 1) / kFusedTile;
+    const int64_t want = ntasks > 0 ? 3648 / ntasks : 1;
+    if (want <= 1 || ntile <= 1) return 1;
+    const int64_t per = (ntile + want - 1) / want;
+    return (int)((ntile + per - 1) / per);
+}
+
+// Full tiles and 32 rows a block where that gives four blocks per SM (608);
+// below that a product is the time of one block, most of it its expensive
+// pairs, so the tiles are halved down to 32 columns, then the rows down to 4,
+// until the blocks are that many.
+FusedSplit fused_split(const std::vector<int64_t> &rows, int64_t max_ncol)
+{
+    FusedSplit f;
+    auto tasks = [&]() {
+        int64_t n = 0;
+        for (int64_t c : rows) n += (c + f.rows - 1) / f.rows;
+        return n;
+    };
+    auto tiles = [&]() { return (max_ncol + f.cols - 1) / f.cols; };
+    int64_t nt = tasks();
+    while (f.cols > 32 && nt * tiles() < 608) f.cols /= 2;
+    while (f.rows > 4 && nt * tiles() < 608) {
+        f.rows /= 2;
+        nt = tasks();
+    }
+    f.parts = f.cols == kFusedTile ? fused_parts(nt, max_ncol) : (int)std::max<int64_t>(1, tiles());
+    return f;
+}
+
 void build_tree(const Geometry &g, double leaf_edge, Tree &t)
 {
     const int64_t n = g.n;

@@ -99,6 +99,19 @@ struct Tree {
 void build_tree(const Geometry &g, double leaf_edge, Tree &t);
 double auto_leaf_edge(const Geometry &g, const bem_params &p);
 
+// ---------------------------------------------------------------- recomputed product
+constexpr int kFusedRows = 32;       // rows per block at most (the lanes of a warp)
+constexpr int kFusedTile = 256;      // columns staged per pass at most
+// Blocks of the recomputed near-field product: leaves of rows[t] rows cut into
+// chunks of at most `rows`, times `parts` parts of at most max_ncol columns in
+// tiles of `cols`.
+struct FusedSplit {
+    int rows = kFusedRows, cols = kFusedTile, parts = 1;
+};
+FusedSplit fused_split(const std::vector<int64_t> &rows, int64_t max_ncol);
+// Parts of whole tiles of kFusedTile columns for ntasks row tasks.
+int fused_parts(int64_t ntasks, int64_t max_ncol);
+
 // ---------------------------------------------------------------- per-frequency plan
 struct FarLevel {
     int depth = 0;
