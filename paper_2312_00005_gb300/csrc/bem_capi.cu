@@ -1872,9 +1872,18 @@ const double *upload_points(bem_mesh_impl &M, const double *pts, int64_t n)
     return M.ptsbuf.p;
 }
 
-// Parts of the elements of a direct field sum: blocks enough for several
-// rounds on every SM (at most 64 parts, which one thread per point adds).
-int field_parts(int64_t M_pts, int64_t n) { return std::min(64, fused_parts((M_pts + 31) / 32, n)); }
+// Blocks of a direct field sum: the recomputed product's split of M_pts rows
+// and n columns (at most 64 parts of full tiles), cut finer only below about one
+// block per SM, since most calls have far pairs alone and adding the parts then
+// shows (200 points around 5120 elements: 280 blocks 71 us a call, 560 80, 1120
+// 82; 33 points: 65, 68 and 78; 3000 points at a surface of 320 elements, the
+// other way round: 324, 251).
+FusedSplit field_split(int64_t M_pts, int64_t n)
+{
+    FusedSplit f = fused_split({M_pts}, n, 128);
+    if (f.cols == kFusedTile) f.parts = std::min(64, f.parts);
+    return f;
+}
 
 // to waits for what from holds (the mesh's event is recorded anew each time)
 void join_streams(bem_mesh_impl &M, cudaStream_t from, cudaStream_t to)
@@ -3351,22 +3360,22 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
             return BEM_OK;
         }
         const double *dp = upload_points(M, pts, M_pts);
-        const int S = field_parts(M_pts, n);
+        const FusedSplit fs = field_split(M_pts, n);
+        const int S = fs.parts;
         if (S > 1) M.fieldpart.alloc((size_t)M_pts * S);
         {
             KTimer kt_("k_field", s);
-            k_field<<<dim3(nblocks(M_pts, 32), (unsigned)S), kFusedThreads, 0, s>>>(M.elem(), M.Q.p, dp, M_pts, (float)k,
-                                                                      (float)M.prm.tau, M.tmp.p, M.tmp2.p,
-                                                                      sdev, n_src,
-                                                                      M.fieldpart.p, (float2 *)out_dev,
-                                                                      fr(M).err.p);
+            k_field<<<dim3(nblocks(M_pts, fs.rows), (unsigned)S), kFusedThreads, 0, s>>>(
+                M.elem(), M.Q.p, dp, M_pts, fs.rows, fs.cols, (float)k, (float)M.prm.tau, M.tmp.p, M.tmp2.p, sdev, n_src,
+                M.fieldpart.p, (float2 *)out_dev, fr(M).err.p);
         }
         ck_launch("k_field");
         if (S > 1) {
             {
                 KTimer kt_("k_field", s);
-                k_field_finish<<<nblocks(M_pts, 128), 128, 0, s>>>(dp, M_pts, S, (float)k, sdev, n_src,
-                                                                  M.fieldpart.p, (float2 *)out_dev);
+                const int lanes = M_pts <= kFinishWarps ? 32 : 1;
+                k_field_finish<<<nblocks(lanes * M_pts, 128), 128, 0, s>>>(
+                    dp, M_pts, S, lanes, (float)k, sdev, n_src, M.fieldpart.p, (float2 *)out_dev);
             }
             ck_launch("k_field_finish");
         }
@@ -3410,12 +3419,13 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         const double k = wavenumber(freq_hz, c);
         const float inv_omega_rho = (float)(1.0 / (2.0 * 3.14159265358979323846 * freq_hz * rho));
         const double *dp = upload_points(M, pts, M_pts);
-        const int S = field_parts(M_pts, n);
+        const FusedSplit fs = field_split(M_pts, n);
+        const int S = fs.parts;
         if (S > 1) M.fieldpart.alloc((size_t)M_pts * S * 3);
         {
             KTimer kt_("k_field_velocity", s);
-            k_field_velocity<<<dim3(nblocks(M_pts, 32), (unsigned)S), kFusedThreads, 0, s>>>(
-                M.elem(), M.Q.p, dp, M_pts, (float)k, (float)M.prm.tau, inv_omega_rho, M.tmp.p, M.tmp2.p,
+            k_field_velocity<<<dim3(nblocks(M_pts, fs.rows), (unsigned)S), kFusedThreads, 0, s>>>(
+                M.elem(), M.Q.p, dp, M_pts, fs.rows, fs.cols, (float)k, (float)M.prm.tau, inv_omega_rho, M.tmp.p, M.tmp2.p,
                 sdev, n_src,
                 M.fieldpart.p, (float2 *)v_out_dev, fr(M).err.p);
         }
@@ -3423,8 +3433,9 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         if (S > 1) {
             {
                 KTimer kt_("k_field_velocity", s);
-                k_field_velocity_finish<<<nblocks(M_pts, 128), 128, 0, s>>>(
-                    dp, M_pts, S, (float)k, inv_omega_rho, sdev, n_src, M.fieldpart.p, (float2 *)v_out_dev);
+                const int lanes = M_pts <= kFinishWarps ? 32 : 1;
+                k_field_velocity_finish<<<nblocks(lanes * M_pts, 128), 128, 0, s>>>(
+                    dp, M_pts, S, lanes, (float)k, inv_omega_rho, sdev, n_src, M.fieldpart.p, (float2 *)v_out_dev);
             }
             ck_launch("k_field_velocity_finish");
         }

@@ -18,6 +18,16 @@ __device__ __forceinline__ float2 warp_sum(float2 v)
     return v;
 }
 
+// the sum over the lanes that differ by multiples of w (a power of two)
+__device__ __forceinline__ float2 lanes_sum(float2 v, int w)
+{
+    for (int o = w; o < 32; o <<= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
+
 // ------------------------------------------------------------------ near field
 // Expensive pairs (heavy_rt2) of the stored near field, listed by kind so
 // that the warps of k_near_store_heavy take pairs of one kind: 0 = self term,
@@ -631,66 +641,170 @@ __device__ __forceinline__ void bm_point_sel(float3 d, float3 nx, float3 ny, flo
 // in 20..23 and the children taken from the whole element down, two bits
 // each, in 0..19 (the first in bits 0, 1).
 constexpr int kPartDepth = 10;
+__device__ __forceinline__ SubTri child_triangle(const SubTri &s, unsigned i)
+{
+    const float mx01 = 0.5f * (s.x0 + s.x1), my01 = 0.5f * (s.y0 + s.y1);
+    const float mx12 = 0.5f * (s.x1 + s.x2), my12 = 0.5f * (s.y1 + s.y2);
+    const float mx20 = 0.5f * (s.x2 + s.x0), my20 = 0.5f * (s.y2 + s.y0);
+    switch (i) {
+        case 0: return SubTri{s.x0, s.y0, mx01, my01, mx20, my20, s.depth + 1};
+        case 1: return SubTri{mx01, my01, s.x1, s.y1, mx12, my12, s.depth + 1};
+        case 2: return SubTri{mx20, my20, mx12, my12, s.x2, s.y2, s.depth + 1};
+        default: return SubTri{mx01, my01, mx12, my12, mx20, my20, s.depth + 1};
+    }
+}
+// The triangle whose child i is s: exact, as the coordinates are multiples of
+// 2^-kPartDepth.
+__device__ __forceinline__ SubTri parent_triangle(const SubTri &s, unsigned i)
+{
+    switch (i) {
+        case 0:
+            return SubTri{s.x0, s.y0, 2.f * s.x1 - s.x0, 2.f * s.y1 - s.y0, 2.f * s.x2 - s.x0, 2.f * s.y2 - s.y0,
+                          s.depth - 1};
+        case 1:
+            return SubTri{2.f * s.x0 - s.x1, 2.f * s.y0 - s.y1, s.x1, s.y1, 2.f * s.x2 - s.x1, 2.f * s.y2 - s.y1,
+                          s.depth - 1};
+        case 2:
+            return SubTri{2.f * s.x0 - s.x2, 2.f * s.y0 - s.y2, 2.f * s.x1 - s.x2, 2.f * s.y1 - s.y2, s.x2, s.y2,
+                          s.depth - 1};
+        default:
+            return SubTri{s.x0 + s.x2 - s.x1, s.y0 + s.y2 - s.y1, s.x0 + s.x1 - s.x2, s.y0 + s.y1 - s.y2,
+                          s.x1 + s.x2 - s.x0, s.y1 + s.y2 - s.y0, s.depth - 1};
+    }
+}
 __device__ __forceinline__ SubTri part_triangle(unsigned code, int depth)
 {
-    SubTri s{0.f, 0.f, 1.f, 0.f, 0.f, 1.f, depth};
-    for (int d = 0; d < depth; ++d) {
-        const float mx01 = 0.5f * (s.x0 + s.x1), my01 = 0.5f * (s.y0 + s.y1);
-        const float mx12 = 0.5f * (s.x1 + s.x2), my12 = 0.5f * (s.y1 + s.y2);
-        const float mx20 = 0.5f * (s.x2 + s.x0), my20 = 0.5f * (s.y2 + s.y0);
-        switch ((code >> (2 * d)) & 3) {
-            case 0: s = SubTri{s.x0, s.y0, mx01, my01, mx20, my20, depth}; break;
-            case 1: s = SubTri{mx01, my01, s.x1, s.y1, mx12, my12, depth}; break;
-            case 2: s = SubTri{mx20, my20, mx12, my12, s.x2, s.y2, depth}; break;
-            default: s = SubTri{mx01, my01, mx12, my12, mx20, my20, depth}; break;
-        }
-    }
+    SubTri s{0.f, 0.f, 1.f, 0.f, 0.f, 1.f, 0};
+    for (int d = 0; d < depth; ++d) s = child_triangle(s, (code >> (2 * d)) & 3u);
     return s;
 }
-// The parts under one rule of element j seen from midpoint i (Sec. 3.1.3's
-// subdivision, the decisions of integrate_subdivided), without integrating:
-// their number, and their codes (with `row` set in the upper bits) when out
-// is given.  0 when the element is subdivided deeper than a code can say
-// (the caller then takes the general rule, which also reports the limit).
-__device__ __noinline__ int cut_pair(const NearArgs &a, int64_t i, int64_t j, unsigned *out, unsigned row)
+// The parts under one rule of element j seen from x (D0 = x_j - x, xd the FP64
+// point; Sec. 3.1.3's subdivision, the decisions of integrate_regular_acc),
+// without integrating: their number, and the first cap codes in out.  0 when the element is subdivided deeper than a
+// code can say (the caller then takes the general rule, which also reports the
+// limit).
+__device__ __forceinline__ int cut_element(const ElemDev &E, const QuadTables &Q, int64_t j, float3 D0, const double *xd,
+                                           unsigned *out, int cap)
 {
-    const QuadTables &Q = *a.Q;
-    const float4 ch = a.E.chi[j];
-    const float3 e1 = f3(a.E.e1[j]), e2 = f3(a.E.e2[j]);
-    const float3 D0 = add3(sub3f(f3(ch), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i])));
-    const float3 base = add3(D0, f3(a.E.va[j]));
-    const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
-    int m = whole_rule(a.E, j, D0, ch.w, xd, Q);
+    const float area = E.chi[j].w;
+    const float3 e1 = f3(E.e1[j]), e2 = f3(E.e2[j]);
+    const float3 base = add3(D0, f3(E.va[j]));
+    int m = whole_rule(E, j, D0, area, xd, Q);
     if (m > 0) {
-        if (out) *out = row | (unsigned)m << 24;
+        if (cap > 0) *out = (unsigned)m << 24;
         return 1;
     }
-    int n = 0, depth = 1;
-    unsigned path = 0;                     // the part at hand: child path[depth - 1] of its parent ...
+    // depth first through the children; up: the parent of the part at hand
+    SubTri up{0.f, 0.f, 1.f, 0.f, 0.f, 1.f, 0};
+    int n = 0;
+    unsigned path = 0;                     // child path[d] taken at depth d ...
     if (Q.max_depth < 1) return 0;
     for (;;) {
-        const SubTri s = part_triangle(path, depth);
+        const int depth = up.depth + 1;
+        const SubTri s = child_triangle(up, (path >> (2 * up.depth)) & 3u);
         const float cx = (s.x0 + s.x1 + s.x2) * (1.0f / 3.0f), cy = (s.y0 + s.y1 + s.y2) * (1.0f / 3.0f);
-        m = sub_rule(a.E, j, mad3(cy, e2, mad3(cx, e1, base)), ch.w * exp2f(-2.0f * (float)depth), s, xd, Q);
+        m = sub_rule(E, j, mad3(cy, e2, mad3(cx, e1, base)), area * exp2f(-2.0f * (float)depth), s, xd, Q);
         if (m == 0) {
             if (depth >= kPartDepth || depth >= Q.max_depth) return 0;
-            ++depth;                       // down to its first child
+            up = s;                        // down to its first child
             continue;
         }
-        if (out) out[n] = row | (unsigned)m << 24 | (unsigned)depth << 20 | path;
+        if (n < cap) out[n] = (unsigned)m << 24 | (unsigned)depth << 20 | path;
         ++n;
         // the next sibling, or the next one of the nearest ancestor that has one
-        while (depth > 0 && ((path >> (2 * (depth - 1))) & 3u) == 3u) {
-            path &= ~(3u << (2 * (depth - 1)));
-            --depth;
+        while (((path >> (2 * up.depth)) & 3u) == 3u) {
+            path &= ~(3u << (2 * up.depth));
+            if (up.depth == 0) return n;
+            up = parent_triangle(up, (path >> (2 * (up.depth - 1))) & 3u);
         }
-        if (depth == 0) return n;
-        path += 1u << (2 * (depth - 1));
+        path += 1u << (2 * up.depth);
     }
+}
+// The same of the pair of elements (i, j).
+__device__ __noinline__ int cut_pair(const NearArgs &a, int64_t i, int64_t j, unsigned *out, int cap)
+{
+    const double xd[3] = {a.E.cd[3 * i], a.E.cd[3 * i + 1], a.E.cd[3 * i + 2]};
+    const float3 D0 = add3(sub3f(f3(a.E.chi[j]), f3(a.E.chi[i])), sub3f(f3(a.E.clo[j]), f3(a.E.clo[i])));
+    return cut_element(a.E, *a.Q, j, D0, xd, out, cap);
 }
 
 // first point of order m in a table of orders 1 to 6: 0, 1, 5, 14, 30, 55
 __device__ __forceinline__ int rule_at(int m) { return (m - 1) * m * (2 * m - 1) / 6; }
+// (xi, eta, 2 w) of point v of the orders 1 to 6 in a row
+__device__ __forceinline__ float4 rule_point(const QuadTables &Q, int v)
+{
+    int m = 1;
+    while (rule_at(m + 1) <= v) ++m;
+    const int u = v - rule_at(m);
+    return make_float4(Q.tri_xi[m][u], Q.tri_eta[m][u], 2.0f * Q.tri_w[m][u], 0.f);
+}
+constexpr int kCutKept = 96;                             // codes of a pair that its thread keeps (else cut again)
+constexpr int kPartBytes = kFusedParts * 10;           // the parts of a block's queued pairs, in shared memory
+// A block's nq queued pairs, kFusedThreads at a time: cut into parts
+// (cut(pair, out, cap): their number, and the first cap codes), the parts sorted
+// by order, integrated part by part (part(pair, code)); pairs whose parts
+// found no room go into another round, pairs that cannot be cut are taken whole
+// (whole(pair)).  Called by the whole block; buf: kPartBytes of shared memory,
+// pn: 8 counters.
+template <class Cut, class Part, class Whole>
+__device__ __forceinline__ void work_queue(int nq, unsigned char *buf, int *pn, Cut cut, Part part, Whole whole)
+{
+    int *pq = reinterpret_cast<int *>(buf);                        // part: its pair
+    unsigned *pc = reinterpret_cast<unsigned *>(pq + kFusedParts); // ... its code
+    unsigned short *po = reinterpret_cast<unsigned short *>(pc + kFusedParts);   // parts by order
+    int q = threadIdx.x, np = -1;                      // this thread's next pair and its parts (-1: not counted)
+    unsigned codes[kCutKept];
+    while (__syncthreads_or(q < nq)) {
+        if (threadIdx.x < 8) pn[threadIdx.x] = 0;
+        __syncthreads();
+        if (q < nq) {
+            if (np < 0) np = cut(q, codes, kCutKept);
+            if (np > 0 && np <= kFusedParts) {
+                const int at = atomicAdd(&pn[0], np);
+                if (at + np <= kFusedParts) {
+                    if (np > kCutKept) cut(q, pc + at, np);
+                    for (int u = at; u < at + np; ++u) {
+                        if (np <= kCutKept) pc[u] = codes[u - at];
+                        pq[u] = q;
+                        atomicAdd(&pn[(pc[u] >> 24) & 7], 1);
+                    }
+                    q += kFusedThreads;
+                    np = -1;
+                } else {
+                    for (int u = at; u < min(at + np, kFusedParts); ++u) pc[u] = 0;   // order 0: no part
+                }
+            } else {
+                whole(q);
+                q += kFusedThreads;
+                np = -1;
+            }
+        }
+        __syncthreads();
+        const int n_all = min(pn[0], kFusedParts);
+        int start[8];                                  // first slot of an order: the longest first
+        start[7] = 0;
+        start[6] = 0;
+#pragma unroll
+        for (int m = 5; m >= 1; --m) start[m] = start[m + 1] + pn[m + 1];
+        const int n_parts = start[1] + pn[1];
+        __syncthreads();
+        if (threadIdx.x < 8) pn[threadIdx.x] = 0;
+        __syncthreads();
+        for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
+            const int m = (pc[u] >> 24) & 7;
+            if (m == 0) continue;
+            int at = start[1];
+#pragma unroll
+            for (int v = 2; v <= 6; ++v)
+                if (m == v) at = start[v];
+            po[at + atomicAdd(&pn[m], 1)] = (unsigned short)u;
+        }
+        __syncthreads();
+        for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) part(pq[po[u]], pc[po[u]]);
+    }
+    __syncthreads();
+}
+
 // The part's share of A_ij, to FP32 rounding; rule: (xi, eta, 2 w) of the
 // points of orders 1 to 6.
 __device__ __forceinline__ float2 part_entry(const NearArgs &a, int64_t i, int64_t j, unsigned code, const float4 *rule)
@@ -770,14 +884,11 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     // the staged tile (a transposed product stages rows: no vertices and
     // coefficients), and afterwards the parts of the queued pairs
     constexpr int kTileArrays = kT ? 3 : 7;
-    constexpr int kTileBytes = kTileArrays * kFusedTile * 16, kPartBytes = kFusedParts * 10;
+    constexpr int kTileBytes = kTileArrays * kFusedTile * 16;
     __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
     float4 *s_hi = reinterpret_cast<float4 *>(s_buf), *s_lo = s_hi + kFusedTile, *s_n = s_lo + kFusedTile;
     float4 *s_va = kT ? s_hi : s_n + kFusedTile, *s_e1 = kT ? s_hi : s_va + kFusedTile;
     float4 *s_e2 = kT ? s_hi : s_e1 + kFusedTile, *s_c = kT ? s_hi : s_e2 + kFusedTile;
-    int *s_pj = reinterpret_cast<int *>(s_buf);                        // part: staged element
-    unsigned *s_pc = reinterpret_cast<unsigned *>(s_pj + kFusedParts); // ... row, order, depth, path
-    unsigned short *s_po = reinterpret_cast<unsigned short *>(s_pc + kFusedParts);   // parts by order
     __shared__ float2 s_x[NR][kFold ? 1 : kFusedTile];
     __shared__ int s_j[kFusedTile];
     __shared__ int s_qj[kFusedQueue];                  // expensive pairs: staged element and row
@@ -810,12 +921,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     if (threadIdx.x < kFusedRows)
 #pragma unroll
         for (int r = 0; r < NR; ++r) s_h[r][threadIdx.x] = make_double2(0.0, 0.0);
-    if (threadIdx.x < 91) {
-        int m = 1;
-        while (rule_at(m + 1) <= (int)threadIdx.x) ++m;
-        const int v = threadIdx.x - rule_at(m);
-        s_rule[threadIdx.x] = make_float4(Q.tri_xi[m][v], Q.tri_eta[m][v], 2.0f * Q.tri_w[m][v], 0.f);
-    }
+    if (threadIdx.x < 91) s_rule[threadIdx.x] = rule_point(Q, threadIdx.x);
     // this lane's element
     const float4 ehi = a.E.chi[e], elo = a.E.clo[e], en = a.E.nrm[e];
     float3 eva = make_float3(0.f, 0.f, 0.f), ee1 = eva, ee2 = eva;
@@ -843,71 +949,22 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     float2 acc[NR], accq = make_float2(0.f, 0.f);      // kT: acc[0] the p sum, accq the q sum
 #pragma unroll
     for (int r = 0; r < NR; ++r) acc[r] = make_float2(0.f, 0.f);
-    // the queued pairs, kFusedThreads at a time: cut into parts, the parts
-    // sorted by order, the parts integrated; pairs whose parts found no room go
-    // into another round (called by the whole block after a barrier; takes the
+    // the queued pairs (called by the whole block after a barrier; takes the
     // staged tile's place)
     auto drain = [&]() {
-        const int nq = min(s_qn, kFusedQueue);
-        int q = threadIdx.x;                           // this thread's next pair
-        while (__syncthreads_or(q < nq)) {
-            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
-            __syncthreads();
-            if (q < nq) {
-                const int row = s_qr[q], wj = s_qj[q];
-                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
-                const int np = cut_pair(a, i, j, nullptr, 0);
-                if (np > 0 && np <= kFusedParts) {
-                    const int at = atomicAdd(&s_pn[0], np);
-                    if (at + np <= kFusedParts) {
-                        unsigned *pc = s_pc + at;
-                        cut_pair(a, i, j, pc, (unsigned)row << 27);
-                        for (int u = 0; u < np; ++u) {
-                            s_pj[at + u] = wj;
-                            atomicAdd(&s_pn[(pc[u] >> 24) & 7], 1);
-                        }
-                        q += kFusedThreads;
-                    } else {
-                        for (int u = at; u < min(at + np, kFusedParts); ++u) s_pc[u] = 0;   // order 0: no part
-                    }
-                } else {
-                    // cut deeper than a code can say
-                    float2 v;
-                    if (general_entry(a, i, j, &v)) add_entry<NR>(&s_h[0][row], x, a.E.n, wj, v);
-                    else atomicMin(err, (int)j);
-                    q += kFusedThreads;
-                }
-            }
-            __syncthreads();
-            const int n_all = min(s_pn[0], kFusedParts);
-            int start[8];                              // first slot of an order: the longest first
-            start[7] = 0;
-            start[6] = 0;
-#pragma unroll
-            for (int m = 5; m >= 1; --m) start[m] = start[m + 1] + s_pn[m + 1];
-            const int n_parts = start[1] + s_pn[1];
-            __syncthreads();
-            if (threadIdx.x < 8) s_pn[threadIdx.x] = 0;
-            __syncthreads();
-            for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
-                const int m = (s_pc[u] >> 24) & 7;
-                if (m == 0) continue;
-                int at = start[1];
-#pragma unroll
-                for (int v = 2; v <= 6; ++v)
-                    if (m == v) at = start[v];
-                s_po[at + atomicAdd(&s_pn[m], 1)] = (unsigned short)u;
-            }
-            __syncthreads();
-            for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) {
-                const int pi = s_po[u], wj = s_pj[pi];
-                const unsigned pc = s_pc[pi];
-                const int row = pc >> 27;
-                const int64_t i = kT ? wj : e0 + row, j = kT ? e0 + row : wj;
-                add_entry<NR>(&s_h[0][row], x, a.E.n, wj, part_entry(a, i, j, pc, s_rule));
-            }
-        }
-        __syncthreads();
+        auto row_of = [&](int q) { return kT ? (int64_t)s_qj[q] : e0 + s_qr[q]; };
+        auto col_of = [&](int q) { return kT ? e0 + s_qr[q] : (int64_t)s_qj[q]; };
+        work_queue(
+            min(s_qn, kFusedQueue), s_buf, s_pn,
+            [&](int q, unsigned *out, int cap) { return cut_pair(a, row_of(q), col_of(q), out, cap); },
+            [&](int q, unsigned code) {
+                add_entry<NR>(&s_h[0][s_qr[q]], x, a.E.n, s_qj[q], part_entry(a, row_of(q), col_of(q), code, s_rule));
+            },
+            [&](int q) {                               // cut deeper than a code can say
+                float2 v;
+                if (general_entry(a, row_of(q), col_of(q), &v)) add_entry<NR>(&s_h[0][s_qr[q]], x, a.E.n, s_qj[q], v);
+                else atomicMin(err, (int)col_of(q));
+            });
         if (threadIdx.x == 0) s_qn = 0;
     };
     const int nc = a.N.ncol[t];
@@ -1064,19 +1121,18 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         Ee = warp_sum(Ee);
         if (lane == 0) add_entry<NR>(&s_h[0][row], x, a.E.n, j, self_entry(G, Ee, k, ik_inv, a.tau, a.cp[j], a.cq[j]));
     }
-    // the lanes' sums of a row in (warp, side-by-side column) order
+    // the sums of a row: columns side by side in a warp, then the warps in order
     float2 *red = reinterpret_cast<float2 *>(s_buf);
     float2 *dst = out + (int64_t)part * NR * a.E.n;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         __syncthreads();
-        red[threadIdx.x] = acc[r];
+        red[threadIdx.x] = lanes_sum(acc[r], w);
         __syncthreads();
         if (threadIdx.x < cnt) {
             const double2 h = s_h[r][threadIdx.x];
             float2 v = make_float2((float)h.x, (float)h.y);
-            for (int q = 0; q < kW; ++q)
-                for (int u = 0; u < R; ++u) v = cadd(v, red[q * 32 + u * w + threadIdx.x]);
+            for (int q = 0; q < kW; ++q) v = cadd(v, red[q * 32 + threadIdx.x]);
             dst[r * a.E.n + e0 + threadIdx.x] = v;
         }
     }
@@ -2341,92 +2397,166 @@ __device__ __noinline__ bool field_entry(const ElemDev &E, const QuadTables &Q, 
     return ok;
 }
 
+// x_j - x of element j and a point x.
+__device__ __forceinline__ float3 point_to(const ElemDev &E, int64_t j, const double *xd)
+{
+    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
+    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
+                                   (float)(xd[2] - (double)xhi.z));
+    return add3(sub3f(f3(E.chi[j]), xhi), sub3f(f3(E.clo[j]), xlo));
+}
+__device__ __noinline__ int cut_point(const ElemDev &E, const QuadTables &Q, int64_t j, const double *xd, unsigned *out,
+                                      int cap)
+{
+    return cut_element(E, Q, j, point_to(E, j, xd), xd, out, cap);
+}
+// The contribution of a part of element j at x.
+template <bool kGrad>
+__device__ __forceinline__ void field_part(const ElemDev &E, int64_t j, const double *xd, unsigned code,
+                                           const float4 *rule, float k, float2 p, float2 q, float2 *v)
+{
+    const int m = (code >> 24) & 7, depth = (code >> 20) & 15;
+    const SubTri T = part_triangle(code, depth);
+    const float3 g1 = f3(E.e1[j]), g2 = f3(E.e2[j]), ny = f3(E.nrm[j]);
+    const float3 base = add3(point_to(E, j, xd), f3(E.va[j]));
+    const float sa = E.chi[j].w * exp2f(-2.0f * (float)depth);
+    const float sx1 = T.x1 - T.x0, sy1 = T.y1 - T.y0, sx2 = T.x2 - T.x0, sy2 = T.y2 - T.y0;
+    FieldPair<kGrad> f(k);
+    const int r1 = rule_at(m + 1);
+    for (int u = rule_at(m); u < r1; ++u) {
+        const float4 rl = rule[u];
+        const float px = T.x0 + rl.x * sx1 + rl.y * sx2, py = T.y0 + rl.x * sy1 + rl.y * sy2;
+        f.acc.point(mad3(py, g2, mad3(px, g1, base)), ny, sa * rl.z);
+    }
+#pragma unroll
+    for (int a = 0; a < FieldPair<kGrad>::kN; ++a) v[a] = make_float2(0.f, 0.f);
+    f.add(v, p, q);
+}
+
 // Direct sum over every element at M points: p (k_field) or v (k_field_
 // velocity).  Bound by FP32 / SFU issue.  As in the recomputed product, a lane
-// holds a point, the elements are staged in shared memory and read as
-// broadcasts, and the far pairs (one quadrature point, nearly all) are
-// evaluated in place; the others are queued per block and worked off by all
-// its threads when the queue has filled and at the end, their sums FP64
-// additions.  Block (x, y) takes 32 points and every gridDim.y-th part of the
-// elements; with several parts they go to part[(m S + s) N + a] and the finish
-// kernels add them in order.  Lanes over the elements, one point per block
-// (112 bytes of element data through L1 per pair): 1000 points and 5120
-// elements 64 + 72 us (field + velocity); this 40 + 60; 8000 points and 8000
-// elements 640 -> 280 us.
+// holds a point, the elements are staged in shared memory in tiles of `cols`
+// and read as broadcasts, and the pairs under one rule of order 1 to 3 are
+// evaluated in place; the others (subdivided elements, orders 4 to 6, distances
+// within rounding of a threshold) are queued per block and worked off as there
+// (work_queue), their sums FP64 additions.  Block (x, y) takes `rows` points and every gridDim.y-th part of
+// the elements; with several parts they go to part[(m S + s) N + a] and the
+// finish kernels add them in order.  rows, cols and the parts are
+// fused_split's: few points or few elements get small blocks.
+// Calls (host part of about 60 us included) on 5120 elements: 3000 points 0.2 m
+// off the surface 139 us, a millimetre off it 345; with one point per block and
+// lanes over the elements (112 bytes of element data through L1 per pair) 232
+// and 915.  200 points at a surface of 320 elements 130 and 186 us; with orders
+// 2 and 3 queued as well, and pairs worked off whole, one per thread, 1758.
 template <bool kGrad>
 __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q, const double *__restrict__ pts,
-                                           int64_t M, float k, float tau, float inv_omega_rho,
-                                           const float2 *__restrict__ p, const float2 *__restrict__ q,
+                                           int64_t M, int rows, int cols, float k, float tau, float inv_omega_rho,
+                                           const float2 *__restrict__ p, const float2 *__restrict__ qs,
                                            const SourceDev *__restrict__ src, int nsrc, float2 *__restrict__ part,
                                            float2 *__restrict__ out, int *err)
 {
     constexpr int kW = kFusedThreads / 32, kN = FieldPair<kGrad>::kN;
-    __shared__ float4 s_hi[kFusedTile], s_lo[kFusedTile], s_n[kFusedTile], s_pq[kFusedTile];
+    // the staged tile, and afterwards the parts of the queued pairs
+    constexpr int kTileBytes = 7 * kFusedTile * 16;
+    __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
+    float4 *s_hi = reinterpret_cast<float4 *>(s_buf), *s_lo = s_hi + kFusedTile, *s_n = s_lo + kFusedTile;
+    float4 *s_pq = s_n + kFusedTile, *s_va = s_pq + kFusedTile, *s_e1 = s_va + kFusedTile, *s_e2 = s_e1 + kFusedTile;
+    __shared__ float4 s_rule[91];                      // (xi, eta, 2 w) of orders 1 to 6
+    __shared__ int s_pn[8];
     __shared__ int s_qj[kFieldQueue];
     __shared__ unsigned char s_qr[kFieldQueue];
     __shared__ int s_qn;
     __shared__ double2 s_h[kN][32];
     __shared__ double s_x[32][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t m0 = (int64_t)blockIdx.x * 32;
-    const int cnt = (int)min((int64_t)32, M - m0);
+    const int64_t m0 = (int64_t)blockIdx.x * rows;
+    const int cnt = (int)min((int64_t)rows, M - m0);
     int w = 1;
     while (w < cnt) w <<= 1;
-    const int R = 32 / w, sub = lane / w, rr = lane % w;   // R elements side by side for fewer than 32 points
+    const int R = 32 / w, sub = lane / w, rr = lane % w;   // R elements side by side for w < 32 points
     const bool live = rr < cnt;
     if (threadIdx.x < 32) {
 #pragma unroll
         for (int a = 0; a < kN; ++a) s_h[a][threadIdx.x] = make_double2(0.0, 0.0);
         for (int a = 0; a < 3; ++a) s_x[threadIdx.x][a] = (int)threadIdx.x < cnt ? pts[3 * (m0 + threadIdx.x) + a] : 0.0;
     }
+    if (threadIdx.x < 91) s_rule[threadIdx.x] = rule_point(Q, threadIdx.x);
     if (threadIdx.x == 0) s_qn = 0;
     __syncthreads();
     const double *xd = s_x[live ? rr : 0];
     const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
     const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
                                    (float)(xd[2] - (double)xhi.z));
-    const float rt1 = fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2);   // R2[1] = 0 with m_max = 1
-    auto general = [&](int row, int j) {
-        float2 v[kN];
-        if (!field_entry<kGrad>(E, Q, j, s_x[row], k, p[j], q[j], v)) {
-            atomicMin(err, j);
-            return;
-        }
-#pragma unroll
-        for (int a = 0; a < kN; ++a) {
-            atomicAdd(&s_h[a][row].x, (double)v[a].x);
-            atomicAdd(&s_h[a][row].y, (double)v[a].y);
-        }
-    };
-    // (called by the whole block after a barrier)
+    // thresholds on r~^2 as in the recomputed product
+    const float rt1 = fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2);
+    const float rt1lo = Q.R2[1] * (1.0f - 2e-5f), rt2hi = Q.R2[2] * (1.0f + 2e-5f), rt2lo = Q.R2[2] * (1.0f - 2e-5f);
+    const float rth = Q.m_max > 3 ? Q.heavy_rt2 : Q.whole_rt2;
+    // the queued pairs (called by the whole block after a barrier; takes the
+    // staged tile's place)
     auto drain = [&]() {
-        const int n = min(s_qn, kFieldQueue);
-        for (int u = threadIdx.x; u < n; u += kFusedThreads) general(s_qr[u], s_qj[u]);
-        __syncthreads();
+        auto add = [&](int row, const float2 *v) {
+#pragma unroll
+            for (int a = 0; a < kN; ++a) {
+                atomicAdd(&s_h[a][row].x, (double)v[a].x);
+                atomicAdd(&s_h[a][row].y, (double)v[a].y);
+            }
+        };
+        work_queue(
+            min(s_qn, kFieldQueue), s_buf, s_pn,
+            [&](int q, unsigned *out, int cap) { return cut_point(E, Q, s_qj[q], s_x[s_qr[q]], out, cap); },
+            [&](int q, unsigned code) {
+                float2 v[kN];
+                field_part<kGrad>(E, s_qj[q], s_x[s_qr[q]], code, s_rule, k, p[s_qj[q]], qs[s_qj[q]], v);
+                add(s_qr[q], v);
+            },
+            [&](int q) {                               // cut deeper than a code can say
+                float2 v[kN];
+                if (field_entry<kGrad>(E, Q, s_qj[q], s_x[s_qr[q]], k, p[s_qj[q]], qs[s_qj[q]], v)) add(s_qr[q], v);
+                else atomicMin(err, s_qj[q]);
+            });
         if (threadIdx.x == 0) s_qn = 0;
     };
     float2 acc[kN];
 #pragma unroll
     for (int a = 0; a < kN; ++a) acc[a] = make_float2(0.f, 0.f);
-    const int S = gridDim.y, sl = blockIdx.y;
-    const int64_t ntile = (E.n + kFusedTile - 1) / kFusedTile;
+    const int S = gridDim.y, sl = blockIdx.y, chunk = cols / kW;
+    const int64_t ntile = (E.n + cols - 1) / cols;
     const int64_t tb = ntile * sl / S, te = ntile * (sl + 1) / S;
-    for (int64_t tile = tb; tile < te; ++tile) {
-        __syncthreads();
-        if (s_qn > kFieldQueue / 2) drain();               // the same in every thread: no pushes since the barrier
-        const int64_t j = tile * kFusedTile + threadIdx.x;
-        if (j < E.n) {
+    unsigned pend = 0;                                 // elements of this lane that found the queue full
+    for (int64_t tile = tb;; ++tile) {
+        // as in the recomputed product (s_qn is the same in every thread: no
+        // pushes since the barrier)
+        for (;;) {
+            const bool full = __syncthreads_or(pend != 0);
+            if (!full && tile < te && s_qn <= kFieldQueue / 2) break;
+            drain();
+            __syncthreads();
+            if (!full) break;
+            for (unsigned left = pend; left; left &= left - 1) {
+                const int b = __ffs((int)left) - 1, slot = atomicAdd(&s_qn, 1);
+                if (slot >= kFieldQueue) break;
+                s_qj[slot] = (int)((tile - 1) * cols) + warp * chunk + b;
+                s_qr[slot] = (unsigned char)rr;
+                pend &= ~(1u << b);
+            }
+        }
+        if (tile >= te) break;
+        const int64_t j = tile * cols + threadIdx.x;
+        if ((int)threadIdx.x < cols && j < E.n) {
             const float4 h = E.chi[j];
             float4 l = E.clo[j];
             l.w = __frcp_rn(h.w);
-            const float2 pj = p[j], qj = q[j];
+            const float2 pj = p[j], qj = qs[j];
             s_hi[threadIdx.x] = h;
             s_lo[threadIdx.x] = l;
             s_n[threadIdx.x] = E.nrm[j];
+            s_va[threadIdx.x] = E.va[j];
+            s_e1[threadIdx.x] = E.e1[j];
+            s_e2[threadIdx.x] = E.e2[j];
             s_pq[threadIdx.x] = make_float4(pj.x, pj.y, qj.x, qj.y);
         }
         __syncthreads();
-        const int c0 = warp * 32, c1 = (int)min((int64_t)c0 + 32, E.n - tile * kFusedTile);
+        const int c0 = warp * chunk, c1 = (int)min((int64_t)c0 + chunk, E.n - tile * cols);
         float2 ta[kN];                                      // the tile's own sum first
 #pragma unroll
         for (int a = 0; a < kN; ++a) ta[a] = make_float2(0.f, 0.f);
@@ -2436,40 +2566,49 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
             const float4 eh = s_hi[c], el = s_lo[c];
             float3 D0;
             const float rt2 = pair_rt2(f3(eh), f3(el), xhi, xlo, el.w, D0);
-            if (rt2 > rt1) {
-                const float4 pq = s_pq[c];
-                FieldPair<kGrad> f(k);
-                f.acc.point(D0, f3(s_n[c]), eh.w);
-                f.add(ta, make_float2(pq.x, pq.y), make_float2(pq.z, pq.w));
-            } else {
-                const int je = (int)(tile * kFusedTile) + c;
+            int code = 0;
+            if (rt2 > rt1) code = 1;
+            else if (rt2 > rth && rt2 < rt1lo && (rt2 > rt2hi || rt2 < rt2lo)) code = rt2 > rt2hi ? 2 : 3;
+            if (code == 0) {
                 const int slot = atomicAdd(&s_qn, 1);
                 if (slot < kFieldQueue) {
-                    s_qj[slot] = je;
+                    s_qj[slot] = (int)(tile * cols) + c;
                     s_qr[slot] = (unsigned char)rr;
                 } else {
-                    general(rr, je);
+                    pend |= 1u << (c - c0);
+                }
+                continue;
+            }
+            const float4 pq = s_pq[c];
+            const float3 ny = f3(s_n[c]);
+            FieldPair<kGrad> f(k);
+            if (code == 1) {
+                f.acc.point(D0, ny, eh.w);
+            } else {
+                const float3 g1 = f3(s_e1[c]), g2 = f3(s_e2[c]), base = add3(D0, f3(s_va[c]));
+                const int u1 = code == 2 ? 5 : 14;
+                for (int u = code == 2 ? 1 : 5; u < u1; ++u) {
+                    const float4 rl = s_rule[u];
+                    f.acc.point(mad3(rl.y, g2, mad3(rl.x, g1, base)), ny, eh.w * rl.z);
                 }
             }
+            f.add(ta, make_float2(pq.x, pq.y), make_float2(pq.z, pq.w));
         }
 #pragma unroll
         for (int a = 0; a < kN; ++a) acc[a] = cadd(acc[a], ta[a]);
     }
-    __syncthreads();
-    drain();
-    // the lanes' sums of a point in (warp, side-by-side element) order
+    // the sums of a point: elements side by side in a warp, then the warps in order
     float2 *red = reinterpret_cast<float2 *>(s_hi);
     float2 tot[kN];
 #pragma unroll
     for (int a = 0; a < kN; ++a) {
         __syncthreads();
-        red[threadIdx.x] = acc[a];
+        red[threadIdx.x] = lanes_sum(acc[a], w);
         __syncthreads();
         if ((int)threadIdx.x < cnt) {
             const double2 h = s_h[a][threadIdx.x];
             float2 v = make_float2((float)h.x, (float)h.y);
-            for (int u = 0; u < kW; ++u)
-                for (int t = 0; t < R; ++t) v = cadd(v, red[u * 32 + t * w + threadIdx.x]);
+            for (int u = 0; u < kW; ++u) v = cadd(v, red[u * 32 + threadIdx.x]);
             tot[a] = cscale(v, tau);                        // tau on the integral part (Eq. BIE_I)
         }
     }
@@ -2497,12 +2636,12 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
 }
 
 __global__ void __launch_bounds__(kFusedThreads, 3) k_field(ElemDev E, const QuadTables *__restrict__ Q,
-                                                         const double *__restrict__ pts, int64_t M, float k, float tau,
-                                                         const float2 *__restrict__ p, const float2 *__restrict__ q,
+                                                         const double *__restrict__ pts, int64_t M, int rows, int cols,
+                                                         float k, float tau, const float2 *__restrict__ p, const float2 *__restrict__ q,
                                                          const SourceDev *__restrict__ src, int nsrc,
                                                          float2 *__restrict__ part, float2 *__restrict__ out, int *err)
 {
-    field_body<false>(E, *Q, pts, M, k, tau, 0.f, p, q, src, nsrc, part, out, err);
+    field_body<false>(E, *Q, pts, M, rows, cols, k, tau, 0.f, p, q, src, nsrc, part, out, err);
 }
 
 // Particle velocity at field points, v = grad p / (i w rho) (Eq. utopandv),
@@ -2510,27 +2649,36 @@ __global__ void __launch_bounds__(kFusedThreads, 3) k_field(ElemDev E, const Qua
 // (Eq. BIE_I, lambda = 1, differentiated under the integral; the element
 // rules of the field).  out: [M][3] (x, y, z components).
 __global__ void __launch_bounds__(kFusedThreads, 3) k_field_velocity(ElemDev E, const QuadTables *__restrict__ Q,
-                                                                  const double *__restrict__ pts, int64_t M, float k,
-                                                                  float tau, float inv_omega_rho,
+                                                                  const double *__restrict__ pts, int64_t M, int rows,
+                                                                  int cols, float k, float tau, float inv_omega_rho,
                                                                   const float2 *__restrict__ p,
                                                                   const float2 *__restrict__ q,
                                                                   const SourceDev *__restrict__ src, int nsrc,
                                                                   float2 *__restrict__ part, float2 *__restrict__ out,
                                                                   int *err)
 {
-    field_body<true>(E, *Q, pts, M, k, tau, inv_omega_rho, p, q, src, nsrc, part, out, err);
+    field_body<true>(E, *Q, pts, M, rows, cols, k, tau, inv_omega_rho, p, q, src, nsrc, part, out, err);
 }
 
-// The S partial sums of each field point in slice order, plus the incident
-// field; one thread per point.
-__global__ void k_field_finish(const double *__restrict__ pts, int64_t M, int S, float k,
+// The S partial sums of a point, `stride` apart, by one thread, or by a warp
+// (every lane takes part; the lanes are added in a fixed tree).
+__device__ __forceinline__ float2 finish_sum(const float2 *__restrict__ part, int stride, int S, int lanes)
+{
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int s = threadIdx.x % lanes; s < S; s += lanes) v = cadd(v, part[s * stride]);
+    return lanes > 1 ? warp_sum(v) : v;
+}
+
+// The S partial sums of each field point, plus the incident field.
+__global__ void k_field_finish(const double *__restrict__ pts, int64_t M, int S, int lanes, float k,
                                const SourceDev *__restrict__ src, int nsrc, const float2 *__restrict__ part,
                                float2 *__restrict__ out)
 {
-    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t m = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lanes;
     if (m >= M) return;
-    float2 v = part[m * S];
-    for (int s = 1; s < S; ++s) v = cadd(v, part[m * S + s]);
+    const float2 v = finish_sum(part + m * S, 1, S, lanes);
+    if (threadIdx.x % lanes > 0) return;
     const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
     double br = v.x, bi = v.y;
     field_incident(xd, k, src, nsrc, br, bi);
@@ -2612,21 +2760,21 @@ __global__ void k_field_eval_finish(const double *__restrict__ pts, int64_t M, f
     out[perm[m]] = make_float2((float)br, (float)bi);
 }
 
-// The S partial gradients of each field point in slice order, the incident
-// gradient and the scaling to the velocity; one thread per point.
-__global__ void k_field_velocity_finish(const double *__restrict__ pts, int64_t M, int S, float k,
+// The S partial gradients of each field point, the incident gradient and the
+// scaling to the velocity.
+__global__ void k_field_velocity_finish(const double *__restrict__ pts, int64_t M, int S, int lanes, float k,
                                         float inv_omega_rho, const SourceDev *__restrict__ src, int nsrc,
                                         const float2 *__restrict__ part, float2 *__restrict__ out)
 {
-    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t m = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lanes;
     if (m >= M) return;
     double gr[3], gi[3];
     for (int a = 0; a < 3; ++a) {
-        float2 v = part[(m * S) * 3 + a];
-        for (int s = 1; s < S; ++s) v = cadd(v, part[(m * S + s) * 3 + a]);
+        const float2 v = finish_sum(part + m * S * 3 + a, 3, S, lanes);
         gr[a] = v.x;
         gi[a] = v.y;
     }
+    if (threadIdx.x % lanes > 0) return;
     const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
     incident_grad(xd, k, src, nsrc, gr, gi);
     for (int a = 0; a < 3; ++a)

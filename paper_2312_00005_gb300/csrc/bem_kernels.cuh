@@ -375,15 +375,18 @@ struct DTableArgs {
 __global__ void k_dtable(DTableArgs a);
 __global__ void k_rhs(const double *cd, const float4 *nrm, int64_t n, double k, const SourceDev *src, int nsrc,
                       float2 *b);
-__global__ void k_field(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, float tau,
-                        const float2 *p, const float2 *q, const SourceDev *src, int nsrc, float2 *part, float2 *out,
+__global__ void k_field(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, int rows, int cols, float k,
+                        float tau, const float2 *p, const float2 *q, const SourceDev *src, int nsrc, float2 *part, float2 *out,
                         int *err);
-__global__ void k_field_finish(const double *pts, int64_t M, int S, float k, const SourceDev *src, int nsrc,
+// The finish kernels take one thread per point, or a warp (lanes 32) up to
+// kFinishWarps points, where one thread's sum of the parts is the longer chain.
+constexpr int kFinishWarps = 512;
+__global__ void k_field_finish(const double *pts, int64_t M, int S, int lanes, float k, const SourceDev *src, int nsrc,
                                const float2 *part, float2 *out);
-__global__ void k_field_velocity(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, float k, float tau,
-                                 float inv_omega_rho, const float2 *p, const float2 *q, const SourceDev *src, int nsrc,
+__global__ void k_field_velocity(ElemDev E, const QuadTables *Q, const double *pts, int64_t M, int rows, int cols,
+                                 float k, float tau, float inv_omega_rho, const float2 *p, const float2 *q, const SourceDev *src, int nsrc,
                                  float2 *part, float2 *out, int *err);
-__global__ void k_field_velocity_finish(const double *pts, int64_t M, int S, float k, float inv_omega_rho,
+__global__ void k_field_velocity_finish(const double *pts, int64_t M, int S, int lanes, float k, float inv_omega_rho,
                                         const SourceDev *src, int nsrc, const float2 *part, float2 *out);
 __global__ void k_gather(const float2 *x, const int64_t *perm, int64_t n, float2 *y);
 __global__ void k_gather2(const float2 *x0, const float2 *x1, const int64_t *perm, int64_t n, float2 *y0, float2 *y1);

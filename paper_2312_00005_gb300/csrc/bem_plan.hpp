@@ -104,11 +104,11 @@ constexpr int kFusedRows = 32;       // rows per block at most (the lanes of a w
 constexpr int kFusedTile = 256;      // columns staged per pass at most
 // Blocks of the recomputed near-field product: leaves of rows[t] rows cut into
 // chunks of at most `rows`, times `parts` parts of at most max_ncol columns in
-// tiles of `cols`.
+// tiles of `cols`, so that there are at least `blocks` where the sizes allow.
 struct FusedSplit {
     int rows = kFusedRows, cols = kFusedTile, parts = 1;
 };
-FusedSplit fused_split(const std::vector<int64_t> &rows, int64_t max_ncol);
+FusedSplit fused_split(const std::vector<int64_t> &rows, int64_t max_ncol, int64_t blocks = 608);
 // Parts of whole tiles of kFusedTile columns for ntasks row tasks.
 int fused_parts(int64_t ntasks, int64_t max_ncol);
 

@@ -1,0 +1,78 @@
+"""Direct field and velocity where most or many pairs are not one-point pairs:
+points within a fraction of an element of the surface, and coarse surfaces
+seen from a few elements away, for point and element counts around the blocks'
+edges (4 to 32 points, 32 to 256 elements), against the oracle; the same call
+gives the same bits; and the time of points at the surface grows with their
+number (a block's queue must not become a serial chain).
+
+Bounds: 2e-5 of the largest value for every point (FP32 entries and sums), as
+for the direct field elsewhere."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2312_00005_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+C, RHO, F = 343.0, 1.21, 1200.0
+
+
+@pytest.fixture(scope="module")
+def bem():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_00005_gb300 import bemfmm
+    bemfmm.lib()
+    return bemfmm
+
+
+def _state(bem, nu, m, radius, **kw):
+    nodes, tris = inputs.geodesic_sphere(nu)
+    n = tris.shape[0]
+    p, q = (torch.tensor(v, dtype=torch.complex64, device="cuda")
+            for v in (inputs.random_complex(n, 1), inputs.random_complex(n, 2) * 20))
+    pts = inputs.fibonacci_sphere(m, radius) if m > 1 else np.array([[0.0, 0.0, radius]])
+    return 0.1 * nodes, tris, p, q, pts, bem.Mesh(0.1 * nodes, tris, field_mode=1, **kw)
+
+
+@pytest.mark.parametrize("nu,m,radius,kw", [
+    (1, 1, 0.101, {}), (2, 5, 0.101, {}), (2, 32, 0.13, {}), (4, 33, 0.3, {}), (4, 200, 0.1005, {}), (9, 4, 0.101, {}),
+    (9, 65, 0.101, {}), (4, 100, 0.101, {"quad_tol": 1e-6}), (4, 100, 0.102, {"m_max": 2}), (16, 700, 0.1002, {}),
+])
+def test_points_at_the_surface_match_oracle(bem, nu, m, radius, kw):
+    nodes, tris, p, q, pts, mesh = _state(bem, nu, m, radius, **kw)
+    f = mesh.evaluate(F, p, q, pts, c=C, rho=RHO)
+    v = mesh.evaluate_velocity(F, p, q, pts, c=C, rho=RHO)
+    for _ in range(4):
+        assert torch.equal(mesh.evaluate(F, p, q, pts, c=C, rho=RHO), f)
+        assert torch.equal(mesh.evaluate_velocity(F, p, q, pts, c=C, rho=RHO), v)
+    mesh.close()
+    ph, qh = (t.cpu().numpy().astype(np.complex128) for t in (p, q))
+    fo = oracle.field(nodes, tris, F, ph, qh, pts, c=C, params=kw)
+    vo = oracle.field_velocity(nodes, tris, F, ph, qh, pts, c=C, rho=RHO, params=kw)
+    assert np.abs(f.cpu().numpy() - fo).max() < 2e-5 * np.abs(fo).max()
+    assert np.abs(v.cpu().numpy() - vo).max() < 2e-5 * np.abs(vo).max()
+
+
+def test_few_points_at_the_surface_are_not_a_serial_chain(bem):
+    """200 points on a 320-element surface take well under the time of 3000
+    (they took as long when a block of 32 points worked off all its pairs)."""
+    t = {}
+    for m in (200, 3000):
+        _, _, p, q, pts, mesh = _state(bem, 4, m, 0.101)
+        for _ in range(3):
+            mesh.evaluate(F, p, q, pts)
+        ev = []
+        for _ in range(10):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            mesh.evaluate(F, p, q, pts)
+            b.record()
+            b.synchronize()
+            ev.append(a.elapsed_time(b))
+        t[m] = float(np.median(ev))
+        mesh.close()
+    print("ms by points", t)
+    assert t[200] < 0.7 * t[3000], t
