@@ -18,6 +18,34 @@ __device__ __forceinline__ float2 warp_sum(float2 v)
     return v;
 }
 
+// A sum of complex FP32 terms with its rounding errors beside it (two-sum), good
+// to about 2^-45: the sums of a row's partial sums, whose FP64 additions cost 9 us
+// of the 276 of a recomputed product on 5120 elements (a plain FP32 sum of 20
+// parts loses a tenth of the product's accuracy instead).
+struct Sum2 {
+    float2 s, e;
+    __device__ __forceinline__ Sum2() : s(make_float2(0.f, 0.f)), e(make_float2(0.f, 0.f)) {}
+    __device__ __forceinline__ explicit Sum2(double2 v) : s(make_float2((float)v.x, (float)v.y))
+    {
+        e = make_float2((float)(v.x - (double)s.x), (float)(v.y - (double)s.y));
+    }
+    static __device__ __forceinline__ void add1(float &s, float &e, float a)
+    {
+        const float t = __fadd_rn(s, a), b = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b)));
+        s = t;
+    }
+    __device__ __forceinline__ void add(float2 a)
+    {
+        add1(s.x, e.x, a.x);
+        add1(s.y, e.y, a.y);
+    }
+    __device__ __forceinline__ float2 value() const { return make_float2(s.x + e.x, s.y + e.y); }
+    __device__ __forceinline__ double2 value_d() const
+    {
+        return make_double2((double)s.x + (double)e.x, (double)s.y + (double)e.y);
+    }
+};
 // the sum over the lanes that differ by multiples of w (a power of two)
 __device__ __forceinline__ float2 lanes_sum(float2 v, int w)
 {
@@ -1130,10 +1158,9 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         red[threadIdx.x] = lanes_sum(acc[r], w);
         __syncthreads();
         if (threadIdx.x < cnt) {
-            const double2 h = s_h[r][threadIdx.x];
-            float2 v = make_float2((float)h.x, (float)h.y);
-            for (int q = 0; q < kW; ++q) v = cadd(v, red[q * 32 + threadIdx.x]);
-            dst[r * a.E.n + e0 + threadIdx.x] = v;
+            Sum2 v(s_h[r][threadIdx.x]);
+            for (int q = 0; q < kW; ++q) v.add(red[q * 32 + threadIdx.x]);
+            dst[r * a.E.n + e0 + threadIdx.x] = v.value();
         }
     }
 }
@@ -1160,9 +1187,10 @@ __global__ void k_near_fused_sum(const float2 *__restrict__ part, int S, int64_t
     if (skip_now(skip)) return;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    float2 v = part[i];
-    for (int s = 1; s < S; ++s) v = cadd(v, part[(int64_t)s * n + i]);
-    y[i] = v;
+    Sum2 v;
+#pragma unroll 4
+    for (int s = 0; s < S; ++s) v.add(part[(int64_t)s * n + i]);
+    y[i] = v.value();
 }
 
 // Row scaling of Eq. SystemI (Sec. 3.2, the solver's row-scaling
@@ -2606,10 +2634,9 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
         red[threadIdx.x] = lanes_sum(acc[a], w);
         __syncthreads();
         if ((int)threadIdx.x < cnt) {
-            const double2 h = s_h[a][threadIdx.x];
-            float2 v = make_float2((float)h.x, (float)h.y);
-            for (int u = 0; u < kW; ++u) v = cadd(v, red[u * 32 + threadIdx.x]);
-            tot[a] = cscale(v, tau);                        // tau on the integral part (Eq. BIE_I)
+            Sum2 v(s_h[a][threadIdx.x]);
+            for (int u = 0; u < kW; ++u) v.add(red[u * 32 + threadIdx.x]);
+            tot[a] = cscale(v.value(), tau);                // tau on the integral part (Eq. BIE_I)
         }
     }
     if ((int)threadIdx.x >= cnt) return;
@@ -2662,12 +2689,19 @@ __global__ void __launch_bounds__(kFusedThreads, 3) k_field_velocity(ElemDev E, 
 
 // The S partial sums of a point, `stride` apart, by one thread, or by a warp
 // (every lane takes part; the lanes are added in a fixed tree).
-__device__ __forceinline__ float2 finish_sum(const float2 *__restrict__ part, int stride, int S, int lanes)
+__device__ __forceinline__ double2 finish_sum(const float2 *__restrict__ part, int stride, int S, int lanes)
 {
-    float2 v = make_float2(0.f, 0.f);
-#pragma unroll 8
-    for (int s = threadIdx.x % lanes; s < S; s += lanes) v = cadd(v, part[s * stride]);
-    return lanes > 1 ? warp_sum(v) : v;
+    Sum2 v;
+#pragma unroll 4
+    for (int s = threadIdx.x % lanes; s < S; s += lanes) v.add(part[s * stride]);
+    if (lanes > 1)
+        for (int o = 16; o > 0; o >>= 1) {
+            const float2 t = make_float2(__shfl_xor_sync(0xffffffffu, v.s.x, o), __shfl_xor_sync(0xffffffffu, v.s.y, o));
+            const float2 u = make_float2(__shfl_xor_sync(0xffffffffu, v.e.x, o), __shfl_xor_sync(0xffffffffu, v.e.y, o));
+            v.add(t);
+            v.e = cadd(v.e, u);
+        }
+    return v.value_d();
 }
 
 // The S partial sums of each field point, plus the incident field.
@@ -2677,7 +2711,7 @@ __global__ void k_field_finish(const double *__restrict__ pts, int64_t M, int S,
 {
     const int64_t m = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lanes;
     if (m >= M) return;
-    const float2 v = finish_sum(part + m * S, 1, S, lanes);
+    const double2 v = finish_sum(part + m * S, 1, S, lanes);
     if (threadIdx.x % lanes > 0) return;
     const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
     double br = v.x, bi = v.y;
@@ -2770,7 +2804,7 @@ __global__ void k_field_velocity_finish(const double *__restrict__ pts, int64_t 
     if (m >= M) return;
     double gr[3], gi[3];
     for (int a = 0; a < 3; ++a) {
-        const float2 v = finish_sum(part + m * S * 3 + a, 3, S, lanes);
+        const double2 v = finish_sum(part + m * S * 3 + a, 3, S, lanes);
         gr[a] = v.x;
         gi[a] = v.y;
     }
