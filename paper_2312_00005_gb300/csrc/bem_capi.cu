@@ -222,6 +222,33 @@ void dev_malloc(void **p, size_t bytes)
     g_live_bytes += (int64_t)bytes;
 }
 
+// Host memory whose copies to the device have been queued, by stream: a copy
+// from pageable memory may read it after the call that queued it has returned,
+// so it is kept until the thread that queued it has waited for the stream.
+thread_local std::vector<std::pair<cudaStream_t, std::shared_ptr<const void>>> t_kept;
+
+void keep_until_wait(cudaStream_t s, std::shared_ptr<const void> v) { t_kept.emplace_back(s, std::move(v)); }
+
+void let_go(cudaStream_t s)
+{
+    t_kept.erase(std::remove_if(t_kept.begin(), t_kept.end(), [s](const auto &k) { return k.first == s; }),
+                 t_kept.end());
+}
+
+// Waits for the stream and lets go of what was kept for it.
+void wait_stream(cudaStream_t s, const char *what = "sync")
+{
+    ck(cudaStreamSynchronize(s), what);
+    let_go(s);
+}
+// The same where a call is given up: its copies from the caller's memory end
+// before it returns.
+void settle(cudaStream_t s)
+{
+    if (cudaStreamSynchronize(s) == cudaSuccess) let_go(s);
+    else (void)cudaGetLastError();
+}
+
 template <typename T>
 struct DevArr {
     T *p = nullptr;
@@ -253,7 +280,15 @@ struct DevArr {
         std::swap(n, o.n);
         std::swap(cap, o.cap);
     }
-    void upload(const std::vector<T> &v, cudaStream_t s)
+    // Copies of v, which is kept until the stream has been waited for, and of a
+    // vector that the caller holds that long.
+    void upload(std::vector<T> &&v, cudaStream_t s)
+    {
+        auto kept = std::make_shared<std::vector<T>>(std::move(v));
+        keep_until_wait(s, kept);
+        upload_held(*kept, s);
+    }
+    void upload_held(const std::vector<T> &v, cudaStream_t s)
     {
         alloc(v.size());
         if (!v.empty()) ck(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s), "H2D");
@@ -519,6 +554,8 @@ struct bem_mesh_impl {
     }
     ~bem_mesh_impl()
     {
+        for (cudaStream_t x : {s, s_setup})
+            if (x) settle(x);
         for (int t = 0; t < kStepsPerGraph; ++t) {
             if (ev_orth[t]) cudaEventDestroy(ev_orth[t]);
             if (ev_giv[t]) cudaEventDestroy(ev_giv[t]);
@@ -584,7 +621,7 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         leaf_start[t] = Lf.start[t];
         Ls->max_ncol = std::max(Ls->max_ncol, ncol[t]);
     }
-    Ls->leaf_start.upload(leaf_start, s);
+    Ls->leaf_start.upload(std::vector<int64_t>(leaf_start), s);
     {
         // disaggregation tasks: each leaf split into ranges of at most
         // kDisTask elements of nearly equal size, largest first
@@ -597,7 +634,7 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         }
         std::stable_sort(dt.begin(), dt.end(), [](int2 u, int2 v) { return u.y - u.x > v.y - v.x; });
         Ls->n_dis_tasks = (int)dt.size();
-        Ls->dis_tasks.upload(dt, s);
+        Ls->dis_tasks.upload(std::move(dt), s);
     }
     {
         // block-Jacobi sub-blocks: each leaf split into ceil(count / kBjMax)
@@ -615,15 +652,15 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         }
         if (off > INT_MAX) throw Fail{set_err(BEM_E_ARG, "block-Jacobi blocks exceed the 32-bit offset range")};
         Ls->bj_entries = off;
-        Ls->bj.upload(Ls->h_bj, s);
+        Ls->bj.upload_held(Ls->h_bj, s);
     }
     Ls->nnz = row_ptr[M.n];
     Ls->h_row_ptr = row_ptr;   // for the transposed product's rows, built when first needed
-    Ls->leaf_of.upload(leaf_of, s);
-    Ls->run_ptr.upload(run_ptr, s);
-    Ls->ncol.upload(ncol, s);
-    Ls->runs.upload(runs, s);
-    Ls->row_ptr.upload(row_ptr, s);
+    Ls->leaf_of.upload(std::move(leaf_of), s);
+    Ls->run_ptr.upload(std::move(run_ptr), s);
+    Ls->ncol.upload(std::vector<int>(ncol), s);
+    Ls->runs.upload(std::move(runs), s);
+    Ls->row_ptr.upload_held(Ls->h_row_ptr, s);
     {
         // at most `entries` values per item (and kSpmvMaxItemRows rows), a
         // leaf's rows split evenly
@@ -651,11 +688,11 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         ck(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, M.device), "attribute");
         const int64_t per_sm = row_ptr[M.n] > 2500 * M.n ? 8 : 4;
         const int64_t fine = std::max(kSpmvMinEntries, row_ptr[M.n] / (per_sm * nsm));
-        const std::vector<int4> items = cut(std::min(kSpmvItemEntries, fine)), multi = cut(kSpmvItemEntries);
+        std::vector<int4> items = cut(std::min(kSpmvItemEntries, fine)), multi = cut(kSpmvItemEntries);
         Ls->n_spmv_items = (int)items.size();
-        Ls->spmv_items.upload(items, s);
+        Ls->spmv_items.upload(std::move(items), s);
         Ls->n_multi_items = (int)multi.size();
-        Ls->multi_items.upload(multi, s);
+        Ls->multi_items.upload(std::move(multi), s);
         Ls->fused = fused_split(Lf.count, Ls->max_ncol);
         std::vector<int4> ft;
         for (int t = 0; t < nl; ++t) {
@@ -665,21 +702,19 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
                 ft.push_back(make_int4(t, (int)(a + cnt * q / nch), (int)(a + cnt * (q + 1) / nch), 0));
         }
         Ls->n_fused = (int)ft.size();
-        Ls->fused_tasks.upload(ft, s);
-        ck(cudaStreamSynchronize(s), "sync");   // items and ft are uploaded before they go
+        Ls->fused_tasks.upload(std::move(ft), s);
     }
     std::vector<AggTask> all_tasks;
     std::vector<int2> all_reds, all_targets;
     for (const FarLevel &FL : F.far) {
         const int lev_index = (int)Ls->lev.size();
         auto D = std::make_unique<ListsLevelDev>();
-        D->il_ptr.upload(FL.il_ptr, s);
-        D->il_src.upload(FL.il_src, s);
-        D->il_off.upload(FL.il_off, s);
-        D->offs.upload(FL.offsets, s);
+        D->il_ptr.upload_held(FL.il_ptr, s);
+        D->il_src.upload_held(FL.il_src, s);
+        D->il_off.upload_held(FL.il_off, s);
+        D->offs.upload_held(FL.offsets, s);
         std::vector<int> is_src(FL.nc, 0);
         for (int v : FL.il_src) is_src[v] = 1;
-        D->is_src.upload(is_src, s);
         // aggregation tasks: chunks of at most kAggChunk elements of each
         // source cluster, of nearly equal size (each plan expands them into
         // ranges of direction pairs for its expansion lengths)
@@ -708,10 +743,11 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
         D->ntasks = (int)tasks.size();
         D->nred = (int)red_c.size();
         D->nextra = extra;
-        D->tasks.upload(tasks, s);
-        D->red_ptr.upload(red_ptr, s);
-        D->red_c.upload(red_c, s);
         all_tasks.insert(all_tasks.end(), tasks.begin(), tasks.end());
+        D->is_src.upload(std::move(is_src), s);
+        D->tasks.upload(std::move(tasks), s);
+        D->red_ptr.upload(std::move(red_ptr), s);
+        D->red_c.upload(std::move(red_c), s);
         for (int q = 0; q < D->nred; ++q) all_reds.push_back(make_int2(lev_index, q));
         for (int c = 0; c < FL.nc; ++c)
             if (FL.il_ptr[c + 1] > FL.il_ptr[c]) all_targets.push_back(make_int2(lev_index, c));
@@ -720,13 +756,13 @@ std::shared_ptr<Lists> upload_lists(bem_mesh_impl &M, FreqPlan &&fp)
     Ls->n_tasks = (int)all_tasks.size();
     Ls->n_reds = (int)all_reds.size();
     Ls->n_targets = (int)all_targets.size();
-    Ls->h_tasks = all_tasks;
-    Ls->all_reds.upload(all_reds, s);
-    Ls->all_targets.upload(all_targets, s);
-    Ls->h_targets = all_targets;
+    Ls->h_tasks = std::move(all_tasks);
+    Ls->h_targets = std::move(all_targets);
+    Ls->all_reds.upload(std::move(all_reds), s);
+    Ls->all_targets.upload_held(Ls->h_targets, s);
     Ls->red_cnt.alloc(std::max(1, Ls->n_reds));
     ck(cudaMemsetAsync(Ls->red_cnt.p, 0, std::max(1, Ls->n_reds) * sizeof(unsigned int), s), "memset");
-    ck(cudaStreamSynchronize(s), "sync");
+    wait_stream(s);
     return Ls;
 }
 
@@ -749,10 +785,10 @@ const DepthDev *depth_data(bem_mesh_impl &M, int depth)
         dz[i] = make_float4((float)(L.z[3 * cc] - M.g.cen[3 * e]), (float)(L.z[3 * cc + 1] - M.g.cen[3 * e + 1]),
                             (float)(L.z[3 * cc + 2] - M.g.cen[3 * e + 2]), 0.f);
     }
-    D->cstart.upload(cst, fr(M).s);
-    D->dz.upload(dz, fr(M).s);
-    D->elem_cl.upload(ecl, fr(M).s);
-    ck(cudaStreamSynchronize(fr(M).s), "sync");
+    D->cstart.upload(std::move(cst), fr(M).s);
+    D->dz.upload(std::move(dz), fr(M).s);
+    D->elem_cl.upload(std::move(ecl), fr(M).s);
+    wait_stream(fr(M).s);
     const DepthDev *r = D.get();
     M.depth_dev[depth] = std::move(D);
     return r;
@@ -770,7 +806,7 @@ int level_L(const bem_mesh_impl &M, int depth, double k)
 void recycle_plan(bem_mesh_impl &M)
 {
     if (!fr(M).plan) return;
-    ck(cudaStreamSynchronize(fr(M).s), "sync");
+    wait_stream(fr(M).s);
     M.spare_val.swap(fr(M).plan->val);
     for (auto &L : fr(M).plan->lev) {
         for (DevArr<float2> *b : {&L->D, &L->M, &L->Lam, &L->ph}) {
@@ -822,8 +858,8 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
         std::vector<float4> dirs(D->nd);
         for (int q = 0; q < D->nd; ++q)
             dirs[q] = make_float4((float)sd[3 * q], (float)sd[3 * q + 1], (float)sd[3 * q + 2], (float)sw[q]);
-        D->dirs.upload(dirs, s);
-        D->dirs_d.upload(sd, s);
+        D->dirs.upload(std::move(dirs), s);
+        D->dirs_d.upload(std::move(sd), s);
         take_spare(M, D->D, (size_t)D->noff * D->nd);
         take_spare(M, D->M, (size_t)(D->nc + D->ll->nextra) * D->nd);
         take_spare(M, D->Lam, (size_t)D->nc * D->nd);
@@ -900,9 +936,9 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
                 u.p0 = p0;
                 at.push_back(u);
             }
-        P->agg_tasks.upload(at, s);
-        A.tasks = P->agg_tasks.p;
         A.ntasks = (int)at.size();
+        P->agg_tasks.upload(std::move(at), s);
+        A.tasks = P->agg_tasks.p;
         if (M.prm.far_precision == 1) {
             std::vector<AggTask> tt;
             for (const AggTask &t : P->lists->h_tasks)
@@ -911,8 +947,8 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
                     u.p0 = p0;
                     tt.push_back(u);
                 }
-            P->agg_tasks_tc.upload(tt, s);
             P->n_tc_tasks = (int)tt.size();
+            P->agg_tasks_tc.upload(std::move(tt), s);
         }
     }
     A.reds = P->lists->all_reds.p;
@@ -925,9 +961,9 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
         std::vector<int4> tg;
         for (const int2 &lt : P->lists->h_targets)
             for (int nu0 = 0; nu0 < P->lev[lt.x]->nd; nu0 += kTransferDirs) tg.push_back(make_int4(lt.x, lt.y, nu0, 0));
-        P->tgroups.upload(tg, s);
-        A.tgroups = P->tgroups.p;
         A.ntgroups = (int)tg.size();
+        P->tgroups.upload(std::move(tg), s);
+        A.tgroups = P->tgroups.p;
     }
     A.red_cnt = P->lists->red_cnt.p;
     for (size_t l = 0; l < P->lev.size(); ++l) {
@@ -936,7 +972,7 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
         A.lev[l].mplane = (int64_t)(P->lev[l]->nc + P->lev[l]->ll->nextra) * P->lev[l]->nd;
         A.lev[l].lplane = (int64_t)P->lev[l]->nc * P->lev[l]->nd;
     }
-    ck(cudaStreamSynchronize(s), "sync");
+    wait_stream(s);
 }
 
 void autotune_leaf_depth(bem_mesh_impl &M, double k);
@@ -1075,8 +1111,7 @@ void ensure_coeffs(bem_mesh_impl &M, double omega, double c, double rho, const d
     F.coef_key.clear();
     for (DevArr<float2> *a : {&F.cp, &F.cq, &F.cp0, &F.cq0, &F.z, &F.aq}) a->alloc(M.n);
     if (M.has_admi) {
-        std::vector<double> h(adm, adm + 2 * ((size_t)M.max_region + 1));
-        F.adm.upload(h, F.s);
+        F.adm.upload(std::vector<double>(adm, adm + 2 * ((size_t)M.max_region + 1)), F.s);
     }
     {
         KTimer kt_("k_coeffs", F.s);
@@ -1093,7 +1128,7 @@ void ensure_coeffs(bem_mesh_impl &M, double omega, double c, double rho, const d
 void check_err(bem_mesh_impl &M)
 {
     ck(cudaMemcpyAsync(fr(M).h_err, fr(M).err.p, sizeof(int), cudaMemcpyDeviceToHost, fr(M).s), "D2H err");
-    ck(cudaStreamSynchronize(fr(M).s), "sync");
+    wait_stream(fr(M).s);
     const int e = *fr(M).h_err;
     if (e != kNoErr) {
         char buf[160];
@@ -1111,7 +1146,7 @@ void check_tc_fault(bem_mesh_impl &M)
 {
     if (M.prm.far_precision != 1) return;
     ck(cudaMemcpyAsync(M.h_err + 2, M.tc_fault.p, sizeof(int), cudaMemcpyDeviceToHost, M.s), "D2H fault");
-    ck(cudaStreamSynchronize(M.s), "sync");
+    wait_stream(M.s);
     if (M.h_err[2]) {
         ck(cudaMemsetAsync(M.tc_fault.p, 0, sizeof(int), M.s), "memset");
         g_err = "tensor-core aggregation: the wait for the tensor cores gave up";
@@ -1149,21 +1184,21 @@ void store_near(bem_mesh_impl &M, Plan &P, const float2 *cp, const float2 *cq)
         ck_launch("k_near_classify");
         unsigned long long hk[kHeavyKinds], ho[kHeavyKinds];
         ck(cudaMemcpyAsync(hk, cnt.p, sizeof hk, cudaMemcpyDeviceToHost, fr(M).s), "D2H");
-        ck(cudaStreamSynchronize(fr(M).s), "sync");
+        wait_stream(fr(M).s);
         unsigned long long h = 0;
         for (int q = 0; q < kHeavyKinds; ++q) {
             ho[q] = h;
             h += hk[q];
         }
         Ls.heavy.alloc(std::max<unsigned long long>(h, 1));
-        ck(cudaMemcpyAsync(off.p, ho, sizeof ho, cudaMemcpyHostToDevice, fr(M).s), "H2D");
+        off.upload(std::vector<unsigned long long>(ho, ho + kHeavyKinds), fr(M).s);
         ck(cudaMemsetAsync(cnt.p, 0, kHeavyKinds * sizeof(unsigned long long), fr(M).s), "memset");
         {
             KTimer kt_("k_near_classify", fr(M).s);
             k_near_classify<<<nblocks(M.n, 8), 256, 0, fr(M).s>>>(a, Ls.heavy.p, cnt.p, off.p);
         }
         ck_launch("k_near_classify");
-        ck(cudaStreamSynchronize(fr(M).s), "sync");
+        wait_stream(fr(M).s);
         Ls.n_heavy = (int64_t)h;
     }
     {
@@ -1299,17 +1334,18 @@ void ensure_pairs(bem_mesh_impl &M)
                 q[q.size() - 2].y = lt.y;
             }
         }
+        std::vector<int> np;
         for (size_t l = 0; l < P.lev.size(); ++l) {
             ListsLevelDev &L = *Ls.lev[l];
-            L.pair.upload(pt[l], s);
+            np.push_back((int)(pt[l].size() / 2));
+            L.pair.upload(std::move(pt[l]), s);
             L.pair_ent.alloc(L.il_src.n);
-            if (!pt[l].empty())
-                k_pair_lists<<<(unsigned)(pt[l].size() / 2), 128, 0, s>>>(L.il_ptr.p, L.il_src.p, L.il_off.p, L.pair.p,
-                                                                    L.pair_ent.p);
+            if (np[l] > 0)
+                k_pair_lists<<<(unsigned)np[l], 128, 0, s>>>(L.il_ptr.p, L.il_src.p, L.il_off.p, L.pair.p, L.pair_ent.p);
         }
         ck_launch("k_pair_lists");
-        ck(cudaStreamSynchronize(s), "sync");
-        for (size_t l = 0; l < P.lev.size(); ++l) Ls.lev[l]->npairs = (int)(pt[l].size() / 2);
+        wait_stream(s);
+        for (size_t l = 0; l < P.lev.size(); ++l) Ls.lev[l]->npairs = np[l];
     }
     std::vector<int4> tp;
     for (size_t l = 0; l < P.lev.size(); ++l) {
@@ -1319,10 +1355,11 @@ void ensure_pairs(bem_mesh_impl &M)
         for (int g = 0; g < L.npairs; ++g)
             for (int nu0 = 0; nu0 < P.lev[l]->nd; nu0 += 32) tp.push_back(make_int4((int)l, g, nu0, 0));
     }
-    P.tpairs.upload(tp, s);
-    ck(cudaStreamSynchronize(s), "sync");
+    const int ntp = (int)tp.size();
+    P.tpairs.upload(std::move(tp), s);
+    wait_stream(s);
     P.hargs.tpairs = P.tpairs.p;
-    P.hargs.ntpairs = (int)tp.size();
+    P.hargs.ntpairs = ntp;
 }
 
 // Room for nr right-hand sides in the current plan's M and Lambda buffers
@@ -1541,11 +1578,11 @@ void ensure_transposed_rows(bem_mesh_impl &M)
         rptr[t + 1] = (int)ri.size();
     }
     cudaStream_t s = fr(M).s;
-    Ls.trow_ptr.upload(rptr, s);
-    Ls.h_trow_ptr = rptr;
-    Ls.trow_i.upload(ri, s);
-    Ls.trow_off.upload(roff, s);
-    ck(cudaStreamSynchronize(s), "sync");
+    Ls.h_trow_ptr = std::move(rptr);
+    Ls.trow_ptr.upload_held(Ls.h_trow_ptr, s);
+    Ls.trow_i.upload(std::move(ri), s);
+    Ls.trow_off.upload(std::move(roff), s);
+    wait_stream(s);
     Ls.tsym = true;
     Ls.trow_ready = true;
 }
@@ -1589,7 +1626,7 @@ void ensure_transposed_values(bem_mesh_impl &M)
                                             P.valT.p);
     }
     ck_launch("k_near_transpose");
-    ck(cudaStreamSynchronize(s), "sync");
+    wait_stream(s);
     P.valT_valid = true;
 }
 
@@ -1701,9 +1738,9 @@ void autotune_leaf_depth(bem_mesh_impl &M, double k)
     DevArr<float2> tcp, tcq, tx, ty;
     std::vector<float2> h1(n, make_float2(1.f, 0.f)), h0(n, make_float2(0.f, 0.f)), hx(n);
     for (int64_t i = 0; i < n; ++i) hx[i] = make_float2(std::cos(0.37 * i), std::sin(0.11 * i));
-    tcp.upload(h1, M.s);
-    tcq.upload(h0, M.s);
-    tx.upload(hx, M.s);
+    tcp.upload(std::move(h1), M.s);
+    tcq.upload(std::move(h0), M.s);
+    tx.upload(std::move(hx), M.s);
     ty.alloc(n);
     // events destroyed on every exit (a failed allocation throws from here)
     struct Events {
@@ -1857,7 +1894,7 @@ SourceDev *upload_sources(bem_mesh_impl &M, const bem_source *srcs, int n)
     };
     if (v.empty() || v.size() != M.src_key.size() || !std::equal(v.begin(), v.end(), M.src_key.begin(), same)) {
         M.src_key.clear();
-        M.srcbuf.upload(v, M.s);
+        M.srcbuf.upload(std::vector<SourceDev>(v), M.s);
         M.src_key.swap(v);
     }
     return M.srcbuf.p;
@@ -2136,12 +2173,19 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
             ty[i] = M->bct[j];
         }
         cudaStream_t s = M->s;
-        M->chi.upload(chi, s); M->clo.upload(clo, s); M->nrm.upload(nr, s);
-        M->va.upload(va, s); M->e1.upload(e1, s); M->e2.upload(e2, s);
-        M->cd.upload(cd, s); M->vad.upload(vad, s); M->e1d.upload(e1d, s); M->e2d.upload(e2d, s);
-        M->ad.upload(ad, s);
-        M->perm.upload(M->t.perm, s);
-        M->type.upload(ty, s);
+        M->chi.upload(std::move(chi), s);
+        M->clo.upload(std::move(clo), s);
+        M->nrm.upload(std::move(nr), s);
+        M->va.upload(std::move(va), s);
+        M->e1.upload(std::move(e1), s);
+        M->e2.upload(std::move(e2), s);
+        M->cd.upload(std::move(cd), s);
+        M->vad.upload(std::move(vad), s);
+        M->e1d.upload(std::move(e1d), s);
+        M->e2d.upload(std::move(e2d), s);
+        M->ad.upload(std::move(ad), s);
+        M->perm.upload_held(M->t.perm, s);
+        M->type.upload(std::move(ty), s);
         ck(cudaFuncSetAttribute(k_near_spmv_items, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024),
            "cudaFuncSetAttribute");
         ck(cudaFuncSetAttribute(k_near_spmv_items_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2158,8 +2202,7 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
         M->tc_fault.alloc(1);
         ck(cudaMemsetAsync(M->tc_fault.p, 0, sizeof(int), s), "memset");
 
-        std::vector<QuadTables> qt(1, make_tables(p));
-        M->Q.upload(qt, s);
+        M->Q.upload(std::vector<QuadTables>(1, make_tables(p)), s);
         {
             for (Frame *F : {&M->cur, &M->next}) {
                 F->err.alloc(1);
@@ -2180,11 +2223,10 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
                     M->max_region = std::max(M->max_region, rg[i]);
                 }
             }
-            M->bcv_d.upload(bv, s);
-            M->region_d.upload(rg, s);
-            ck(cudaStreamSynchronize(s), "sync");
+            M->bcv_d.upload(std::move(bv), s);
+            M->region_d.upload(std::move(rg), s);
         }
-        ck(cudaStreamSynchronize(s), "sync");
+        wait_stream(s);
         *out = M.release();
         return BEM_OK;
     } catch (Fail &f) {
@@ -2199,7 +2241,6 @@ int bem_mesh_destroy(void *mesh)
     if (!mesh) return set_err(BEM_E_ARG, "mesh is NULL");
     auto *M = (bem_mesh_impl *)mesh;
     cudaSetDevice(M->device);
-    if (M->s) cudaStreamSynchronize(M->s);
     delete M;
     return BEM_OK;
 }
@@ -2272,12 +2313,16 @@ int bem_matvec_host(void *mesh, double freq_hz, const bem_medium *medium, const 
         const size_t bytes = (size_t)M.n * n_rhs * sizeof(float2);
         ck(cudaMemcpyAsync(M.bvec.p, x_host, bytes, cudaMemcpyHostToDevice, us), "H2D x");
         int st = bem_matvec(mesh, freq_hz, medium, admittance, n_regions, M.bvec.p, M.uvec.p, n_rhs, stream);
-        if (st < 0) return st;
+        if (st < 0) {
+            settle(us);
+            return st;
+        }
         ck(cudaMemcpyAsync(y_host, M.uvec.p, bytes, cudaMemcpyDeviceToHost, us), "D2H y");
-        ck(cudaStreamSynchronize(us), "sync");
+        wait_stream(us);
         resolve_timing();
         return st;
     } catch (Fail &f) {
+        settle((cudaStream_t)stream);
         return f.code;
     }
 }
@@ -2354,7 +2399,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
             h.tol = tol;
             h.maxit = max_iter;
         }
-        ck(cudaMemcpyAsync(M.st.p, hs.data(), nr * sizeof(GmresState), cudaMemcpyHostToDevice, s), "H2D st");
+        M.st.upload(std::move(hs), s);
     }
     ck(cudaMemsetAsync(M.uvec.p, 0, (size_t)nr * n * sizeof(float2), s), "memset x");
     ck(cudaMemsetAsync(M.H.p, 0, M.H.bytes(), s), "memset H");
@@ -2541,7 +2586,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
         if (use_graph) {
             ck(cudaGraphLaunch(gexec, s), "graph launch");
             ck(cudaMemcpyAsync(M.h_st, M.st.p, nr * sizeof(GmresState), cudaMemcpyDeviceToHost, s), "D2H st");
-            ck(cudaStreamSynchronize(s), "sync st");
+            wait_stream(s, "sync st");
             g_launches.fetch_add(per_graph * (uint64_t)std::max(0, M.h_st[0].bodies));
             for (int r = 0; r < nr; ++r) R.hp[r] = M.h_st[r];
         } else {
@@ -2550,7 +2595,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
             for (int launched = 0; launched < max_graphs; ++launched) {
                 arnoldi_steps(1);
                 ck(cudaMemcpyAsync(M.h_st, M.st.p, nr * sizeof(GmresState), cudaMemcpyDeviceToHost, s), "D2H st");
-                ck(cudaStreamSynchronize(s), "sync st");
+                wait_stream(s, "sync st");
                 bool all_done = true;
                 for (int r = 0; r < nr; ++r) {
                     R.hp[r] = M.h_st[r];
@@ -2591,7 +2636,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
         start(M.w.p, 0);
         ck(cudaMemsetAsync(M.H.p, 0, M.H.bytes(), s), "memset H");
         ck(cudaMemcpyAsync(M.h_st, M.st.p, nr * sizeof(GmresState), cudaMemcpyDeviceToHost, s), "D2H st");
-        ck(cudaStreamSynchronize(s), "sync");
+        wait_stream(s);
         bool all_done = true;
         for (int r = 0; r < nr; ++r) all_done = all_done && M.h_st[r].done;
         if (all_done) {
@@ -2669,7 +2714,7 @@ GmresResult run_refined(bem_mesh_impl &M, double tol, int32_t max_iter, int nr)
             ck_launch("k_refine_residual");
         }
         ck(cudaMemcpyAsync(hp.data(), part.p, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H norms");
-        ck(cudaStreamSynchronize(s), "sync");
+        wait_stream(s);
         for (int r = 0; r < nr; ++r) {
             double v = 0.0;
             for (int q = 0; q < nparts; ++q) v += hp[(size_t)r * nparts + q];
@@ -2811,7 +2856,7 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
         // the preconditioned right-hand side (the refinement of a
         // mixed-precision solve preconditions each inner residual instead)
         if (M.prm.far_precision != 1) precondition_rhs(M, M.bvec.p, nr);
-        ck(cudaStreamSynchronize(s), "sync");
+        wait_stream(s);
         auto t_rhs = std::chrono::steady_clock::now();
         GmresResult R;
         {
@@ -2831,7 +2876,7 @@ int solve_frame(bem_mesh_impl &M, double freq_hz, const bem_medium *medium, cons
         }
         check_err(M);
         join_streams(M, s, us);
-        ck(cudaStreamSynchronize(us), "sync");
+        wait_stream(us);
         resolve_timing();
         bool all_conv = true;
         for (int r = 0; r < nr; ++r) all_conv = all_conv && R.conv[r];
@@ -2910,7 +2955,7 @@ int bem_solve(void *mesh, double freq_hz, const bem_medium *medium, const double
         cudaStream_t us = (cudaStream_t)stream;
         join_streams(M, us, M.s);
         prepare(M, freq_hz, medium, admittance, n_regions);
-        ck(cudaStreamSynchronize(M.s), "sync");
+        wait_stream(M.s);
         return solve_frame(M, freq_hz, medium, srcs, n_src, tol, max_iter, p_dev, q_dev, info, us, t0,
                            std::chrono::steady_clock::now());
     } catch (Fail &f) {
@@ -2932,7 +2977,7 @@ int bem_solve_multi(void *mesh, double freq_hz, const bem_medium *medium, const 
         cudaStream_t us = (cudaStream_t)stream;
         join_streams(M, us, M.s);
         prepare(M, freq_hz, medium, admittance, n_regions);
-        ck(cudaStreamSynchronize(M.s), "sync");
+        wait_stream(M.s);
         return solve_frame(M, freq_hz, medium, srcs, n_rhs, tol, max_iter, p_dev, q_dev, infos, us, t0,
                            std::chrono::steady_clock::now(), n_rhs);
     } catch (Fail &f) {
@@ -2962,7 +3007,7 @@ int bem_solve_sweep(void *mesh, const double *freqs_hz, int32_t n_freq, const be
         auto t0 = std::chrono::steady_clock::now();
         {
             prepare(M, freqs_hz[0], medium, admittance, n_regions);
-            ck(cudaStreamSynchronize(M.s), "sync");
+            wait_stream(M.s);
         }
         for (int32_t i = 0; i < n_freq; ++i) {
             auto t_setup = std::chrono::steady_clock::now();
@@ -2978,11 +3023,13 @@ int bem_solve_sweep(void *mesh, const double *freqs_hz, int32_t n_freq, const be
                     try {
                         ck(cudaSetDevice(M.device), "cudaSetDevice");
                         prepare(M, fn, medium, admittance, n_regions);
-                        ck(cudaStreamSynchronize(M.s_setup), "sync");
+                        wait_stream(M.s_setup);
                     } catch (Fail &f) {
                         next_code = f.code;
                         next_msg = g_err;
+                        settle(M.s_setup);
                     } catch (std::exception &e) {
+                        settle(M.s_setup);
                         next_code = BEM_E_INTERNAL;
                         next_msg = e.what();
                     }
@@ -3000,7 +3047,7 @@ int bem_solve_sweep(void *mesh, const double *freqs_hz, int32_t n_freq, const be
                                                 (float2 *)field_dev + (int64_t)i * n_pts, stream);
                     if (se < 0) throw Fail{se};
                 }
-                ck(cudaStreamSynchronize(us), "sync");
+                wait_stream(us);
             } catch (Fail &f) {
                 abandon_capture(M);
                 const std::string msg = g_err;
@@ -3047,7 +3094,9 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         !memcmp(pts, V.key_pts.data(), 3 * (size_t)np * sizeof(double)))
         return;
     V.valid = false;
-    EvalPlan ep;
+    const auto plan = std::make_shared<EvalPlan>();
+    keep_until_wait(s, plan);
+    EvalPlan &ep = *plan;
     const std::string msg = build_eval_plan(M.g, M.t, M.prm, k, M.leaf_depth, pts, np, kMaxTableL, ep);
     if (!msg.empty()) throw Fail{set_err(BEM_E_ARG, msg)};
     if ((int)ep.far.size() > kMaxFarLevels)
@@ -3056,13 +3105,12 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
     std::vector<double> hp(3 * (size_t)np);
     for (int64_t i = 0; i < np; ++i)
         for (int a = 0; a < 3; ++a) hp[3 * i + a] = pts[3 * ep.perm[i] + a];
-    V.pts.upload(hp, s);
-    V.perm.upload(ep.perm, s);
+    V.perm.upload_held(ep.perm, s);
     const int npl = (int)ep.leaf_start.size() - 1;
     std::vector<int> pleaf((size_t)np);
     for (int c = 0; c < npl; ++c)
         for (int64_t i = ep.leaf_start[c]; i < ep.leaf_start[c + 1]; ++i) pleaf[i] = c;
-    V.pleaf.upload(pleaf, s);
+    V.pleaf.upload(std::move(pleaf), s);
     const Level &EL = M.t.lv[ep.leaf_depth];
     std::vector<int> nptr(npl + 1, 0), ntot(npl, 0);
     std::vector<int2> nruns;                   // (first element, first position in the leaf's list)
@@ -3078,9 +3126,9 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         nptr[c + 1] = (int)nruns.size();
         ntot[c] = pos;
     }
-    V.ntot.upload(ntot, s);
-    V.nptr.upload(nptr, s);
-    V.nruns.upload(nruns, s);
+    V.ntot.upload(std::move(ntot), s);
+    V.nptr.upload(std::move(nptr), s);
+    V.nruns.upload(std::move(nruns), s);
     V.vnear.alloc(np);
     V.vall.alloc(np);
     V.np = np;
@@ -3115,20 +3163,20 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
             std::vector<float4> dirs(nd);
             for (int q2 = 0; q2 < nd; ++q2)
                 dirs[q2] = make_float4((float)sd[3 * q2], (float)sd[3 * q2 + 1], (float)sd[3 * q2 + 2], (float)sw[q2]);
-            Ld.dirs.upload(dirs, s);
-            Ld.dirs_d.upload(sd, s);
-            Ld.il_ptr.upload(F.il_ptr, s);
-            Ld.il_src.upload(F.il_src, s);
-            Ld.il_off.upload(F.il_off, s);
-            Ld.offs.upload(F.offsets, s);
-            Ld.pcl.upload(F.pcl, s);
+            Ld.dirs.upload(std::move(dirs), s);
+            Ld.dirs_d.upload(std::move(sd), s);
+            Ld.il_ptr.upload_held(F.il_ptr, s);
+            Ld.il_src.upload_held(F.il_src, s);
+            Ld.il_off.upload_held(F.il_off, s);
+            Ld.offs.upload_held(F.offsets, s);
+            Ld.pcl.upload_held(F.pcl, s);
             std::vector<float4> dzp((size_t)np);
             for (int64_t i = 0; i < np; ++i) {
                 const int c = F.pcl[i];
                 dzp[i] = make_float4((float)(F.zp[3 * c] - hp[3 * i]), (float)(F.zp[3 * c + 1] - hp[3 * i + 1]),
                                      (float)(F.zp[3 * c + 2] - hp[3 * i + 2]), 0.f);
             }
-            Ld.dzp.upload(dzp, s);
+            Ld.dzp.upload(std::move(dzp), s);
             // aggregation tasks over this level's source clusters: element
             // chunks of at most kAggChunk (split clusters summed by the last
             // block) times ranges of kAggThreads direction pairs
@@ -3158,8 +3206,9 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
             }
             for (size_t q2 = 0; q2 < red_c.size(); ++q2) reds.push_back(make_int2((int)l, (int)q2));
             Ld.nextra = extra;
-            Ld.red_ptr.upload(red_ptr, s);
-            Ld.red_c.upload(red_c, s);
+            const int nred = (int)red_c.size();
+            Ld.red_ptr.upload(std::move(red_ptr), s);
+            Ld.red_c.upload(std::move(red_c), s);
             Ld.Mx.alloc((size_t)(Ld.nc + extra) * nd);
             Ld.Lam.alloc((size_t)Ld.npc * nd);
             Ld.D.alloc((size_t)Ld.noff * nd);
@@ -3179,7 +3228,7 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
             f.k = (float)k;
             f.red_ptr = Ld.red_ptr.p;
             f.red_c = Ld.red_c.p;
-            f.nred = (int)red_c.size();
+            f.nred = nred;
             f.dirs = Ld.dirs.p;
             f.il_ptr = Ld.il_ptr.p;
             f.il_src = Ld.il_src.p;
@@ -3200,18 +3249,18 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         }
         ta.start[ta.nlev] = nb;
         A.nlev = (int)ep.far.size();
-        V.tasks.upload(tasks, s);
-        A.tasks = V.tasks.p;
         A.ntasks = (int)tasks.size();
-        V.reds.upload(reds, s);
-        A.reds = V.reds.p;
+        V.tasks.upload(std::move(tasks), s);
+        A.tasks = V.tasks.p;
         A.nreds = (int)reds.size();
-        V.red_cnt.alloc(std::max<size_t>(1, reds.size()));
-        ck(cudaMemsetAsync(V.red_cnt.p, 0, std::max<size_t>(1, reds.size()) * sizeof(unsigned int), s), "memset");
+        V.reds.upload(std::move(reds), s);
+        A.reds = V.reds.p;
+        V.red_cnt.alloc(std::max(1, A.nreds));
+        ck(cudaMemsetAsync(V.red_cnt.p, 0, std::max(1, A.nreds) * sizeof(unsigned int), s), "memset");
         A.red_cnt = V.red_cnt.p;
-        V.tgroups.upload(tg, s);
-        A.tgroups = V.tgroups.p;
         A.ntgroups = (int)tg.size();
+        V.tgroups.upload(std::move(tg), s);
+        A.tgroups = V.tgroups.p;
         if (nb > 0) {
             {
                 KTimer kt_("k_dtable", s);
@@ -3228,8 +3277,8 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
             for (int64_t q2 = 0; q2 < nch; ++q2)
                 dt.push_back(make_int2((int)(a + cnt * q2 / nch), (int)(a + cnt * (q2 + 1) / nch)));
         }
-        V.dtasks.upload(dt, s);
         V.n_dtasks = (int)dt.size();
+        V.dtasks.upload(std::move(dt), s);
         V.zeros.alloc(np);
         ck(cudaMemsetAsync(V.zeros.p, 0, np * sizeof(float4), s), "memset");
         da.n = np;
@@ -3240,7 +3289,8 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
         da.tasks = V.dtasks.p;
         da.rowf = nullptr;
     }
-    ck(cudaStreamSynchronize(s), "sync");   // the host vectors above are uploaded before they go
+    V.pts.upload(std::move(hp), s);
+    wait_stream(s);
     V.key_pts.assign(pts, pts + 3 * np);
     V.key_k = k;
     V.key_depth = M.leaf_depth;
@@ -3384,6 +3434,7 @@ int bem_evaluate(void *mesh, double freq_hz, const bem_medium *medium, const bem
         resolve_timing();
         return BEM_OK;
     } catch (Fail &f) {
+        settle(M.s);
         return f.code;
     }
 }
@@ -3444,6 +3495,7 @@ int bem_evaluate_velocity(void *mesh, double freq_hz, const bem_medium *medium, 
         resolve_timing();
         return BEM_OK;
     } catch (Fail &f) {
+        settle(M.s);
         return f.code;
     }
 }
@@ -3497,15 +3549,14 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         // (tau folded in as for the unknowns' coefficients)
         if (M.adjreg.n != (size_t)n) {
             // the same for every gradient of the mesh
-            std::vector<float2> h0((size_t)n, make_float2(0.f, 0.f)), hq((size_t)n, make_float2(tau, 0.f));
-            M.adj_cp.upload(h0, s);
-            M.adj_cq.upload(hq, s);
+            M.adj_cp.upload(std::vector<float2>((size_t)n, make_float2(0.f, 0.f)), s);
+            M.adj_cq.upload(std::vector<float2>((size_t)n, make_float2(tau, 0.f)), s);
             std::vector<int> reg((size_t)n);
             for (int64_t i = 0; i < n; ++i) {
                 const int64_t e = M.t.perm[i];
                 reg[i] = M.bct[e] == BEM_ADMI ? M.region[e] : -1;
             }
-            M.adjreg.upload(reg, s);
+            M.adjreg.upload(std::move(reg), s);
         }
         matvec_t_internal(M, M.adj_cp.p, M.adj_cq.p, M.uvec.p, M.w.p, false, false, nullptr, s);
         // per-region sums and the loss
@@ -3523,7 +3574,7 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         ck(cudaMemcpyAsync(hacc.data(), M.adjacc.p, nacc * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H acc");
         check_err(M);
         join_streams(M, s, us);
-        ck(cudaStreamSynchronize(s), "sync");
+        wait_stream(s);
         resolve_timing();
         *loss = hacc[2 * n_regions];
         for (int r = 0; r < 2 * n_regions; ++r) grad[r] = hacc[r];
@@ -3540,6 +3591,7 @@ int bem_admittance_gradient(void *mesh, double freq_hz, const bem_medium *medium
         return fwd;
     } catch (Fail &f) {
         abandon_capture(M);
+        settle(M.s);
         return f.code;
     }
 }
@@ -3613,7 +3665,7 @@ int bem_krylov_basis(void *mesh, int32_t plane, void *v_dev, int32_t max_cols, i
         if (!M.st.p || !M.V.p || plane < 0 || (size_t)(plane + 1) > M.st.n)
             return set_err(BEM_E_ARG, "no GMRES state for this right-hand side");
         ck(cudaSetDevice(M.device), "cudaSetDevice");
-        ck(cudaStreamSynchronize(M.s), "sync");
+        wait_stream(M.s);
         GmresState st;
         ck(cudaMemcpy(&st, M.st.p + plane, sizeof st, cudaMemcpyDeviceToHost), "D2H state");
         const int64_t n = M.n;
@@ -3724,7 +3776,7 @@ int bem_mesh_blocks(void *mesh, double freq_hz, const bem_medium *medium, int32_
         ck(cudaSetDevice(M.device), "cudaSetDevice");
         ensure_work(M);
         build_plan_dev(M, freq_hz, c);
-        ck(cudaStreamSynchronize(M.s), "sync");
+        wait_stream(M.s);
         const Lists &L = *fr(M).plan->lists;
         for (size_t b = 0; b < L.h_bj.size(); ++b) {
             const int4 B = L.h_bj[b];
@@ -3747,7 +3799,7 @@ int bem_mesh_stats(void *mesh, double freq_hz, const bem_medium *medium, bem_pla
         ck(cudaSetDevice(M.device), "cudaSetDevice");
         ensure_work(M);
         build_plan_dev(M, freq_hz, c);
-        ck(cudaStreamSynchronize(M.s), "sync");
+        wait_stream(M.s);
         Plan &P = *fr(M).plan;
         fill_stats(M.g, M.t, P.fp(), M.prm, out);
         for (size_t l = 0; l < P.lev.size() && l < 16; ++l) out->L[l] = P.lev[l]->L;
