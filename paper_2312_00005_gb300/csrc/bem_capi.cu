@@ -1922,9 +1922,23 @@ FusedSplit field_split(int64_t M_pts, int64_t n)
     return f;
 }
 
-// to waits for what from holds (the mesh's event is recorded anew each time)
+// to waits for what from holds.  The mesh's event, recorded anew each time,
+// serves the streams of its device; while another device is current, that
+// device's streams (its default stream above all) need an event of theirs.
 void join_streams(bem_mesh_impl &M, cudaStream_t from, cudaStream_t to)
 {
+    int dev = M.device;
+    if (from != M.s) ck(cudaGetDevice(&dev), "cudaGetDevice");
+    if (dev != M.device) {
+        cudaEvent_t ev;
+        ck(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
+        const bool theirs = cudaEventRecord(ev, from) == cudaSuccess;
+        const cudaError_t e = theirs ? cudaStreamWaitEvent(to, ev, 0) : cudaSuccess;
+        cudaEventDestroy(ev);
+        ck(e, "wait");
+        if (theirs) return;
+        (void)cudaGetLastError();   // a stream of the mesh's device
+    }
     ck(cudaEventRecord(M.ev_user, from), "record");
     ck(cudaStreamWaitEvent(to, M.ev_user, 0), "wait");
 }

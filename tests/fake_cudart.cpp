@@ -328,6 +328,11 @@ int main(int argc, char **argv)
         if (!m) return 1;
         if (what == "devices") {
             // the caller's current device is another one, the stream its default
+            // one or one of the mesh's device
+            cudaStream_t own;
+            cudaStreamCreateWithFlags(&own, 0);
+            cudaSetDevice(0);
+            ok("matvec", bem_matvec(m, 1000.0, nullptr, adm, 2, x.data(), y.data(), 1, own));
             cudaSetDevice(0);
             ok("matvec", bem_matvec(m, 1000.0, nullptr, adm, 2, x.data(), y.data(), 1, nullptr));
             cudaSetDevice(0);

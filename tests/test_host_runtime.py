@@ -1,7 +1,8 @@
 """The library's host code on a CUDA runtime without a GPU (fake_cudart.cpp):
 no host memory is freed while a queued copy has still to read it, through mesh
-creation, products, solves, sweeps, fields and gradients.  Linked from the
-objects of the build (built again where they are missing)."""
+creation, products, solves, sweeps, fields and gradients; and a handle of one
+device is usable while another device is current.  Linked from the objects of
+the build (built again where they are missing)."""
 import os
 import shutil
 import subprocess
@@ -41,3 +42,8 @@ def test_host_memory_outlives_its_copies(program, nu):
     r = subprocess.run([exe, "uploads", *files[nu]], capture_output=True, text=True, timeout=300)
     print(r.stdout)
     assert r.returncode == 0 and "errors 0, freed in flight 0" in r.stdout, (r.returncode, r.stdout, r.stderr[-1000:])
+
+def test_handle_of_another_device_than_the_current(program):
+    exe, files = program
+    r = subprocess.run([exe, "devices", *files[4]], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "errors 0" in r.stdout, (r.returncode, r.stdout, r.stderr[-1000:])
