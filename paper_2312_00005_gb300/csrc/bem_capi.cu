@@ -1219,6 +1219,14 @@ void store_near(bem_mesh_impl &M, Plan &P, const float2 *cp, const float2 *cq)
     check_err(M);
 }
 
+// Whether the near field of the current unknowns' product is recomputed (no
+// stored values, or a transposed product without the rows' mirror).
+bool near_recomputed(bem_mesh_impl &M, bool transposed)
+{
+    const Plan &P = *fr(M).plan;
+    return !M.prm.near_store || P.fp().direct || (transposed && !P.lists->trow_ready);
+}
+
 // Room for the column parts of a recomputed product with nr right-hand sides
 // (also before a graph capture, which may not allocate).
 void ensure_fused(bem_mesh_impl &M, int nr)
@@ -2371,7 +2379,7 @@ GmresResult run_gmres(bem_mesh_impl &M, double tol, int32_t max_iter, bool trans
     GmresResult R;
     if (transposed) M.rowf.alloc(n);   // before the Arnoldi steps are captured (no allocation in a capture)
     if (nr > 1) ensure_planes(M, nr);
-    ensure_fused(M, nr);
+    if (near_recomputed(M, transposed)) ensure_fused(M, nr);
     // GMRES workspace, nr planes of each
     const int64_t vplane = (int64_t)(m + 1) * n, hplane = (int64_t)(m + 1) * m;
     M.V.alloc((size_t)nr * vplane);
