@@ -411,23 +411,28 @@ def residual_vs_fp64(W, p, args, nrows=48):
     return {"fp64_residual_sampled_rows": float(np.linalg.norm(Ap - b) / np.linalg.norm(b)), "rows": nrows}
 
 
-# DRAM traffic of one k_near_spmv_items launch from an ncu capture of this
-# workload with the tree the timed run chooses (leaf depth 4):
-# dram__bytes_read.sum 288.65 MB + dram__bytes_write.sum 2.79 MB = 291.44 MB,
-# 1.013 x the algorithmic 287.7 MB, taken with
+# DRAM traffic of one k_near_spmv_items launch from ncu captures of this
+# workload with the tree the timed run chooses (leaf depth 4), taken with
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum \
 #       --clock-control none -k regex:k_near_spmv_items -s 45 -c 1 \
 #       python bench.py --steps 1 --warmup 3 --no-cpu-baseline --leaf-edge 0.0126
-# Valid only while the kernel's source and launch and the plan (near_nnz)
-# are the ones captured (the source hash below guards it).
+# "bytes": with items of 65,536 values, 288.65 + 2.79 MB; "items_bytes": with the
+# items of the present cut (1220 blocks), dram__bytes_read.sum 288.66 MB +
+# dram__bytes_write.sum 2.80 MB = 291.47 MB, 1.013 x the algorithmic 287.7 MB.
+# Each is valid only for the kernel's source and launch and the plan (near_nnz)
+# captured, the second also only for the cut (the hashes below guard them).
 SPMV_TRAFFIC = {"source_sha256": "072a1b81091cecf996027de780a3b1aa872908dd1618af338cd09a6791df839c",
-                "near_nnz": 35925668, "bytes": 291443712}
+                "near_nnz": 35925668, "bytes": 291443712,
+                "items_sha256": "c0873ef043113922b579aa433de79a0b7fb3b9da5ea17087a44b7fef12d4f975", "items_bytes": 291468800}
+
+
+def _csrc(name):
+    return open(os.path.join(ROOT, "paper_2312_00005_gb300", "csrc", name)).read()
 
 
 def _spmv_source_hash():
     import hashlib
-    src = open(os.path.join(ROOT, "paper_2312_00005_gb300", "csrc", "bem_kernels.cu")).read()
-    capi = open(os.path.join(ROOT, "paper_2312_00005_gb300", "csrc", "bem_capi.cu")).read()
+    src, capi = _csrc("bem_kernels.cu"), _csrc("bem_capi.cu")
     i0 = src.index("__device__ __forceinline__ float2 spmv_segment(")
     i1 = src.index("\n}\n", src.index("k_near_spmv_items(NearArgs a"))
     # the forward product's launches (the transposed product also streams
@@ -437,12 +442,34 @@ def _spmv_source_hash():
     return hashlib.sha256((src[i0:i1] + "\n".join(launch)).encode()).hexdigest()
 
 
+def _spmv_items_hash():
+    """Of what cuts the captured launch's items (upload_lists and its constants)."""
+    import hashlib
+    capi = _csrc("bem_capi.cu")
+    i0 = capi.index("auto cut = [&](int64_t entries)")
+    cut = [ln.split("//")[0].strip() for ln in capi[i0:capi.index("Ls->n_spmv_items", i0)].splitlines()]
+    const = [ln.split("//")[0].strip() for f in ("bem_capi.cu", "bem_kernels.cuh") for ln in _csrc(f).splitlines()
+             if "constexpr" in ln and "kSpmv" in ln]
+    return hashlib.sha256("\n".join(filter(None, cut + const)).encode()).hexdigest()
+
+
 def spmv_traffic(nnz):
     t = SPMV_TRAFFIC
     if t["bytes"] is None or t["near_nnz"] != nnz:
         return None
     try:
         return t["bytes"] if _spmv_source_hash() == t["source_sha256"] else None
+    except (OSError, ValueError):
+        return None
+
+
+def spmv_items_traffic(nnz):
+    """The traffic of the launch as it is cut now."""
+    t = SPMV_TRAFFIC
+    if spmv_traffic(nnz) is None:
+        return None
+    try:
+        return t["items_bytes"] if _spmv_items_hash() == t["items_sha256"] else None
     except (OSError, ValueError):
         return None
 
@@ -460,7 +487,7 @@ def roofline(kernels, stats, n, peaks, peak_src):
         byts = 8 * nnz + 16 * n
         ach = byts / avg_s / 1e9
         return {"kernel": name, "bound": "hbm", "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s",
-                "frac": round(ach / hbm, 4), "traffic": spmv_traffic(nnz), "algorithmic_bytes": byts,
+                "frac": round(ach / hbm, 4), "traffic": spmv_items_traffic(nnz), "algorithmic_bytes": byts,
                 "peak_source": peak_src}
     return {"kernel": name, "bound": None, "achieved": None, "peak": None, "unit": None, "frac": None,
             "traffic": None, "avg_us": kernels[name]["avg_us"], "peak_source": peak_src}
