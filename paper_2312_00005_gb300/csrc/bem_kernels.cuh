@@ -331,15 +331,18 @@ __global__ void k_transfer_split(const __grid_constant__ LevelsArgs A, const int
 // The same for 2 right-hand sides (M and Lambda planes mplane and lplane
 // apart): each D value is loaded once for both.  One block per half of a group
 // of directions; kTransferWarps warps per target, or one (s) from
-// kTransferManyBlocks blocks on, where the blocks alone fill the GPU.
-constexpr int kTransferManyBlocks = 20000;
+// kTransferManyBlocks blocks on, where the blocks alone fill the GPU (four warps
+// and one: 10,580 elements, 7900 blocks: 27.8 and 31.6 us; 20,480, 23,400: 80.4 and
+// 84.1; 28,880, 32,700: 105.4 and 106.9; 40,500, 36,000: 117.8 and 115.4; 81,920,
+// 93,300: 320 and 317; 158,420, 144,000: 577 and 578).
+constexpr int kTransferManyBlocks = 34000;
 __global__ void k_transfer_m2(const __grid_constant__ LevelsArgs A, const int *skip);
 __global__ void k_transfer_m2s(const __grid_constant__ LevelsArgs A, const int *skip);
 // For 4 right-hand sides: one block per pair of targets and 32 directions;
 // kTransferWarps warps, or kPairManyWarps (s) from kPairManyBlocks blocks on,
-// where the blocks alone fill the GPU (pairs with every source tested: 10,580
-// elements, 4,800 blocks: 43.2 us with four warps, 49.5 with two; 40,500, 17,400
-// blocks: 182 and 178; 158,420, 70,000 blocks: 855 and 827).
+// where the blocks alone fill the GPU (four warps and two: 10,580 elements, 3800
+// blocks: 43.0 and 47.2 us; 20,480, 11,600: 128.3 and 129.5; 28,880, 15,900: 168.3
+// and 164.0; 40,500, 17,400: 180 and 173; 158,420, 70,000: 842 and 796).
 constexpr int kPairManyBlocks = 12000;
 constexpr int kPairManyWarps = 2;
 __global__ void k_pair_lists(const int *il_ptr, const int *il_src, const int *il_off, int4 *pair, int4 *ent);
