@@ -923,8 +923,7 @@ void finish_plan(bem_mesh_impl &M, Plan &Pl)
             P->has_phases = true;
         }
     }
-    LevelsArgs &A = P->hargs;
-    memset(&A, 0, sizeof A);
+    LevelsArgs &A = P->hargs;                 // zeroed with the plan
     A.nlev = (int)P->lev.size();
     {
         // aggregation blocks for this plan's expansion lengths: every

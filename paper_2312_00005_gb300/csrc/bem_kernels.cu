@@ -895,8 +895,7 @@ __device__ __forceinline__ void add_entry(double2 *h, const float2 *__restrict__
 // tiles; with several parts, k_near_fused_sum adds them in order.  NR right-
 // hand sides share every entry.  One warp per row with lanes over the columns
 // (96 bytes of element data per pair through L1, all rules mixed in a warp)
-// took 721 us on 5120 elements; this takes 281 us (four blocks per SM; with
-// three 283, and 352 with half as many parts).
+// took 721 us on 5120 elements; this takes 254 us.
 // kT: the transposed product (the lists read backwards): a lane holds
 // column j, the rows i whose leaves are in the near list of j's own leaf are
 // staged, y_j = cp_j sum_i Kp_ij x_i + cq_j sum_i Kq_ij x_i.
@@ -3029,37 +3028,35 @@ __device__ void gm_givens_warp(const GmresArgs &a, double nn, int j)
 
 // ------------------------------------------------------------------ Gram-Schmidt
 // Classical Gram-Schmidt with selective reorthogonalisation (DGKS: a second
-// pass when ||w_1|| < 0.1 ||w||) for Arnoldi column j, in three launches with
-// no block ever waiting for another:
-//   k_gs_dots    w = (far + near part of A v_j); each block adds its partial
-//                dots V_l^H w into column j of H and its partial ||w||^2
-//                into acc (FP64 atomics);
+// pass when ||w_1|| < ||w|| / sqrt(2), gs_second_pass) for Arnoldi column j, in
+// three launches with no block ever waiting for another:
+//   k_gs_dots    v_j is scaled to unit norm (it was stored as it came; rnorm = 1 /
+//                ||v_j|| is k_gm_givens's of the step before) and so is w = far +
+//                near part of the product; each block adds its partial dots V_l^H
+//                w into column j of H and its partial ||w||^2 into acc (FP64
+//                atomics);
 //   k_gs_update  w_1 = w - V h and its partial ||w_1||^2; the DGKS test on
 //                the sums (||w_1||^2 = ||w||^2 - |h|^2 by Pythagoras; exact
-//                enough to decide, since the sums are) asks for a second pass
-//                rarely, and only then the block adds the dots V_l^H w_1;
+//                enough to decide, since the sums are), and where it asks for a
+//                second pass the block adds the dots V_l^H w_1;
 //   k_gs_finish  the decision read from the state (k_gs_update's block 0
-//                leaves it there); without a second pass v_{j+1} = w_1 /
-//                ||w_1|| and the next product's inputs; with one h_2 is
-//                added to column j of H, w_2 = w_1 - V h_2 and its partial
-//                ||w_2||^2 are formed, and the last block to finish (an
-//                arrival counter) forms v_{j+1} = w_2 / ||w_2|| for every
-//                row (second passes are rare).
+//                leaves it there); without a second pass w_1 is v_{j+1}; with one
+//                h_2 is added to column j of H and w_2 = w_1 - V h_2, with its
+//                partial ||w_2||^2, is.  Every block stores its rows of v_{j+1},
+//                unnormalised, and the next product's inputs (gs_store).
 // Every norm is summed from the vector itself, never estimated (when w_1 is
 // mostly rounding noise inside span(V), ||w_1||^2 - |h_2|^2 would cancel to
 // nothing and fake a breakdown of the Arnoldi process).
 // Every block of k_gs_update takes the same decision from the same FP64
-// sums.  Block b owns
-// rows [b R, b R + R) of every vector (R about 64: the basis comes from HBM,
-// since each product streams the stored near field through L2, so many
-// blocks keep many loads in flight), with FP32 sums within a block.  The
+// sums.  Block b owns rows [b R, b R + R) of every vector (R 64 or 128: the basis
+// comes from HBM, since each product streams the stored near field through L2, so
+// many blocks keep many loads in flight), with FP32 sums within a block.  The
 // FP64 sums of the blocks' FP32 partials are exact whenever the partials span
 // fewer than 29 binary orders of magnitude, so they do not depend on the
-// order in which the blocks add them.  acc ([4]: ||w||^2, ||w_1||^2,
-// ||w_2||^2, arrival counter) and h2 alternate between two copies by the
-// parity of j: the normalising block clears the copy of step j + 1
-// (k_gm_start clears both at the start of a cycle, where H is cleared too).
-// The Givens step (k_gm_givens) follows on a side stream.
+// order in which the blocks add them.  acc ([4]: ||w||^2, ||w_1||^2, ||w_2||^2,
+// unused) and h2 alternate between two copies by the parity of j: step j clears
+// the copy of step j + 1 (k_gm_start clears both at the start of a cycle, where H
+// is cleared too).  The Givens step (k_gm_givens) follows on a side stream.
 __device__ __forceinline__ int gs_rows(const GsArgs &a, int64_t &r0)
 {
     r0 = (int64_t)blockIdx.x * a.rows;

@@ -46,7 +46,6 @@ struct GmresState {
     double bnorm, beta, resid, tol, hn;
     int reorth;              // second Gram-Schmidt pass needed for the current column
     int n_reorth;            // columns that needed it
-    int fault;               // unused (kept zero)
     float rnorm;             // 1 / ||v_{j+1}||, for k_gs_dots (its FP64 root and division off every block's path)
     // Skip flag of the product kernels: a copy of done taken by k_gs_dots
     // (in stream order before the next product).  done itself is set by
@@ -448,7 +447,7 @@ struct GsArgs {
     GmresArgs g;             // g.nblk = gridDim.x
     PrepArgs next;           // inputs of the next product, formed from V_{j+1}
     const float2 *wnear;     // near-field part of the product (g.w holds the far part)
-    double *acc;             // [2][4] per parity of j: ||w||^2, ||w_1||^2, ||w_2||^2, arrival counter
+    double *acc;             // [2][4] per parity of j: ||w||^2, ||w_1||^2, ||w_2||^2, unused
     double2 *h2;             // [2][m + 1] per parity of j: second-pass dots V^H w_1
     int rows;                // rows of the basis per block
 };

@@ -324,7 +324,8 @@ double auto_leaf_edge(const Geometry &g, const bem_params &p)
 }
 
 // Blocks enough for several rounds of four per SM, and whole tiles in each part
-// (5120 elements: 20 parts of one tile 283 us, 10 of two 352 us).
+// (5120 elements: 20 parts of one tile 283 us, 10 of two 352 us, before the
+// queues were worked off part by part without a second cut).
 int fused_parts(int64_t ntasks, int64_t max_ncol)
 {
     const int64_t ntile = (max_ncol + kFusedTile - 1) / kFusedTile;

@@ -40,6 +40,8 @@ def _state(bem, nu, m, radius, **kw):
 @pytest.mark.parametrize("nu,m,radius,kw", [
     (1, 1, 0.101, {}), (2, 5, 0.101, {}), (2, 32, 0.13, {}), (4, 33, 0.3, {}), (4, 200, 0.1005, {}), (9, 4, 0.101, {}),
     (9, 65, 0.101, {}), (4, 100, 0.101, {"quad_tol": 1e-6}), (4, 100, 0.102, {"m_max": 2}), (16, 700, 0.1002, {}),
+    # full blocks in which most pairs are expensive: more than the queue holds
+    (4, 6000, 0.13, {"quad_tol": 1e-6}),
 ])
 def test_points_at_the_surface_match_oracle(bem, nu, m, radius, kw):
     nodes, tris, p, q, pts, mesh = _state(bem, nu, m, radius, **kw)
