@@ -463,6 +463,7 @@ struct EvalDev {
     DevArr<unsigned int> red_cnt;
     DevArr<int4> tgroups;
     DevArr<int> pleaf, nptr, ntot;
+    DevArr<int> close;            // points with expensive near pairs: their number, then the points
     DevArr<double> pts;
     DevArr<int64_t> perm;
     DevArr<float4> wts, zeros;
@@ -3151,6 +3152,7 @@ void field_fmm_plan(bem_mesh_impl &M, double k, const double *pts, int64_t np, c
     V.nptr.upload(std::move(nptr), s);
     V.nruns.upload(std::move(nruns), s);
     V.vnear.alloc(np);
+    V.close.alloc(1 + (size_t)np);
     V.vall.alloc(np);
     V.np = np;
     V.npl = npl;
@@ -3356,13 +3358,20 @@ void field_fmm(bem_mesh_impl &M, double k, const double *pts, int64_t np, const 
             ck_launch("k_aggregate");
         }
     }
+    ck(cudaMemsetAsync(V.close.p, 0, sizeof(int), s), "memset");
     {
         KTimer kt_("k_field_near", s);
         k_field_near<<<(unsigned)np, 32 * kFieldNearWarps, 0, s>>>(M.elem(), M.Q.p, V.pts.p, (float)k, p, q, V.pleaf.p,
-                                                                   V.nptr.p, V.ntot.p, V.nruns.p, V.vnear.p,
-                                                                   fr(M).err.p);
+                                                                   V.nptr.p, V.ntot.p, V.nruns.p, V.vnear.p, V.close.p);
     }
     ck_launch("k_field_near");
+    {
+        KTimer kt_("k_field_near_close", s);
+        k_field_near_close<<<(unsigned)std::min<int64_t>(np, kFieldCloseBlocks), 32 * kFieldNearWarps, 0, s>>>(
+            M.elem(), M.Q.p, V.pts.p, (float)k, p, q, V.pleaf.p, V.nptr.p, V.ntot.p, V.nruns.p, V.vnear.p, V.close.p,
+            fr(M).err.p);
+    }
+    ck_launch("k_field_near_close");
     const float2 *vres = V.vnear.p;
     if (V.far) {
         if (V.A.ntgroups > 0) {

@@ -768,18 +768,18 @@ __device__ __forceinline__ float4 rule_point(const QuadTables &Q, int v)
 }
 constexpr int kCutKept = 96;                             // codes of a pair that its thread keeps (else cut again)
 constexpr int kPartBytes = kFusedParts * 10;           // the parts of a block's queued pairs, in shared memory
-// A block's nq queued pairs, kFusedThreads at a time: cut into parts
+// A block's nq queued pairs, kThreads (its threads) at a time: cut into parts
 // (cut(pair, out, cap): their number, and the first cap codes), the parts sorted
 // by order, integrated part by part (part(pair, code)); pairs whose parts
 // found no room go into another round, pairs that cannot be cut are taken whole
-// (whole(pair)).  Called by the whole block; buf: kPartBytes of shared memory,
-// pn: 8 counters.
-template <class Cut, class Part, class Whole>
+// (whole(pair)).  Called by the whole block; buf: 10 kParts bytes of shared
+// memory, pn: 8 counters.
+template <int kThreads, int kParts, class Cut, class Part, class Whole>
 __device__ __forceinline__ void work_queue(int nq, unsigned char *buf, int *pn, Cut cut, Part part, Whole whole)
 {
     int *pq = reinterpret_cast<int *>(buf);                        // part: its pair
-    unsigned *pc = reinterpret_cast<unsigned *>(pq + kFusedParts); // ... its code
-    unsigned short *po = reinterpret_cast<unsigned short *>(pc + kFusedParts);   // parts by order
+    unsigned *pc = reinterpret_cast<unsigned *>(pq + kParts); // ... its code
+    unsigned short *po = reinterpret_cast<unsigned short *>(pc + kParts);   // parts by order
     int q = threadIdx.x, np = -1;                      // this thread's next pair and its parts (-1: not counted)
     unsigned codes[kCutKept];
     while (__syncthreads_or(q < nq)) {
@@ -787,28 +787,28 @@ __device__ __forceinline__ void work_queue(int nq, unsigned char *buf, int *pn, 
         __syncthreads();
         if (q < nq) {
             if (np < 0) np = cut(q, codes, kCutKept);
-            if (np > 0 && np <= kFusedParts) {
+            if (np > 0 && np <= kParts) {
                 const int at = atomicAdd(&pn[0], np);
-                if (at + np <= kFusedParts) {
+                if (at + np <= kParts) {
                     if (np > kCutKept) cut(q, pc + at, np);
                     for (int u = at; u < at + np; ++u) {
                         if (np <= kCutKept) pc[u] = codes[u - at];
                         pq[u] = q;
                         atomicAdd(&pn[(pc[u] >> 24) & 7], 1);
                     }
-                    q += kFusedThreads;
+                    q += kThreads;
                     np = -1;
                 } else {
-                    for (int u = at; u < min(at + np, kFusedParts); ++u) pc[u] = 0;   // order 0: no part
+                    for (int u = at; u < min(at + np, kParts); ++u) pc[u] = 0;   // order 0: no part
                 }
             } else {
                 whole(q);
-                q += kFusedThreads;
+                q += kThreads;
                 np = -1;
             }
         }
         __syncthreads();
-        const int n_all = min(pn[0], kFusedParts);
+        const int n_all = min(pn[0], kParts);
         int start[8];                                  // first slot of an order: the longest first
         start[7] = 0;
         start[6] = 0;
@@ -818,7 +818,7 @@ __device__ __forceinline__ void work_queue(int nq, unsigned char *buf, int *pn, 
         __syncthreads();
         if (threadIdx.x < 8) pn[threadIdx.x] = 0;
         __syncthreads();
-        for (int u = threadIdx.x; u < n_all; u += kFusedThreads) {
+        for (int u = threadIdx.x; u < n_all; u += kThreads) {
             const int m = (pc[u] >> 24) & 7;
             if (m == 0) continue;
             int at = start[1];
@@ -828,7 +828,7 @@ __device__ __forceinline__ void work_queue(int nq, unsigned char *buf, int *pn, 
             po[at + atomicAdd(&pn[m], 1)] = (unsigned short)u;
         }
         __syncthreads();
-        for (int u = threadIdx.x; u < n_parts; u += kFusedThreads) part(pq[po[u]], pc[po[u]]);
+        for (int u = threadIdx.x; u < n_parts; u += kThreads) part(pq[po[u]], pc[po[u]]);
     }
     __syncthreads();
 }
@@ -981,7 +981,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
     auto drain = [&]() {
         auto row_of = [&](int q) { return kT ? (int64_t)s_qj[q] : e0 + s_qr[q]; };
         auto col_of = [&](int q) { return kT ? e0 + s_qr[q] : (int64_t)s_qj[q]; };
-        work_queue(
+        work_queue<kFusedThreads, kFusedParts>(
             min(s_qn, kFusedQueue), s_buf, s_pn,
             [&](int q, unsigned *out, int cap) { return cut_pair(a, row_of(q), col_of(q), out, cap); },
             [&](int q, unsigned code) {
@@ -2528,7 +2528,7 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
                 atomicAdd(&s_h[a][row].y, (double)v[a].y);
             }
         };
-        work_queue(
+        work_queue<kFusedThreads, kFusedParts>(
             min(s_qn, kFieldQueue), s_buf, s_pn,
             [&](int q, unsigned *out, int cap) { return cut_point(E, Q, s_qj[q], s_x[s_qr[q]], out, cap); },
             [&](int q, unsigned code) {
@@ -2733,48 +2733,168 @@ __global__ void k_field_weights(int64_t n, const float2 *__restrict__ p, const f
     wts[i] = make_float4(-A * qv.x, -A * qv.y, k * A * pv.y, -k * A * pv.x);
 }
 
+// Rule of the pair of a point and an element: 1 to 3 where one regular rule of
+// that order serves the whole element, else 0, an expensive pair (thresholds on
+// r~^2 as in the recomputed product; FP64 within rounding of R_1 and R_2).
+__device__ __forceinline__ int light_rule(const ElemDev &E, const QuadTables &Q, int j, float3 D0, float area, float rt2,
+                                          const double *xd)
+{
+    if (rt2 > fmaxf(Q.R2[1] * (1.0f + 2e-5f), Q.whole_rt2)) return 1;
+    if (!(rt2 > (Q.m_max > 3 ? Q.heavy_rt2 : Q.whole_rt2))) return 0;
+    if (rt2 < Q.R2[1] * (1.0f - 2e-5f)) {
+        if (rt2 > Q.R2[2] * (1.0f + 2e-5f)) return 2;
+        if (rt2 < Q.R2[2] * (1.0f - 2e-5f)) return 3;
+    }
+    const int code = whole_rule(E, j, D0, area, xd, Q);
+    return code <= 3 ? code : 0;
+}
 // Near part of the field at points (internal point order): the element rules
-// of the direct sum over the point's leaf near list, one warp per point; v_m =
-// sum_j H_j p_j - G_j q_j.  The list's runs (first element, first position)
-// are walked by position, so that all lanes have an element whatever the
-// runs' lengths (a run is often a leaf of a dozen elements).  kFieldNearWarps
-// warps share a point: the points nearest to the surface have lists many times
-// the mean, and set the kernel's length (24,874 points, one warp each 74 us,
-// four 46).
-__global__ void k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, float k,
-                             const float2 *__restrict__ p, const float2 *__restrict__ q,
-                             const int *__restrict__ pleaf, const int *__restrict__ nptr, const int *__restrict__ ntot,
-                             const int2 *__restrict__ nruns, float2 *__restrict__ v, int *err)
+// of the direct sum over the point's leaf near list, kFieldNearWarps warps per
+// point; v_m = sum_j H_j p_j - G_j q_j.  The list's runs (first element, first
+// position) are walked by position, so that all lanes have an element whatever
+// the runs' lengths (a run is often a leaf of a dozen elements).  The pairs of
+// orders 1 to 3 here, with few registers and one barrier, since most points have
+// no others; the points close to the surface are listed in close (their number
+// first) for k_field_near_close.  24,874 points around 20,480 elements: 35 us, and
+// 6 for the empty second launch (all rules in one kernel, 92 registers: 43; one
+// warp per point 74).
+__global__ void __launch_bounds__(32 * kFieldNearWarps)
+k_field_near(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, float k,
+             const float2 *__restrict__ p, const float2 *__restrict__ q, const int *__restrict__ pleaf,
+             const int *__restrict__ nptr, const int *__restrict__ ntot, const int2 *__restrict__ nruns,
+             float2 *__restrict__ v, int *__restrict__ close)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t m = blockIdx.x;
-    const QuadTables &Q = *Qp;
-    const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
-    const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
-    const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
-                                   (float)(xd[2] - (double)xhi.z));
     const int pl = pleaf[m], tot = ntot[pl], r1 = nptr[pl + 1];
-    int r = nptr[pl];
+    if (tot == 0) {                                    // far from every element
+        if (threadIdx.x == 0) v[m] = make_float2(0.f, 0.f);
+        return;
+    }
     float2 acc = make_float2(0.f, 0.f);
-    for (int c = threadIdx.x; c < tot; c += 32 * kFieldNearWarps) {
-        while (r + 1 < r1 && nruns[r + 1].y <= c) ++r;
-        const int2 run = nruns[r];
-        const int64_t j = run.x + (c - run.y);
-        float2 G = make_float2(0.f, 0.f), H = make_float2(0.f, 0.f);
-        if (!integrate_regular<true>(E, j, xhi, xlo, xd, make_float3(0.f, 0.f, 1.f), k, 1.0f / k, Q, G, H)) {
-            atomicMin(err, (int)j);
-            continue;
+    bool expensive = false;
+    if ((int)threadIdx.x < tot) {                      // (the point's FP64 conversions are most of a short list)
+        const QuadTables &Q = *Qp;
+        const double xd[3] = {pts[3 * m], pts[3 * m + 1], pts[3 * m + 2]};
+        const float3 xhi = make_float3((float)xd[0], (float)xd[1], (float)xd[2]);
+        const float3 xlo = make_float3((float)(xd[0] - (double)xhi.x), (float)(xd[1] - (double)xhi.y),
+                                       (float)(xd[2] - (double)xhi.z));
+        int r = nptr[pl];
+        for (int c = threadIdx.x; c < tot; c += 32 * kFieldNearWarps) {
+            while (r + 1 < r1 && nruns[r + 1].y <= c) ++r;
+            const int2 run = nruns[r];
+            const int j = run.x + (c - run.y);
+            const float4 h = E.chi[j];
+            const float3 ny = f3(E.nrm[j]);
+            float3 D0;
+            const float rt2 = pair_rt2(f3(h), f3(E.clo[j]), xhi, xlo, __frcp_rn(h.w), D0);
+            const int code = light_rule(E, Q, j, D0, h.w, rt2, xd);
+            FieldPair<false> f(k);
+            if (code == 1) {
+                f.acc.point(D0, ny, h.w);
+            } else if (code > 1) {
+                const float3 g1 = f3(E.e1[j]), g2 = f3(E.e2[j]), base = add3(D0, f3(E.va[j]));
+                for (int u = 0; u < code * code; ++u)
+                    f.acc.point(mad3(Q.tri_eta[code][u], g2, mad3(Q.tri_xi[code][u], g1, base)), ny,
+                                2.0f * h.w * Q.tri_w[code][u]);
+            } else {
+                expensive = true;
+            }
+            f.add(&acc, p[j], q[j]);
         }
-        acc = cadd(acc, csub(cmul(H, p[j]), cmul(G, q[j])));
     }
     __shared__ float2 red[kFieldNearWarps];
     acc = warp_sum(acc);
     if (lane == 0) red[warp] = acc;
-    __syncthreads();
+    const bool any = __syncthreads_or(expensive);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int w = 1; w < kFieldNearWarps; ++w) acc = cadd(acc, red[w]);
         v[m] = acc;
+        if (any) close[1 + atomicAdd(close, 1)] = (int)m;
+    }
+}
+
+// The expensive pairs of the listed points, added to v: a block goes over a
+// point's list again, queues them and works them off part by part (work_queue).
+// 5000 points a millimetre off 1280 elements: 630 us a call (lanes that took such
+// a pair whole, as the general rule does: 957).
+__global__ void __launch_bounds__(32 * kFieldNearWarps, 5)
+k_field_near_close(ElemDev E, const QuadTables *__restrict__ Qp, const double *__restrict__ pts, float k,
+                   const float2 *__restrict__ p, const float2 *__restrict__ q, const int *__restrict__ pleaf,
+                   const int *__restrict__ nptr, const int *__restrict__ ntot, const int2 *__restrict__ nruns,
+                   float2 *__restrict__ v, const int *__restrict__ close, int *err)
+{
+    constexpr int kT = 32 * kFieldNearWarps;
+    static_assert(kFieldNearQueue >= 4 * kT, "two passes of pushes find room above the half");
+    __shared__ __align__(16) unsigned char s_buf[10 * kFieldNearParts];
+    __shared__ float4 s_rule[91];                      // (xi, eta, 2 w) of orders 1 to 6
+    __shared__ int s_qj[kFieldNearQueue], s_qn, s_pn[8];
+    __shared__ double s_x[3];
+    __shared__ double2 s_h;
+    const QuadTables &Q = *Qp;
+    const int n = *close;
+    if (blockIdx.x >= n) return;
+    if (threadIdx.x < 91) s_rule[threadIdx.x] = rule_point(Q, threadIdx.x);
+    auto add = [&](float2 u) {
+        atomicAdd(&s_h.x, (double)u.x);
+        atomicAdd(&s_h.y, (double)u.y);
+    };
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+        const int m = close[1 + i];
+        __syncthreads();                               // the point before has been written
+        if (threadIdx.x < 3) s_x[threadIdx.x] = pts[3 * (int64_t)m + threadIdx.x];
+        if (threadIdx.x == 0) {
+            s_qn = 0;
+            s_h = make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+        const int pl = pleaf[m], tot = ntot[pl], r1 = nptr[pl + 1];
+        const float3 xhi = make_float3((float)s_x[0], (float)s_x[1], (float)s_x[2]);
+        const float3 xlo = make_float3((float)(s_x[0] - (double)xhi.x), (float)(s_x[1] - (double)xhi.y),
+                                       (float)(s_x[2] - (double)xhi.z));
+        int r = nptr[pl];
+        bool half = false;                             // this thread queued a pair beyond half of the queue
+        for (int c0 = 0, pass = 1; c0 < tot; c0 += kT, ++pass) {
+            const int c = c0 + threadIdx.x;
+            if (c < tot) {
+                while (r + 1 < r1 && nruns[r + 1].y <= c) ++r;
+                const int2 run = nruns[r];
+                const int j = run.x + (c - run.y);
+                const float4 h = E.chi[j];
+                float3 D0;
+                const float rt2 = pair_rt2(f3(h), f3(E.clo[j]), xhi, xlo, __frcp_rn(h.w), D0);
+                if (light_rule(E, Q, j, D0, h.w, rt2, s_x) == 0) {
+                    const int slot = atomicAdd(&s_qn, 1);
+                    s_qj[slot] = j;
+                    half = half || slot >= kFieldNearQueue / 2;
+                }
+            }
+            // a barrier every second pass
+            const bool last = c0 + kT >= tot;
+            if (!last && (pass & 1)) continue;
+            if (!__syncthreads_or(half) && !last) continue;
+            work_queue<kT, kFieldNearParts>(
+                s_qn, s_buf, s_pn, [&](int u, unsigned *out, int cap) { return cut_point(E, Q, s_qj[u], s_x, out, cap); },
+                [&](int u, unsigned code) {
+                    float2 w;
+                    field_part<false>(E, s_qj[u], s_x, code, s_rule, k, p[s_qj[u]], q[s_qj[u]], &w);
+                    add(w);
+                },
+                [&](int u) {                           // cut deeper than a code can say
+                    float2 w;
+                    if (field_entry<false>(E, Q, s_qj[u], s_x, k, p[s_qj[u]], q[s_qj[u]], &w)) add(w);
+                    else atomicMin(err, s_qj[u]);
+                });
+            if (threadIdx.x == 0) s_qn = 0;
+            half = false;
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            Sum2 t(s_h);
+            t.add(v[m]);
+            v[m] = t.value();
+        }
     }
 }
 

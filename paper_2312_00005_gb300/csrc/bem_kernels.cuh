@@ -399,10 +399,16 @@ __global__ void k_coeffs(int64_t n, const int *type, const double2 *bcv, const i
                          float2 *z, float2 *aq);
 // FMM evaluation of the field at points (see the definitions)
 constexpr int kFieldNearWarps = 4;     // warps per point
+constexpr int kFieldCloseBlocks = 760; // blocks of the close points' kernel: five per SM
+constexpr int kFieldNearQueue = 512;   // expensive pairs queued per point
+constexpr int kFieldNearParts = 1024;  // ... and their parts, per pass over the queue
 __global__ void k_field_weights(int64_t n, const float2 *p, const float2 *q, const float4 *chi, float k, float4 *wts);
 __global__ void k_field_near(ElemDev E, const QuadTables *Q, const double *pts, float k, const float2 *p,
                              const float2 *q, const int *pleaf, const int *nptr, const int *ntot, const int2 *nruns,
-                             float2 *v, int *err);
+                             float2 *v, int *close);
+__global__ void k_field_near_close(ElemDev E, const QuadTables *Q, const double *pts, float k, const float2 *p,
+                                   const float2 *q, const int *pleaf, const int *nptr, const int *ntot,
+                                   const int2 *nruns, float2 *v, const int *close, int *err);
 __global__ void k_field_eval_finish(const double *pts, int64_t M, float k, float tau, const SourceDev *src, int nsrc,
                                     const float2 *v, const int64_t *perm, float2 *out);
 
