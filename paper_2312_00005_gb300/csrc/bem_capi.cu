@@ -1474,8 +1474,11 @@ void matvec_internal(bem_mesh_impl &M, const float2 *cp, const float2 *cq, bool 
         const int cw = std::max(2, std::min(ncp, M.prm.near_chunk > 0 ? M.prm.near_chunk : kSpmvMultiChunk));
         if (P.lists->n_multi_items > 0) {
             KTimer kt_("k_near_spmv", s);
-            k_near_spmv_items_multi<<<P.lists->n_multi_items, kSpmvMultiThreads, (size_t)nr * cw * sizeof(float2), s>>>(
-                na, P.lists->multi_items.p, P.val.p, M.xint.p, M.ynear.p, nr, n, cw, skip);
+            const bool chosen = M.prm.near_chunk > 0;
+            auto product = chosen ? k_near_spmv_items_multi_s : k_near_spmv_items_multi;
+            product<<<P.lists->n_multi_items, chosen ? kChunkThreads : kSpmvMultiThreads,
+                      (size_t)nr * cw * sizeof(float2), s>>>(na, P.lists->multi_items.p, P.val.p, M.xint.p, M.ynear.p, nr,
+                                                             n, cw, skip);
         }
         ck_launch("k_near_spmv");
     } else if (use_store && M.prm.near_store && !P.fp().direct) {
@@ -2210,9 +2213,10 @@ int bem_mesh_create(const double *nodes, int64_t n_nodes, const int32_t *tris, i
         M->type.upload(std::move(ty), s);
         ck(cudaFuncSetAttribute(k_near_spmv_items, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024),
            "cudaFuncSetAttribute");
-        ck(cudaFuncSetAttribute(k_near_spmv_items_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(kMaxPlanes * 4096 * sizeof(float2))),
-           "cudaFuncSetAttribute");
+        for (auto product : {k_near_spmv_items_multi, k_near_spmv_items_multi_s})
+            ck(cudaFuncSetAttribute(product, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kMaxPlanes * 4096 * sizeof(float2))),
+               "cudaFuncSetAttribute");
 
         ck(cudaFuncSetAttribute(k_gm_backsolve, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kBacksolveCols * (kBacksolveCols + 1) / 2 * (int)sizeof(double2)),

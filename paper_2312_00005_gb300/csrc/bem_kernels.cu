@@ -577,15 +577,13 @@ __device__ __forceinline__ void spmv_segment_multi(const float2 *__restrict__ v,
     for (int r = 0; r < kMaxPlanes; ++r) out[r] = warp_sum(cadd(acc0[r], acc1[r]));
 }
 
-__global__ void __launch_bounds__(kSpmvMultiThreads) k_near_spmv_items_multi(NearArgs a, const int4 *__restrict__ items,
-                                                                        const float2 *__restrict__ val,
-                                                                        const float2 *__restrict__ x,
-                                                                        float2 *__restrict__ y, int nr, int64_t plane,
-                                                                        int cw, const int *skip)
+template <int kThreads>
+__device__ __forceinline__ void spmv_items_multi_body(const NearArgs &a, const int4 *__restrict__ items,
+                                                      const float2 *__restrict__ val, const float2 *__restrict__ x,
+                                                      float2 *__restrict__ y, int nr, int64_t plane, int cw)
 {
-    if (skip_now(skip)) return;
     extern __shared__ float2 xs[];            // [nr][cw]: one chunk of the leaf's columns
-    constexpr int kW = kSpmvMultiThreads / 32;
+    constexpr int kW = kThreads / 32;
     __shared__ float2 part[kMaxPlanes][kSpmvMaxItemRows][kW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 W = items[blockIdx.x];
@@ -593,7 +591,7 @@ __global__ void __launch_bounds__(kSpmvMultiThreads) k_near_spmv_items_multi(Nea
     const int nc = a.N.ncol[t];
     const int ncp = (nc + 1) & ~1;
     const int run0 = a.N.run_ptr[t], run1 = a.N.run_ptr[t + 1];
-    for (int q = threadIdx.x; q < kMaxPlanes * kSpmvMaxItemRows * kW; q += kSpmvMultiThreads)
+    for (int q = threadIdx.x; q < kMaxPlanes * kSpmvMaxItemRows * kW; q += kThreads)
         (&part[0][0][0])[q] = make_float2(0.f, 0.f);
     const int64_t i0 = a.N.leaf_start[t] + W.y;
     const int nrow = min(W.z - W.y, kSpmvMaxItemRows);
@@ -631,7 +629,7 @@ __global__ void __launch_bounds__(kSpmvMultiThreads) k_near_spmv_items_multi(Nea
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < nrow * nr; q += kSpmvMultiThreads) {
+    for (int q = threadIdx.x; q < nrow * nr; q += kThreads) {
         const int row = q % nrow, pl = q / nrow;
         float2 sum = part[pl][row][0];
 #pragma unroll
@@ -639,6 +637,18 @@ __global__ void __launch_bounds__(kSpmvMultiThreads) k_near_spmv_items_multi(Nea
         y[pl * plane + i0 + row] = sum;
     }
 }
+
+#define BEM_SPMV_MULTI_KERNEL(NAME, THREADS)                                                                          \
+    __global__ void __launch_bounds__(THREADS)                                                                       \
+        NAME(NearArgs a, const int4 *__restrict__ items, const float2 *__restrict__ val, const float2 *__restrict__ x, \
+             float2 *__restrict__ y, int nr, int64_t plane, int cw, const int *skip)                                 \
+    {                                                                                                                 \
+        if (skip_now(skip)) return;                                                                                   \
+        spmv_items_multi_body<THREADS>(a, items, val, x, y, nr, plane, cw);                                           \
+    }
+BEM_SPMV_MULTI_KERNEL(k_near_spmv_items_multi, kSpmvMultiThreads)
+BEM_SPMV_MULTI_KERNEL(k_near_spmv_items_multi_s, kChunkThreads)
+#undef BEM_SPMV_MULTI_KERNEL
 
 // ------------------------------------------------------------------ recomputed near field
 // Kp and / or Kq of bm_point at one quadrature point (needp, needq uniform

@@ -211,11 +211,17 @@ __global__ void k_near_transpose(const int64_t *leaf_start, const int *trow_ptr,
 // Eight warps share a chunk of 1024 (four planes: 71 us on 10,580 elements,
 // 594 on 158,420); with four warps and 512 the block waits more often for its
 // columns (102 and 602 us), larger chunks leave too few blocks on an SM beside
-// the far-field kernels (alone 64 us, but 10 % slower GMRES steps).
+// the far-field kernels (alone 64 us, but 10 % slower GMRES steps).  Four warps (s)
+// with a chunk of the caller's choice, mostly a smaller one (256 columns and one
+// plane: 167 us and 231 with eight on 20,480 elements, 216 and 251 on 40,500, 102
+// and 96 on 10,580).
 constexpr int kSpmvMultiChunk = 1024;
 constexpr int kSpmvMultiThreads = 256;
+constexpr int kChunkThreads = 128;
 __global__ void k_near_spmv_items_multi(NearArgs a, const int4 *items, const float2 *val, const float2 *x, float2 *y,
                                         int nr, int64_t plane, int cw, const int *skip);
+__global__ void k_near_spmv_items_multi_s(NearArgs a, const int4 *items, const float2 *val, const float2 *x, float2 *y,
+                                          int nr, int64_t plane, int cw, const int *skip);
 // Near-field product with recomputed entries for 1, 2 or 4 right-hand sides
 // (planes n apart in x and out) and its transpose: blocks of tasks (leaf,
 // first row, end row; at most kFusedRows rows; tasks null: one leaf holds
