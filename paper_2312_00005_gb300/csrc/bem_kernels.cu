@@ -1029,7 +1029,7 @@ __device__ __forceinline__ void near_fused_body(const NearArgs &a, const int4 *_
         // every thread: no pushes since the barrier)
         for (;;) {
             const bool full = __syncthreads_or(pend != 0);
-            if (!full && tile < te && s_qn <= kFusedQueue / 2) break;
+            if (!full && (tile < te ? s_qn <= kFusedQueue / 2 : s_qn == 0)) break;
             drain();
             __syncthreads();
             if (!full) break;
@@ -2473,8 +2473,10 @@ __device__ __forceinline__ void field_part(const ElemDev &E, int64_t j, const do
 // Direct sum over every element at M points: p (k_field) or v (k_field_
 // velocity).  Bound by FP32 / SFU issue.  As in the recomputed product, a lane
 // holds a point, the elements are staged in shared memory in tiles of `cols`
-// and read as broadcasts, and the pairs under one rule of order 1 to 3 are
-// evaluated in place; the others (subdivided elements, orders 4 to 6, distances
+// and read as broadcasts (their vertices, which order 1 does not need, from
+// global memory: staged, far points took 4 % longer and points at the surface 3 %
+// less), and the pairs under one rule of order 1 to 3 are evaluated in place; the
+// others (subdivided elements, orders 4 to 6, distances
 // within rounding of a threshold) are queued per block and worked off as there
 // (work_queue), their sums FP64 additions.  Block (x, y) takes `rows` points and every gridDim.y-th part of
 // the elements; with several parts they go to part[(m S + s) N + a] and the
@@ -2494,10 +2496,10 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
 {
     constexpr int kW = kFusedThreads / 32, kN = FieldPair<kGrad>::kN;
     // the staged tile, and afterwards the parts of the queued pairs
-    constexpr int kTileBytes = 7 * kFusedTile * 16;
-    __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
+    constexpr int kTileBytes = 4 * kFusedTile * 16;
+    __shared__ __align__(16) unsigned char s_buf[kTileBytes > 10 * kFieldParts ? kTileBytes : 10 * kFieldParts];
     float4 *s_hi = reinterpret_cast<float4 *>(s_buf), *s_lo = s_hi + kFusedTile, *s_n = s_lo + kFusedTile;
-    float4 *s_pq = s_n + kFusedTile, *s_va = s_pq + kFusedTile, *s_e1 = s_va + kFusedTile, *s_e2 = s_e1 + kFusedTile;
+    float4 *s_pq = s_n + kFusedTile;
     __shared__ float4 s_rule[91];                      // (xi, eta, 2 w) of orders 1 to 6
     __shared__ int s_pn[8];
     __shared__ int s_qj[kFieldQueue];
@@ -2538,7 +2540,7 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
                 atomicAdd(&s_h[a][row].y, (double)v[a].y);
             }
         };
-        work_queue<kFusedThreads, kFusedParts>(
+        work_queue<kFusedThreads, kFieldParts>(
             min(s_qn, kFieldQueue), s_buf, s_pn,
             [&](int q, unsigned *out, int cap) { return cut_point(E, Q, s_qj[q], s_x[s_qr[q]], out, cap); },
             [&](int q, unsigned code) {
@@ -2565,7 +2567,7 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
         // pushes since the barrier)
         for (;;) {
             const bool full = __syncthreads_or(pend != 0);
-            if (!full && tile < te && s_qn <= kFieldQueue / 2) break;
+            if (!full && (tile < te ? s_qn <= kFieldQueue / 2 : s_qn == 0)) break;
             drain();
             __syncthreads();
             if (!full) break;
@@ -2587,9 +2589,6 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
             s_hi[threadIdx.x] = h;
             s_lo[threadIdx.x] = l;
             s_n[threadIdx.x] = E.nrm[j];
-            s_va[threadIdx.x] = E.va[j];
-            s_e1[threadIdx.x] = E.e1[j];
-            s_e2[threadIdx.x] = E.e2[j];
             s_pq[threadIdx.x] = make_float4(pj.x, pj.y, qj.x, qj.y);
         }
         __syncthreads();
@@ -2622,7 +2621,8 @@ __device__ __forceinline__ void field_body(const ElemDev &E, const QuadTables &Q
             if (code == 1) {
                 f.acc.point(D0, ny, eh.w);
             } else {
-                const float3 g1 = f3(s_e1[c]), g2 = f3(s_e2[c]), base = add3(D0, f3(s_va[c]));
+                const int64_t je = tile * cols + c;
+                const float3 g1 = f3(E.e1[je]), g2 = f3(E.e2[je]), base = add3(D0, f3(E.va[je]));
                 const int u1 = code == 2 ? 5 : 14;
                 for (int u = code == 2 ? 1 : 5; u < u1; ++u) {
                     const float4 rl = s_rule[u];

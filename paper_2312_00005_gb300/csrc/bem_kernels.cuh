@@ -231,8 +231,13 @@ __global__ void k_near_spmv_items_multi_s(NearArgs a, const int4 *items, const f
 // cols and parts.
 constexpr int kFusedThreads = 256;
 constexpr int kFusedQueue = 1024;        // expensive pairs queued per block
-constexpr int kFieldQueue = 2048;        // near pairs of field points queued per block
-constexpr int kFusedParts = 2560;        // ... and their parts under one rule, per kFusedThreads pairs
+constexpr int kFusedParts = 2560;        // ... and their parts under one rule, per pass over the queue
+// The same for the direct field: with 25 kB of shared memory a block (1600 parts)
+// a call of 50 to 1000 far points takes 62 to 86 us on 1280 and 5120 elements, with
+// 40 kB (2560 and a queue of 2048) 66 to 90, by the SMs' change of carve-out
+// between the call's kernels.
+constexpr int kFieldQueue = 1024;
+constexpr int kFieldParts = 1600;
 __global__ void k_near_fused_1(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
                                int *err, const int *skip);
 __global__ void k_near_fused_2(NearArgs a, const int4 *tasks, int rows, int cols, const float2 *x, float2 *out,
